@@ -469,7 +469,7 @@ __device__ __forceinline__ void batch_body(const BArgs& A, unsigned char* smem, 
       for (int i = blockIdx.x; i < n; i += gridDim.x) {
         if (!in_cycle(A.st, i, c)) continue;
         const BInst& I = A.inst[i];
-        tiles::coarse_levels_block<float, 2, true, double>(I.cl, I.L[I.lc].b, I.L[I.lc].u, I.inv64, smem);
+        tiles::coarse_levels_block<float, true, double>(I.cl, I.L[I.lc].b, I.L[I.lc].u, I.inv64, smem, false);
       }
       if (!grid_barrier(A.bar, A.err, A.extra_arrivals, A.spin_limit)) return;
       for (int l = A.LC - 1; l >= 0; --l) {
@@ -537,7 +537,8 @@ size_t batch_smem(const std::vector<csff_plan*>& plans) {
   size_t s = std::max(tiles::down_smem_elems<16>(ng, false), tiles::up_smem_elems<16>(ng, false));
   for (csff_plan* P : plans) {
     int lc = P->fused_lc;
-    s = std::max(s, tiles::coarse_levels_elems(P->lv, lc));
+    const size_t c = tiles::coarse_block_bytes(P->lv, lc, sizeof(float2), sizeof(double2), false);
+    s = std::max(s, (c + sizeof(float2) - 1) / sizeof(float2));
   }
   return s * sizeof(float2);
 }

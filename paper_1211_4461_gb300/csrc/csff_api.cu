@@ -391,7 +391,7 @@ csff_status run_fused_from(csff_plan* P, int l0, cx<T>* u, const cx<T>* b, bool 
     const cx<T>* bl = (l == l0) ? b : bbuf<T>(F);
     CK(csff::launch_down2<T>(F, C, in, zero_init || l > l0, bl, tbuf<T>(F), bbuf<T>(C), s, l == 0), "fused down");
   }
-  CK(csff::launch_coarse_levels<T>(P->dim, P->lv, lc, cinv<T>(P), coarse_fp64(P) ? P->coarse_inv : nullptr,
+  CK(csff::launch_coarse_levels<T>(P->lv, lc, cinv<T>(P), coarse_fp64(P) ? P->coarse_inv : nullptr,
                                    bbuf<T>(P->lv[lc]), ubuf<T>(P->lv[lc]), s),
      "coarse levels");
   for (int l = lc - 1; l >= l0; --l) {
@@ -899,8 +899,8 @@ csff_status csff_plan_create(const csff_problem* prob, const csff_opts* opts, vo
     for (int l = 0; l < (int)P->lv.size(); ++l)
       if (P->lv[l].n <= 33) { lc = l; break; }
     if (lc < 0) lc = (int)P->lv.size() - 1;
-    if (lc >= 1 && csff::coarse_levels_smem(d, P->lv, lc, 8) <= 200 * 1024) {
-      cudaError_t e = csff::prepare_fused(d, P->lv, lc);
+    if (lc >= 1 && csff::coarse_block_fits(P->lv, lc)) {
+      cudaError_t e = csff::prepare_fused();
       if (e != cudaSuccess) return fail(csff::cuda_fail(e, "fused kernel attributes"));
       P->fused_lc = lc;
     }

@@ -310,7 +310,8 @@ cudaError_t launch_gmres_step(int dim, const Level& L, int m, cx<T>* u, const cx
                               double2* part, int part_cap, GmState* S, cudaStream_t s);
 
 // ---- fused 2D V(1,1) RB-GS kernels (mg_fused.cu) ----------------------------
-size_t coarse_levels_smem(int dim, const std::vector<Level>& lv, int lc, int real_bytes);
+// whether the levels from lc on may run in the one-CTA block
+bool coarse_block_fits(const std::vector<Level>& lv, int lc);
 // finest: the launch works on the plan's finest level (a profiling family of its own)
 template <typename T>
 cudaError_t launch_down2(const Level& F, const Level& Cl, const cx<T>* u_in, bool zero_init, const cx<T>* b,
@@ -321,10 +322,10 @@ cudaError_t launch_up2(const Level& F, const Level& Cl, const cx<T>* u_in, const
 // inv64 (FP32 cycles only, may be null): the FP64 inverse, applied in FP64
 // to the coarsest right-hand side in place of inv
 template <typename T>
-cudaError_t launch_coarse_levels(int dim, const std::vector<Level>& lv, int lc, const cx<T>* inv,
-                                 const double2* inv64, const cx<T>* b, cx<T>* u, cudaStream_t s);
+cudaError_t launch_coarse_levels(const std::vector<Level>& lv, int lc, const cx<T>* inv, const double2* inv64,
+                                 const cx<T>* b, cx<T>* u, cudaStream_t s);
 // dynamic shared-memory opt-in of the fused kernels on the current device
-cudaError_t prepare_fused(int dim, const std::vector<Level>& lv, int lc);
+cudaError_t prepare_fused();
 // true while a graph is being captured (profiling brackets are suppressed)
 extern thread_local bool g_capturing;
 // kernel families currently timed (csff_prof_begin mask)

@@ -45,12 +45,13 @@ __global__ void __launch_bounds__(NT, tile_min_ctas<T, TC>()) k_up2(const cx<T>*
   tiles::up_tile<T, TC, false, G1>(blockIdx.x * TC, blockIdx.y * TC, u_in, ec, b, K, c, m, mc, u_out, smem_raw);
 }
 
-template <typename T, int D, typename TI = T>
-__global__ void __launch_bounds__(1024) k_coarse_levels(CoarseLevels L, const cx<T>* __restrict__ b_top,
-                                                        cx<T>* __restrict__ u_top, const cx<TI>* __restrict__ inv) {
-  extern __shared__ unsigned char smem_raw[];
-  pdl_prologue();
-  tiles::coarse_levels_block<T, D, false, TI>(L, b_top, u_top, inv, smem_raw);
+template <typename T, typename TI = T>
+__global__ void __launch_bounds__(tiles::COARSE_NT, 1) k_coarse_levels(CoarseLevels L, const cx<T>* __restrict__ b_top,
+                                                                    cx<T>* __restrict__ u_top,
+                                                                    const cx<TI>* __restrict__ inv, int staged) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  // the block waits for its predecessor itself, after its table copies
+  tiles::coarse_levels_block<T, false, TI>(L, b_top, u_top, inv, smem_raw, staged != 0);
 }
 
 template <typename T> const cx<T>* qt(const Level& L);
@@ -146,41 +147,43 @@ cudaError_t launch_up2(const Level& F, const Level& Cl, const cx<T>* u_in, const
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-size_t coarse_levels_smem(int dim, const std::vector<Level>& lv, int lc, int real_bytes) {
-  return tiles::coarse_levels_elems(lv, lc) * 2 * real_bytes;
+bool coarse_block_fits(const std::vector<Level>& lv, int lc) {
+  size_t n = 0;
+  for (size_t l = lc; l < lv.size(); ++l) n += (size_t)lv[l].N;
+  return n * 5 * sizeof(double2) <= 200 * 1024;
 }
 
 template <typename T>
-cudaError_t launch_coarse_levels(int dim, const std::vector<Level>& lv, int lc, const cx<T>* inv,
-                                 const double2* inv64, const cx<T>* b, cx<T>* u, cudaStream_t s) {
+cudaError_t launch_coarse_levels(const std::vector<Level>& lv, int lc, const cx<T>* inv, const double2* inv64,
+                                 const cx<T>* b, cx<T>* u, cudaStream_t s) {
   CoarseLevels L{};
   L.nl = (int)lv.size() - lc;
   if (L.nl > 8 || L.nl < 1) return cudaErrorInvalidValue;
   for (int i = 0; i < L.nl; ++i) {
     const Level& v = lv[lc + i];
+    if (i < L.nl - 1 && v.m > 2 * tiles::COARSE_ROW - 1) return cudaErrorInvalidValue;
     L.m[i] = v.m;
     L.q[i] = qt<T>(v);
     L.dinv[i] = dt<T>(v);
     L.c[i] = v.c;
     L.c32[i] = make_float2((float)v.c.x, (float)v.c.y);
   }
-  size_t sm = coarse_levels_smem(dim, lv, lc, sizeof(T));
+  const bool wide = sizeof(T) == 4 && inv64;
+  const size_t el = sizeof(cx<T>), ei = wide ? sizeof(double2) : el;
+  const bool st = tiles::coarse_inv_staged(lv, lc, el, ei);
+  const size_t sm = tiles::coarse_block_bytes(lv, lc, el, ei, st);
+  const dim3 nt(tiles::COARSE_NT);
   ProfScope ps(mg_family<T>(), s, (double)sizeof(cx<T>) * 2.0 * lv[lc].N, 0);
   cudaError_t e;
-  if (sizeof(T) == 4 && inv64)
-    e = (dim == 2) ? launch_pdl(k_coarse_levels<T, 2, double>, dim3(1), dim3(1024), sm, s, L, b, u, inv64)
-                   : launch_pdl(k_coarse_levels<T, 3, double>, dim3(1), dim3(1024), sm, s, L, b, u, inv64);
-  else
-    e = (dim == 2) ? launch_pdl(k_coarse_levels<T, 2>, dim3(1), dim3(1024), sm, s, L, b, u, inv)
-                   : launch_pdl(k_coarse_levels<T, 3>, dim3(1), dim3(1024), sm, s, L, b, u, inv);
+  if (wide) e = launch_pdl(k_coarse_levels<T, double>, dim3(1), nt, sm, s, L, b, u, inv64, (int)st);
+  else e = launch_pdl(k_coarse_levels<T>, dim3(1), nt, sm, s, L, b, u, inv, (int)st);
   count_launch();
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 // Opt the fused kernels into the dynamic shared memory they need (done at plan
-// creation on the plan's device; the coarse-level kernel gets the plan's size
-// or the largest size set so far, whichever is larger).
-cudaError_t prepare_fused(int dim, const std::vector<Level>& lv, int lc) {
+// creation on the plan's device).
+cudaError_t prepare_fused() {
   const int kMax = 227 * 1024;
   cudaError_t e;
   // the tiles stay below the default 48 KB (FP64: no factor windows; FP32:
@@ -195,21 +198,10 @@ cudaError_t prepare_fused(int dim, const std::vector<Level>& lv, int lc) {
                     tiles::down_smem_elems<8>(0, true) * 16 <= 48 * 1024 &&
                     tiles::up_smem_elems<8>(0, true) * 16 <= 48 * 1024,
                 "fused tile shared memory");
-  size_t s8 = coarse_levels_smem(dim, lv, lc, 8);
-  if (s8 > (size_t)kMax) return cudaErrorInvalidValue;
-  if (dim == 2) {
-    if ((e = cudaFuncSetAttribute(k_coarse_levels<float, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMax)) ||
-        (e = cudaFuncSetAttribute(k_coarse_levels<float, 2, double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  kMax)) ||
-        (e = cudaFuncSetAttribute(k_coarse_levels<double, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMax)))
-      return e;
-  } else {
-    if ((e = cudaFuncSetAttribute(k_coarse_levels<float, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMax)) ||
-        (e = cudaFuncSetAttribute(k_coarse_levels<float, 3, double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  kMax)) ||
-        (e = cudaFuncSetAttribute(k_coarse_levels<double, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMax)))
-      return e;
-  }
+  if ((e = cudaFuncSetAttribute(k_coarse_levels<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMax)) ||
+      (e = cudaFuncSetAttribute(k_coarse_levels<float, double>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMax)) ||
+      (e = cudaFuncSetAttribute(k_coarse_levels<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMax)))
+    return e;
   return cudaSuccess;
 }
 
@@ -218,8 +210,8 @@ cudaError_t prepare_fused(int dim, const std::vector<Level>& lv, int lc) {
                                        cx<T>*, cudaStream_t, bool);                                        \
   template cudaError_t launch_up2<T>(const Level&, const Level&, const cx<T>*, const cx<T>*, const cx<T>*,   \
                                      cx<T>*, cudaStream_t, bool);                                          \
-  template cudaError_t launch_coarse_levels<T>(int, const std::vector<Level>&, int, const cx<T>*,           \
-                                               const double2*, const cx<T>*, cx<T>*, cudaStream_t);
+  template cudaError_t launch_coarse_levels<T>(const std::vector<Level>&, int, const cx<T>*, const double2*, \
+                                               const cx<T>*, cx<T>*, cudaStream_t);
 CSFF_FUSED_INST(double)
 CSFF_FUSED_INST(float)
 

@@ -531,22 +531,6 @@ __device__ void down_tile(int P0x, int P0y, const cx<T>* u_in, int zero_init, co
   __syncthreads();   // shared memory is reused by the next tile
 }
 
-// Linear interpolation along one axis from a coarse window whose first entry
-// is coarse interior index e0 (coarse values outside [0, mc) are zero).
-template <typename T>
-__device__ __forceinline__ int interp_w(int p, int e0, int mc, int* ci, T* w) {
-  int i = p + 1, n = 0;
-  if ((i & 1) == 0) {
-    int I = i >> 1;
-    if (I >= 1 && I <= mc) { ci[n] = I - 1 - e0; w[n] = (T)1; ++n; }
-  } else {
-    int I0 = (i - 1) >> 1, I1 = I0 + 1;
-    if (I0 >= 1 && I0 <= mc) { ci[n] = I0 - 1 - e0; w[n] = (T)0.5; ++n; }
-    if (I1 >= 1 && I1 <= mc) { ci[n] = I1 - 1 - e0; w[n] = (T)0.5; ++n; }
-  }
-  return n;
-}
-
 // up tile: u = u_in + P e_c, one RB-GS sweep, write owned points.  Window
 // colour 0 is red (ox + oy even).  In the per-level kernel the tile itself
 // waits for the kernel before it (which writes only e_c), after issuing the
@@ -650,8 +634,27 @@ __device__ void up_tile(int P0x, int P0y, const cx<T>* u_in, const cx<T>* ec, co
 }
 
 // ---------------------------------------------------------------------------
-// All levels from lc down to the coarsest and back in one CTA.  Level data
-// (u, b, r and the coefficients) lives in shared memory.
+// All levels from lc down to the coarsest and back in one CTA.
+//
+// Bound by latency: one CTA, a chain of short phases, each a few shared loads,
+// a handful of dependent multiply-adds and a barrier (FP64 cycles and the FP64
+// coarsest product: by the one SM's FP64 pipe, two operations a clock).  So
+// the phases are few and lean:
+//  - a 16-lane row per grid row (the smoothing levels have m <= 31, at most 16
+//    points of a colour a row), windows with a ring of zeros: no index
+//    division and no test of a neighbour;
+//  - the red half sweep from zero, u = d^{-1} b, is folded into the load of b
+//    and into the full weighting that forms it;
+//  - as in the tiles, the residual is formed at the red points only (zero at
+//    the black ones) and the prolongation is needed at the black points only;
+//    here it is folded into the red half sweep, which adds the neighbour sum
+//    of the interpolated correction: its black result overwrites the rest;
+//  - the tables and, where it fits, the coarsest inverse are copied to shared
+//    memory before the wait for the predecessor kernel.
+// 33^2, 17^2 and 9^2 levels: 9.4 us a launch with FP32 levels and the FP64
+// product, 27.6 us all in FP64 (18.5 and 89 us when every point decoded its
+// index, formed the residual of both colours and prolonged in phases of its
+// own).
 // ---------------------------------------------------------------------------
 struct CoarseLevels {
   int nl;                       // number of levels handled (last = coarsest)
@@ -666,49 +669,21 @@ template <typename T> __device__ __forceinline__ cx<T> level_c(const CoarseLevel
 template <> __device__ __forceinline__ double2 level_c<double>(const CoarseLevels& L, int l) { return L.c[l]; }
 template <> __device__ __forceinline__ float2 level_c<float>(const CoarseLevels& L, int l) { return L.c32[l]; }
 
-template <typename T, int D>
-__device__ __forceinline__ cx<T> apply_s(const cx<T>* u, int m, int ix, int iy, int iz, int idx, cx<T> q,
-                                         cx<T> c) {
-  using C = cx<T>;
-  C s = zero_c<T>();
-  if (ix > 0) s = xadd(s, u[idx - 1]);
-  if (ix < m - 1) s = xadd(s, u[idx + 1]);
-  if (iy > 0) s = xadd(s, u[idx - m]);
-  if (iy < m - 1) s = xadd(s, u[idx + m]);
-  if (D == 3) {
-    if (iz > 0) s = xadd(s, u[idx - m * m]);
-    if (iz < m - 1) s = xadd(s, u[idx + m * m]);
-  }
-  C uj = u[idx];
-  C t = xsub(xscale(uj, (T)(2 * D)), s);
-  return xsub(xmul(c, t), xmul(q, uj));
-}
+constexpr int COARSE_NT = 512;      // threads of the per-level kernel (the persistent kernel's CTAs have NT)
+constexpr int COARSE_ROW = 16;      // lanes per grid row: points of a colour in a row of a smoothing level
+constexpr size_t COARSE_STAGE_LIMIT = 200 * 1024;
 
-template <int D>
-__device__ __forceinline__ void decode(int i, int m, int& ix, int& iy, int& iz) {
-  ix = i % m;
-  int r = i / m;
-  if (D == 3) { iy = r % m; iz = r / m; } else { iy = r; iz = 0; }
-}
-
-template <typename T, int D>
-__device__ void rbgs_s(cx<T>* u, const cx<T>* b, const cx<T>* q, const cx<T>* dinv, cx<T> c, int m, int N) {
-  for (int colour = 0; colour < 2; ++colour) {
-    for (int i = threadIdx.x; i < N; i += blockDim.x) {
-      int ix, iy, iz;
-      decode<D>(i, m, ix, iy, iz);
-      if (((ix + iy + iz + D) & 1) != colour) continue;
-      cx<T> rj = xsub(b[i], apply_s<T, D>(u, m, ix, iy, iz, i, q[i], c));
-      u[i] = xadd(u[i], xmul(dinv[i], rj));
-    }
-    __syncthreads();
-  }
-}
-
-inline size_t coarse_levels_elems(const std::vector<Level>& lv, int lc) {
+// shared memory of the block: per smoothing level u, b, r, q, 1/d on (m+2)^2
+// padded grids, for the coarsest u (padded) and b (m^2, in the product's type)
+// and, when staged, the inverse
+inline size_t coarse_block_bytes(const std::vector<Level>& lv, int lc, size_t el, size_t el_inv, bool staged) {
   size_t n = 0;
-  for (size_t l = lc; l < lv.size(); ++l) n += 5 * (size_t)lv[l].N;
-  return n;
+  for (size_t l = lc; l < lv.size(); ++l) n += (l + 1 < lv.size() ? 5 : 1) * (size_t)(lv[l].m + 2) * (lv[l].m + 2);
+  n = ((n * el + 15) & ~(size_t)15) + (size_t)lv.back().N * el_inv;
+  return n + (staged ? (size_t)lv.back().N * lv.back().N * el_inv : 0);
+}
+inline bool coarse_inv_staged(const std::vector<Level>& lv, int lc, size_t el, size_t el_inv) {
+  return coarse_block_bytes(lv, lc, el, el_inv, true) <= COARSE_STAGE_LIMIT;
 }
 
 template <typename T> __device__ __forceinline__ cx<T> to_cx(double2 v);
@@ -716,166 +691,173 @@ template <> __device__ __forceinline__ double2 to_cx<double>(double2 v) { return
 template <> __device__ __forceinline__ float2 to_cx<float>(double2 v) {
   return make_float2(__double2float_rn(v.x), __double2float_rn(v.y));
 }
+template <typename T> __device__ __forceinline__ cx<T> to_cx(float2 v) { return v; }
 template <typename TI, typename T> __device__ __forceinline__ cx<TI> widen(cx<T> v) {
   return mk<cx<TI>>((TI)v.x, (TI)v.y);
 }
 
+// sum of the four neighbours of padded index i (pitch W): x-1, x+1, y-1, y+1
+template <typename C> __device__ __forceinline__ C nbr_sum(const C* u, int i, int W) {
+  return xadd(xadd(xadd(u[i - 1], u[i + 1]), u[i - W]), u[i + W]);
+}
+
 // TI: the arithmetic of the coarsest product (T, or double for FP32 cycles
-// whose coarsest solve runs in FP64; the product is then rounded to T once)
-template <typename T, int D, bool COH, typename TI = T>
+// whose coarsest solve runs in FP64; the product is then rounded to T once).
+// staged: the launch's shared memory has room for the inverse.
+template <typename T, bool COH, typename TI = T>
 __device__ void coarse_levels_block(const CoarseLevels& L, const cx<T>* b_top, cx<T>* u_top,
-                                    const cx<TI>* __restrict__ inv, unsigned char* smem_raw) {
+                                    const cx<TI>* __restrict__ inv, unsigned char* smem_raw, bool staged) {
   using C = cx<T>;
-  C* base = reinterpret_cast<C*>(smem_raw);
-  C* U[8];
-  C* B[8];
-  C* R[8];
-  C* Qs[8];
-  C* Ds[8];
-  int N[8];
-  {
-    C* p = base;
-    for (int l = 0; l < L.nl; ++l) {
-      N[l] = L.m[l] * L.m[l] * (D == 3 ? L.m[l] : 1);
-      U[l] = p; p += N[l];
-      B[l] = p; p += N[l];
-      R[l] = p; p += N[l];
-      Qs[l] = p; p += N[l];
-      Ds[l] = p; p += N[l];
+  using CI = cx<TI>;
+  const int t = threadIdx.x, nt = blockDim.x, last = L.nl - 1;
+  C* const base = reinterpret_cast<C*>(smem_raw);
+  const int n = L.m[last] * L.m[last];
+  // tables to shared memory, zero iterates with their rings
+  C* p = base;
+  for (int l = 0; l <= last; ++l) {
+    const int m = L.m[l], W = m + 2, A = W * W;
+    for (int i = t; i < A; i += nt) p[i] = zero_c<T>();
+    if (l < last) {
+      const C* q = reinterpret_cast<const C*>(L.q[l]);
+      const C* dv = reinterpret_cast<const C*>(L.dinv[l]);
+      const int x = t & 31;
+      if (x < m)
+        for (int y = t >> 5; y < m; y += nt >> 5) {
+          const int g = y * m + x, s = (y + 1) * W + x + 1;
+          if constexpr (COH) {
+            p[3 * A + s] = q[g];
+            p[4 * A + s] = dv[g];
+          } else {
+            cp_async_s<(int)sizeof(C)>(smem_addr(p + 3 * A + s), q + g);
+            cp_async_s<(int)sizeof(C)>(smem_addr(p + 4 * A + s), dv + g);
+          }
+        }
+      p += 5 * A;
     }
   }
-  // every global read up front; the phases below touch shared memory only.
-  // Each thread's first point of every level is loaded into registers before
-  // any store, so those loads are in flight together; the rest follow.
-  {
-    const int t = threadIdx.x;
-    C qv[8], dv[8];
-#pragma unroll
-    for (int l = 0; l < 8; ++l)
-      if (l < L.nl && t < N[l]) {
-        qv[l] = reinterpret_cast<const C*>(L.q[l])[t];
-        dv[l] = reinterpret_cast<const C*>(L.dinv[l])[t];
+  C* const Ulast = p;
+  CI* const Bc = reinterpret_cast<CI*>(
+      smem_raw + (((size_t)(p - base) + (size_t)(L.m[last] + 2) * (L.m[last] + 2)) * sizeof(C) + 15) / 16 * 16);
+  const CI* iv = inv;
+  if constexpr (!COH) {
+    if (staged) {
+      CI* d = Bc + n;
+      for (int i = t; i < n * n; i += nt) cp_async_s<(int)sizeof(CI)>(smem_addr(d + i), inv + i);
+      iv = d;
+    }
+    cp_async_wait_all();
+    __syncthreads();
+    pdl_prologue();
+    pdl_trigger();      // the up tile copies its own window before it waits for this block
+  } else {
+    __syncthreads();
+  }
+  // b of the top level, with its red half sweep from zero
+  if (last > 0) {
+    const int m = L.m[0], W = m + 2, A = W * W, x = t & 31;
+    if (x < m)
+      for (int y = t >> 5; y < m; y += nt >> 5) {
+        const C v = ld<COH>(b_top + y * m + x);
+        const int s = (y + 1) * W + x + 1;
+        base[A + s] = v;
+        if (((x + y) & 1) == 0) base[s] = xmul(base[4 * A + s], v);
       }
-    const C bv = (t < N[0]) ? ld<COH>(b_top + t) : zero_c<T>();
-#pragma unroll
-    for (int l = 0; l < 8; ++l)
-      if (l < L.nl && t < N[l]) {
-        Qs[l][t] = qv[l];
-        Ds[l][t] = dv[l];
-      }
-    if (t < N[0]) {
-      B[0][t] = bv;
-      U[0][t] = zero_c<T>();
-    }
-  }
-  for (int l = 0; l < L.nl; ++l) {
-    const C* q = reinterpret_cast<const C*>(L.q[l]);
-    const C* dv = reinterpret_cast<const C*>(L.dinv[l]);
-    for (int i = threadIdx.x + blockDim.x; i < N[l]; i += blockDim.x) {
-      Qs[l][i] = q[i];
-      Ds[l][i] = dv[i];
-    }
-  }
-  for (int i = threadIdx.x + blockDim.x; i < N[0]; i += blockDim.x) {
-    B[0][i] = ld<COH>(b_top + i);
-    U[0][i] = zero_c<T>();
+  } else {
+    for (int i = t; i < n; i += nt) Bc[i] = widen<TI, T>(ld<COH>(b_top + i));
   }
   __syncthreads();
-  const T w1[3] = {(T)0.25, (T)0.5, (T)0.25};
-  const int last = L.nl - 1;
+  const int j = t % COARSE_ROW, y0 = t / COARSE_ROW, dy = nt / COARSE_ROW;
+  p = base;
   for (int l = 0; l < last; ++l) {
-    const int m = L.m[l], mc = L.m[l + 1];
+    const int m = L.m[l], mc = L.m[l + 1], W = m + 2, A = W * W, Wc = mc + 2, Ac = Wc * Wc;
     const C c = level_c<T>(L, l);
-    if (l > 0)
-      for (int i = threadIdx.x; i < N[l]; i += blockDim.x) U[l][i] = zero_c<T>();
-    __syncthreads();
-    rbgs_s<T, D>(U[l], B[l], Qs[l], Ds[l], c, m, N[l]);
-    for (int i = threadIdx.x; i < N[l]; i += blockDim.x) {
-      int ix, iy, iz;
-      decode<D>(i, m, ix, iy, iz);
-      R[l][i] = xsub(B[l][i], apply_s<T, D>(U[l], m, ix, iy, iz, i, Qs[l][i], c));
+    C *U = p, *B = p + A, *R = p + 2 * A, *Q = p + 3 * A, *D = p + 4 * A;
+    C* const next = p + 5 * A;
+    for (int iy = y0 + 1; iy <= m; iy += dy) {               // black
+      const int ix = 2 * j + ((iy & 1) ? 2 : 1), i = iy * W + ix;
+      if (ix <= m) U[i] = xmul(D[i], xfma(B[i], c, nbr_sum(U, i, W)));
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < N[l + 1]; i += blockDim.x) {
-      int px, py, pz;
-      decode<D>(i, mc, px, py, pz);
-      C acc = zero_c<T>();
-      for (int oz = (D == 3 ? -1 : 0); oz <= (D == 3 ? 1 : 0); ++oz)
-        for (int oy = -1; oy <= 1; ++oy)
-          for (int ox = -1; ox <= 1; ++ox) {
-            int fx = 2 * px + 1 + ox, fy = 2 * py + 1 + oy, fz = (D == 3) ? 2 * pz + 1 + oz : 0;
-            T w = w1[ox + 1] * w1[oy + 1] * ((D == 3) ? w1[oz + 1] : (T)1);
-            acc = xadd(acc, xscale(R[l][(fz * m + fy) * m + fx], w));
-          }
-      B[l + 1][i] = acc;
+    for (int iy = y0 + 1; iy <= m; iy += dy) {               // residual at the red points
+      const int ix = 2 * j + ((iy & 1) ? 1 : 2), i = iy * W + ix;
+      if (ix <= m) {
+        const C d = xsub(xscale(c, (T)4), Q[i]);
+        R[i] = xfma(xfms(B[i], d, U[i]), c, nbr_sum(U, i, W));
+      }
     }
     __syncthreads();
+    for (int Y = y0 + 1; Y <= mc; Y += dy) {                 // full weighting of the red residuals
+      const int X = j + 1;
+      if (X > mc) continue;
+      const C* r = R + 2 * Y * W + 2 * X;
+      const C corners = xadd(xadd(r[-W - 1], r[-W + 1]), xadd(r[W - 1], r[W + 1]));
+      const C v = xfma_r(xscale(corners, (T)0.0625), r[0], (T)0.25);
+      if (l + 1 < last) {
+        const int s = Y * Wc + X;
+        next[Ac + s] = v;
+        if (((X + Y) & 1) == 0) next[s] = xmul(next[4 * Ac + s], v);
+      } else {
+        Bc[(Y - 1) * mc + X - 1] = widen<TI, T>(v);
+      }
+    }
+    __syncthreads();
+    p = next;
   }
-  // coarsest: u = inv b (the inverse itself comes from FP64 Gauss-Jordan)
-  if constexpr (sizeof(TI) == sizeof(T)) {
-    // in the cycle's precision: one warp per row, lanes split the columns
-    const int n = N[last];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    for (int i = warp; i < n; i += nw) {
-      C acc = zero_c<T>();
-      const C* row = inv + (long long)i * n;
-      for (int j = lane; j < n; j += 32) acc = xadd(acc, xmul(row[j], B[last][j]));
-      for (int o = 16; o > 0; o >>= 1) {
+  // coarsest: u = inv b (the inverse itself comes from FP64 Gauss-Jordan).
+  // Each row over four consecutive lanes (columns j = p mod 4), fused
+  // multiply-add chains, two shuffles: FP64 work is scarce
+  {
+    const int ml = L.m[last];
+    for (int k = t; k < ((4 * n + 31) & ~31); k += nt) {
+      const int i = k >> 2, part = k & 3;
+      CI acc = mk<CI>((TI)0, (TI)0);
+      if (i < n) {
+        const CI* row = iv + (long long)i * n;
+        for (int col = part; col < n; col += 4) acc = xfma(acc, row[col], Bc[col]);
+      }
+#pragma unroll
+      for (int o = 1; o <= 2; o <<= 1) {
         acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
         acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
       }
-      if (lane == 0) U[last][i] = acc;
-    }
-    __syncthreads();
-  } else {
-    // in FP64 (FP32 cycles of the FP64 refinement): FP64 work is scarce, so
-    // each row is split over four consecutive lanes only (columns j = p mod 4),
-    // each lane a chain of fused multiply-adds; two shuffles join the parts and
-    // the row's sum is rounded once to the cycle's precision
-    const int n = N[last];
-    for (int t = threadIdx.x; t < ((4 * n + 31) & ~31); t += blockDim.x) {
-      const int i = t >> 2, part = t & 3;
-      double re = 0.0, im = 0.0;
-      if (i < n) {
-        const double2* row = reinterpret_cast<const double2*>(inv) + (long long)i * n;
-        for (int j = part; j < n; j += 4) {
-          const double2 a = row[j];
-          const double bx = (double)B[last][j].x, by = (double)B[last][j].y;
-          re = fma(a.x, bx, fma(-a.y, by, re));
-          im = fma(a.x, by, fma(a.y, bx, im));
-        }
+      if (i < n && part == 0) {
+        const C v = to_cx<T>(acc);
+        if (last == 0) u_top[i] = v;
+        else Ulast[(i / ml + 1) * (ml + 2) + i % ml + 1] = v;
       }
-      re += __shfl_xor_sync(0xffffffffu, re, 1);
-      im += __shfl_xor_sync(0xffffffffu, im, 1);
-      re += __shfl_xor_sync(0xffffffffu, re, 2);
-      im += __shfl_xor_sync(0xffffffffu, im, 2);
-      if (i < n && part == 0) U[last][i] = to_cx<T>(make_double2(re, im));
     }
     __syncthreads();
   }
+  C* E = Ulast;
   for (int l = last - 1; l >= 0; --l) {
-    const int m = L.m[l], mc = L.m[l + 1];
+    const int m = L.m[l], W = m + 2, A = W * W, Wc = L.m[l + 1] + 2;
     const C c = level_c<T>(L, l);
-    for (int i = threadIdx.x; i < N[l]; i += blockDim.x) {
-      int ix, iy, iz;
-      decode<D>(i, m, ix, iy, iz);
-      int cxi[2], cyi[2], czi[2] = {0, 0};
-      T wx[2], wy[2], wz[2] = {(T)1, (T)0};
-      int nx = interp_w<T>(ix, 0, mc, cxi, wx);
-      int ny = interp_w<T>(iy, 0, mc, cyi, wy);
-      int nz = (D == 3) ? interp_w<T>(iz, 0, mc, czi, wz) : 1;
-      C acc = zero_c<T>();
-      for (int a = 0; a < nz; ++a)
-        for (int bq = 0; bq < ny; ++bq)
-          for (int cq = 0; cq < nx; ++cq)
-            acc = xadd(acc, xscale(U[l + 1][(czi[a] * mc + cyi[bq]) * mc + cxi[cq]], wx[cq] * wy[bq] * wz[a]));
-      U[l][i] = xadd(U[l][i], acc);
+    C *U = E - 5 * A, *B = U + A, *D = U + 4 * A;
+    // red, with the neighbour sum of the interpolated correction: at a cell
+    // centre (odd node indices) the four corners; at a coarse node twice its
+    // value and half of each of its four neighbours
+    for (int iy = y0 + 1; iy <= m; iy += dy) {
+      const int ix = 2 * j + ((iy & 1) ? 1 : 2), i = iy * W + ix;
+      if (ix > m) continue;
+      const C* e = E + (iy >> 1) * Wc + (ix >> 1);
+      C pe;
+      if (iy & 1) pe = xadd(xadd(e[0], e[1]), xadd(e[Wc], e[Wc + 1]));
+      else pe = xfma_r(xscale(e[0], (T)2), xadd(xadd(e[-1], e[1]), xadd(e[-Wc], e[Wc])), (T)0.5);
+      const C v = xmul(D[i], xfma(B[i], c, xadd(nbr_sum(U, i, W), pe)));
+      U[i] = v;
+      if (l == 0) u_top[(iy - 1) * m + ix - 1] = v;
     }
     __syncthreads();
-    rbgs_s<T, D>(U[l], B[l], Qs[l], Ds[l], c, m, N[l]);
+    for (int iy = y0 + 1; iy <= m; iy += dy) {               // black
+      const int ix = 2 * j + ((iy & 1) ? 2 : 1), i = iy * W + ix;
+      if (ix > m) continue;
+      const C v = xmul(D[i], xfma(B[i], c, nbr_sum(U, i, W)));
+      if (l == 0) u_top[(iy - 1) * m + ix - 1] = v;
+      else U[i] = v;
+    }
+    __syncthreads();
+    E = U;
   }
-  for (int i = threadIdx.x; i < N[0]; i += blockDim.x) u_top[i] = U[0][i];
-  __syncthreads();
 }
 
 }  // namespace tiles
