@@ -32,6 +32,7 @@ __global__ void __launch_bounds__(NT, tile_min_ctas<T, TC>()) k_down2(const cx<T
                                               int m, int mc, cx<T>* __restrict__ u_out, cx<T>* __restrict__ bc) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   pdl_prologue();
+  if (tiles::early_trigger()) pdl_trigger();
   tiles::down_tile<T, TC, false, G1>(blockIdx.x * TC, blockIdx.y * TC, u_in, zero_init, b, K, c, m, mc, u_out, bc,
                                  smem_raw);
 }

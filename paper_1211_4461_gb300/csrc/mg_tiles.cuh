@@ -28,6 +28,16 @@ template <int TC> struct Geo {
 };
 constexpr int NT = 256;
 
+// Small launches (at most one tile an SM: the levels from 129^2 down) let their
+// dependents be set up as soon as they have passed their own wait: the next
+// kernel's CTAs find free slots and copy what they can meanwhile.  257^2 map
+// 939 -> 868 us, 1025^2 map 2316 -> 2213 us.  With the 256 tiles of the 257^2
+// and 513^2 levels included the 1025^2 map took 2343 us: the waiting CTAs of
+// the next level then hold slots and bandwidth that the running one needs.
+#ifdef __CUDACC__
+__device__ __forceinline__ bool early_trigger() { return gridDim.x * gridDim.y <= 152u; }
+#endif
+
 // Coefficients of one fine level as the tile bodies see them: the diagonal
 // d = 2D c - q and its inverse.  FP64 cycles read the plan's FP64 tables
 // (q, dinv); FP32 cycles form them from separable per-axis factors,
@@ -552,6 +562,7 @@ __device__ void up_tile(int P0x, int P0y, const cx<T>* u_in, const cx<T>* ec, co
   if constexpr (!COH) {
     load_window<T, UW, COH, false>(ox, oy, m, u_in, false, b, K, U, B, X);
     pdl_prologue();
+    if (early_trigger()) pdl_trigger();
   }
   // coarse window: asynchronous copies (per-level kernels) or loads held in
   // registers across the fine window's loads (persistent kernel)
