@@ -12,7 +12,7 @@ ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 BUILD = os.path.join(ROOT, "_build")
 LIB = os.path.join(PKG, "libcsff.so")
-SOURCES = ["csff_api.cu", "mg_kernels.cu", "mg_fused.cu", "farfield.cu", "batch.cu", "learned.cu", "noalloc.cu",
+SOURCES = ["csff_api.cu", "mg_kernels.cu", "mg_fused.cu", "mg_split3.cu", "farfield.cu", "batch.cu", "learned.cu", "noalloc.cu",
            "gmres.cu", "partial_wave.cu", "refine_df.cu"]
 # every header under csrc/ and the public one: an edit to any of them rebuilds every object
 HEADERS = sorted(f for f in os.listdir(CSRC) if f.endswith((".h", ".cuh"))) + [

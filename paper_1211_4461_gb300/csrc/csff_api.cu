@@ -304,21 +304,23 @@ csff_status smooth(csff_plan* P, int l, cx<T>* u, const cx<T>* b, int sweeps) {
   return CSFF_OK;
 }
 
+template <typename T> csff_status coarsest_solve(csff_plan* P, const cx<T>* b, cx<T>* u) {
+  if constexpr (sizeof(T) == 4) {
+    if (coarse_fp64(P)) {
+      CK(csff::launch_coarse_solve_f64(P->coarse_inv, P->coarse_N, b, u, P->stream), "coarse solve");
+      return CSFF_OK;
+    }
+  }
+  CK(csff::launch_coarse_solve<T>(cinv<T>(P), P->coarse_N, b, u, P->stream), "coarse solve");
+  return CSFF_OK;
+}
+
 // One V(nu1, nu2) cycle on level l for A_l u = b (Sec. 4).
 template <typename T>
 csff_status vcycle(csff_plan* P, int l, cx<T>* u, const cx<T>* b) {
   const int nl = (int)P->lv.size();
   cudaStream_t s = P->stream;
-  if (l == nl - 1) {
-    if constexpr (sizeof(T) == 4) {
-      if (coarse_fp64(P)) {
-        CK(csff::launch_coarse_solve_f64(P->coarse_inv, P->coarse_N, b, u, s), "coarse solve");
-        return CSFF_OK;
-      }
-    }
-    CK(csff::launch_coarse_solve<T>(cinv<T>(P), P->coarse_N, b, u, s), "coarse solve");
-    return CSFF_OK;
-  }
+  if (l == nl - 1) return coarsest_solve<T>(P, b, u);
   Level& L = P->lv[l];
   Level& C = P->lv[l + 1];
   CS(smooth<T>(P, l, u, b, P->opts.nu1));
@@ -432,12 +434,29 @@ csff_status run_vcycle_learned(csff_plan* P, float2* u, const float2* b, bool ze
   return CSFF_OK;
 }
 
-// One V-cycle at the finest level: the fused 2D V(1,1) RB-GS kernels when the
-// plan qualifies, else the general per-step kernels.  zero_init: the iterate
-// enters as zero (the correction equation of a refinement step).
+// The 3D V(1,1) RB-GS cycle on colour-split arrays.  first/last: of the cycles
+// run on one right-hand side (the iterate stays split in between).
 template <typename T>
-csff_status run_vcycle(csff_plan* P, cx<T>* u, const cx<T>* b, bool zero_init) {
+csff_status run_split3(csff_plan* P, cx<T>* u, const cx<T>* b, bool zero_init, bool first, bool last) {
+  const cx<T>* none = nullptr;
+  cx<T>* no = nullptr;
+  CK(csff::launch_split3_down<T>(P->lv, first && !zero_init ? u : none, b, zero_init, first, P->stream), "split down");
+  Level& C = P->lv.back();
+  CS(coarsest_solve<T>(P, bbuf<T>(C), ubuf<T>(C)));
+  CK(csff::launch_split3_up<T>(P->lv, last ? u : no, false, P->stream), "split up");
+  return CSFF_OK;
+}
+
+// One V-cycle at the finest level: the fused 2D V(1,1) RB-GS kernels or the
+// colour-split 3D ones when the plan qualifies, else the general per-step
+// kernels.  zero_init: the iterate enters as zero (the correction equation of
+// a refinement step); first, last: of a run of cycles on one right-hand side,
+// between which only this function touches u.
+template <typename T>
+csff_status run_vcycle(csff_plan* P, cx<T>* u, const cx<T>* b, bool zero_init, bool first = true, bool last = true) {
   const int lc = P->fused_lc;
+  const bool learned = sizeof(T) == 4 && P->net && !P->learned_off;
+  if ((sizeof(T) == 4 ? P->split32 : P->split64) && !learned) return run_split3<T>(P, u, b, zero_init, first, last);
   if constexpr (sizeof(T) == 4) {
     if (P->net && !P->learned_off) {
       if (lc > P->learned_levels) return run_vcycle_learned(P, u, b, zero_init);
@@ -469,7 +488,7 @@ csff_status step_fp64(csff_plan* P, int eb) {
 csff_status step_mixed(csff_plan* P, int n) {
   Level& L = P->lv[0];
   cudaStream_t s = P->stream;
-  for (int c = 0; c < n; ++c) CS(run_vcycle<float>(P, L.u32, L.b32, c == 0));
+  for (int c = 0; c < n; ++c) CS(run_vcycle<float>(P, L.u32, L.b32, c == 0, c == 0, c == n - 1));
   CK(csff::launch_df_update(P->dfu, L.u32, L.N, s), "update");
   CK(csff::launch_df_residual(P->dim, L, P->dfu, P->dfb, P->dfq, L.b32, P->dfpart, P->red_out, s), "residual");
   CK(cudaMemcpyAsync(P->red_host, P->red_out, sizeof(double), cudaMemcpyDeviceToHost, s), "read norm");
@@ -492,7 +511,7 @@ void destroy_graphs(csff_plan* P) {
 csff_status step_mixed64(csff_plan* P, int n) {
   Level& L = P->lv[0];
   cudaStream_t s = P->stream;
-  for (int c = 0; c < n; ++c) CS(run_vcycle<float>(P, L.u32, L.b32, c == 0));
+  for (int c = 0; c < n; ++c) CS(run_vcycle<float>(P, L.u32, L.b32, c == 0, c == 0, c == n - 1));
   CK(csff::launch_update64_fixed(L.u64, L.u32, L.N, P->refine_eb, s), "update");
   CK(csff::launch_refine_residual(P->dim, L, L.u64, L.b64, P->refine_eb, L.b32, P->red, P->red_blocks, P->red_out,
                                   s),
@@ -668,6 +687,36 @@ csff_status solve_mixed(csff_plan* P, int eb, double nb, csff_info* info, const 
   return result;
 }
 
+template <typename T> csff::Split3<T>& split_of(Level& L);
+template <> csff::Split3<float>& split_of<float>(Level& L) { return L.s32; }
+template <> csff::Split3<double>& split_of<double>(Level& L) { return L.s64; }
+
+// The colour-split arrays of every level above the coarsest: one allocation a
+// level, and 1/d by colour.  Slots outside the domain hold zero: on the finest
+// level every pass writes whole rows, below it the full weighting does not.
+template <typename T> csff_status alloc_split3(csff_plan* P) {
+  for (size_t l = 0; l + 1 < P->lv.size(); ++l) {
+    Level& L = P->lv[l];
+    csff::Split3<T>& S = split_of<T>(L);
+    const size_t half = (size_t)L.m * L.m * csff::split3_pitch(L.m);
+    const size_t total = (l == 0 ? 7 : 8) * half;
+    cx<T>* base = nullptr;
+    CS(dev_alloc(P, &base, total));
+    S.base = base;
+    if (l > 0) CK(cudaMemsetAsync(base, 0, total * sizeof(cx<T>), P->stream), "zero split arrays");
+    S.ur = base;
+    S.ub = base + half;
+    S.br = base + 2 * half;
+    S.bb = base + 3 * half;
+    S.dr = base + 4 * half;
+    S.db = base + 5 * half;
+    if (l == 0) S.delta = base + 6 * half;
+    else S.e = base + 6 * half;
+    CK(csff::split3_coefs<T>(L, P->prob.k * P->prob.k, P->stream), "split coefficients");
+  }
+  return CSFF_OK;
+}
+
 csff_status check_level(const csff_plan* P, int level, int arith) {
   if (!P) return invalid("plan is NULL");
   if (level < 0 || level >= (int)P->lv.size()) return invalid("level out of range");
@@ -745,7 +794,7 @@ void csff_plan_destroy(csff_plan* P) {
   for (Level& L : P->lv)
     for (void* p : {(void*)L.q64, (void*)L.dinv64, (void*)L.q32, (void*)L.dinv32, (void*)L.u64, (void*)L.t64,
                     (void*)L.b64, (void*)L.r64, (void*)L.u32, (void*)L.t32, (void*)L.b32, (void*)L.r32,
-                    (void*)L.fac32})
+                    (void*)L.fac32, L.s32.base, L.s64.base})
       if (p) cudaFree(p);
   for (double2* p : P->chi_tab)
     if (p) cudaFree(p);
@@ -891,6 +940,13 @@ csff_status csff_plan_create(const csff_problem* prob, const csff_opts* opts, vo
       }
       P->gm_v = v;
     }
+  }
+  // colour-split V(1,1) RB-GS path (3D), in the precision of the plan's cycles
+  if (d == 3 && opts->smoother == CSFF_SMOOTHER_RBGS && opts->nu1 == 1 && opts->nu2 == 1 && P->lv.size() > 1) {
+    const bool mixed = P->opts.precision == CSFF_PREC_MIXED;
+    csff_status s = mixed ? alloc_split3<float>(P) : alloc_split3<double>(P);
+    if (s != CSFF_OK) return fail(s);
+    (mixed ? P->split32 : P->split64) = true;
   }
   // fused V(1,1) RB-GS path (2D): the levels from the first with n <= 33 run in
   // one CTA; at least one fused fine level is needed
@@ -1180,6 +1236,10 @@ static csff_status user_q_levels(csff_plan* P) {
   cudaStream_t s = P->stream;
   for (size_t l = 1; l < P->lv.size(); ++l) CK(csff::launch_inject_q(P->dim, P->lv[l - 1], P->lv[l], s), "inject q");
   for (const Level& L : P->lv) CK(csff::launch_coefs_from_q(P->dim, L, s), "coefficients");
+  for (size_t l = 0; l + 1 < P->lv.size(); ++l) {
+    if (P->split32) CK(csff::split3_coefs<float>(P->lv[l], P->prob.k * P->prob.k, s), "split coefficients");
+    if (P->split64) CK(csff::split3_coefs<double>(P->lv[l], P->prob.k * P->prob.k, s), "split coefficients");
+  }
   const Level& Lc = P->lv.back();
   std::vector<double2> qc((size_t)Lc.N);
   CK(cudaMemcpyAsync(qc.data(), Lc.q64, sizeof(double2) * qc.size(), cudaMemcpyDeviceToHost, s), "read q");

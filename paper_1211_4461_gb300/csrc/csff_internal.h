@@ -69,6 +69,16 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
 // ---------------------------------------------------------------------------
 // plan internals
 // ---------------------------------------------------------------------------
+// Colour-split arrays of a 3D level (mg_split3.cu): iterate, right-hand side
+// and 1/d by colour (red, black), the black change of a sweep (finest level),
+// and the level's correction in natural order, rows 2 split3_pitch apart.
+template <typename T> struct Split3 {
+  cx<T> *ur = nullptr, *ub = nullptr, *br = nullptr, *bb = nullptr, *dr = nullptr, *db = nullptr;
+  cx<T> *delta = nullptr, *e = nullptr;
+  cx<T> d0{};                    // FP32: dr, db hold 1/d - d0
+  void* base = nullptr;          // the one allocation behind them
+};
+
 struct Level {
   int n = 0, m = 0;
   long long N = 0;       // m^d
@@ -87,6 +97,8 @@ struct Level {
   // work buffers
   double2 *u64 = nullptr, *t64 = nullptr, *b64 = nullptr, *r64 = nullptr;
   float2 *u32 = nullptr, *t32 = nullptr, *b32 = nullptr, *r32 = nullptr;
+  Split3<float> s32;
+  Split3<double> s64;
 };
 
 // Far-field scratch (grown on demand): g = chi (u_in + u); x/y/z phase
@@ -153,6 +165,8 @@ struct csff_plan {
   double log_rhs_max = 0, log_ff_max = 0;
   // fused V(1,1) RB-GS path (2D): levels >= fused_lc run in one CTA; -1 = unfused
   int fused_lc = -1;
+  // colour-split 3D V(1,1) RB-GS cycles: their arrays exist in FP32 / FP64
+  bool split32 = false, split64 = false;
   // CUDA graphs of solver steps (FP64 cycle, or mixed refinement step of a
   // given cycle count), captured on an internal stream and kept by key; the
   // oldest is replaced when all slots are taken
@@ -301,6 +315,22 @@ cudaError_t launch_refine_residual(int dim, const Level& L, const double2* u, co
                                    float2* r32, double* partial, int nblk, double* out, cudaStream_t s);
 cudaError_t launch_update64_fixed(double2* u, const float2* e, long long N, int s_exp, cudaStream_t s);
 cudaError_t launch_scale_to32(const double2* v, long long N, int s_exp, float2* r32, cudaStream_t s);
+
+// ---- 3D V(1,1) cycles on colour-split arrays (mg_split3.cu) ----------------------
+int split3_pitch(int m);                       // slots of a row of one colour
+// 1/d by colour from dinv64 (k2: the wavenumber's square, without potential)
+template <typename T> cudaError_t split3_coefs(Level& L, double k2, cudaStream_t s);
+// the levels down to the coarsest right-hand side (b32/b64 of the last level);
+// new_b: b differs from the last call's; u: the natural iterate, or null when it
+// is still in the split arrays (or zero_init)
+template <typename T>
+cudaError_t launch_split3_down(std::vector<Level>& lv, const cx<T>* u, const cx<T>* b, bool zero_init, bool new_b,
+                               cudaStream_t s);
+// and back from the coarsest solution (u32/u64 of the last level); the iterate
+// goes to u_nat (may be null) and, without u_nat or with keep_split, stays in
+// the split arrays
+template <typename T>
+cudaError_t launch_split3_up(std::vector<Level>& lv, cx<T>* u_nat, bool keep_split, cudaStream_t s);
 
 // ---- GMRES(m) smoothing step (gmres.cu) ----------------------------------------
 // u += V y for the GMRES(m) minimiser from u; V holds m+1 vectors of L.N

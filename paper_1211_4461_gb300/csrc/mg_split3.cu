@@ -1,0 +1,444 @@
+// 3D V(1,1) red-black Gauss-Seidel cycles on colour-split arrays (Sec. 4).
+//
+// Bound by memory traffic: a half sweep reads the other colour of u, its own
+// colour of b and 1/d and writes its own colour of u.  With the colours
+// interleaved every one of those streams moves whole cache lines, both colours
+// of each array; split by colour a half sweep moves half as much.
+//
+// Layout: row (iy, iz) of a colour holds its points in order, x = 2 j + o in
+// slot j with o the row's parity of the colour (red: (iy + iz + 1) mod 2, black
+// the other), HP slots a row (a multiple of four; slots outside the domain are
+// zero).  The six neighbours of slot j lie in the other colour's array: slots
+// j + o - 1 and j + o of the same row, slot j of the rows above, below, before
+// and behind.  A thread takes two slots of a row (one 16-byte access in FP32).
+//
+// A cycle has four passes per level instead of eight:
+//  - the red half sweep from zero, u = d^{-1} b, is folded into the full
+//    weighting that forms b;
+//  - no residual array: after the black half sweep every black equation holds
+//    and the red residual is r = c sum_nbr delta, delta the change of the black
+//    values since the red half sweep (their values themselves when the iterate
+//    entered as zero), because the red half sweep left d u = b + c sum_nbr u_old.
+//    Full weighting of r (centre 1/8, the twelve red edge points 1/32) then is
+//    one 38-point sum over delta: 1/4 at the 6 points at distance (1,0,0), 3/32
+//    at the 8 at (1,1,1), 1/32 at the 24 at (2,1,0), times c;
+//  - the prolongation is needed at the black points only, as neighbours of the
+//    red half sweep (the black half sweep overwrites them): the red half sweep
+//    adds the interpolated correction's neighbour sum, formed from the coarse
+//    values directly;
+//  - the last black half sweep writes both colours in natural order.
+// 257^3 FP32 cycle through the public call (natural order in and out): 411 us,
+// 670 with interleaved colours; a half sweep of 255^3 48 us, 80 before (copy
+// rate: 39), the 38-point full weighting 39 us, residual and full weighting
+// 123 before, the prolonging half sweep 74, both passes 125 before.
+#include "csff_internal.h"
+
+namespace csff {
+namespace {
+
+template <typename T> struct Pair { cx<T> a, b; };
+template <typename T> __device__ __forceinline__ cx<T> zc() { return mk<cx<T>>((T)0, (T)0); }
+__device__ __forceinline__ Pair<float> ld2(const float2* p) {
+  const float4 v = *reinterpret_cast<const float4*>(p);
+  return Pair<float>{make_float2(v.x, v.y), make_float2(v.z, v.w)};
+}
+__device__ __forceinline__ Pair<double> ld2(const double2* p) { return Pair<double>{p[0], p[1]}; }
+__device__ __forceinline__ void st2(float2* p, float2 a, float2 b) {
+  *reinterpret_cast<float4*>(p) = make_float4(a.x, a.y, b.x, b.y);
+}
+__device__ __forceinline__ void st2(double2* p, double2 a, double2 b) {
+  p[0] = a;
+  p[1] = b;
+}
+// a + b c for complex values, a chain of fused multiply-adds
+template <typename C> __device__ __forceinline__ C cfma(C a, C b, C c) {
+  return mk<C>(fma(b.x, c.x, fma(-b.y, c.y, a.x)), fma(b.x, c.y, fma(b.y, c.x, a.y)));
+}
+
+// d^{-1} t.  FP32 cycles hold d^{-1} as d0 + dv, d0 the level's FP32 value
+// without the potential and dv the FP32 difference: rounding d^{-1} itself
+// shifts every equation by the same 2^-25 |d|, which the folded residual (no
+// explicit b - A u) would pass to the coarse levels as a residual.
+__device__ __forceinline__ float2 dinv_mul(float2 d0, float2 dv, float2 t) { return cfma(cmul(d0, t), dv, t); }
+__device__ __forceinline__ double2 dinv_mul(double2, double2 dv, double2 t) { return cmul(dv, t); }
+
+// coordinates of a thread: slot pair, row, plane
+struct At { int j, iy, iz; long long row; };
+__device__ __forceinline__ bool at(int m, int HP, At& p) {
+  p.j = 2 * (int)(blockIdx.x * blockDim.x + threadIdx.x);
+  p.iy = blockIdx.y * blockDim.y + threadIdx.y;
+  p.iz = blockIdx.z;
+  p.row = (long long)p.iz * m + p.iy;
+  return p.j < HP && p.iy < m;
+}
+
+// b (both colours) and, when u_nat, the black points of u from natural order;
+// with dr (the iterate enters as zero) the red half sweep u = d^{-1} b
+template <typename T>
+__global__ void k3s_import(const cx<T>* __restrict__ b_nat, const cx<T>* __restrict__ u_nat,
+                           const cx<T>* __restrict__ dr, cx<T> d0, int m, int HP, cx<T>* __restrict__ br,
+                           cx<T>* __restrict__ bb, cx<T>* __restrict__ ub, cx<T>* __restrict__ ur) {
+  using C = cx<T>;
+  pdl_prologue();
+  At p;
+  if (!at(m, HP, p)) return;
+  const int o = (p.iy + p.iz + 1) & 1;                 // red parity of the row
+  const C* row = b_nat + p.row * m;
+  const int x = 2 * p.j;
+  C v[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) v[k] = x + k < m ? row[x + k] : zc<T>();
+  const long long s = p.row * HP + p.j;
+  const C r0 = o ? v[1] : v[0], r1 = o ? v[3] : v[2];
+  st2(br + s, r0, r1);
+  st2(bb + s, o ? v[0] : v[1], o ? v[2] : v[3]);
+  if (dr) {
+    const Pair<T> d = ld2(dr + s);
+    st2(ur + s, dinv_mul(d0, d.a, r0), dinv_mul(d0, d.b, r1));
+  }
+  if (u_nat) {
+    const C* ru = u_nat + p.row * m;
+    const int x0 = x + 1 - o, x1 = x0 + 2;
+    st2(ub + s, x0 < m ? ru[x0] : zc<T>(), x1 < m ? ru[x1] : zc<T>());
+  }
+}
+
+// a level's d^{-1} by colour: FP64 as stored; FP32 as the difference to d0 of
+// 1 / (6 c - q) with c the FP32 value that the sweeps multiply by, to first
+// order in dc, six times the rounding of c (relative 2^-25: its square and the
+// rounding of this term lie far below the result's)
+template <typename T>
+__global__ void k3s_split(const double2* __restrict__ dinv, float2 dc, cx<T> d0, int m, int HP,
+                          cx<T>* __restrict__ red, cx<T>* __restrict__ black) {
+  using C = cx<T>;
+  At p;
+  if (!at(m, HP, p)) return;
+  const int o = (p.iy + p.iz + 1) & 1, x = 2 * p.j;
+  C v[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    v[k] = zc<T>();
+    if (x + k < m) {
+      const long long i = p.row * m + x + k;
+      if constexpr (sizeof(T) == 8) {
+        v[k] = dinv[i];
+      } else {
+        const double2 di = dinv[i];
+        const float2 f = make_float2((float)di.x, (float)di.y), t = cmul(cmul(f, f), dc);
+        v[k] = make_float2((float)(di.x - (double)d0.x) - t.x, (float)(di.y - (double)d0.y) - t.y);
+      }
+    }
+  }
+  const long long s = p.row * HP + p.j;
+  st2(red + s, o ? v[1] : v[0], o ? v[3] : v[2]);
+  st2(black + s, o ? v[0] : v[1], o ? v[2] : v[3]);
+}
+
+// Neighbour sum of the interpolated correction P e at the red slots j, j + 1 of
+// row (iy, iz).  Node indices: a red node has an even number of odd indices.
+// All even (a coarse node K): 3 e_K + 1/2 sum of its six coarse neighbours.
+// Two odd: with S4 the sum of the four coarse corners around the point in the
+// plane of its odd axes, 5/4 S4 + 1/8 (S4 one coarse plane up and one down the
+// even axis).  e: coarse values, x first, rows pe elements apart, mc a side.
+template <typename T>
+__device__ __forceinline__ Pair<T> prolong_nbr(const cx<T>* __restrict__ e, int pe, int mc, int j, int iy, int iz) {
+  using C = cx<T>;
+  const bool oy = !(iy & 1), oz = !(iz & 1);           // odd node indices
+  const int Y = (iy + 1) >> 1, Z = (iz + 1) >> 1;      // coarse node at or below
+  auto rowp = [&](int y, int z) -> const C* {
+    return (y >= 1 && y <= mc && z >= 1 && z <= mc) ? e + ((long long)(z - 1) * mc + (y - 1)) * pe - 1 : nullptr;
+  };
+  auto val = [&](const C* r, int X) -> C { return (r && X >= 1 && X <= mc) ? r[X] : zc<T>(); };
+  Pair<T> out;
+  if (oy == oz) {                                      // x even: coarse columns j + 1 and j + 2
+    const int X = j + 1;
+    if (!oy) {
+      const C* r = rowp(Y, Z);
+      const C e0 = val(r, X - 1), e1 = val(r, X), e2 = val(r, X + 1), e3 = val(r, X + 2);
+      C a = cadd(e0, e2), b = cadd(e1, e3);
+      const C *r1 = rowp(Y - 1, Z), *r2 = rowp(Y + 1, Z), *r3 = rowp(Y, Z - 1), *r4 = rowp(Y, Z + 1);
+      a = cadd(a, cadd(cadd(val(r1, X), val(r2, X)), cadd(val(r3, X), val(r4, X))));
+      b = cadd(b, cadd(cadd(val(r1, X + 1), val(r2, X + 1)), cadd(val(r3, X + 1), val(r4, X + 1))));
+      out.a = cadd(cscale(e1, (T)3), cscale(a, (T)0.5));
+      out.b = cadd(cscale(e2, (T)3), cscale(b, (T)0.5));
+    } else {
+      const C *r1 = rowp(Y, Z), *r2 = rowp(Y + 1, Z), *r3 = rowp(Y, Z + 1), *r4 = rowp(Y + 1, Z + 1);
+      C s[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        s[k] = cadd(cadd(val(r1, X - 1 + k), val(r2, X - 1 + k)), cadd(val(r3, X - 1 + k), val(r4, X - 1 + k)));
+      out.a = cadd(cscale(s[1], (T)1.25), cscale(cadd(s[0], s[2]), (T)0.125));
+      out.b = cadd(cscale(s[2], (T)1.25), cscale(cadd(s[1], s[3]), (T)0.125));
+    }
+  } else {                                             // x odd: between coarse columns j and j + 1 (j + 1 and j + 2)
+    C t0[3], t1[3];                                    // S4 at the even axis' plane below, at, above
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const C *r1, *r2;
+      if (oy) {
+        r1 = rowp(Y, Z - 1 + k);
+        r2 = rowp(Y + 1, Z - 1 + k);
+      } else {
+        r1 = rowp(Y - 1 + k, Z);
+        r2 = rowp(Y - 1 + k, Z + 1);
+      }
+      const C c0 = cadd(val(r1, j), val(r2, j)), c1 = cadd(val(r1, j + 1), val(r2, j + 1)),
+              c2 = cadd(val(r1, j + 2), val(r2, j + 2));
+      t0[k] = cadd(c0, c1);
+      t1[k] = cadd(c1, c2);
+    }
+    out.a = cadd(cscale(t0[1], (T)1.25), cscale(cadd(t0[0], t0[2]), (T)0.125));
+    out.b = cadd(cscale(t1[1], (T)1.25), cscale(cadd(t1[0], t1[2]), (T)0.125));
+  }
+  return out;
+}
+
+// One colour of a sweep: u <- d^{-1} (b + c sum_nbr u), uo the other colour.
+//  PLAIN: u
+//  PROLONG (red): the neighbours are u + P e
+//  DELTA (black): also delta = u_new - u_old
+//  NAT (black): both colours to nat in natural order (rows nat_pitch apart); the
+//  split black values too when u
+enum Mode { PLAIN, PROLONG, DELTA, NAT };
+template <typename T, int COLOUR, int MODE>
+__global__ void k3s_sweep(const cx<T>* __restrict__ uo, const cx<T>* __restrict__ b, const cx<T>* __restrict__ dinv,
+                          cx<T> c, cx<T> d0, int m, int HP, cx<T>* u, cx<T>* __restrict__ delta,
+                          const cx<T>* __restrict__ e, int pe, int mc, cx<T>* __restrict__ nat, int nat_pitch) {
+  using C = cx<T>;
+  pdl_prologue();
+  At p;
+  if (!at(m, HP, p)) return;
+  const int o = (p.iy + p.iz + 1 + COLOUR) & 1;
+  const long long s = p.row * HP + p.j;
+  const long long plane = (long long)m * HP;
+  const Pair<T> zero{zc<T>(), zc<T>()};
+  const Pair<T> mid = ld2(uo + s);
+  const int je = o ? p.j + 2 : p.j - 1;                 // the row's third neighbour slot
+  const C edge = (je >= 0 && je < HP) ? uo[s + (je - p.j)] : zc<T>();
+  const Pair<T> yl = p.iy > 0 ? ld2(uo + s - HP) : zero, yr = p.iy < m - 1 ? ld2(uo + s + HP) : zero;
+  const Pair<T> zl = p.iz > 0 ? ld2(uo + s - plane) : zero, zr = p.iz < m - 1 ? ld2(uo + s + plane) : zero;
+  const Pair<T> bv = ld2(b + s), dv = ld2(dinv + s);
+  Pair<T> old = zero;
+  if constexpr (MODE == DELTA) old = ld2(u + s);
+  // x - 1 and x + 1 of both slots
+  const C a0 = o ? mid.a : edge, a1 = o ? mid.b : mid.a, b0 = o ? mid.b : mid.a, b1 = o ? edge : mid.b;
+  // pairs first: fewer roundings of large partial sums
+  C s0 = cadd(cadd(cadd(a0, a1), cadd(yl.a, yr.a)), cadd(zl.a, zr.a));
+  C s1 = cadd(cadd(cadd(b0, b1), cadd(yl.b, yr.b)), cadd(zl.b, zr.b));
+  if constexpr (MODE == PROLONG) {
+    const Pair<T> q = prolong_nbr<T>(e, pe, mc, p.j, p.iy, p.iz);
+    s0 = cadd(s0, q.a);
+    s1 = cadd(s1, q.b);
+  }
+  const int x0 = 2 * p.j + o, x1 = x0 + 2;
+  const C v0 = x0 < m ? dinv_mul(d0, dv.a, cfma(bv.a, c, s0)) : zc<T>();
+  const C v1 = x1 < m ? dinv_mul(d0, dv.b, cfma(bv.b, c, s1)) : zc<T>();
+  if (MODE != NAT || u) st2(u + s, v0, v1);
+  if constexpr (MODE == DELTA) st2(delta + s, csub(v0, old.a), csub(v1, old.b));
+  if constexpr (MODE == NAT) {
+    C* n = nat + p.row * nat_pitch + 2 * p.j;
+    const C w[4] = {o ? mid.a : v0, o ? v0 : mid.a, o ? mid.b : v1, o ? v1 : mid.b};
+    if (nat_pitch == 2 * HP) {
+      st2(n, w[0], w[1]);
+      st2(n + 2, w[2], w[3]);
+    } else {
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (2 * p.j + k < m) n[k] = w[k];
+    }
+  }
+}
+
+// Full weighting of the red residual c sum_nbr delta into the coarse level:
+// its b in both colours and the red half sweep u = d^{-1} b from zero, or (the
+// coarsest level, nat) b in natural order.  A thread takes the coarse points
+// P, P + 1 (P even) of a row: one of them red.
+template <typename T>
+__global__ void k3s_restrict(const cx<T>* __restrict__ delta, int m, int HP, cx<T> c, int mc, int HPc,
+                             cx<T>* __restrict__ br, cx<T>* __restrict__ bb, const cx<T>* __restrict__ dr,
+                             cx<T> d0, cx<T>* __restrict__ ur, cx<T>* __restrict__ nat) {
+  using C = cx<T>;
+  pdl_prologue();
+  const int P = 2 * (int)(blockIdx.x * blockDim.x + threadIdx.x);
+  const int Yc = blockIdx.y * blockDim.y + threadIdx.y, Zc = blockIdx.z;
+  if (P >= mc || Yc >= mc) return;
+  const int fy = 2 * Yc + 1, fz = 2 * Zc + 1;
+  const Pair<T> zero{zc<T>(), zc<T>()};
+  auto rowp = [&](int dy, int dz) -> const C* {
+    const int y = fy + dy, z = fz + dz;
+    return (y >= 0 && y < m && z >= 0 && z < m) ? delta + ((long long)z * m + y) * HP + P : nullptr;
+  };
+  // slots P, P + 1 of a row; the pair's neighbours: slot P - 1 and P + 2
+  auto pair = [&](const C* r) { return r ? ld2(r) : zero; };
+  auto right = [&](const C* r) { return (r && P + 2 < HP) ? r[2] : zc<T>(); };
+  auto left = [&](const C* r) { return (r && P > 0) ? r[-1] : zc<T>(); };
+  C f0 = zc<T>(), f1 = f0, g0 = f0, g1 = f0, h0 = f0, h1 = f0;      // distance (1,0,0), (1,1,1), (2,1,0)
+  auto add = [](C& x, C& y, C u, C v) { x = cadd(x, u); y = cadd(y, v); };
+  {                                                    // own row: x offsets -1 and +1
+    const C* r = rowp(0, 0);
+    const Pair<T> v = ld2(r);
+    add(f0, f1, cadd(v.a, v.b), cadd(v.b, right(r)));
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {                        // one unit off in y or z: x offset 0, and -2, +2
+    const int s = (k & 1) ? 1 : -1;
+    const C* r = (k < 2) ? rowp(s, 0) : rowp(0, s);
+    const Pair<T> v = pair(r);
+    add(f0, f1, v.a, v.b);
+    add(h0, h1, cadd(left(r), v.b), cadd(v.a, right(r)));
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {                        // one unit off in both: x offsets -1 and +1
+    const C* r = rowp((k & 1) ? 1 : -1, (k & 2) ? 1 : -1);
+    const Pair<T> v = pair(r);
+    add(g0, g1, cadd(v.a, v.b), cadd(v.b, right(r)));
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {                        // two units off in one: x offsets -1 and +1
+    const int s = (k & 1) ? 2 : -2;
+    const C* r = (k < 2) ? rowp(s, 0) : rowp(0, s);
+    const Pair<T> v = pair(r);
+    add(h0, h1, cadd(v.a, v.b), cadd(v.b, right(r)));
+  }
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {                        // two and one: x offset 0
+    const int s = (k & 1) ? 1 : -1, s2 = (k & 2) ? 2 : -2;
+    const Pair<T> v = pair((k & 4) ? rowp(s2, s) : rowp(s, s2));
+    add(h0, h1, v.a, v.b);
+  }
+  const C w0 = cadd(cadd(cscale(f0, (T)0.25), cscale(g0, (T)0.09375)), cscale(h0, (T)0.03125));
+  const C w1 = cadd(cadd(cscale(f1, (T)0.25), cscale(g1, (T)0.09375)), cscale(h1, (T)0.03125));
+  const C v0 = cmul(c, w0), v1 = P + 1 < mc ? cmul(c, w1) : zc<T>();
+  const long long row = (long long)Zc * mc + Yc;
+  if (nat) {
+    nat[row * mc + P] = v0;
+    if (P + 1 < mc) nat[row * mc + P + 1] = v1;
+    return;
+  }
+  const int o = (Yc + Zc + 1) & 1;                     // red parity of the coarse row
+  const long long s = row * HPc + (P >> 1);
+  const C vr = o ? v1 : v0;
+  br[s] = vr;
+  bb[s] = o ? v0 : v1;
+  ur[s] = dinv_mul(d0, dr[s], vr);
+}
+
+struct Shape { dim3 g, b; };
+// threads along x cover a row's slot pairs, rows fill the block up to 256
+// threads (128 on small levels, whose passes last one CTA's lifetime)
+Shape shape(int pairs, int m) {
+  const int tx = pairs < 128 ? pairs : 128;
+  const int want = m >= 127 ? 256 : 128;
+  int ty = want / tx;
+  ty = ty < 1 ? 1 : (ty > m ? m : ty);
+  return Shape{dim3((pairs + tx - 1) / tx, (m + ty - 1) / ty, m), dim3(tx, ty)};
+}
+
+template <typename T> Split3<T>& sp(Level& L);
+template <> Split3<float>& sp<float>(Level& L) { return L.s32; }
+template <> Split3<double>& sp<double>(Level& L) { return L.s64; }
+template <typename T> cx<T>* nat_u(Level& L);
+template <> float2* nat_u<float>(Level& L) { return L.u32; }
+template <> double2* nat_u<double>(Level& L) { return L.u64; }
+template <typename T> cx<T>* nat_b(Level& L);
+template <> float2* nat_b<float>(Level& L) { return L.b32; }
+template <> double2* nat_b<double>(Level& L) { return L.b64; }
+
+}  // namespace
+
+int split3_pitch(int m) { return ((m + 1) / 2 + 3) / 4 * 4; }
+
+template <typename T>
+cudaError_t split3_coefs(Level& L, double k2, cudaStream_t s) {
+  const int HP = split3_pitch(L.m);
+  const Shape h = shape(HP / 2, L.m);
+  Split3<T>& S = sp<T>(L);
+  const cx<T> c = mk<cx<T>>((T)L.c.x, (T)L.c.y);
+  const double dx = 6.0 * (double)c.x - k2, dy = 6.0 * (double)c.y, den = dx * dx + dy * dy;
+  S.d0 = den > 0.0 ? mk<cx<T>>((T)(dx / den), (T)(-dy / den)) : mk<cx<T>>((T)0, (T)0);
+  const float2 dc = make_float2((float)(6.0 * ((double)c.x - L.c.x)), (float)(6.0 * ((double)c.y - L.c.y)));
+  k3s_split<T><<<h.g, h.b, 0, s>>>(L.dinv64, dc, S.d0, L.m, HP, S.dr, S.db);
+  count_launch();
+  return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t launch_split3_down(std::vector<Level>& lv, const cx<T>* u, const cx<T>* b, bool zero_init, bool new_b,
+                               cudaStream_t s) {
+  cudaError_t e = cudaSuccess;
+  int launches = 0;
+  auto ok = [&](cudaError_t r) { ++launches; if (e == cudaSuccess) e = r; };
+  const int nl = (int)lv.size();
+  const double S = sizeof(cx<T>);
+  for (int l = 0; l + 1 < nl && e == cudaSuccess; ++l) {
+    Level &L = lv[l], &C = lv[l + 1];
+    Split3<T>&F = sp<T>(L), &G = sp<T>(C);
+    const int m = L.m, HP = split3_pitch(m), HPc = split3_pitch(C.m);
+    const cx<T> c = mk<cx<T>>((T)L.c.x, (T)L.c.y);
+    const Shape h = shape(HP / 2, m), hc = shape((C.m + 1) / 2, C.m);
+    const cx<T>* none = nullptr;
+    cx<T>* no = nullptr;
+    const bool zero = zero_init || l > 0;
+    ProfScope ps(mg_family<T>(), s, (zero ? 3.5 : 6.0) * S * L.N + S * C.N, 0);
+    if (l == 0) {
+      if (new_b || u)
+        ok(launch_pdl(k3s_import<T>, h.g, h.b, 0, s, b, zero ? none : u, zero ? (const cx<T>*)F.dr : none, F.d0, m, HP, F.br,
+                      F.bb, F.ub, F.ur));
+      if (!zero)
+        ok(launch_pdl(k3s_sweep<T, 0, PLAIN>, h.g, h.b, 0, s, (const cx<T>*)F.ub, (const cx<T>*)F.br,
+                      (const cx<T>*)F.dr, c, F.d0, m, HP, F.ur, no, none, 0, 0, no, 0));
+    }
+    if (zero)
+      ok(launch_pdl(k3s_sweep<T, 1, PLAIN>, h.g, h.b, 0, s, (const cx<T>*)F.ur, (const cx<T>*)F.bb, (const cx<T>*)F.db,
+                    c, F.d0, m, HP, F.ub, no, none, 0, 0, no, 0));
+    else
+      ok(launch_pdl(k3s_sweep<T, 1, DELTA>, h.g, h.b, 0, s, (const cx<T>*)F.ur, (const cx<T>*)F.bb, (const cx<T>*)F.db,
+                    c, F.d0, m, HP, F.ub, F.delta, none, 0, 0, no, 0));
+    ok(launch_pdl(k3s_restrict<T>, hc.g, hc.b, 0, s, (const cx<T>*)(zero ? F.ub : F.delta), m, HP, c, C.m, HPc, G.br,
+                  G.bb, (const cx<T>*)G.dr, G.d0, G.ur, l + 2 == nl ? nat_b<T>(C) : no));
+  }
+  count_launch(launches);
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t launch_split3_up(std::vector<Level>& lv, cx<T>* u_nat, bool keep_split, cudaStream_t s) {
+  cudaError_t e = cudaSuccess;
+  int launches = 0;
+  auto ok = [&](cudaError_t r) { ++launches; if (e == cudaSuccess) e = r; };
+  const int nl = (int)lv.size();
+  const double S = sizeof(cx<T>);
+  for (int l = nl - 2; l >= 0 && e == cudaSuccess; --l) {
+    Level &L = lv[l], &C = lv[l + 1];
+    Split3<T>&F = sp<T>(L), &G = sp<T>(C);
+    const int m = L.m, HP = split3_pitch(m);
+    const cx<T> c = mk<cx<T>>((T)L.c.x, (T)L.c.y);
+    const Shape h = shape(HP / 2, m);
+    const bool last = l + 2 == nl;
+    const cx<T>* ev = last ? nat_u<T>(C) : G.e;
+    const cx<T>* none = nullptr;
+    cx<T>* no = nullptr;
+    ProfScope ps(mg_family<T>(), s, 5.0 * S * L.N + S * C.N, 0);
+    ok(launch_pdl(k3s_sweep<T, 0, PROLONG>, h.g, h.b, 0, s, (const cx<T>*)F.ub, (const cx<T>*)F.br,
+                  (const cx<T>*)F.dr, c, F.d0, m, HP, F.ur, no, ev, last ? C.m : 2 * split3_pitch(C.m), C.m, no, 0));
+    if (l == 0 && !u_nat)
+      ok(launch_pdl(k3s_sweep<T, 1, PLAIN>, h.g, h.b, 0, s, (const cx<T>*)F.ur, (const cx<T>*)F.bb, (const cx<T>*)F.db,
+                    c, F.d0, m, HP, F.ub, no, none, 0, 0, no, 0));
+    else
+      ok(launch_pdl(k3s_sweep<T, 1, NAT>, h.g, h.b, 0, s, (const cx<T>*)F.ur, (const cx<T>*)F.bb, (const cx<T>*)F.db,
+                    c, F.d0, m, HP, l == 0 && keep_split ? F.ub : no, no, none, 0, 0, l == 0 ? u_nat : F.e,
+                    l == 0 ? m : 2 * HP));
+  }
+  count_launch(launches);
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+#define CSFF_SPLIT3_INST(T)                                                                                      \
+  template cudaError_t split3_coefs<T>(Level&, double, cudaStream_t);                                                 \
+  template cudaError_t launch_split3_down<T>(std::vector<Level>&, const cx<T>*, const cx<T>*, bool, bool,        \
+                                             cudaStream_t);                                                     \
+  template cudaError_t launch_split3_up<T>(std::vector<Level>&, cx<T>*, bool, cudaStream_t);
+CSFF_SPLIT3_INST(float)
+CSFF_SPLIT3_INST(double)
+
+}  // namespace csff

@@ -1,0 +1,74 @@
+"""Edges of the kernels' size ranges against the CPU oracle: one V-cycle on
+grids whose coarse-level block has one to four levels, even and odd coarsest
+grids, staged and unstaged coarsest inverses, and the far-field and learned
+paths at tile remainders."""
+import math
+
+import numpy as np
+import pytest
+
+import workloads as W
+from oracle import csff_oracle as O
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def csff():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1211_4461_gb300 as m
+    return m
+
+
+def _problem(dim, n, k, R=5.0):
+    return W.problem(dim, n, R, math.pi / 6, k, [W.gauss(-0.7, 1.5), W.gauss(-0.3, 1.0, (0.5, -0.4, 0.2))])
+
+
+def _vcycle_pair(csff, prob, opts, dtype, seed=3):
+    plan = csff.Plan(prob, opts)
+    u0 = W.rand_complex(plan.N, seed)
+    b = W.rand_complex(plan.N, seed + 1)
+    np_t = np.complex128 if dtype == torch.complex128 else np.complex64
+    u = torch.from_numpy(u0.astype(np_t)).cuda()
+    bt = torch.from_numpy(b.astype(np_t)).cuda()
+    plan.vcycle(u, bt)
+    plan.close()
+    levels = O.make_hierarchy(O.problem_from_dict(prob), opts["coarsest_n"])
+    shape = (levels[0].m,) * prob["dim"]
+    ref = O.vcycle(levels, O.coarse_factor(levels[-1]), 0, u0.astype(np_t).astype(np.complex128).reshape(shape),
+                   b.astype(np_t).astype(np.complex128).reshape(shape), O.opts_from_dict(opts))
+    return u.cpu().numpy().astype(np.complex128).ravel(), ref.ravel()
+
+
+# coarsest grids of 3 (one unknown), 4 and 6 (even), 9 (inverse staged), 17 and
+# 18 (the FP64 inverse does not fit shared memory; 18: the block is the direct
+# solve alone)
+@pytest.mark.parametrize("n,coarsest", [(65, 3), (49, 4), (41, 6), (65, 9), (65, 17), (69, 18)])
+@pytest.mark.parametrize("prec", ["fp64", "df", "mixed64"])
+def test_vcycle_over_coarse_blocks(csff, n, coarsest, prec):
+    opts = {"smoother": "rbgs", "omega": 1.0, "nu1": 1, "nu2": 1, "coarsest_n": coarsest, "rel_tol": 1e-8,
+            "max_cycles": 100, "precision": "fp64" if prec == "fp64" else "mixed",
+            "refine_fp64": int(prec == "mixed64")}
+    got, ref = _vcycle_pair(csff, _problem(2, n, 1.0), opts,
+                            torch.complex128 if prec == "fp64" else torch.complex64)
+    # FP64: rounding of a cycle's few dozen operations a point and of the
+    # coarsest inverse; FP32: the same in 2^-24, coefficients included
+    tol = 1e-11 if prec == "fp64" else 1e-4
+    assert np.linalg.norm(got - ref) <= tol * np.linalg.norm(ref)
+
+
+# 3D V(1,1) cycles on colour-split arrays: rows of one slot pair (5 nodes) up
+# to several, row lengths that are no multiple of the pitch's four slots, one
+# level above the direct solve and several, even coarsest grids
+@pytest.mark.parametrize("n,coarsest", [(5, 3), (7, 4), (9, 3), (13, 4), (21, 6), (29, 8), (33, 5)])
+@pytest.mark.parametrize("prec", ["fp64", "df", "mixed64"])
+def test_vcycle_3d_by_colour(csff, n, coarsest, prec):
+    opts = {"smoother": "rbgs", "omega": 1.0, "nu1": 1, "nu2": 1, "coarsest_n": coarsest, "rel_tol": 1e-8,
+            "max_cycles": 100, "precision": "fp64" if prec == "fp64" else "mixed",
+            "refine_fp64": int(prec == "mixed64")}
+    got, ref = _vcycle_pair(csff, _problem(3, n, 1.0, R=3.0), opts,
+                            torch.complex128 if prec == "fp64" else torch.complex64)
+    tol = 1e-11 if prec == "fp64" else 1e-4
+    assert np.linalg.norm(got - ref) <= tol * np.linalg.norm(ref)
