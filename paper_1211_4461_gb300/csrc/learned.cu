@@ -299,23 +299,18 @@ __global__ void __launch_bounds__(128) k_conv_tc(Geom g, const __nv_bfloat16* __
 }
 
 // ---- loss: E = mask (r - A y); per-patch sums |E|^2 and |r|^2 over the mask
-__device__ __forceinline__ bool in_mask(const Geom& g, long long p, int margin) {
-  int j = (int)(p % g.W);
-  int i = (int)((p / g.W) % g.H);
-  return i >= margin && i < g.H - margin && j >= margin && j < g.W - margin;
+__device__ __forceinline__ bool in_mask(const Geom& g, Pix c, int margin) {
+  return c.i >= margin && c.i < g.H - margin && c.j >= margin && c.j < g.W - margin;
 }
 
-__device__ __forceinline__ float2 apply_A_patch(const Geom& g, const float2* v, long long p, float2 q, float2 c,
-                                                bool conj_in) {
-  auto ld = [&](long long k) {
-    float2 x = v[k];
-    return conj_in ? make_float2(x.x, -x.y) : x;
-  };
+// (A v)(p) for the patch operator c (4 v - sum_nbr v) - q v, v read through ld
+template <typename LD>
+__device__ __forceinline__ float2 apply_A_patch(const Geom& g, LD ld, Pix pc, long long p, float2 q, float2 c) {
   float2 s = make_float2(0.f, 0.f);
   for (int t = 0; t < 4; ++t) {
     int a = (t == 0) ? 0 : (t == 1) ? 2 : 1;
     int b = (t == 2) ? 0 : (t == 3) ? 2 : 1;
-    long long k = nbr(g, p, a, b);
+    long long k = nbr_at(g, pc, p, a, b);
     if (k >= 0) s = cadd(s, ld(k));
   }
   float2 vj = ld(p);
@@ -323,133 +318,267 @@ __device__ __forceinline__ float2 apply_A_patch(const Geom& g, const float2* v, 
   return csub(cmul(c, t), cmul(q, vj));
 }
 
-__global__ void k_loss1(Geom g, const float2* __restrict__ y, const float2* __restrict__ r,
-                        const float2* __restrict__ q, const float2* __restrict__ cpatch, int margin,
-                        float2* __restrict__ E, double* __restrict__ sums /* [B][2]: |E|^2, |r|^2 */) {
-  long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (p >= g.npix()) return;
-  int bpatch = (int)(p / ((long long)g.H * g.W));
-  float2 e = make_float2(0.f, 0.f);
-  if (in_mask(g, p, margin)) {
-    float2 rv = r[p];
-    e = csub(rv, apply_A_patch(g, y, p, q[p], cpatch[bpatch], false));
-    atomicAdd(&sums[2 * bpatch + 0], (double)e.x * e.x + (double)e.y * e.y);
-    atomicAdd(&sums[2 * bpatch + 1], (double)rv.x * rv.x + (double)rv.y * rv.y);
-  }
-  E[p] = e;
-}
-
-// dy = -conj(A conj(G)), G = 2 E / (S_r B)   (A is complex symmetric)
-__global__ void k_loss2(Geom g, const float2* __restrict__ E, const double* __restrict__ sums,
-                        const float2* __restrict__ q, const float2* __restrict__ cpatch, float2* __restrict__ G,
-                        float2* __restrict__ dy, int phase) {
-  long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (p >= g.npix()) return;
-  int bpatch = (int)(p / ((long long)g.H * g.W));
-  if (phase == 0) {
-    double sr = sums[2 * bpatch + 1];
-    float sc = sr > 0 ? (float)(2.0 / (sr * g.B)) : 0.f;
-    G[p] = cscale(E[p], sc);
-  } else {
-    float2 a = apply_A_patch(g, G, p, q[p], cpatch[bpatch], true);
-    dy[p] = make_float2(-a.x, a.y);     // -conj(a)
-  }
-}
-
-// input gradient of layer 3: dh2[c] = sum_o sum_ab w3[o][c][a][b] dy[o](p - (a-1, b-1)), masked by h2 > 0
-__global__ void k_bwd3(Geom g, const float2* __restrict__ dy, const __nv_bfloat16* __restrict__ w3,
-                       const __nv_bfloat16* __restrict__ h2, float* __restrict__ dh2) {
-  __shared__ float ws[NP3];
-  for (int i = threadIdx.x; i < NP3; i += blockDim.x) ws[i] = __bfloat162float(w3[i]);
-  __syncthreads();
-  long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (p >= g.npix()) return;
-  float acc[16];
-#pragma unroll
-  for (int c = 0; c < 16; ++c) acc[c] = 0.f;
-  for (int a = 0; a < 3; ++a)
-    for (int b = 0; b < 3; ++b) {
-      long long q = nbr(g, p, 2 - a, 2 - b);      // out pixel p - (a-1, b-1)
-      if (q < 0) continue;
-      float2 d = dy[q];
-#pragma unroll
-      for (int c = 0; c < 16; ++c)
-        acc[c] = fmaf(ws[(0 * 16 + c) * 9 + a * 3 + b], d.x, fmaf(ws[(1 * 16 + c) * 9 + a * 3 + b], d.y, acc[c]));
+// Blocks bpp a patch; the sums are reduced over the CTA before one atomic each:
+// an atomic per pixel on two counters a patch took 97 us for 32 patches of 64^2.
+__global__ void __launch_bounds__(NTH) k_loss1(Geom g, const float2* __restrict__ y, const float2* __restrict__ r,
+                                               const float2* __restrict__ q, const float2* __restrict__ cpatch,
+                                               int margin, int bpp, float2* __restrict__ E,
+                                               double* __restrict__ sums /* [B][2]: |E|^2, |r|^2 */) {
+  __shared__ double2 sh[NTH / 32];
+  const int hw = g.H * g.W, bpatch = blockIdx.x / bpp;
+  const int i = (blockIdx.x - bpatch * bpp) * NTH + threadIdx.x;
+  double2 acc = make_double2(0.0, 0.0);
+  if (i < hw) {
+    const long long p = (long long)bpatch * hw + i;
+    const Pix pc{i / g.W, i % g.W};
+    float2 e = make_float2(0.f, 0.f);
+    if (in_mask(g, pc, margin)) {
+      const float2 rv = r[p];
+      e = csub(rv, apply_A_patch(g, [&](long long k) { return y[k]; }, pc, p, q[p], cpatch[bpatch]));
+      acc.x = (double)e.x * e.x + (double)e.y * e.y;
+      acc.y = (double)rv.x * rv.x + (double)rv.y * rv.y;
     }
-#pragma unroll
-  for (int c = 0; c < 16; ++c) dh2[p * 16 + c] = __bfloat162float(h2[p * 16 + c]) > 0.f ? acc[c] : 0.f;
+    E[p] = e;
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
+    acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
+  }
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
+  __syncthreads();
+  if (threadIdx.x < 2) {
+    double v = 0.0;
+    for (int w = 0; w < NTH / 32; ++w) v += threadIdx.x ? sh[w].y : sh[w].x;
+    if (v != 0.0) atomicAdd(&sums[2 * bpatch + threadIdx.x], v);
+  }
 }
 
-// input gradient of layer 2, masked by h1 > 0
-__global__ void k_bwd2(Geom g, const float* __restrict__ dh2, const __nv_bfloat16* __restrict__ w2,
-                       const __nv_bfloat16* __restrict__ h1, float* __restrict__ dh1) {
-  __shared__ float ws[NP2];
-  for (int i = threadIdx.x; i < NP2; i += blockDim.x) ws[i] = __bfloat162float(w2[i]);
+// dy = -conj(A conj(G)), G = 2 E / (S_r B) formed as it is read (A is complex
+// symmetric)
+__global__ void __launch_bounds__(NTH) k_loss2(Geom g, const float2* __restrict__ E, const double* __restrict__ sums,
+                                               const float2* __restrict__ q, const float2* __restrict__ cpatch,
+                                               int bpp, float2* __restrict__ dy) {
+  const int hw = g.H * g.W, bpatch = blockIdx.x / bpp;
+  const int i = (blockIdx.x - bpatch * bpp) * NTH + threadIdx.x;
+  if (i >= hw) return;
+  const long long p = (long long)bpatch * hw + i;
+  const Pix pc{i / g.W, i % g.W};
+  const double sr = sums[2 * bpatch + 1];
+  const float sc = sr > 0 ? (float)(2.0 / (sr * g.B)) : 0.f;
+  auto ld = [&](long long k) {
+    const float2 x = cscale(E[k], sc);
+    return make_float2(x.x, -x.y);
+  };
+  const float2 a = apply_A_patch(g, ld, pc, p, q[p], cpatch[bpatch]);
+  dy[p] = make_float2(-a.x, a.y);     // -conj(a)
+}
+
+__device__ __forceinline__ void unpack16(const __nv_bfloat16* src, float* x) {
+  const uint4 a = reinterpret_cast<const uint4*>(src)[0], b = reinterpret_cast<const uint4*>(src)[1];
+  const __nv_bfloat162* pa = reinterpret_cast<const __nv_bfloat162*>(&a);
+  const __nv_bfloat162* pb = reinterpret_cast<const __nv_bfloat162*>(&b);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const float2 fa = __bfloat1622float2(pa[i]), fb = __bfloat1622float2(pb[i]);
+    x[2 * i] = fa.x;
+    x[2 * i + 1] = fa.y;
+    x[8 + 2 * i] = fb.x;
+    x[8 + 2 * i + 1] = fb.y;
+  }
+}
+
+// acc[0..15] += v w[0..15] on the packed two-lane instructions (w: 16-byte
+// broadcast loads, four for 16 multiply-adds)
+__device__ __forceinline__ void fma16(float2 (&acc)[8], float v, const float4* w) {
+  const float2 vv = make_float2(v, v);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const float4 x = w[k];
+    acc[2 * k] = __ffma2_rn(vv, make_float2(x.x, x.y), acc[2 * k]);
+    acc[2 * k + 1] = __ffma2_rn(vv, make_float2(x.z, x.w), acc[2 * k + 1]);
+  }
+}
+// acc masked by h > 0, as four 16-byte stores
+__device__ __forceinline__ void store16_mask(float* dst, const __nv_bfloat16* h, const float2 (&acc)[8]) {
+  float hv[16];
+  unpack16(h, hv);
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+    reinterpret_cast<float4*>(dst)[k] =
+        make_float4(hv[4 * k] > 0.f ? acc[2 * k].x : 0.f, hv[4 * k + 1] > 0.f ? acc[2 * k].y : 0.f,
+                    hv[4 * k + 2] > 0.f ? acc[2 * k + 1].x : 0.f, hv[4 * k + 3] > 0.f ? acc[2 * k + 1].y : 0.f);
+}
+
+// Input gradients, each pixel's 16 channels in a thread's registers; the
+// weights sit in shared memory as [tap][out][in], so the 16 input weights of
+// one (tap, output channel) are four broadcast loads.  A 16-byte shared load
+// costs as many cycles as four plain ones even when it is a broadcast, so
+// layer 2 (2304 multiply-adds a pixel) is bound by them and a thread takes two
+// pixels: 24 us for 32 patches of 64^2, 31 with one pixel, 83 with scalar loads.
+constexpr int BW_NT = 128;
+// layer 3: dh2[c] = sum_o sum_ab w3[o][c][a][b] dy[o](p - (a-1, b-1)), masked by h2 > 0
+__global__ void __launch_bounds__(BW_NT) k_bwd3(Geom g, const float2* __restrict__ dy,
+                                                const __nv_bfloat16* __restrict__ w3,
+                                                const __nv_bfloat16* __restrict__ h2, float* __restrict__ dh2) {
+  __shared__ __align__(16) float ws[9][2][16];
+  for (int i = threadIdx.x; i < NP3; i += BW_NT) ws[i % 9][i / 144][(i / 9) % 16] = __bfloat162float(w3[i]);
   __syncthreads();
-  long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  const long long p = blockIdx.x * (long long)BW_NT + threadIdx.x;
   if (p >= g.npix()) return;
-  float acc[16];
+  const Pix pc = pix_of(g, p);
+  float2 acc[8];
 #pragma unroll
-  for (int c = 0; c < 16; ++c) acc[c] = 0.f;
-  for (int a = 0; a < 3; ++a)
-    for (int b = 0; b < 3; ++b) {
-      long long q = nbr(g, p, 2 - a, 2 - b);
-      if (q < 0) continue;
-      const float* d = dh2 + q * 16;
+  for (int c = 0; c < 8; ++c) acc[c] = make_float2(0.f, 0.f);
 #pragma unroll
-      for (int o = 0; o < 16; ++o) {
-        float dv = d[o];
+  for (int t = 0; t < 9; ++t) {
+    const long long q = nbr_at(g, pc, p, 2 - t / 3, 2 - t % 3);      // out pixel p - (a-1, b-1)
+    if (q < 0) continue;
+    const float2 d = dy[q];
+    fma16(acc, d.x, reinterpret_cast<const float4*>(&ws[t][0][0]));
+    fma16(acc, d.y, reinterpret_cast<const float4*>(&ws[t][1][0]));
+  }
+  store16_mask(dh2 + p * 16, h2 + p * 16, acc);
+}
+
+// layer 2, masked by h1 > 0; the CTA's pixels are [2 BW_NT blockIdx, ..), a
+// thread's two BW_NT apart
+__global__ void __launch_bounds__(BW_NT) k_bwd2(Geom g, const float* __restrict__ dh2,
+                                                const __nv_bfloat16* __restrict__ w2,
+                                                const __nv_bfloat16* __restrict__ h1, float* __restrict__ dh1) {
+  __shared__ __align__(16) float ws[9][16][16];
+  for (int i = threadIdx.x; i < NP2; i += BW_NT) {
+    const int t = i >> 8, o = (i >> 4) & 15, c = i & 15;
+    ws[t][o][c] = __bfloat162float(w2[(o * 16 + c) * 9 + t]);
+  }
+  __syncthreads();
+  const long long np = g.npix(), p0 = blockIdx.x * (long long)(2 * BW_NT) + threadIdx.x, p1 = p0 + BW_NT;
+  if (p0 >= np) return;
+  const Pix c0 = pix_of(g, p0), c1 = p1 < np ? pix_of(g, p1) : Pix{0, 0};
+  float2 acc0[8], acc1[8];
 #pragma unroll
-        for (int c = 0; c < 16; ++c) acc[c] = fmaf(ws[(o * 16 + c) * 9 + a * 3 + b], dv, acc[c]);
+  for (int c = 0; c < 8; ++c) acc0[c] = acc1[c] = make_float2(0.f, 0.f);
+  const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int t = 0; t < 9; ++t) {
+    const long long q0 = nbr_at(g, c0, p0, 2 - t / 3, 2 - t % 3);
+    const long long q1 = p1 < np ? nbr_at(g, c1, p1, 2 - t / 3, 2 - t % 3) : -1;
+#pragma unroll
+    for (int o4 = 0; o4 < 4; ++o4) {
+      const float4 u = q0 >= 0 ? reinterpret_cast<const float4*>(dh2 + q0 * 16)[o4] : z;
+      const float4 v = q1 >= 0 ? reinterpret_cast<const float4*>(dh2 + q1 * 16)[o4] : z;
+      const float d0[4] = {u.x, u.y, u.z, u.w}, d1[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const float4* w = reinterpret_cast<const float4*>(&ws[t][4 * o4 + k][0]);
+        const float4 w4[4] = {w[0], w[1], w[2], w[3]};
+        fma16(acc0, d0[k], w4);
+        fma16(acc1, d1[k], w4);
       }
     }
-#pragma unroll
-  for (int c = 0; c < 16; ++c) dh1[p * 16 + c] = __bfloat162float(h1[p * 16 + c]) > 0.f ? acc[c] : 0.f;
+  }
+  store16_mask(dh1 + p0 * 16, h1 + p0 * 16, acc0);
+  if (p1 < np) store16_mask(dh1 + p1 * 16, h1 + p1 * 16, acc1);
 }
 
-// weight gradient: dw[o][c][a][b] += sum_p dout[p][o] in[c](p + (a-1, b-1)).
+// Weight gradient: dw[o][c][a][b] += sum_p dout[p][o] in[c](p + (a-1, b-1)).
 // INKIND 0: input is bf16(r) (2 channels from float2); 1: bf16 activations.
 // DKIND 0: dout is float2 (2 channels); 1: float[16].
-template <int CIN, int COUT, int INKIND, int DKIND>
-__global__ void k_wgrad(Geom g, const void* __restrict__ in, const void* __restrict__ dout, float* __restrict__ dw) {
-  constexpr int NPAR = COUT * CIN * 9;
-  constexpr int TP = 128;                          // pixels per block
-  __shared__ float sd[TP * COUT];
-  const long long p0 = (long long)blockIdx.x * TP;
-  for (int i = threadIdx.x; i < TP * COUT; i += blockDim.x) {
-    long long p = p0 + i / COUT;
-    int o = i % COUT;
-    float v = 0.f;
-    if (p < g.npix()) {
-      if (DKIND == 0) {
-        float2 d = reinterpret_cast<const float2*>(dout)[p];
-        v = (o == 0) ? d.x : d.y;
-      } else {
-        v = reinterpret_cast<const float*>(dout)[p * COUT + o];
-      }
-    }
-    sd[i] = v;
-  }
+// A thread owns one input channel c and OV output channels and keeps the nine
+// taps' sums of each in registers (9 OV multiply-adds for one vector load of
+// dout and three new input values: the other six taps slide along the row).
+// The threads of a group, (COUT / OV) CIN of them, walk WG_SEG pixels of an
+// image row; the block's groups join in shared memory before one atomic per
+// parameter.  Bound by the latency of a segment's loads and, in layer 2, by
+// the FP32 pipe (302 M multiply-adds for 32 patches of 64^2).  The three
+// layers are ranges of one launch's blocks, since layers 1 and 3 alone fill a
+// fraction of the chip: 47 us, 22 + 20 + 39 launched one by one, 850 with a
+// thread per parameter walking its pixels.
+constexpr int WG_NT = 256, WG_SEG = 32;
+template <int CIN, int COUT, int OV, int INKIND, int DKIND>
+__device__ __forceinline__ void wgrad_body(const Geom& g, const void* __restrict__ in, const void* __restrict__ dout,
+                                           float* __restrict__ dw, int block, int nblocks, float* sh) {
+  constexpr int TPG = COUT / OV * CIN, NG = WG_NT / TPG, NPAR = COUT * CIN * 9;
+  const int grp = threadIdx.x / TPG, l = threadIdx.x % TPG, c = l % CIN, o0 = l / CIN * OV;
+  for (int i = threadIdx.x; i < NPAR; i += WG_NT) sh[i] = 0.f;
   __syncthreads();
-  for (int par = threadIdx.x; par < NPAR; par += blockDim.x) {
-    int o = par / (CIN * 9), rem = par % (CIN * 9), c = rem / 9, ab = rem % 9, a = ab / 3, b = ab % 3;
-    float acc = 0.f;
-    for (int t = 0; t < TP; ++t) {
-      long long p = p0 + t;
-      if (p >= g.npix()) break;
-      long long q = nbr(g, p, a, b);
-      if (q < 0) continue;
-      float x;
-      if (INKIND == 0) {
-        float2 v = reinterpret_cast<const float2*>(in)[q];
-        x = bf(c == 0 ? v.x : v.y);
-      } else {
-        x = __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(in)[q * CIN + c]);
-      }
-      acc = fmaf(sd[t * COUT + o], x, acc);
+  auto input = [&](long long q) -> float {
+    if constexpr (INKIND == 0) {
+      const float2 v = reinterpret_cast<const float2*>(in)[q];
+      return bf(c == 0 ? v.x : v.y);
+    } else {
+      return __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(in)[q * CIN + c]);
     }
-    atomicAdd(&dw[par], acc);
+  };
+  float acc[OV][9];
+#pragma unroll
+  for (int o = 0; o < OV; ++o)
+#pragma unroll
+    for (int t = 0; t < 9; ++t) acc[o][t] = 0.f;
+  const int nseg = (g.W + WG_SEG - 1) / WG_SEG;
+  const long long units = (long long)g.B * g.H * nseg;
+  for (long long un = block * (long long)NG + grp; un < units; un += (long long)nblocks * NG) {
+    const long long row = un / nseg;
+    const int j0 = (int)(un - row * nseg) * WG_SEG, j1 = min(j0 + WG_SEG, g.W), i = (int)(row % g.H);
+    const long long p0 = row * g.W;
+    float x[3][3];                            // input rows i - 1 .. i + 1, columns j - 1 .. j + 1
+    bool in_row[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      in_row[a] = i + a - 1 >= 0 && i + a - 1 < g.H;
+      const long long q = p0 + (long long)(a - 1) * g.W + j0;
+      x[a][1] = in_row[a] && j0 > 0 ? input(q - 1) : 0.f;
+      x[a][2] = in_row[a] ? input(q) : 0.f;
+    }
+#pragma unroll 4
+    for (int j = j0; j < j1; ++j) {
+      const long long p = p0 + j;
+      float d[OV];
+      if constexpr (DKIND == 0) {
+        const float2 v = reinterpret_cast<const float2*>(dout)[p];
+        d[0] = v.x;
+        d[1] = v.y;
+      } else {
+        const float4 v = *reinterpret_cast<const float4*>(reinterpret_cast<const float*>(dout) + p * COUT + o0);
+        d[0] = v.x;
+        d[1] = v.y;
+        d[2] = v.z;
+        d[3] = v.w;
+      }
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        x[a][0] = x[a][1];
+        x[a][1] = x[a][2];
+        x[a][2] = (in_row[a] && j + 1 < g.W) ? input(p + (long long)(a - 1) * g.W + 1) : 0.f;
+      }
+#pragma unroll
+      for (int o = 0; o < OV; ++o)
+#pragma unroll
+        for (int t = 0; t < 9; ++t) acc[o][t] = fmaf(d[o], x[t / 3][t % 3], acc[o][t]);
+    }
   }
+#pragma unroll
+  for (int o = 0; o < OV; ++o)
+#pragma unroll
+    for (int t = 0; t < 9; ++t) {
+#pragma unroll
+      for (int k = 16; k >= TPG; k >>= 1) acc[o][t] += __shfl_xor_sync(0xffffffffu, acc[o][t], k);
+      if (TPG >= 32 || (threadIdx.x & 31) < TPG) atomicAdd(&sh[((o0 + o) * CIN + c) * 9 + t], acc[o][t]);
+    }
+  __syncthreads();
+  for (int i = threadIdx.x; i < NPAR; i += WG_NT) atomicAdd(&dw[i], sh[i]);
+}
+
+// layer 1 on the first n1 blocks, layer 3 on the next n3 (their few long
+// segments start first), layer 2 on the rest
+__global__ void __launch_bounds__(WG_NT, 3) k_wgrad(Geom g, const float2* __restrict__ r,
+                                                 const __nv_bfloat16* __restrict__ h1,
+                                                 const __nv_bfloat16* __restrict__ h2, const float2* __restrict__ dy,
+                                                 const float* __restrict__ dh2, const float* __restrict__ dh1,
+                                                 float* __restrict__ dw, int n1, int n3) {
+  __shared__ float sh[NP2];
+  const int b = blockIdx.x;
+  if (b < n1) wgrad_body<2, 16, 4, 0, 1>(g, r, dh1, dw, b, n1, sh);
+  else if (b < n1 + n3) wgrad_body<16, 2, 2, 1, 0>(g, h2, dy, dw + NP1 + NP2, b - n1, n3, sh);
+  else wgrad_body<16, 16, 4, 1, 1>(g, h1, dh2, dw + NP1, b - n1 - n3, gridDim.x - n1 - n3, sh);
 }
 
 __global__ void k_adam(float* w, float* m, float* v, const float* gr, __nv_bfloat16* wb, int n, float lr,
@@ -534,19 +663,6 @@ __device__ __forceinline__ long long nbr3(const Geom3& g, Vox v, long long p, in
   return p + ((long long)(a - 1) * g.H + (b - 1)) * g.W + (e - 1);
 }
 
-__device__ __forceinline__ void unpack16(const __nv_bfloat16* src, float* x) {
-  const uint4 a = reinterpret_cast<const uint4*>(src)[0], b = reinterpret_cast<const uint4*>(src)[1];
-  const __nv_bfloat162* pa = reinterpret_cast<const __nv_bfloat162*>(&a);
-  const __nv_bfloat162* pb = reinterpret_cast<const __nv_bfloat162*>(&b);
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const float2 fa = __bfloat1622float2(pa[i]), fb = __bfloat1622float2(pb[i]);
-    x[2 * i] = fa.x;
-    x[2 * i + 1] = fa.y;
-    x[8 + 2 * i] = fb.x;
-    x[8 + 2 * i + 1] = fb.y;
-  }
-}
 __device__ __forceinline__ void store16_relu(__nv_bfloat16* dst, const float* acc) {
   __align__(16) __nv_bfloat16 hv[16];
 #pragma unroll
@@ -885,7 +1001,7 @@ struct csff_net {
   __nv_bfloat16 *h1 = nullptr, *h2 = nullptr;
   float *dh1 = nullptr, *dh2 = nullptr;
   float2 *y = nullptr, *E = nullptr, *G = nullptr, *dy = nullptr;
-  double* sums = nullptr;
+  double* sums = nullptr;        // behind grad, in its allocation
   int cap_b = 0;
   float2* cpatch = nullptr;
   int* tcerr = nullptr;          // set when a tensor-core layer's wait ran out
@@ -903,6 +1019,9 @@ csff_status ninvalid(const char* s) {
   csff::set_error(s);
   return CSFF_ERR_INVALID_ARG;
 }
+
+// the weight gradient and, behind it, the loss sums of B patches
+size_t red_bytes(const csff_net* N, int B) { return sizeof(float) * N->nparam + sizeof(double) * 2 * B; }
 
 csff_status ensure_scratch(csff_net* N, long long npix, int B, bool train) {
   if (npix >= (1ll << 31)) return ninvalid("more than 2^31 pixels");
@@ -927,9 +1046,15 @@ csff_status ensure_scratch(csff_net* N, long long npix, int B, bool train) {
     N->cap = cap;
   }
   if (B > N->cap_b) {
-    if (N->sums) cudaFree(N->sums);
+    if (N->grad) cudaFree(N->grad);
+    N->grad = nullptr;
+    N->sums = nullptr;
+    N->cap_b = 0;
     if (N->cpatch) cudaFree(N->cpatch);
-    NK(cudaMalloc((void**)&N->sums, sizeof(double) * 2 * B), "net sums");
+    N->cpatch = nullptr;
+    static_assert(csff::NPARAM % 2 == 0 && csff::NPARAM3 % 2 == 0, "the sums' alignment");
+    NK(cudaMalloc((void**)&N->grad, red_bytes(N, B)), "net gradient and sums");
+    N->sums = reinterpret_cast<double*>(N->grad + N->nparam);
     NK(cudaMalloc((void**)&N->cpatch, sizeof(float2) * B), "net patch constants");
     N->cap_b = B;
   }
@@ -996,8 +1121,28 @@ csff_status forward3(csff_net* N, csff::Geom3 g, const float2* r, float scale, f
   return CSFF_OK;
 }
 
+// loss and gradient to the host (either may be null) in one copy
+csff_status read_loss(csff_net* N, int B, float* loss_host, float* grad_host, cudaStream_t s) {
+  if (!loss_host && !grad_host) return CSFF_OK;
+  const size_t ng = sizeof(float) * N->nparam, from = grad_host ? 0 : ng, bytes = red_bytes(N, loss_host ? B : 0) - from;
+  std::vector<unsigned char> h(bytes);
+  NK(cudaMemcpyAsync(h.data(), reinterpret_cast<unsigned char*>(N->grad) + from, bytes, cudaMemcpyDeviceToHost, s),
+     "loss and gradient");
+  NK(cudaStreamSynchronize(s), "sync");
+  if (grad_host) std::memcpy(grad_host, h.data(), ng);
+  if (loss_host) {
+    double L = 0, v[2];
+    for (int b = 0; b < B; ++b) {
+      std::memcpy(v, h.data() + (ng - from) + sizeof(v) * b, sizeof(v));
+      L += v[1] > 0 ? v[0] / v[1] : 0.0;
+    }
+    *loss_host = (float)(L / B);
+  }
+  return CSFF_OK;
+}
+
 csff_status loss_grad3(csff_net* N, csff::Geom3 g, const float2* r, const float2* q, const double* c_host, int margin,
-                       float* loss_host, cudaStream_t s) {
+                       float* loss_host, float* grad_host, cudaStream_t s) {
   using namespace csff;
   const long long np = g.npix();
   csff_status st = ensure_scratch(N, np, g.B, true);
@@ -1005,8 +1150,7 @@ csff_status loss_grad3(csff_net* N, csff::Geom3 g, const float2* r, const float2
   std::vector<float2> cp(g.B);
   for (int b = 0; b < g.B; ++b) cp[b] = make_float2((float)c_host[2 * b], (float)c_host[2 * b + 1]);
   NK(cudaMemcpyAsync(N->cpatch, cp.data(), sizeof(float2) * g.B, cudaMemcpyHostToDevice, s), "patch constants");
-  NK(cudaMemsetAsync(N->sums, 0, sizeof(double) * 2 * g.B, s), "sums");
-  NK(cudaMemsetAsync(N->grad, 0, sizeof(float) * NPARAM3, s), "grad");
+  NK(cudaMemsetAsync(N->grad, 0, red_bytes(N, g.B), s), "gradient and sums");
   st = forward3(N, g, r, 1.f, N->y, 0, s);
   if (st != CSFF_OK) return st;
   const __nv_bfloat16* w2 = N->wb + NP31;
@@ -1022,15 +1166,7 @@ csff_status loss_grad3(csff_net* N, csff::Geom3 g, const float2* r, const float2
   k3_wgrad<2, 16, 0, 1><<<wb_blocks, NTH, 0, s>>>(g, r, N->dh1, N->grad);
   count_launch(8);
   NK(cudaGetLastError(), "3D net backward");
-  if (loss_host) {
-    std::vector<double> sums(2 * g.B);
-    NK(cudaMemcpyAsync(sums.data(), N->sums, sizeof(double) * 2 * g.B, cudaMemcpyDeviceToHost, s), "loss");
-    NK(cudaStreamSynchronize(s), "sync");
-    double L = 0;
-    for (int b = 0; b < g.B; ++b) L += sums[2 * b + 1] > 0 ? sums[2 * b] / sums[2 * b + 1] : 0.0;
-    *loss_host = (float)(L / g.B);
-  }
-  return CSFF_OK;
+  return read_loss(N, g.B, loss_host, grad_host, s);
 }
 
 // one Adam step on N->grad
@@ -1064,7 +1200,7 @@ csff_status forward_mma(csff_net* N, csff::Geom g, const float2* r, float2* y, c
 
 // loss and weight gradient (into N->grad) for a batch of patches
 csff_status loss_grad(csff_net* N, csff::Geom g, const float2* r, const float2* q, const double* c_host, int margin,
-                      float* loss_host, cudaStream_t s) {
+                      float* loss_host, float* grad_host, cudaStream_t s) {
   using namespace csff;
   const long long np = g.npix();
   csff_status st = ensure_scratch(N, np, g.B, true);
@@ -1072,32 +1208,23 @@ csff_status loss_grad(csff_net* N, csff::Geom g, const float2* r, const float2* 
   std::vector<float2> cp(g.B);
   for (int b = 0; b < g.B; ++b) cp[b] = make_float2((float)c_host[2 * b], (float)c_host[2 * b + 1]);
   NK(cudaMemcpyAsync(N->cpatch, cp.data(), sizeof(float2) * g.B, cudaMemcpyHostToDevice, s), "patch constants");
-  NK(cudaMemsetAsync(N->sums, 0, sizeof(double) * 2 * g.B, s), "sums");
-  NK(cudaMemsetAsync(N->grad, 0, sizeof(float) * NPARAM, s), "grad");
+  NK(cudaMemsetAsync(N->grad, 0, red_bytes(N, g.B), s), "gradient and sums");
   st = forward_stored(N, g, r, N->y, 0, s);
   if (st != CSFF_OK) return st;
   const __nv_bfloat16* w2 = N->wb + NP1;
   const __nv_bfloat16* w3 = N->wb + NP1 + NP2;
-  k_loss1<<<nblk(np), NTH, 0, s>>>(g, N->y, r, q, N->cpatch, margin, N->E, N->sums);
-  k_loss2<<<nblk(np), NTH, 0, s>>>(g, N->E, N->sums, q, N->cpatch, N->G, N->dy, 0);
-  k_loss2<<<nblk(np), NTH, 0, s>>>(g, N->E, N->sums, q, N->cpatch, N->G, N->dy, 1);
-  k_bwd3<<<nblk(np), NTH, 0, s>>>(g, N->dy, w3, N->h2, N->dh2);
-  k_bwd2<<<nblk(np), NTH, 0, s>>>(g, N->dh2, w2, N->h1, N->dh1);
-  const int wb_blocks = (int)((np + 127) / 128);
-  k_wgrad<16, 2, 1, 0><<<wb_blocks, NTH, 0, s>>>(g, N->h2, N->dy, N->grad + NP1 + NP2);
-  k_wgrad<16, 16, 1, 1><<<wb_blocks, NTH, 0, s>>>(g, N->h1, N->dh2, N->grad + NP1);
-  k_wgrad<2, 16, 0, 1><<<wb_blocks, NTH, 0, s>>>(g, r, N->dh1, N->grad);
-  count_launch(8);
+  const int bpp = (g.H * g.W + NTH - 1) / NTH;
+  k_loss1<<<(unsigned)g.B * bpp, NTH, 0, s>>>(g, N->y, r, q, N->cpatch, margin, bpp, N->E, N->sums);
+  k_loss2<<<(unsigned)g.B * bpp, NTH, 0, s>>>(g, N->E, N->sums, q, N->cpatch, bpp, N->dy);
+  k_bwd3<<<(unsigned)((np + BW_NT - 1) / BW_NT), BW_NT, 0, s>>>(g, N->dy, w3, N->h2, N->dh2);
+  k_bwd2<<<(unsigned)((np + 2 * BW_NT - 1) / (2 * BW_NT)), BW_NT, 0, s>>>(g, N->dh2, w2, N->h1, N->dh1);
+  const long long units = (long long)g.B * g.H * ((g.W + WG_SEG - 1) / WG_SEG);
+  auto wblocks = [&](int groups, int cap) { return (int)std::min<long long>((units + groups - 1) / groups, cap); };
+  const int n2 = wblocks(4, 152 * 4), n3 = wblocks(16, 152), n1 = wblocks(32, 152);
+  k_wgrad<<<n2 + n3 + n1, WG_NT, 0, s>>>(g, r, N->h1, N->h2, N->dy, N->dh2, N->dh1, N->grad, n1, n3);
+  count_launch(5);
   NK(cudaGetLastError(), "net backward");
-  if (loss_host) {
-    std::vector<double> sums(2 * g.B);
-    NK(cudaMemcpyAsync(sums.data(), N->sums, sizeof(double) * 2 * g.B, cudaMemcpyDeviceToHost, s), "loss");
-    NK(cudaStreamSynchronize(s), "sync");
-    double L = 0;
-    for (int b = 0; b < g.B; ++b) L += sums[2 * b + 1] > 0 ? sums[2 * b] / sums[2 * b + 1] : 0.0;
-    *loss_host = (float)(L / g.B);
-  }
-  return CSFF_OK;
+  return read_loss(N, g.B, loss_host, grad_host, s);
 }
 
 }  // namespace
@@ -1136,7 +1263,7 @@ void csff_net_destroy(csff_net* N) {
   if (!N) return;
   for (void* p : {(void*)N->w, (void*)N->m, (void*)N->v, (void*)N->grad, (void*)N->wb, (void*)N->h1, (void*)N->h2,
                   (void*)N->dh1, (void*)N->dh2, (void*)N->y, (void*)N->E, (void*)N->G, (void*)N->dy,
-                  (void*)N->sums, (void*)N->cpatch, (void*)N->tcerr})
+                  (void*)N->cpatch, (void*)N->tcerr})
     if (p) cudaFree(p);
   delete N;
 }
@@ -1200,13 +1327,8 @@ csff_status csff_net_loss_grad(csff_net* N, int B, int H, int W, const void* r_d
   if ((long long)B * H * W >= (1ll << 31)) return ninvalid("more than 2^31 pixels");
   cudaStream_t s = (cudaStream_t)stream;
   csff_status st = loss_grad(N, csff::Geom{B, H, W}, (const float2*)r_dev, (const float2*)q_dev, c_host, margin,
-                             loss_host, s);
-  if (st != CSFF_OK) return st;
-  if (grad_host) {
-    NK(cudaMemcpyAsync(grad_host, N->grad, sizeof(float) * csff::NPARAM, cudaMemcpyDeviceToHost, s), "grad");
-    NK(cudaStreamSynchronize(s), "sync");
-  }
-  return CSFF_OK;
+                             loss_host, grad_host, s);
+  return st;
 }
 
 csff_status csff_net_train_step(csff_net* N, int B, int H, int W, const void* r_dev, const void* q_dev,
@@ -1238,13 +1360,9 @@ csff_status csff_net_loss_grad3(csff_net* N, int B, int Z, int H, int W, const v
   const csff::Geom3 g{B, Z, H, W};
   if (g.npix() >= (1ll << 31)) return ninvalid("more than 2^31 voxels");
   cudaStream_t s = (cudaStream_t)stream;
-  csff_status st = loss_grad3(N, g, (const float2*)r_dev, (const float2*)q_dev, c_host, margin, loss_host, s);
-  if (st != CSFF_OK) return st;
-  if (grad_host) {
-    NK(cudaMemcpyAsync(grad_host, N->grad, sizeof(float) * csff::NPARAM3, cudaMemcpyDeviceToHost, s), "grad");
-    NK(cudaStreamSynchronize(s), "sync");
-  }
-  return CSFF_OK;
+  csff_status st = loss_grad3(N, g, (const float2*)r_dev, (const float2*)q_dev, c_host, margin, loss_host,
+                              grad_host, s);
+  return st;
 }
 
 csff_status csff_net_train_step3(csff_net* N, int B, int Z, int H, int W, const void* r_dev, const void* q_dev,

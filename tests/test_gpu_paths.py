@@ -72,3 +72,23 @@ def test_vcycle_3d_by_colour(csff, n, coarsest, prec):
                             torch.complex128 if prec == "fp64" else torch.complex64)
     tol = 1e-11 if prec == "fp64" else 1e-4
     assert np.linalg.norm(got - ref) <= tol * np.linalg.norm(ref)
+
+
+# training gradients: one patch and several, widths around the 256-thread loss
+# blocks and the weight gradient's row groups, non-square patches
+@pytest.mark.parametrize("B,H,Wd,margin", [(1, 9, 9, 4), (1, 1, 1, 0), (2, 17, 15, 3), (5, 16, 16, 2), (3, 33, 40, 4),
+                                           (40, 12, 11, 1)])
+def test_net_gradient_over_patch_shapes(csff, B, H, Wd, margin):
+    import oracle.net_oracle as NO
+    theta = NO.init_params(8)
+    net = csff.Net(theta)
+    r = W.rand_complex((B, H, Wd), 21).astype(np.complex64)
+    q = (W.rand_complex((B, H, Wd), 22, scale=0.3) + 1.4).astype(np.complex64)
+    c = np.array([complex(np.exp(-1j * math.pi / 3) * (1.0 + 0.1 * b)) for b in range(B)])
+    L, g = net.loss_grad(torch.from_numpy(r).cuda(), torch.from_numpy(q).cuda(), c, margin=margin)
+    tb = torch.from_numpy(theta.astype(np.float32)).to(torch.bfloat16).to(torch.float64).numpy()
+    Lo, go = NO.batch_loss_and_grad(tb, list(r.astype(complex)), list(q.astype(complex)), list(c), margin=margin)
+    net.close()
+    # the BF16 rounding of input and activations (2^-9 a value) bounds both
+    assert abs(L - Lo) <= 2e-2 * abs(Lo)
+    assert np.linalg.norm(g - go) <= 5e-2 * np.linalg.norm(go)
