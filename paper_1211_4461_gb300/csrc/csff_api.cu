@@ -278,7 +278,7 @@ csff_status smooth(csff_plan* P, int l, cx<T>* u, const cx<T>* b, int sweeps) {
   if (P->opts.smoother == CSFF_SMOOTHER_GMRES) {
     for (int i = 0; i < sweeps; ++i)
       CK(csff::launch_gmres_step<T>(P->dim, L, P->opts.krylov_m, u, b, reinterpret_cast<cx<T>*>(P->gm_v),
-                                    P->gm_part, P->red_blocks, P->gm, s),
+                                    P->gm_part, s),
          "gmres");
     return CSFF_OK;
   }
@@ -794,7 +794,7 @@ void csff_plan_destroy(csff_plan* P) {
   for (Level& L : P->lv)
     for (void* p : {(void*)L.q64, (void*)L.dinv64, (void*)L.q32, (void*)L.dinv32, (void*)L.u64, (void*)L.t64,
                     (void*)L.b64, (void*)L.r64, (void*)L.u32, (void*)L.t32, (void*)L.b32, (void*)L.r32,
-                    (void*)L.fac32, L.s32.base, L.s64.base})
+                    (void*)L.fac32, (void*)L.kq64, (void*)L.kq32, L.s32.base, L.s64.base})
       if (p) cudaFree(p);
   for (double2* p : P->chi_tab)
     if (p) cudaFree(p);
@@ -804,7 +804,7 @@ void csff_plan_destroy(csff_plan* P) {
   if (P->red) cudaFree(P->red);
   if (P->red_out) cudaFree(P->red_out);
   if (P->red_host) cudaFreeHost(P->red_host);
-  for (void* p : {P->gm_v, (void*)P->gm_part, (void*)P->gm, (void*)P->sep_T, (void*)P->dfu, (void*)P->dfb,
+  for (void* p : {P->gm_v, (void*)P->gm_part, (void*)P->sep_T, (void*)P->dfu, (void*)P->dfb,
                   (void*)P->dfq, (void*)P->dfpart})
     if (p) cudaFree(p);
   csff::free_ff_buffers(P);
@@ -934,11 +934,16 @@ csff_status csff_plan_create(const csff_problem* prob, const csff_opts* opts, vo
     if (P->opts.smoother == CSFF_SMOOTHER_GMRES) {
       double2* v = nullptr;
       if ((s = dev_alloc(P, &v, (size_t)(P->opts.krylov_m + 1) * P->lv[0].N)) ||
-          (s = dev_alloc(P, &P->gm_part, P->red_blocks)) || (s = dev_alloc(P, &P->gm, 1))) {
+          (s = dev_alloc(P, &P->gm_part, (size_t)csff::GM_SLOTS * csff::GM_NB))) {
         if (v) cudaFree(v);
         return fail(s);
       }
       P->gm_v = v;
+      for (Level& L : P->lv) {
+        if ((s = dev_alloc(P, &L.kq64, L.N)) || (s = dev_alloc(P, &L.kq32, L.N))) return fail(s);
+        if ((e = csff::launch_gmres_coefs(L, P->stream)) != cudaSuccess)
+          return fail(csff::cuda_fail(e, "GMRES coefficients"));
+      }
     }
   }
   // colour-split V(1,1) RB-GS path (3D), in the precision of the plan's cycles
@@ -1236,6 +1241,8 @@ static csff_status user_q_levels(csff_plan* P) {
   cudaStream_t s = P->stream;
   for (size_t l = 1; l < P->lv.size(); ++l) CK(csff::launch_inject_q(P->dim, P->lv[l - 1], P->lv[l], s), "inject q");
   for (const Level& L : P->lv) CK(csff::launch_coefs_from_q(P->dim, L, s), "coefficients");
+  if (P->opts.smoother == CSFF_SMOOTHER_GMRES)
+    for (const Level& L : P->lv) CK(csff::launch_gmres_coefs(L, s), "GMRES coefficients");
   for (size_t l = 0; l + 1 < P->lv.size(); ++l) {
     if (P->split32) CK(csff::split3_coefs<float>(P->lv[l], P->prob.k * P->prob.k, s), "split coefficients");
     if (P->split64) CK(csff::split3_coefs<double>(P->lv[l], P->prob.k * P->prob.k, s), "split coefficients");

@@ -94,6 +94,9 @@ struct Level {
   float2* fac32 = nullptr;
   int ng = 0;
   double k2 = 0;
+  // kappa q, kappa = 1 / c (GMRES smoothing)
+  double2* kq64 = nullptr;
+  float2* kq32 = nullptr;
   // work buffers
   double2 *u64 = nullptr, *t64 = nullptr, *b64 = nullptr, *r64 = nullptr;
   float2 *u32 = nullptr, *t32 = nullptr, *b32 = nullptr, *r32 = nullptr;
@@ -126,17 +129,11 @@ struct FFBuffers {
   int *dtce = nullptr, *dtcflag = nullptr;
 };
 
-// Device state of one GMRES(m) smoothing step (gmres.cu): the (m+1) x m
-// Hessenberg matrix, the norms beta = nrm[0] and h_{j+1,j} = nrm[j+1] with their
-// inverses, the least-squares solution y and the number k of columns used.
+// Scratch of a GMRES(m) smoothing step (gmres.cu): the partial sums of the
+// norms of its basis vectors and of their inner products, one a block
 constexpr int GM_MAX = 4;
-struct GmState {
-  double2 H[GM_MAX + 1][GM_MAX];
-  double nrm[GM_MAX + 1];
-  double inv[GM_MAX + 1];
-  double2 y[GM_MAX];
-  int k;
-};
+constexpr int GM_NB = 152;
+constexpr int GM_SLOTS = GM_MAX + 1 + GM_MAX * (GM_MAX + 1) / 2;
 
 }  // namespace csff
 
@@ -189,10 +186,9 @@ struct csff_plan {
   double learned_guard = 0.5;
   bool learned_off = false;       // per-solve fallback to plain RB-GS
   // GMRES(m) smoother: m+1 basis vectors of the finest level (sized for FP64,
-  // shared by every level and both precisions), reduction partials, state
+  // shared by every level and both precisions), reduction partials
   void* gm_v = nullptr;
   double2* gm_part = nullptr;
-  csff::GmState* gm = nullptr;
   // coefficients from user samples (csff_plan_set_potential) and the scratch
   // of csff_separable_sum
   bool user_q = false;
@@ -334,10 +330,11 @@ cudaError_t launch_split3_up(std::vector<Level>& lv, cx<T>* u_nat, bool keep_spl
 
 // ---- GMRES(m) smoothing step (gmres.cu) ----------------------------------------
 // u += V y for the GMRES(m) minimiser from u; V holds m+1 vectors of L.N
-// values, part at least part_cap double2 partial sums, S the step's state.
+// values, part GM_SLOTS * GM_NB partial sums.
+cudaError_t launch_gmres_coefs(const Level& L, cudaStream_t s);     // kq64, kq32 from q64
 template <typename T>
 cudaError_t launch_gmres_step(int dim, const Level& L, int m, cx<T>* u, const cx<T>* b, cx<T>* V,
-                              double2* part, int part_cap, GmState* S, cudaStream_t s);
+                              double2* part, cudaStream_t s);
 
 // ---- fused 2D V(1,1) RB-GS kernels (mg_fused.cu) ----------------------------
 // whether the levels from lc on may run in the one-CTA block
