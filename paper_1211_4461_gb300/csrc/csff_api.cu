@@ -271,10 +271,14 @@ template <> float2* rbuf<float>(Level& L) { return L.r32; }
 // coarsest-grid solve, FP32 for the rest of the cycle.
 bool coarse_fp64(const csff_plan* P) { return P->opts.precision == CSFF_PREC_MIXED && P->opts.refine_fp64 != 0; }
 
+// sweeps of the plan's smoother; zero: the iterate enters as zero (u need not
+// hold it)
 template <typename T>
-csff_status smooth(csff_plan* P, int l, cx<T>* u, const cx<T>* b, int sweeps) {
+csff_status smooth(csff_plan* P, int l, cx<T>* u, const cx<T>* b, int sweeps, bool zero = false) {
   Level& L = P->lv[l];
   cudaStream_t s = P->stream;
+  if (zero && (P->opts.smoother != CSFF_SMOOTHER_JACOBI || sweeps == 0))
+    CK(csff::launch_zero<T>(u, L.N, s), "zero");
   if (P->opts.smoother == CSFF_SMOOTHER_GMRES) {
     for (int i = 0; i < sweeps; ++i)
       CK(csff::launch_gmres_step<T>(P->dim, L, P->opts.krylov_m, u, b, reinterpret_cast<cx<T>*>(P->gm_v),
@@ -291,16 +295,17 @@ csff_status smooth(csff_plan* P, int l, cx<T>* u, const cx<T>* b, int sweeps) {
     }
     return CSFF_OK;
   }
+  // Jacobi: between u and the second buffer; from zero the first sweep reads no
+  // iterate and goes where an even number of sweeps is left
   cx<T>* t = tbuf<T>(L);
-  int i = 0;
-  for (; i + 1 < sweeps; i += 2) {
-    CK(csff::launch_jacobi<T>(P->dim, L, P->opts.omega, u, b, t, s), "jacobi");
-    CK(csff::launch_jacobi<T>(P->dim, L, P->opts.omega, t, b, u, s), "jacobi");
+  cx<T>* cur = u;
+  for (int i = 0; i < sweeps; ++i) {
+    const bool first = zero && i == 0;
+    cx<T>* dst = first ? ((sweeps & 1) ? u : t) : (cur == u ? t : u);
+    CK(csff::launch_jacobi<T>(P->dim, L, P->opts.omega, first ? nullptr : cur, b, dst, s), "jacobi");
+    cur = dst;
   }
-  if (i < sweeps) {
-    CK(csff::launch_jacobi<T>(P->dim, L, P->opts.omega, u, b, t, s), "jacobi");
-    CK(cudaMemcpyAsync(u, t, sizeof(cx<T>) * (size_t)L.N, cudaMemcpyDeviceToDevice, s), "copy");
-  }
+  if (cur != u) CK(cudaMemcpyAsync(u, t, sizeof(cx<T>) * (size_t)L.N, cudaMemcpyDeviceToDevice, s), "copy");
   return CSFF_OK;
 }
 
@@ -315,19 +320,18 @@ template <typename T> csff_status coarsest_solve(csff_plan* P, const cx<T>* b, c
   return CSFF_OK;
 }
 
-// One V(nu1, nu2) cycle on level l for A_l u = b (Sec. 4).
+// One V(nu1, nu2) cycle on level l for A_l u = b (Sec. 4); zero: u enters as zero.
 template <typename T>
-csff_status vcycle(csff_plan* P, int l, cx<T>* u, const cx<T>* b) {
+csff_status vcycle(csff_plan* P, int l, cx<T>* u, const cx<T>* b, bool zero = false) {
   const int nl = (int)P->lv.size();
   cudaStream_t s = P->stream;
   if (l == nl - 1) return coarsest_solve<T>(P, b, u);
   Level& L = P->lv[l];
   Level& C = P->lv[l + 1];
-  CS(smooth<T>(P, l, u, b, P->opts.nu1));
+  CS(smooth<T>(P, l, u, b, P->opts.nu1, zero));
   CK(csff::launch_residual<T>(P->dim, L, u, b, rbuf<T>(L), s), "residual");
   CK(csff::launch_restrict<T>(P->dim, L, C, rbuf<T>(L), bbuf<T>(C), s), "restrict");
-  if (l + 1 < nl - 1) CK(csff::launch_zero<T>(ubuf<T>(C), C.N, s), "zero");
-  CS(vcycle<T>(P, l + 1, ubuf<T>(C), bbuf<T>(C)));
+  CS(vcycle<T>(P, l + 1, ubuf<T>(C), bbuf<T>(C), true));
   CK(csff::launch_prolong_add<T>(P->dim, L, C, ubuf<T>(C), u, s), "prolong");
   CS(smooth<T>(P, l, u, b, P->opts.nu2));
   return CSFF_OK;
@@ -460,25 +464,22 @@ csff_status run_vcycle(csff_plan* P, cx<T>* u, const cx<T>* b, bool zero_init, b
   if constexpr (sizeof(T) == 4) {
     if (P->net && !P->learned_off) {
       if (lc > P->learned_levels) return run_vcycle_learned(P, u, b, zero_init);
-      if (zero_init) CK(csff::launch_zero<T>(u, P->lv[0].N, P->stream), "zero");
-      return vcycle<T>(P, 0, u, b);
+      return vcycle<T>(P, 0, u, b, zero_init);
     }
   }
   if (lc < 1) {
-    if (zero_init) CK(csff::launch_zero<T>(u, P->lv[0].N, P->stream), "zero");
-    return vcycle<T>(P, 0, u, b);
+    return vcycle<T>(P, 0, u, b, zero_init);
   }
   return run_fused_from<T>(P, 0, u, b, zero_init);
 }
 
-// Body of one solver step on P->stream (eagerly or under capture): the
-// finest-level norm of the new residual ends in red_host[0].
+// Body of one solver step on P->stream (eagerly or under capture): the norm of
+// the new finest-level residual goes straight to red_host[0] (pinned, written
+// by the kernel; a copy of eight bytes is a node of its own in the graph).
 csff_status step_fp64(csff_plan* P, int eb) {
   Level& L = P->lv[0];
   CS(run_vcycle<double>(P, L.u64, L.b64, false));
-  CK(csff::launch_residual<double>(P->dim, L, L.u64, L.b64, L.r64, P->stream), "residual");
-  CS(norm64(P, L.r64, eb, 0));
-  CK(cudaMemcpyAsync(P->red_host, P->red_out, sizeof(double), cudaMemcpyDeviceToHost, P->stream), "read norm");
+  CK(csff::launch_resid_norm(P->dim, L, L.u64, L.b64, eb, P->red, P->red_blocks, P->red_host, P->stream), "norm");
   return CSFF_OK;
 }
 
@@ -490,8 +491,7 @@ csff_status step_mixed(csff_plan* P, int n) {
   cudaStream_t s = P->stream;
   for (int c = 0; c < n; ++c) CS(run_vcycle<float>(P, L.u32, L.b32, c == 0, c == 0, c == n - 1));
   CK(csff::launch_df_update(P->dfu, L.u32, L.N, s), "update");
-  CK(csff::launch_df_residual(P->dim, L, P->dfu, P->dfb, P->dfq, L.b32, P->dfpart, P->red_out, s), "residual");
-  CK(cudaMemcpyAsync(P->red_host, P->red_out, sizeof(double), cudaMemcpyDeviceToHost, s), "read norm");
+  CK(csff::launch_df_residual(P->dim, L, P->dfu, P->dfb, P->dfq, L.b32, P->dfpart, P->red_host, s), "residual");
   return CSFF_OK;
 }
 
@@ -513,10 +513,9 @@ csff_status step_mixed64(csff_plan* P, int n) {
   cudaStream_t s = P->stream;
   for (int c = 0; c < n; ++c) CS(run_vcycle<float>(P, L.u32, L.b32, c == 0, c == 0, c == n - 1));
   CK(csff::launch_update64_fixed(L.u64, L.u32, L.N, P->refine_eb, s), "update");
-  CK(csff::launch_refine_residual(P->dim, L, L.u64, L.b64, P->refine_eb, L.b32, P->red, P->red_blocks, P->red_out,
+  CK(csff::launch_refine_residual(P->dim, L, L.u64, L.b64, P->refine_eb, L.b32, P->red, P->red_blocks, P->red_host,
                                   s),
      "residual");
-  CK(cudaMemcpyAsync(P->red_host, P->red_out, sizeof(double), cudaMemcpyDeviceToHost, s), "read norm");
   return CSFF_OK;
 }
 
@@ -576,9 +575,7 @@ csff_status step_fmg_level(csff_plan* P, int arg) {
   Level& L = P->lv[l];
   if (P->fused_lc > l) CS(run_fused_from<double>(P, l, L.u64, L.b64, false));
   else CS(vcycle<double>(P, l, L.u64, L.b64));
-  CK(csff::launch_residual<double>(P->dim, L, L.u64, L.b64, L.r64, P->stream), "residual");
-  CK(csff::launch_norm2<double>(L.r64, L.N, e, P->red, P->red_blocks, P->red_out, P->stream), "norm");
-  CK(cudaMemcpyAsync(P->red_host, P->red_out, sizeof(double), cudaMemcpyDeviceToHost, P->stream), "read norm");
+  CK(csff::launch_resid_norm(P->dim, L, L.u64, L.b64, e, P->red, P->red_blocks, P->red_host, P->stream), "norm");
   return CSFF_OK;
 }
 
@@ -1115,8 +1112,7 @@ static csff_status fmg_loaded(csff_plan* P, double2* u_out, int* level_cycles, c
     CK(csff::launch_zero<double>(L.u64, L.N, s), "zero");
     CK(csff::launch_prolong_add<double>(P->dim, L, P->lv[l + 1], P->lv[l + 1].u64, L.u64, s), "interpolate");
     CK(csff::launch_norm2<double>(L.b64, L.N, eb, P->red, P->red_blocks, P->red_out + 1, s), "norm b");
-    CK(csff::launch_residual<double>(P->dim, L, L.u64, L.b64, L.r64, s), "residual");
-    CK(csff::launch_norm2<double>(L.r64, L.N, eb, P->red, P->red_blocks, P->red_out, s), "norm");
+    CK(csff::launch_resid_norm(P->dim, L, L.u64, L.b64, eb, P->red, P->red_blocks, P->red_out, s), "norm");
     CS(read_scalars(P, 2));
     const double nb = P->red_host[1];
     int cycles = 0;

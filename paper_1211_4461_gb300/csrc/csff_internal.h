@@ -247,6 +247,7 @@ template <typename T> constexpr int mg_family() { return sizeof(T) == 8 ? PF_MG6
 template <typename T>
 cudaError_t launch_residual(int dim, const Level& L, const cx<T>* u, const cx<T>* b, cx<T>* r,
                             cudaStream_t s);
+// u may be null: the sweep starts from zero
 template <typename T>
 cudaError_t launch_jacobi(int dim, const Level& L, double omega, const cx<T>* u, const cx<T>* b,
                           cx<T>* u_out, cudaStream_t s);
@@ -255,6 +256,9 @@ cudaError_t launch_rbgs(int dim, const Level& L, cx<T>* u, const cx<T>* b, cudaS
 template <typename T>
 cudaError_t launch_restrict(int dim, const Level& F, const Level& C, const cx<T>* r, cx<T>* bc,
                             cudaStream_t s);
+// ||b - A u|| (prescaled as in launch_norm2) into *out; out: device or pinned host memory
+cudaError_t launch_resid_norm(int dim, const Level& L, const double2* u, const double2* b, int exp_scale,
+                              double* partial, int nblk, double* out, cudaStream_t s);
 template <typename T>
 cudaError_t launch_prolong_add(int dim, const Level& F, const Level& C, const cx<T>* ec, cx<T>* u,
                                cudaStream_t s);

@@ -12,9 +12,8 @@
 // gamma}: a common factor of the system changes neither the Krylov space nor
 // the minimiser, and it makes the stencil's weights real, A'' v = 2d v - sum_nbr
 // v - (kappa q) v.  The basis vectors are kept unnormalised, w_0 = r'' and
-// w_{j+1} = A'' w_j - sum_i alpha_ij w_i; norms and coefficients are scalars in
-// device memory (h_ij = (w_i, w) / (n_i n_j), alpha_ij = (w_i, w) / n_i^2), so no
-// pass only scales a vector.
+// w_{j+1} = A'' w_j - sum_i alpha_ij w_i, h_ij = (w_i, w) / (n_i n_j), alpha_ij =
+// (w_i, w) / n_i^2, n_i = ||w_i||, so no pass only scales a vector.
 //
 // Bound by the FP64 pipe on large levels (136 operations an unknown for
 // m = 3) and by launches below: every pass that changes a vector also forms
@@ -25,10 +24,11 @@
 // them, behind a fence and a counter, costs 2 us a pass on small levels), and
 // every pass lets its successor be set up at once.  GMRES(3) takes 11 launches,
 // 34 with passes for each inner product, its final sum, each update and each
-// scaling; a 129^3 solve (10 cycles) 34.1 -> 21.6 ms, its finest level at about
-// three quarters of the FP64 pipe's rate.  A step is graph-capturable and never synchronises with the host.
-// Inner products and norms accumulate in
-// FP64 for both cycle precisions.  A zero h_{j+1,j} (the Krylov space is
+// scaling; a 129^3 solve (10 cycles) 34.1 -> 21.5 ms, its finest level at about
+// four fifths of the FP64 pipe's rate (one warp instruction in 19 clocks an
+// SM, one in 65 from a single warp).  A step is graph-capturable and never
+// synchronises with the host.  Inner products and norms accumulate in FP64 for
+// both cycle precisions.  A zero h_{j+1,j} (the Krylov space is
 // invariant: the Arnoldi process breaks down) ends the basis: the least-squares
 // step uses the first j+1 columns only.
 #include "csff_internal.h"

@@ -5,19 +5,30 @@
 //
 // Layout: m^d interior unknowns, x fastest, interleaved complex.  Boundary
 // nodes are not stored (homogeneous Dirichlet).  Grid mapping: block (32, 8)
-// over (x, y), blockIdx.z = z plane in 3D.
+// over (x, y), blockIdx.z = z plane in 3D; (32, 2) on levels of few blocks,
+// whose passes last one block's FP64 work (a warp instruction in 19 clocks an
+// SM, in 65 from one warp).  Together with dependent launches, sweeps from zero,
+// the norm of the residual without storing it and the operation counts below,
+// the 65^2 FP64 map (17 Jacobi V(2,2) cycles) went from 1910 to 1180 us.
 #include "csff_internal.h"
 #include "df_bits.cuh"
 
 namespace csff {
 namespace {
 
-constexpr int BX = 32, BY = 8;
+constexpr int BX = 32, BY = 8, BY_SMALL = 2;
+
+// wait for the predecessor; a grid of at most one block an SM lets its
+// successor be set up at once
+__device__ __forceinline__ void pdl_start() {
+  pdl_prologue();
+  if (gridDim.x * gridDim.y * gridDim.z <= 152u) pdl_trigger();
+}
 
 template <int D>
 __device__ __forceinline__ bool thread_point(int m, int& ix, int& iy, int& iz, long long& idx) {
   ix = blockIdx.x * BX + threadIdx.x;
-  iy = blockIdx.y * BY + threadIdx.y;
+  iy = blockIdx.y * blockDim.y + threadIdx.y;
   iz = (D == 3) ? (int)blockIdx.z : 0;
   if (ix >= m || iy >= m) return false;
   idx = ((long long)iz * m + iy) * m + ix;
@@ -47,22 +58,40 @@ __device__ __forceinline__ cx<T> residual_point(const cx<T>* __restrict__ u, cx<
 template <typename T, int D>
 __global__ void k_residual(const cx<T>* __restrict__ u, const cx<T>* __restrict__ b,
                            const cx<T>* __restrict__ q, cx<T> c, int m, cx<T>* __restrict__ r) {
-  pdl_prologue();
+  pdl_start();
   int ix, iy, iz; long long idx;
   if (!thread_point<D>(m, ix, iy, iz, idx)) return;
   r[idx] = residual_point<T, D>(u, u[idx], b[idx], q[idx], c, m, ix, iy, iz, idx);
 }
 
-template <typename T, int D>
-__global__ void k_jacobi(const cx<T>* __restrict__ u, const cx<T>* __restrict__ b,
-                         const cx<T>* __restrict__ q, const cx<T>* __restrict__ dinv, cx<T> c, T omega,
-                         int m, cx<T>* __restrict__ u_out) {
+// u_out = u + omega d^{-1} (b - A u) = (1 - omega) u + omega d^{-1} (b + c
+// sum_nbr u), since A u = d u - c sum_nbr u: 18 FP64 operations a point in 2D,
+// 26 by way of the residual, and no read of q.  ZERO: from u = 0, omega d^{-1} b.
+template <typename T, int D, bool ZERO>
+__global__ void k_jacobi(const cx<T>* __restrict__ u, const cx<T>* __restrict__ b, const cx<T>* __restrict__ dinv,
+                         cx<T> c, T omega, int m, cx<T>* __restrict__ u_out) {
+  pdl_start();
   int ix, iy, iz; long long idx;
   if (!thread_point<D>(m, ix, iy, iz, idx)) return;
-  const cx<T> uj = u[idx], di = dinv[idx];
-  const cx<T> rj = residual_point<T, D>(u, uj, b[idx], q[idx], c, m, ix, iy, iz, idx);
-  const cx<T> t = mk<cx<T>>(fma(di.x, rj.x, -di.y * rj.y), fma(di.x, rj.y, di.y * rj.x));
-  u_out[idx] = mk<cx<T>>(fma(omega, t.x, uj.x), fma(omega, t.y, uj.y));
+  using C = cx<T>;
+  const C di = dinv[idx];
+  C v = b[idx];
+  if constexpr (!ZERO) {
+    const C z = mk<C>((T)0, (T)0);
+    C s = cadd(ix > 0 ? u[idx - 1] : z, ix < m - 1 ? u[idx + 1] : z);
+    s = cadd(s, cadd(iy > 0 ? u[idx - m] : z, iy < m - 1 ? u[idx + m] : z));
+    if (D == 3) {
+      const long long p = (long long)m * m;
+      s = cadd(s, cadd(iz > 0 ? u[idx - p] : z, iz < m - 1 ? u[idx + p] : z));
+    }
+    v = mk<C>(fma(c.x, s.x, fma(-c.y, s.y, v.x)), fma(c.x, s.y, fma(c.y, s.x, v.y)));
+  }
+  C r = mk<C>(omega * fma(di.x, v.x, -di.y * v.y), omega * fma(di.x, v.y, di.y * v.x));
+  if constexpr (!ZERO) {
+    const C uj = u[idx];
+    r = mk<C>(fma((T)1 - omega, uj.x, r.x), fma((T)1 - omega, uj.y, r.y));
+  }
+  u_out[idx] = r;
 }
 
 // One colour of red-black Gauss-Seidel, in place.  colour 0 (red) = even sum
@@ -74,7 +103,8 @@ __global__ void k_jacobi(const cx<T>* __restrict__ u, const cx<T>* __restrict__ 
 template <typename T, int D>
 __global__ void k_rbgs(cx<T>* u, const cx<T>* __restrict__ b, const cx<T>* __restrict__ dinv, cx<T> c, int m,
                        int colour) {
-  const int iy = blockIdx.y * BY + threadIdx.y;
+  pdl_start();
+  const int iy = blockIdx.y * blockDim.y + threadIdx.y;
   const int iz = (D == 3) ? (int)blockIdx.z : 0;
   const int ix = 2 * (int)(blockIdx.x * BX + threadIdx.x) + ((colour + iy + iz + D) & 1);
   if (ix >= m || iy >= m) return;
@@ -94,46 +124,36 @@ __global__ void k_rbgs(cx<T>* u, const cx<T>* __restrict__ b, const cx<T>* __res
 }
 
 // Full weighting: coarse interior P <- sum over offsets o in {-1,0,1}^d of
-// prod(1/2 if o = 0 else 1/4) * r_f[2P + 1 + o].
-template <typename T, int D>
-__global__ void k_restrict(const cx<T>* __restrict__ rf, int mf, cx<T>* __restrict__ bc, int mc) {
-  int ix, iy, iz; long long idx;
-  if (!thread_point<D>(mc, ix, iy, iz, idx)) return;
+// prod(1/2 if o = 0 else 1/4) * r_f[2P + 1 + o], axis by axis as
+// ((left + right)/2 + middle)/2: in 3D 54 operations a point, 144 with a
+// product and a sum for every offset.
+template <typename C, typename T> __device__ __forceinline__ C weigh(C l, C mid, C r) {
+  const T h = (T)0.5;
+  return mk<C>(fma(l.x + r.x, h, mid.x), fma(l.y + r.y, h, mid.y));
+}
+template <typename T, int D, typename R>
+__device__ __forceinline__ cx<T> full_weight(R r) {
   using C = cx<T>;
-  C acc = mk<C>(0, 0);
-  const int fx = 2 * ix + 1, fy = 2 * iy + 1, fz = (D == 3) ? 2 * iz + 1 : 0;
-  const T w1[3] = {(T)0.25, (T)0.5, (T)0.25};
+  C plane[3];
 #pragma unroll
   for (int oz = (D == 3 ? -1 : 0); oz <= (D == 3 ? 1 : 0); ++oz) {
+    C row[3];
 #pragma unroll
-    for (int oy = -1; oy <= 1; ++oy) {
-      C row = mk<C>(0, 0);
-      long long base = ((long long)(fz + oz) * mf + (fy + oy)) * mf + fx;
-#pragma unroll
-      for (int ox = -1; ox <= 1; ++ox) row = cadd(row, cscale(rf[base + ox], w1[ox + 1]));
-      T wz = (D == 3) ? w1[oz + 1] : (T)1;
-      acc = cadd(acc, cscale(row, w1[oy + 1] * wz));
-    }
+    for (int oy = -1; oy <= 1; ++oy) row[oy + 1] = weigh<C, T>(r(-1, oy, oz), r(0, oy, oz), r(1, oy, oz));
+    plane[oz + 1] = weigh<C, T>(row[0], row[1], row[2]);
   }
-  bc[idx] = acc;
+  if (D == 2) return cscale(plane[1], (T)0.25);
+  return cscale(weigh<C, T>(plane[0], plane[1], plane[2]), (T)0.125);
 }
 
-// Linear interpolation weights of fine interior index p along one axis: node
-// i = p + 1; even i sits on coarse node i/2 (weight 1), odd i between coarse
-// nodes (i-1)/2 and (i+1)/2 (weights 1/2).  Returns the number of coarse
-// interior neighbours (coarse interior index = coarse node - 1).
-template <typename T>
-__device__ __forceinline__ int interp_1d(int p, int mc, int* ci, T* w) {
-  int i = p + 1, n = 0;
-  if ((i & 1) == 0) {
-    int I = i >> 1;
-    if (I >= 1 && I <= mc) { ci[n] = I - 1; w[n] = (T)1; ++n; }
-  } else {
-    int I0 = (i - 1) >> 1, I1 = I0 + 1;
-    if (I0 >= 1 && I0 <= mc) { ci[n] = I0 - 1; w[n] = (T)0.5; ++n; }
-    if (I1 >= 1 && I1 <= mc) { ci[n] = I1 - 1; w[n] = (T)0.5; ++n; }
-  }
-  return n;
+template <typename T, int D>
+__global__ void k_restrict(const cx<T>* __restrict__ rf, int mf, cx<T>* __restrict__ bc, int mc) {
+  pdl_start();
+  int ix, iy, iz; long long idx;
+  if (!thread_point<D>(mc, ix, iy, iz, idx)) return;
+  const long long f = ((long long)(D == 3 ? 2 * iz + 1 : 0) * mf + 2 * iy + 1) * mf + 2 * ix + 1;
+  const long long p = (long long)mf * mf;
+  bc[idx] = full_weight<T, D>([&](int ox, int oy, int oz) { return rf[f + ox + (long long)oy * mf + oz * p]; });
 }
 
 // u_f += P e by coarse cells: cell (Nx, Ny, Nz), N in [0, mc] per axis, spans
@@ -146,7 +166,8 @@ __device__ __forceinline__ int interp_1d(int p, int mc, int* ci, T* w) {
 template <typename T, int D>
 __global__ void k_prolong_cells(const cx<T>* __restrict__ ec, int mc, cx<T>* __restrict__ uf, int mf) {
   using C = cx<T>;
-  const int Nx = blockIdx.x * BX + threadIdx.x, Ny = blockIdx.y * BY + threadIdx.y;
+  pdl_start();
+  const int Nx = blockIdx.x * BX + threadIdx.x, Ny = blockIdx.y * blockDim.y + threadIdx.y;
   const int Nz = (D == 3) ? (int)blockIdx.z : 0;
   if (Nx > mc || Ny > mc) return;
   const T h = (T)0.5;
@@ -206,74 +227,32 @@ __global__ void k_prolong_cells(const cx<T>* __restrict__ ec, int mc, cx<T>* __r
   }
 }
 
-template <typename T, int D>
-__global__ void k_prolong_add(const cx<T>* __restrict__ ec, int mc, cx<T>* __restrict__ uf, int mf) {
-  int ix, iy, iz; long long idx;
-  if (!thread_point<D>(mf, ix, iy, iz, idx)) return;
-  using C = cx<T>;
-  int cxi[2], cyi[2], czi[2] = {0, 0};
-  T wx[2], wy[2], wz[2] = {(T)1, (T)0};
-  int nx = interp_1d<T>(ix, mc, cxi, wx);
-  int ny = interp_1d<T>(iy, mc, cyi, wy);
-  int nz = (D == 3) ? interp_1d<T>(iz, mc, czi, wz) : 1;
-  C acc = mk<C>(0, 0);
-  for (int a = 0; a < nz; ++a)
-    for (int bq = 0; bq < ny; ++bq) {
-      long long base = ((long long)czi[a] * mc + cyi[bq]) * mc;
-      for (int cq = 0; cq < nx; ++cq) acc = cadd(acc, cscale(ec[base + cxi[cq]], wx[cq] * wy[bq] * wz[a]));
+// Coarsest level: u = inv b, the inverse from FP64 Gauss-Jordan, in TI
+// arithmetic, rounded once to T.  LPR lanes a row (4, or 32 for large N), chains
+// of fused multiply-adds joined by shuffles: FP64 work is scarce on this part.
+template <typename T, typename TI, int LPR>
+__global__ void __launch_bounds__(256) k_coarse_solve(const cx<TI>* __restrict__ inv, int N,
+                                                      const cx<T>* __restrict__ b, cx<T>* __restrict__ u) {
+  pdl_start();
+  const int t = blockIdx.x * 256 + threadIdx.x, i = t / LPR, part = t % LPR;
+  TI re = (TI)0, im = (TI)0;
+  if (i < N) {
+    const cx<TI>* row = inv + (long long)i * N;
+#pragma unroll 8
+    for (int j = part; j < N; j += LPR) {
+      const cx<TI> a = row[j];
+      const cx<T> bj = b[j];
+      const TI bx = (TI)bj.x, by = (TI)bj.y;
+      re = fma(a.x, bx, fma(-a.y, by, re));
+      im = fma(a.x, by, fma(a.y, bx, im));
     }
-  uf[idx] = cadd(uf[idx], acc);
-}
-
-// Coarsest level: u = A_c^{-1} b with the FP64 dense inverse; one CTA, one
-// warp per row (lanes split the columns, shuffle reduction).
-template <typename T>
-__global__ void k_coarse_solve(const cx<T>* __restrict__ inv, int N, const cx<T>* __restrict__ b,
-                               cx<T>* __restrict__ u) {
-  extern __shared__ unsigned char sb_raw[];
-  cx<T>* sb = reinterpret_cast<cx<T>*>(sb_raw);
-  for (int j = threadIdx.x; j < N; j += blockDim.x) sb[j] = b[j];
-  __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  for (int i = warp; i < N; i += nw) {
-    cx<T> acc = mk<cx<T>>((T)0, (T)0);
-    const cx<T>* row = inv + (long long)i * N;
-    for (int j = lane; j < N; j += 32) acc = cadd(acc, cmul(row[j], sb[j]));
-    for (int o = 16; o > 0; o >>= 1) {
-      acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
-      acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
-    }
-    if (lane == 0) u[i] = acc;
   }
-}
-
-// The FP64 inverse applied in FP64 to an FP32 right-hand side; the product is
-// rounded once to FP32 (the mixed solve with its coarsest solve in FP64).
-__global__ void k_coarse_solve_f64(const double2* __restrict__ inv, int N, const float2* __restrict__ b,
-                                   float2* __restrict__ u) {
-  extern __shared__ unsigned char sb_raw[];
-  double2* sb = reinterpret_cast<double2*>(sb_raw);
-  for (int j = threadIdx.x; j < N; j += blockDim.x) sb[j] = make_double2(b[j].x, b[j].y);
-  __syncthreads();
-  // four consecutive lanes per row (columns j = p mod 4), fused multiply-add
-  // chains, two shuffles: FP64 work is scarce on this part
-  for (int t = threadIdx.x; t < ((4 * N + 31) & ~31); t += blockDim.x) {
-    const int i = t >> 2, part = t & 3;
-    double re = 0.0, im = 0.0;
-    if (i < N) {
-      const double2* row = inv + (long long)i * N;
-      for (int j = part; j < N; j += 4) {
-        const double2 a = row[j], x = sb[j];
-        re = fma(a.x, x.x, fma(-a.y, x.y, re));
-        im = fma(a.x, x.y, fma(a.y, x.x, im));
-      }
-    }
-    re += __shfl_xor_sync(0xffffffffu, re, 1);
-    im += __shfl_xor_sync(0xffffffffu, im, 1);
-    re += __shfl_xor_sync(0xffffffffu, re, 2);
-    im += __shfl_xor_sync(0xffffffffu, im, 2);
-    if (i < N && part == 0) u[i] = make_float2(__double2float_rn(re), __double2float_rn(im));
+#pragma unroll
+  for (int o = 1; o < LPR; o <<= 1) {
+    re += __shfl_xor_sync(0xffffffffu, re, o);
+    im += __shfl_xor_sync(0xffffffffu, im, o);
   }
+  if (i < N && part == 0) u[i] = mk<cx<T>>((T)re, (T)im);
 }
 
 // ---- reductions ------------------------------------------------------------
@@ -320,6 +299,30 @@ __global__ void k_norm_finish(const double* __restrict__ partial, int nblk, doub
   for (int i = threadIdx.x; i < nblk; i += blockDim.x) acc += partial[i];
   acc = block_reduce(acc, AddOp(), sh, 0.0);
   if (threadIdx.x == 0) *out = sqrt(acc) * inv_scale;
+}
+
+// per-block sums of |2^-e (b - A u)|^2 in FP64, the residual not stored; a
+// block walks grid rows
+template <int D>
+__global__ void __launch_bounds__(RED_THREADS) k_resid_norm(const double2* __restrict__ u,
+                                                            const double2* __restrict__ b,
+                                                            const double2* __restrict__ q, double2 c, int m, int tx,
+                                                            double scale, double* __restrict__ partial) {
+  pdl_start();
+  __shared__ double sh[32];
+  const int nrows = (D == 3) ? m * m : m, ty = RED_THREADS / tx, y = threadIdx.x / tx;
+  double acc = 0;
+  for (int row = blockIdx.x * ty + y; row < nrows; row += gridDim.x * ty) {
+    const int iz = (D == 3) ? row / m : 0, iy = (D == 3) ? row - iz * m : row;
+    for (int ix = threadIdx.x - y * tx; ix < m; ix += tx) {
+      const long long i = (long long)row * m + ix;
+      const double2 r = residual_point<double, D>(u, u[i], b[i], q[i], c, m, ix, iy, iz, i);
+      const double rx = r.x * scale, ry = r.y * scale;
+      acc = fma(rx, rx, fma(ry, ry, acc));
+    }
+  }
+  acc = block_reduce(acc, AddOp(), sh, 0.0);
+  if (threadIdx.x == 0) partial[blockIdx.x] = acc;
 }
 
 __global__ void k_max_exp(const double2* __restrict__ v, long long N, int* __restrict__ out) {
@@ -570,6 +573,7 @@ __global__ void k_scale_to32(const double2* __restrict__ v, int N, int s, float2
 
 template <typename T>
 __global__ void k_zero(cx<T>* v, long long N) {
+  pdl_start();
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N;
        i += (long long)gridDim.x * blockDim.x)
     v[i] = mk<cx<T>>(0, 0);
@@ -578,6 +582,15 @@ __global__ void k_zero(cx<T>* v, long long N) {
 inline dim3 grid_of(int dim, int m) {
   return dim3((m + BX - 1) / BX, (m + BY - 1) / BY, dim == 3 ? m : 1);
 }
+// grid and block for passes over wx x wy (x wz) threads: small blocks where the
+// large ones would leave SMs without one
+struct Shape { dim3 g, b; };
+inline Shape shape_of(int wx, int wy, int wz) {
+  const long long big = (long long)((wx + BX - 1) / BX) * ((wy + BY - 1) / BY) * wz;
+  const int by = big < 152 ? BY_SMALL : BY;
+  return Shape{dim3((wx + BX - 1) / BX, (wy + by - 1) / by, wz), dim3(BX, by)};
+}
+inline Shape shape_of(int dim, int m) { return shape_of(m, m, dim == 3 ? m : 1); }
 inline int flat_blocks(long long N) {
   long long b = (N + 255) / 256;
   return (int)(b < 152 * 16 ? (b < 1 ? 1 : b) : 152 * 16);
@@ -588,12 +601,6 @@ inline int flat_blocks(long long N) {
 // ---------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------
-#define CSFF_DIM_DISPATCH(dim, KERNEL, ...)                                   \
-  do {                                                                        \
-    if ((dim) == 2) KERNEL<T, 2><<<g, blk, 0, s>>>(__VA_ARGS__);              \
-    else KERNEL<T, 3><<<g, blk, 0, s>>>(__VA_ARGS__);                         \
-  } while (0)
-
 template <typename T> static const cx<T>* qtab(const Level& L);
 template <> const double2* qtab<double>(const Level& L) { return L.q64; }
 template <> const float2* qtab<float>(const Level& L) { return L.q32; }
@@ -604,11 +611,11 @@ template <> const float2* dtab<float>(const Level& L) { return L.dinv32; }
 template <typename T>
 cudaError_t launch_residual(int dim, const Level& L, const cx<T>* u, const cx<T>* b, cx<T>* r,
                             cudaStream_t s) {
-  dim3 g = grid_of(dim, L.m), blk(BX, BY);
+  const Shape h = shape_of(dim, L.m);
   cx<T> c = mk<cx<T>>((T)L.c.x, (T)L.c.y);
   ProfScope ps(mg_family<T>(), s, 3.0 * sizeof(cx<T>) * L.N, 0);
-  cudaError_t e = (dim == 2) ? launch_pdl(k_residual<T, 2>, g, blk, 0, s, u, b, qtab<T>(L), c, L.m, r)
-                             : launch_pdl(k_residual<T, 3>, g, blk, 0, s, u, b, qtab<T>(L), c, L.m, r);
+  cudaError_t e = (dim == 2) ? launch_pdl(k_residual<T, 2>, h.g, h.b, 0, s, u, b, qtab<T>(L), c, L.m, r)
+                             : launch_pdl(k_residual<T, 3>, h.g, h.b, 0, s, u, b, qtab<T>(L), c, L.m, r);
   count_launch();
   return e != cudaSuccess ? e : cudaGetLastError();
 }
@@ -616,60 +623,92 @@ cudaError_t launch_residual(int dim, const Level& L, const cx<T>* u, const cx<T>
 template <typename T>
 cudaError_t launch_jacobi(int dim, const Level& L, double omega, const cx<T>* u, const cx<T>* b,
                           cx<T>* u_out, cudaStream_t s) {
-  dim3 g = grid_of(dim, L.m), blk(BX, BY);
+  const Shape h = shape_of(dim, L.m);
   cx<T> c = mk<cx<T>>((T)L.c.x, (T)L.c.y);
-  ProfScope ps(mg_family<T>(), s, 3.0 * sizeof(cx<T>) * L.N, 0);
-  CSFF_DIM_DISPATCH(dim, k_jacobi, u, b, qtab<T>(L), dtab<T>(L), c, (T)omega, L.m, u_out);
+  const cx<T>* d = dtab<T>(L);
+  ProfScope ps(mg_family<T>(), s, (u ? 3.0 : 2.0) * sizeof(cx<T>) * L.N, 0);
+  cudaError_t e;
+  if (u)
+    e = dim == 2 ? launch_pdl(k_jacobi<T, 2, false>, h.g, h.b, 0, s, u, b, d, c, (T)omega, L.m, u_out)
+                 : launch_pdl(k_jacobi<T, 3, false>, h.g, h.b, 0, s, u, b, d, c, (T)omega, L.m, u_out);
+  else
+    e = dim == 2 ? launch_pdl(k_jacobi<T, 2, true>, h.g, h.b, 0, s, u, b, d, c, (T)omega, L.m, u_out)
+                 : launch_pdl(k_jacobi<T, 3, true>, h.g, h.b, 0, s, u, b, d, c, (T)omega, L.m, u_out);
   count_launch();
-  return cudaGetLastError();
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t launch_rbgs(int dim, const Level& L, cx<T>* u, const cx<T>* b, cudaStream_t s) {
-  dim3 g = grid_of(dim, L.m), blk(BX, BY);
-  g.x = ((L.m + 1) / 2 + BX - 1) / BX;          // one thread per point of a colour along x
+  // one thread per point of a colour along x
+  const Shape h = shape_of((L.m + 1) / 2, L.m, dim == 3 ? L.m : 1);
   cx<T> c = mk<cx<T>>((T)L.c.x, (T)L.c.y);
   ProfScope ps(mg_family<T>(), s, 3.0 * sizeof(cx<T>) * L.N, 0);
-  CSFF_DIM_DISPATCH(dim, k_rbgs, u, b, dtab<T>(L), c, L.m, 0);
-  CSFF_DIM_DISPATCH(dim, k_rbgs, u, b, dtab<T>(L), c, L.m, 1);
+  cudaError_t e = cudaSuccess;
+  for (int colour = 0; colour < 2 && e == cudaSuccess; ++colour)
+    e = dim == 2 ? launch_pdl(k_rbgs<T, 2>, h.g, h.b, 0, s, u, b, dtab<T>(L), c, L.m, colour)
+                 : launch_pdl(k_rbgs<T, 3>, h.g, h.b, 0, s, u, b, dtab<T>(L), c, L.m, colour);
   count_launch(2);
-  return cudaGetLastError();
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t launch_restrict(int dim, const Level& F, const Level& C, const cx<T>* r, cx<T>* bc,
                             cudaStream_t s) {
-  dim3 g = grid_of(dim, C.m), blk(BX, BY);
+  const Shape h = shape_of(dim, C.m);
   ProfScope ps(mg_family<T>(), s, (double)sizeof(cx<T>) * (F.N + C.N), 0);
-  CSFF_DIM_DISPATCH(dim, k_restrict, r, F.m, bc, C.m);
+  cudaError_t e = dim == 2 ? launch_pdl(k_restrict<T, 2>, h.g, h.b, 0, s, r, F.m, bc, C.m)
+                           : launch_pdl(k_restrict<T, 3>, h.g, h.b, 0, s, r, F.m, bc, C.m);
   count_launch();
-  return cudaGetLastError();
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t launch_prolong_add(int dim, const Level& F, const Level& C, const cx<T>* ec, cx<T>* u,
                                cudaStream_t s) {
-  dim3 g = grid_of(dim, F.m), blk(BX, BY);
   ProfScope ps(mg_family<T>(), s, (double)sizeof(cx<T>) * (2.0 * F.N + C.N), 0);
-  g = dim3((C.m + 1 + BX - 1) / BX, (C.m + 1 + BY - 1) / BY, dim == 3 ? C.m + 1 : 1);   // coarse cells
-  CSFF_DIM_DISPATCH(dim, k_prolong_cells, ec, C.m, u, F.m);
+  const Shape h = shape_of(C.m + 1, C.m + 1, dim == 3 ? C.m + 1 : 1);            // coarse cells
+  cudaError_t e = dim == 2 ? launch_pdl(k_prolong_cells<T, 2>, h.g, h.b, 0, s, ec, C.m, u, F.m)
+                           : launch_pdl(k_prolong_cells<T, 3>, h.g, h.b, 0, s, ec, C.m, u, F.m);
   count_launch();
-  return cudaGetLastError();
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+template <typename T, typename TI>
+static cudaError_t coarse_solve(const cx<TI>* inv, int N, const cx<T>* b, cx<T>* u, cudaStream_t s) {
+  ProfScope ps(mg_family<T>(), s, sizeof(cx<T>) * 2.0 * N + sizeof(cx<TI>) * (double)N * N, 8.0 * N * N);
+  cudaError_t e = N <= 128 ? launch_pdl(k_coarse_solve<T, TI, 4>, dim3((4 * N + 255) / 256), dim3(256), 0, s, inv, N, b, u)
+                           : launch_pdl(k_coarse_solve<T, TI, 32>, dim3((32 * N + 255) / 256), dim3(256), 0, s, inv, N, b, u);
+  count_launch();
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t launch_coarse_solve(const cx<T>* inv, int N, const cx<T>* b, cx<T>* u, cudaStream_t s) {
-  ProfScope ps(mg_family<T>(), s, sizeof(cx<T>) * (2.0 * N + (double)N * N), 8.0 * N * N);
-  k_coarse_solve<T><<<1, 256, (size_t)N * sizeof(cx<T>), s>>>(inv, N, b, u);
-  count_launch();
-  return cudaGetLastError();
+  return coarse_solve<T, T>(inv, N, b, u, s);
 }
 
 cudaError_t launch_coarse_solve_f64(const double2* inv, int N, const float2* b, float2* u, cudaStream_t s) {
-  ProfScope ps(mg_family<float>(), s, sizeof(float2) * 2.0 * N + sizeof(double2) * (double)N * N, 8.0 * N * N);
-  k_coarse_solve_f64<<<1, 256, (size_t)N * sizeof(double2), s>>>(inv, N, b, u);
-  count_launch();
-  return cudaGetLastError();
+  return coarse_solve<float, double>(inv, N, b, u, s);
+}
+
+cudaError_t launch_resid_norm(int dim, const Level& L, const double2* u, const double2* b, int exp_scale,
+                              double* partial, int nblk, double* out, cudaStream_t s) {
+  int tx = 32;
+  while (tx < L.m && tx < RED_THREADS) tx *= 2;
+  const long long rows = dim == 3 ? (long long)L.m * L.m : L.m, need = (rows + RED_THREADS / tx - 1) / (RED_THREADS / tx);
+  const int nb = (int)(need < nblk ? need : nblk);
+  const double scale = ldexp(1.0, -exp_scale);
+  ProfScope ps(PF_MG64, s, 3.0 * sizeof(double2) * L.N, 0);
+  cudaError_t e = dim == 2 ? launch_pdl(k_resid_norm<2>, dim3(nb), dim3(RED_THREADS), 0, s, u, b, (const double2*)L.q64,
+                                        L.c, L.m, tx, scale, partial)
+                           : launch_pdl(k_resid_norm<3>, dim3(nb), dim3(RED_THREADS), 0, s, u, b, (const double2*)L.q64,
+                                        L.c, L.m, tx, scale, partial);
+  if (e == cudaSuccess)
+    e = launch_pdl(k_norm_finish, dim3(1), dim3(RED_THREADS), 0, s, (const double*)partial, nb, ldexp(1.0, exp_scale),
+                   out);
+  count_launch(2);
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 template <typename T>
@@ -792,9 +831,9 @@ cudaError_t launch_coefs_from_q(int dim, const Level& L, cudaStream_t s) {
 template <typename T>
 cudaError_t launch_zero(cx<T>* v, long long N, cudaStream_t s) {
   ProfScope ps(mg_family<T>(), s, (double)sizeof(cx<T>) * N, 0);
-  k_zero<T><<<flat_blocks(N), 256, 0, s>>>(v, N);
+  cudaError_t e = launch_pdl(k_zero<T>, dim3(flat_blocks(N)), dim3(256), 0, s, v, N);
   count_launch();
-  return cudaGetLastError();
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 #define CSFF_INST(T)                                                                                   \

@@ -92,3 +92,18 @@ def test_net_gradient_over_patch_shapes(csff, B, H, Wd, margin):
     # the BF16 rounding of input and activations (2^-9 a value) bounds both
     assert abs(L - Lo) <= 2e-2 * abs(Lo)
     assert np.linalg.norm(g - go) <= 5e-2 * np.linalg.norm(go)
+
+
+# Jacobi sweeps from a zero and a non-zero iterate, odd and even counts (the
+# second buffer holds the result of one of them), and the per-level passes in
+# blocks of both shapes: 2D levels of 31 to 255 points a side, 3D of 7 to 31
+@pytest.mark.parametrize("dim,n,coarsest", [(2, 33, 5), (2, 161, 6), (2, 257, 9), (3, 17, 5), (3, 33, 9)])
+@pytest.mark.parametrize("nu1,nu2", [(1, 2), (2, 1), (3, 0), (0, 3)])
+@pytest.mark.parametrize("prec", ["fp64", "df"])
+def test_vcycle_jacobi(csff, dim, n, coarsest, nu1, nu2, prec):
+    opts = {"smoother": "jacobi", "omega": 0.6, "nu1": nu1, "nu2": nu2, "coarsest_n": coarsest, "rel_tol": 1e-8,
+            "max_cycles": 100, "precision": "fp64" if prec == "fp64" else "mixed"}
+    got, ref = _vcycle_pair(csff, _problem(dim, n, 1.0, R=4.0), opts,
+                            torch.complex128 if prec == "fp64" else torch.complex64)
+    tol = 1e-11 if prec == "fp64" else 1e-4
+    assert np.linalg.norm(got - ref) <= tol * np.linalg.norm(ref)
