@@ -106,7 +106,8 @@ struct Level {
 
 // Far-field scratch (grown on demand): g = chi (u_in + u); x/y/z phase
 // tables; stage-1 sums T; angle data; per-row exponents; misc[0] = max
-// exponent of |g|, misc[1] = "a scale was applied" flag.
+// exponent of |g|, misc[1] = "a scale was applied" flag, misc[2] = a wait of
+// the digit contraction ran out.
 struct FFBuffers {
   size_t g = 0, xt = 0, yt = 0, zt = 0, T = 0, al = 0, ux = 0, xr = 0, s1 = 0;
   double2 *dg = nullptr, *dxt = nullptr, *dyt = nullptr, *dzt = nullptr, *dT = nullptr;
@@ -122,6 +123,9 @@ struct FFBuffers {
   int *dxlo = nullptr, *dghi = nullptr;
   unsigned char* dskip = nullptr;
   size_t skip_used = 0;       // flags written by the last 2D far field
+  // digit operands of the tensor-core contraction (ff_digits.cuh)
+  size_t xdig = 0, gdig = 0;
+  unsigned char *dxdig = nullptr, *dgdig = nullptr;
   // tensor-core 3D stage A: pre-swizzled split phase operand, per-column and
   // per-row exponents, [spread_g, spread_P, error word]
   size_t tcb = 0, tce = 0;

@@ -16,12 +16,14 @@
 // s1 + s2 (F = F' 2^(s1+s2)).
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <cmath>
 #include <map>
 #include <vector>
 
 #include "csff_internal.h"
 #include "df_bits.cuh"
+#include "ff_digits.cuh"
 
 namespace csff {
 namespace {
@@ -35,6 +37,11 @@ __device__ __forceinline__ int cexp2(double2 v) {
   if (nzx) e = max(e, bits::exp_field(v.x) == 0x7ff ? 0 : bits::frexp_exp(v.x));
   if (nzy) e = max(e, bits::exp_field(v.y) == 0x7ff ? 0 : bits::frexp_exp(v.y));
   return e + 1;
+}
+
+// a b + c, fused multiply-adds
+__device__ __forceinline__ double2 zfma(double2 a, double2 b, double2 c) {
+  return make_double2(fma(a.x, b.x, fma(-a.y, b.y, c.x)), fma(a.x, b.y, fma(a.y, b.x, c.y)));
 }
 
 // g = chi (u_in + u) at every interior node, and the largest frexp exponent of
@@ -90,12 +97,18 @@ __global__ void k_gfield(Tabs8 tabs, int n_gauss, const double2* __restrict__ ui
   int e = -2000;
   if (ix < m && iy < m) {
     const long long idx = ((long long)iz * m + iy) * m + ix;
+    // chains of fused multiply-adds: 12 operations for one Gaussian, 8 for each
+    // further one (this pass is bound by the FP64 pipe)
     double2 chi = make_double2(0, 0), cu = make_double2(0, 0);
-    for (int q = 0; q < n_gauss; ++q) {
-      chi = cadd(chi, cmul(ex[q][threadIdx.x], eyz[q][threadIdx.y]));
-      cu = cadd(cu, cmul(px[q][threadIdx.x], pyz[q][threadIdx.y]));
+    if (n_gauss > 0) {
+      chi = cmul(ex[0][threadIdx.x], eyz[0][threadIdx.y]);
+      cu = cmul(px[0][threadIdx.x], pyz[0][threadIdx.y]);
     }
-    const double2 v = cadd(cu, cmul(chi, u[idx]));
+    for (int q = 1; q < n_gauss; ++q) {
+      chi = zfma(ex[q][threadIdx.x], eyz[q][threadIdx.y], chi);
+      cu = zfma(px[q][threadIdx.x], pyz[q][threadIdx.y], cu);
+    }
+    const double2 v = zfma(chi, u[idx], cu);
     g[idx] = v;
     e = value_exp(v);
   }
@@ -196,10 +209,15 @@ __device__ __forceinline__ bool df_selected(const int* __restrict__ spread) {
   return sx < DF_NONFINITE && sg < DF_NONFINITE && min(sx, sg) <= DF_SPREAD_LIMIT;
 }
 
+// spread[2]: the largest ex + eg - L over the blocks that the contraction keeps
+__device__ __forceinline__ bool digits_selected(const int* __restrict__ spread) {
+  return spread[0] < DF_NONFINITE && spread[1] < DF_NONFINITE && spread[2] <= digits::MARGIN;
+}
+
 __global__ void __launch_bounds__(256) k_ff_stage1(const double2* __restrict__ X, int M,
                                                    const double2* __restrict__ G, int N, int K,
                                                    double2* __restrict__ T, const int* __restrict__ skip_if_df) {
-  if (skip_if_df && df_selected(skip_if_df)) return;   // the double-float kernel ran
+  if (skip_if_df && (digits_selected(skip_if_df) || df_selected(skip_if_df))) return;   // another kernel ran
   __shared__ double2 As[S1_BK][S1_BM];
   __shared__ double2 Bs[S1_BK][S1_BN + 1];
   const int tid = threadIdx.x;
@@ -250,36 +268,41 @@ __device__ __forceinline__ V bred(V v, Op op, V* sh) {
   for (int j = 1; j < (int)(blockDim.x >> 5); ++j) v = op(v, sh[j]);
   return v;
 }
-// (x, y) summed over the block in the order bred uses, the result in thread
-// 0 only: one pass for both components and no FP64 work for the other threads
+// (x, y) summed over the block of 256, the result in thread 0: halving rounds
+// through shared memory, then one warp (the FP64 pipe takes a warp instruction
+// in 19 clocks, so a butterfly in every warp would cost more than the sums)
 __device__ __forceinline__ double2 bsum2_to0(double x, double y, double2* sh) {
-  for (int o = 16; o > 0; o >>= 1) {
-    x += __shfl_xor_sync(0xffffffffu, x, o);
-    y += __shfl_xor_sync(0xffffffffu, y, o);
-  }
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = make_double2(x, y);
+  double2 v = make_double2(x, y);
+  sh[threadIdx.x] = v;
   __syncthreads();
-  double2 v = make_double2(0.0, 0.0);
-  if (threadIdx.x == 0) {
-    v = sh[0];
-    for (int j = 1; j < (int)(blockDim.x >> 5); ++j) {
-      v.x = v.x + sh[j].x;
-      v.y = v.y + sh[j].y;
+#pragma unroll
+  for (int h = 128; h >= 32; h >>= 1) {
+    if ((int)threadIdx.x < h) {
+      const double2 w = sh[threadIdx.x + h];
+      v.x += w.x;
+      v.y += w.y;
+      sh[threadIdx.x] = v;
     }
+    __syncthreads();
   }
+  if (threadIdx.x < 32)
+    for (int o = 16; o > 0; o >>= 1) {
+      v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
+      v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
+    }
   return v;
 }
 struct MaxI { __device__ int operator()(int a, int b) const { return a > b ? a : b; } };
 
 // Stage 2: one block per angle.
 template <int D>
-__global__ void k_ff_stage2(const double2* __restrict__ T, const int* __restrict__ xrow,
+__global__ void __launch_bounds__(256) k_ff_stage2(const double2* __restrict__ T, const int* __restrict__ xrow,
                             const int* __restrict__ s1, const double2* __restrict__ ytab,
                             const double2* __restrict__ ztab, int m, double2 pref,
                             double2* __restrict__ F, int* __restrict__ Fexp, int write_exp,
                             int* __restrict__ flag) {
   __shared__ int shi[32];
-  __shared__ double2 shd[32];
+  __shared__ double2 shd[256];
   const int a = blockIdx.x;
   const int kx = xrow[a];
   const long long R = (D == 3) ? (long long)m * m : m;
@@ -356,15 +379,14 @@ __device__ __forceinline__ void df_mac2(float2& sh, float2& sl, float2 ah, float
   sl = __fadd2_rn(sl, __fadd2_rn(err, e));
 }
 
-// one warp per (row, block): block exponent of |v| (upper bound), scaled
-// double-float split, and the row-block spread (max - min exponent) into *spread.
+// one warp per (row, block): block exponent of |v| (upper bound) and the
+// row-block spread (max - min exponent) into *spread.
 // elo (block bounds for skipping negligible blocks, see k_ff_df_skip):
 // lo_min != 0 writes the smallest exponent of the block's entries inside the
 // grid (-100000 if one is zero: max(|re|, |im|) >= 2^(e-1) for every entry),
 // else the largest (-100000 for an all-zero block: some entry reaches 2^(e-1)).
-__global__ void k_split_rows(const double2* __restrict__ v, int m, int nrows, float4* __restrict__ vdf,
-                             float2* __restrict__ vsum, int* __restrict__ ev, int* __restrict__ spread,
-                             int* __restrict__ elo, int lo_min) {
+__global__ void k_row_exps(const double2* __restrict__ v, int m, int nrows, int* __restrict__ ev,
+                           int* __restrict__ spread, int* __restrict__ elo, int lo_min) {
   // the spread is reduced over the CTA before one atomic (a per-warp atomic on
   // the one counter serialises in L2)
   __shared__ int wsp[8];
@@ -391,10 +413,9 @@ __global__ void k_split_rows(const double2* __restrict__ v, int m, int nrows, fl
     elow = min(elow, __shfl_xor_sync(0xffffffffu, elow, o));
   }
   const bool bad = __any_sync(0xffffffffu, !fin);   // non-finite: the FP64 kernel runs
-  const int eb = (e == -100000 || bad) ? 0 : e;
   if (active && lane == 0) {
-    ev[(long long)row * nb + b] = eb;
-    if (elo) elo[(long long)row * nb + b] = lo_min ? elow : e;
+    ev[(long long)row * nb + b] = (e == -100000 || bad) ? 0 : e;
+    elo[(long long)row * nb + b] = lo_min ? elow : e;
     wsp[threadIdx.x >> 5] = bad ? DF_NONFINITE : ((e == -100000) ? 0 : e - emin);
   }
   __syncthreads();
@@ -403,21 +424,63 @@ __global__ void k_split_rows(const double2* __restrict__ v, int m, int nrows, fl
     for (int w = 0; w < 8; ++w) sp = max(sp, wsp[w]);
     if (sp > 0) atomicMax(spread, sp);
   }
-  // the scaled splits of re, im and re + im (Gauss's three-product complex
-  // multiply); the scale applies to the values themselves, since 2^-eb alone
-  // overflows for subnormal blocks
-  const bool zero = e == -100000 || bad;
-  float2 re = make_float2(0.f, 0.f), im = re, sm = re;
-  if (!zero) {
-    re = bits::split_scaled(x.x, eb);
-    im = bits::split_scaled(x.y, eb);
-    sm = eb <= 1000 ? bits::split_scaled(x.x + x.y, eb)      // RN(x + y) 2^-eb = RN(x 2^-eb + y 2^-eb)
-                    : bits::split_scaled(ldexp(x.x, -eb) + ldexp(x.y, -eb), 0);
-  }
-  if (active) {
+}
+
+// one warp per (row, block), after k_row_exps: the operands of the
+// double-float contraction (rows scaled per block, split into FP32 pairs)
+__global__ void k_split_rows(const double2* __restrict__ v, int m, int nrows, const int* __restrict__ ev,
+                             const int* __restrict__ spread, float4* __restrict__ vdf, float2* __restrict__ vsum) {
+  if (digits_selected(spread) || !df_selected(spread)) return;
+  const int lane = threadIdx.x & 31, nb = (m + DKB - 1) / DKB;
+  for (int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; warp < nrows * nb; warp += gridDim.x * blockDim.x >> 5) {
+    const int row = warp / nb, b = warp % nb, i = b * DKB + lane;
+    const double2 x = i < m ? v[(long long)row * m + i] : make_double2(0, 0);
+    const int eb = ev[(long long)row * nb + b];
+    // the scaled splits of re, im and re + im (Gauss's three-product complex
+    // multiply); the scale applies to the values themselves, since 2^-eb alone
+    // overflows for subnormal blocks
+    const float2 re = bits::split_scaled(x.x, eb), im = bits::split_scaled(x.y, eb);
+    const float2 sm = eb <= 1000 ? bits::split_scaled(x.x + x.y, eb)      // RN(x + y) 2^-eb = RN(x 2^-eb + y 2^-eb)
+                                 : bits::split_scaled(ldexp(x.x, -eb) + ldexp(x.y, -eb), 0);
     const long long o = (long long)row * nb * DKB + b * DKB + lane;
     vdf[o] = make_float4(re.x, re.y, im.x, im.y);
     vsum[o] = sm;
+  }
+}
+
+// one warp per (row, block), after k_row_exps: the digit operands of
+// k_ff_digits, rows padded with zeros to whole tiles.  PHASE: the two rows (P_re,
+// -P_im), (P_im, P_re) of a phase row in tiles of TK; else a row of g, tiles of TM.
+template <bool PHASE>
+__global__ void k_cut_rows(const double2* __restrict__ v, int m, int nrows, const int* __restrict__ ev,
+                           const int* __restrict__ spread, unsigned char* __restrict__ out) {
+  using namespace digits;
+  if (!digits_selected(spread)) return;
+  constexpr int TR = PHASE ? TK : TM;
+  const int lane = threadIdx.x & 31, nb = (m + KB - 1) / KB, total = (nrows + TR - 1) / TR * TR * nb;
+  for (int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; warp < total; warp += gridDim.x * blockDim.x >> 5) {
+    const int row = warp / nb, b = warp % nb, i = b * KB + lane;
+    uint32_t dig[ND];
+    long long p = 0, q = 0;
+    if (row < nrows && i < m) {
+      const double2 x = v[(long long)row * m + i];
+      const int e = ev[(long long)row * nb + b];
+      p = fixed55(x.x, e);
+      q = fixed55(x.y, e);
+    }
+    cut(p, q, dig);
+    const int r = row % TR;
+    unsigned char* tile = out + ((long long)(row / TR) * nb + b) * (PHASE ? B_SET : ND * A_DIG);
+    const int o = (lane & 3) * 4;
+#pragma unroll
+    for (int s = 0; s < ND; ++s) {
+      if (PHASE) {
+        *reinterpret_cast<uint32_t*>(tile + s * B_DIG + sw(r, lane >> 2) + o) = neg_hi(dig[s]);
+        *reinterpret_cast<uint32_t*>(tile + s * B_DIG + sw(TK + r, lane >> 2) + o) = swap_pair(dig[s]);
+      } else {
+        *reinterpret_cast<uint32_t*>(tile + s * A_DIG + sw(r, lane >> 2) + o) = dig[s];
+      }
+    }
   }
 }
 
@@ -502,8 +565,10 @@ __host__ __device__ constexpr size_t df_skip_smem(int nb) {
 }
 __global__ void k_ff_df_skip(const int* __restrict__ ex, const int* __restrict__ xlo, int M,
                              const int* __restrict__ eg, const int* __restrict__ ghi, int N, int nb,
-                             unsigned char* __restrict__ skip) {
+                             unsigned char* __restrict__ skip, int* __restrict__ margin) {
   __shared__ int Ls[DF_BM * DF_BN];
+  __shared__ int kept;                   // largest ex + eg - L over the blocks kept
+  if (threadIdx.x == 0) kept = 0;
   extern __shared__ int sexp[];          // the tile's rows of ex, xlo, eg, ghi when nb is small
   const int m0 = blockIdx.y * DF_BM, n0 = blockIdx.x * DF_BN;
   constexpr int OUTSIDE = -(1 << 30);    // pair outside the output range: no constraint
@@ -560,8 +625,13 @@ __global__ void k_ff_df_skip(const int* __restrict__ ex, const int* __restrict__
       worst = max(worst, sx[k * ps + b] + sg[r * ps + b] + 6 - L);
     }
     for (int o = 16; o > 0; o >>= 1) worst = max(worst, __shfl_xor_sync(0xffffffffu, worst, o));
-    if (lane == 0) skip[tile * nb + b] = worst < -DF_SKIP_MARGIN ? 1 : 0;
+    if (lane == 0) {
+      skip[tile * nb + b] = worst < -DF_SKIP_MARGIN ? 1 : 0;
+      if (worst - 6 > 0) atomicMax(&kept, worst - 6);
+    }
   }
+  __syncthreads();
+  if (threadIdx.x == 0 && kept > 0) atomicMax(margin, kept);
 }
 
 __global__ void __launch_bounds__(DF_NT, 5) k_ff_stage1_df(const float4* __restrict__ X, const float2* __restrict__ Xs,
@@ -571,7 +641,7 @@ __global__ void __launch_bounds__(DF_NT, 5) k_ff_stage1_df(const float4* __restr
                                                         const int* __restrict__ spread,
                                                         const unsigned char* __restrict__ skip,
                                                         double2* __restrict__ T) {
-  if (!df_selected(spread)) return;      // the FP64 kernel takes this launch
+  if (digits_selected(spread) || !df_selected(spread)) return;      // another kernel takes this launch
   __shared__ float4 As[DF_BM][DKB + 1];
   __shared__ float2 As2[DF_BM][DKB + 1];
   // g rows tx and tx + 16 side by side (the two outputs j of a thread), per
@@ -668,6 +738,245 @@ __global__ void __launch_bounds__(DF_NT, 5) k_ff_stage1_df(const float4* __restr
       T[(long long)gm * N + gn] = make_double2(ldexp(S1 - S2, acc1[i][j].E), ldexp(S3 - S1 - S2, acc1[i][j].E));
     }
   }
+}
+
+// T[k][rho] from the digit operands (ff_digits.cuh): a tile of 128 rho x 16 k a
+// CTA, its kept blocks in order.  Warps 0-15 join the accumulators (TMEM lanes
+// 32 (w mod 4), phase rows [4 (w / 4), +4)), warp 16 loads, warp 17 issues MMAs.
+// A wait that runs out (none should) leaves NaN in the tile and sets *err.
+// Bound by the issue of the MMAs (114 clocks each where the tensor core needs
+// 64; 150 from one thread in a divergent branch) and by the last wave: 184 tiles
+// on 152 SMs at 1025^2.  361 phase rows x 1023 x 1023, every block kept: 125 us,
+// 18 us for cutting the operands; the double-float contraction takes 538.
+__global__ void __launch_bounds__(digits::NT, 1)
+    k_ff_digits(const unsigned char* __restrict__ Ad, const unsigned char* __restrict__ Bd, const int* __restrict__ ex,
+                int M, const int* __restrict__ eg, int N, int nb, const int* __restrict__ spread,
+                const unsigned char* __restrict__ skip, int skip_tiles, double2* __restrict__ T, int* __restrict__ err) {
+  using namespace digits;
+  if (!digits_selected(spread)) return;      // another kernel takes this launch
+  extern __shared__ __align__(1024) unsigned char dsm_raw[];
+  unsigned char* base = dsm_raw + ((1024 - (saddr(dsm_raw) & 1023)) & 1023);
+  const uint32_t sbase = saddr(base), bars = sbase + OFF_BAR;
+  const uint32_t a_full = bars, a_empty = a_full + 8 * NA, b_full = a_empty + 8 * NA, b_empty = b_full + 16,
+                 acc_full = b_empty + 16, acc_empty = acc_full + 16, fin = acc_empty + 16;
+  volatile int* abort = reinterpret_cast<volatile int*>(base + OFF_BAR + 480);
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(base + OFF_BAR + 484);
+  int* n_act_p = reinterpret_cast<int*>(base + OFF_BAR + 488);
+  unsigned short* act = reinterpret_cast<unsigned short*>(base + OFF_ACT);
+  static_assert(8 * (2 * NA + 9) <= 480, "barriers");
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int n0 = blockIdx.x * TM, m0 = blockIdx.y * TK;
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < NA; ++i) {
+      bar_init(a_full + 8 * i, 1);
+      bar_init(a_empty + 8 * i, 1);
+    }
+    for (int i = 0; i < 2; ++i) {
+      bar_init(b_full + 8 * i, 1);
+      bar_init(b_empty + 8 * i, 1);
+      bar_init(acc_full + 8 * i, 1);
+      bar_init(acc_empty + 8 * i, EPI_WARPS);
+    }
+    bar_init(fin, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    *abort = 0;
+  }
+  if (warp == EPI_WARPS + 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(saddr(tslot)), "n"(TMEM_COLS));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  if (warp == 0) {
+    // blocks that one of the tile's skip tiles (16 x 32) keeps
+    int n = 0;
+    const int t0 = blockIdx.x * (TM / DF_BN), t1 = min(t0 + TM / DF_BN, skip_tiles);
+    for (int b0 = 0; b0 < nb; b0 += 32) {
+      const int b = b0 + lane;
+      bool keep = false;
+      if (b < nb)
+        for (int t = t0; t < t1; ++t) keep |= skip[((long long)blockIdx.y * skip_tiles + t) * nb + b] == 0;
+      const unsigned mask = __ballot_sync(0xffffffffu, keep);
+      if (keep) act[n + __popc(mask & ((1u << lane) - 1u))] = (unsigned short)b;
+      n += __popc(mask);
+    }
+    if (lane == 0) *n_act_p = n;
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = *tslot;
+  const int n_act = *n_act_p;
+  static_assert(DF_BM == TK && TM % DF_BN == 0, "skip tiles");
+  if (warp == EPI_WARPS) {
+    // uniform as the MMA warp: one elected lane issues the copies
+    const int n = __reduce_max_sync(0xffffffffu, n_act);
+    int ia = 0, slot = 0;
+    uint32_t eph = 1;                                  // parity of the slot's last release (first round: none awaited)
+    bool ok = true;
+    for (int idx = 0; idx < n; ++idx) {
+      const int p = idx & 1, b = __reduce_max_sync(0xffffffffu, (int)act[idx]);
+      if (idx >= 2) ok = bar_wait(b_empty + 8 * p, (uint32_t)((idx >> 1) - 1) & 1u, abort);
+      if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
+      const unsigned char* src = Ad + ((long long)blockIdx.x * nb + b) * (ND * A_DIG);
+      if (elect_one())
+        bulk_load(sbase + NA * A_DIG + p * B_SET, Bd + ((long long)blockIdx.y * nb + b) * B_SET, B_SET, b_full + 8 * p);
+      __syncwarp();
+#pragma unroll
+      for (int s = 0; s < ND; ++s) {
+        if (ia >= NA) ok = ok && bar_wait(a_empty + 8 * slot, eph, abort);
+        if (__all_sync(0xffffffffu, ok)) {
+          if (elect_one()) bulk_load(sbase + slot * A_DIG, src + s * A_DIG, A_DIG, a_full + 8 * slot);
+          ++ia;
+          if (++slot == NA) {
+            slot = 0;
+            eph ^= 1u;
+          }
+        }
+        __syncwarp();
+      }
+      if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
+    }
+    if (!ok) {
+      // the CTA gives up: its copies land before it ends
+      int never = 0;
+      for (int i = ia > NA ? ia - NA : 0; i < ia; ++i) bar_wait(a_full + 8 * (i % NA), (uint32_t)(i / NA) & 1u, &never);
+      bar_wait(b_full, 0, &never);
+      bar_wait(b_full + 8, 0, &never);
+    }
+    __syncwarp();
+  } else if (warp == EPI_WARPS + 1) {
+    // The whole warp walks the blocks on values that the compiler can prove
+    // uniform (reductions and votes across the warp), one elected lane issues:
+    // the MMAs' operands then stay in uniform registers.  With a single thread
+    // in a divergent branch each MMA cost 150 clocks in register moves.
+    const int n = __reduce_max_sync(0xffffffffu, n_act);
+    const uint32_t tm = __reduce_max_sync(0xffffffffu, tmem);
+    // FP32 accumulator, BF16 A and B, both K-major, M = 128; N per digit of A
+    constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TM >> 4) << 24);
+    int slot = 0;
+    uint32_t aph = 0;
+    bool ok = true;
+    for (int idx = 0; idx < n; ++idx) {
+      const int p = idx & 1;
+      if (idx >= 2) ok = bar_wait(acc_empty + 8 * p, (uint32_t)((idx >> 1) - 1) & 1u, abort);
+      ok = ok && bar_wait(b_full + 8 * p, (uint32_t)(idx >> 1) & 1u, abort);
+      if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
+      const uint32_t sB = sbase + NA * A_DIG + p * B_SET;
+#pragma unroll
+      for (int s = 0; s < ND; ++s) {
+        ok = ok && bar_wait(a_full + 8 * slot, aph, abort);
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        constexpr int TKK = 2 * TK;
+        const uint32_t nd = (uint32_t)(TKK * (ND - s));
+        const uint32_t d = tm + (uint32_t)(p * ACC + TKK * s), sA = sbase + slot * A_DIG;
+        if (__all_sync(0xffffffffu, ok) && elect_one()) {
+#pragma unroll
+          for (int kk = 0; kk < 4; ++kk)
+            mma(d, desc(sA + 32 * kk), desc(sB + 32 * kk), idesc | ((nd >> 3) << 17), (s > 0 || kk > 0) ? 1u : 0u);
+          commit(a_empty + 8 * slot);
+        }
+        __syncwarp();
+        if (++slot == NA) {
+          slot = 0;
+          aph ^= 1u;
+        }
+      }
+      if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
+      if (elect_one()) {
+        commit(b_empty + 8 * p);
+        commit(acc_full + 8 * p);
+      }
+      __syncwarp();
+    }
+    if (!ok) {
+      int never = 0;
+      if (elect_one()) commit(fin);
+      __syncwarp();
+      bar_wait(fin, 0, &never);
+    }
+    __syncwarp();
+  } else {
+    static_assert(EK == 4, "two packed pairs of phase rows a warp");
+    const int lg = warp & 3, kq = EK * (warp >> 2);
+    const int rho = n0 + 32 * lg + lane;
+    const int k0 = m0 + kq;
+    const uint32_t tl = tmem + ((uint32_t)(32 * lg) << 16) + (uint32_t)kq;
+    float2 H[2][2], L[2][2];
+    int E[EK];
+#pragma unroll
+    for (int j = 0; j < 2; ++j) H[0][j] = L[0][j] = H[1][j] = L[1][j] = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int j = 0; j < EK; ++j) E[j] = -100000;
+    bool ok = true;
+    // scale exponents, loaded a block ahead; digit 1 times digit 1 weighs 2^-14
+    int eg1 = 0, ex1[EK];
+    auto scales = [&](int b) {
+      eg1 = (rho < N ? eg[(long long)rho * nb + b] : 0) - 14;
+#pragma unroll
+      for (int j = 0; j < EK; ++j) ex1[j] = k0 + j < M ? ex[(long long)(k0 + j) * nb + b] : 0;
+    };
+    if (n_act > 0) scales(act[0]);
+    for (int idx = 0; idx < n_act; ++idx) {
+      const int p = idx & 1;
+      int es[EK];
+#pragma unroll
+      for (int j = 0; j < EK; ++j) es[j] = eg1 + ex1[j];
+      if (idx + 1 < n_act) scales(act[idx + 1]);
+      // one lane polls: the waits of 512 threads would crowd out the barrier
+      // operations of the two threads that feed the tensor core
+      if (lane == 0) ok = bar_wait(acc_full + 8 * p, (uint32_t)(idx >> 1) & 1u, abort);
+      ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
+      if (!ok) break;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      uint32_t v[2][ND][EK];
+#pragma unroll
+      for (int c = 0; c < 2; ++c)
+#pragma unroll
+        for (int d = 0; d < ND; ++d) CSFF_TMEM_LD4(v[c][d], tl + (uint32_t)(p * ACC + 2 * TK * d + TK * c));
+      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) bar_arrive(acc_empty + 8 * p);
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        // merge into the running sums at the larger of the two exponents
+        const int En0 = max(E[2 * j], es[2 * j]), En1 = max(E[2 * j + 1], es[2 * j + 1]);
+        const float2 fa = make_float2(pow2_or_0(E[2 * j] - En0), pow2_or_0(E[2 * j + 1] - En1));
+        const float2 fs = make_float2(pow2_or_0(es[2 * j] - En0), pow2_or_0(es[2 * j + 1] - En1));
+        E[2 * j] = En0;
+        E[2 * j + 1] = En1;
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          float2 q[ND], h, l, t, e;
+#pragma unroll
+          for (int d = 0; d < ND; ++d)
+            q[d] = make_float2(__uint_as_float(v[c][d][2 * j]), __uint_as_float(v[c][d][2 * j + 1]));
+          join(q, h, l);
+          two_sum(__fmul2_rn(H[c][j], fa), __fmul2_rn(h, fs), t, e);
+          e = __fadd2_rn(e, __ffma2_rn(l, fs, __fmul2_rn(L[c][j], fa)));
+          const float2 hn = __fadd2_rn(t, e);
+          L[c][j] = __ffma2_rn(__ffma2_rn(t, both(-1.f), hn), both(-1.f), e);
+          H[c][j] = hn;
+        }
+      }
+    }
+    if (!ok && lane == 0) atomicOr(err, 1);
+    if (rho < N)
+#pragma unroll
+      for (int j = 0; j < EK; ++j) {
+        if (k0 + j >= M) continue;
+        const float hr = (j & 1) ? H[0][j >> 1].y : H[0][j >> 1].x, lr = (j & 1) ? L[0][j >> 1].y : L[0][j >> 1].x;
+        const float hi = (j & 1) ? H[1][j >> 1].y : H[1][j >> 1].x, li = (j & 1) ? L[1][j >> 1].y : L[1][j >> 1].x;
+        T[(long long)(k0 + j) * N + rho] =
+            !ok ? make_double2(__longlong_as_double(0x7ff8000000000000ll), __longlong_as_double(0x7ff8000000000000ll))
+                : E[j] == -100000 ? make_double2(0.0, 0.0)
+                                  : make_double2(bits::widen(hr, E[j]) + bits::widen(lr, E[j]),
+                                                 bits::widen(hi, E[j]) + bits::widen(li, E[j]));
+      }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (warp == EPI_WARPS + 1)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(TMEM_COLS));
 }
 
 // ---- 3D stage A on the tensor cores ------------------------------------------
@@ -1154,13 +1463,13 @@ csff_status far_field_executed(csff_plan* P, double* executed) {
   *executed = 1.0;
   if (!B.dskip || !B.dspread || B.skip_used == 0) return CSFF_OK;
   std::vector<unsigned char> h(B.skip_used);
-  int sp[2] = {0, 0};
+  int sp[3] = {0, 0, 0};
   cudaError_t e = cudaMemcpyAsync(h.data(), B.dskip, h.size(), cudaMemcpyDeviceToHost, P->stream);
   if (e == cudaSuccess) e = cudaMemcpyAsync(sp, B.dspread, sizeof(sp), cudaMemcpyDeviceToHost, P->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(P->stream);
   if (e != cudaSuccess) return cuda_fail(e, "far-field work");
-  const bool df = sp[0] < DF_NONFINITE && sp[1] < DF_NONFINITE && std::min(sp[0], sp[1]) <= DF_SPREAD_LIMIT;
-  if (!df) return CSFF_OK;
+  const bool finite = sp[0] < DF_NONFINITE && sp[1] < DF_NONFINITE;
+  if (!finite || (std::min(sp[0], sp[1]) > DF_SPREAD_LIMIT && sp[2] > digits::MARGIN)) return CSFF_OK;
   size_t run = 0;
   for (unsigned char c : h) run += c == 0;
   *executed = (double)run / (double)h.size();
@@ -1172,7 +1481,7 @@ void free_ff_buffers(csff_plan* P) {
   for (void* p : {(void*)b.dg, (void*)b.dxt, (void*)b.dyt, (void*)b.dzt, (void*)b.dT, (void*)b.dal,
                   (void*)b.dux, (void*)b.dxr, (void*)b.ds1, (void*)b.dmisc, (void*)b.dxdf, (void*)b.dgdf, (void*)b.dxsm, (void*)b.dgsm,
                   (void*)b.dex, (void*)b.deg, (void*)b.dspread, (void*)b.dtcb, (void*)b.dtce, (void*)b.dtcflag,
-                  (void*)b.dxlo, (void*)b.dghi, (void*)b.dskip})
+                  (void*)b.dxlo, (void*)b.dghi, (void*)b.dskip, (void*)b.dxdig, (void*)b.dgdig})
     if (p) cudaFree(p);
   b = FFBuffers{};
 }
@@ -1234,7 +1543,7 @@ csff_status far_field_one(csff_plan* P, const double* eta_host, const double2* u
           cudaSuccess ||
       (e = cudaMemcpyAsync(B.dux, ux.data(), sizeof(double) * n_ux, cudaMemcpyHostToDevice, s)) != cudaSuccess ||
       (e = cudaMemcpyAsync(B.dxr, xr.data(), sizeof(int) * n_ang, cudaMemcpyHostToDevice, s)) != cudaSuccess ||
-      (e = cudaMemsetAsync(B.dmisc + 1, 0, sizeof(int), s)) != cudaSuccess)
+      (e = cudaMemsetAsync(B.dmisc + 1, 0, 2 * sizeof(int), s)) != cudaSuccess)
     return cuda_fail(e, "upload angles");
 
   Tabs8 t{};
@@ -1380,29 +1689,55 @@ csff_status far_field_one(csff_plan* P, const double* eta_host, const double2* u
       (e = ensure((void**)&B.dxlo, B.xlo, sizeof(int) * (size_t)n_ux * nbk, P)) != cudaSuccess ||
       (e = ensure((void**)&B.dghi, B.ghi, sizeof(int) * (size_t)R * nbk, P)) != cudaSuccess)
     return cuda_fail(e, "far field scratch");
-  if (!B.dspread && (e = cudaMalloc((void**)&B.dspread, 2 * sizeof(int))) != cudaSuccess)
+  if (!B.dspread && (e = cudaMalloc((void**)&B.dspread, 3 * sizeof(int))) != cudaSuccess)
     return cuda_fail(e, "far field scratch");
-  if ((e = cudaMemsetAsync(B.dspread, 0, 2 * sizeof(int), s)) != cudaSuccess) return cuda_fail(e, "memset");
+  // the digit contraction: 2D, where its operands fit (without room for them the
+  // double-float one runs)
+  const int gxt = (int)((R + digits::TM - 1) / digits::TM), gkt = (n_ux + digits::TK - 1) / digits::TK;
+  bool dig = d == 2 && nbk <= digits::MAX_NB &&
+             ensure((void**)&B.dxdig, B.xdig, (size_t)gkt * nbk * digits::B_SET, P) == cudaSuccess &&
+             ensure((void**)&B.dgdig, B.gdig, (size_t)gxt * nbk * digits::ND * digits::A_DIG, P) == cudaSuccess;
+  if (!dig) cudaGetLastError();
+  // [2] starts far over the margin where the digit form may not run
+  if ((e = cudaMemsetAsync(B.dspread, 0, 3 * sizeof(int), s)) != cudaSuccess ||
+      (!dig && (e = cudaMemsetAsync(B.dspread + 2, 1, sizeof(int), s)) != cudaSuccess))
+    return cuda_fail(e, "memset");
   {
     const long long wx = (long long)n_ux * nbk, wg = (long long)R * nbk;
-    k_split_rows<<<(unsigned)((wx * 32 + 255) / 256), 256, 0, s>>>(B.dxt, m, n_ux, B.dxdf, B.dxsm, B.dex,
-                                                                   B.dspread, B.dxlo, 1);
-    k_split_rows<<<(unsigned)((wg * 32 + 255) / 256), 256, 0, s>>>(B.dg, m, (int)R, B.dgdf, B.dgsm, B.deg,
-                                                                   B.dspread + 1, B.dghi, 0);
+    k_row_exps<<<(unsigned)((wx * 32 + 255) / 256), 256, 0, s>>>(B.dxt, m, n_ux, B.dex, B.dspread, B.dxlo, 1);
+    k_row_exps<<<(unsigned)((wg * 32 + 255) / 256), 256, 0, s>>>(B.dg, m, (int)R, B.deg, B.dspread + 1, B.dghi, 0);
     count_launch(2);
   }
   dim3 g1((unsigned)((R + S1_BN - 1) / S1_BN), (n_ux + S1_BM - 1) / S1_BM);
   dim3 gdf((unsigned)((R + DF_BN - 1) / DF_BN), (n_ux + DF_BM - 1) / DF_BM);
   if ((e = ensure((void**)&B.dskip, B.skip, (size_t)gdf.x * gdf.y * nbk, P)) != cudaSuccess)
     return cuda_fail(e, "far field scratch");
-  k_ff_df_skip<<<gdf, 256, df_skip_smem(nbk), s>>>(B.dex, B.dxlo, n_ux, B.deg, B.dghi, (int)R, nbk, B.dskip);
+  k_ff_df_skip<<<gdf, 256, df_skip_smem(nbk), s>>>(B.dex, B.dxlo, n_ux, B.deg, B.dghi, (int)R, nbk, B.dskip,
+                                                   B.dspread + 2);
   count_launch();
+  // the operands of whichever contraction the device selects
+  auto warps = [&](long long rows) { return (unsigned)std::min<long long>((rows * nbk * 32 + 255) / 256, 152 * 8); };
+  k_split_rows<<<warps(n_ux), 256, 0, s>>>(B.dxt, m, n_ux, B.dex, B.dspread, B.dxdf, B.dxsm);
+  k_split_rows<<<warps(R), 256, 0, s>>>(B.dg, m, (int)R, B.deg, B.dspread, B.dgdf, B.dgsm);
+  count_launch(2);
+  if (dig) {
+    if ((e = cudaFuncSetAttribute(k_ff_digits, cudaFuncAttributeMaxDynamicSharedMemorySize, digits::SMEM)) != cudaSuccess)
+      return cuda_fail(e, "far-field contraction attribute");
+    k_cut_rows<true><<<warps((long long)gkt * digits::TK), 256, 0, s>>>(B.dxt, m, n_ux, B.dex, B.dspread, B.dxdig);
+    k_cut_rows<false><<<warps((long long)gxt * digits::TM), 256, 0, s>>>(B.dg, m, (int)R, B.deg, B.dspread, B.dgdig);
+    count_launch(2);
+  }
   if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "far-field skip flags");
   B.skip_used = (size_t)gdf.x * gdf.y * nbk;
   {
     ProfScope ps(PF_FF_CONTRACT, s, 16.0 * ((double)n_ux * m + (double)R * m + (double)n_ux * R),
                  8.0 * (double)n_ux * (double)R * m);
-    // exactly one of the two writes T (device-side range check on the spreads)
+    // exactly one of them writes T (device-side checks on the spreads and margin)
+    if (dig) {
+      k_ff_digits<<<dim3(gxt, gkt), digits::NT, digits::SMEM, s>>>(B.dgdig, B.dxdig, B.dex, n_ux, B.deg, (int)R, nbk, B.dspread, B.dskip, (int)gdf.x, B.dT,
+                                                                    B.dmisc + 2);
+      count_launch();
+    }
     k_ff_stage1_df<<<gdf, DF_NT, 0, s>>>(B.dxdf, B.dxsm, B.dex, n_ux, B.dgdf, B.dgsm, B.deg, (int)R, nbk, B.dspread,
                                          B.dskip, B.dT);
     k_ff_stage1<<<g1, 256, 0, s>>>(B.dxt, n_ux, B.dg, (int)R, m, B.dT, B.dspread);
@@ -1420,11 +1755,15 @@ csff_status far_field_one(csff_plan* P, const double* eta_host, const double2* u
   count_launch();
   if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "far field kernels");
   if (scaled) {
-    int flag = 0;
-    if ((e = cudaMemcpyAsync(&flag, B.dmisc + 1, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
+    int flag[2] = {0, 0};
+    if ((e = cudaMemcpyAsync(flag, B.dmisc + 1, sizeof(flag), cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
         (e = cudaStreamSynchronize(s)) != cudaSuccess)
       return cuda_fail(e, "far field flag");
-    *scaled = flag != 0;
+    *scaled = flag[0] != 0;
+    if (flag[1]) {
+      set_error("far-field contraction: an mbarrier wait ran out");
+      return CSFF_ERR_TIMEOUT;
+    }
   }
   return CSFF_OK;
 }

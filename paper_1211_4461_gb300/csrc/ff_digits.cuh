@@ -1,0 +1,183 @@
+// Stage 1 of the 2D far field on the tensor cores, exactly: both operands are
+// cut into 8-bit digits of a fixed-point representation, every digit product
+// and its sums are integers that FP32 accumulation holds without rounding, and
+// the digit sums join in double-float arithmetic.
+//
+// Representation.  As in the double-float form, each row of either operand is
+// scaled by a power of two per block of 32 nodes, so |x'| < 1 there.  Then
+//   x' = sum_{s=1..7} d_s 2^-(8 s - 1) + r,   |d_s| <= 128,  |r| <= 2^-56,
+// digits balanced (round to nearest), stored as BF16 integers.  A product of two
+// digits is at most 2^14; a block's sum over 64 real terms (32 complex nodes)
+// and the at most 7 digit pairs (s, t) of one diagonal s + t = D stays below
+// 2^23, so the FP32 accumulators hold it exactly.  Diagonals D = 2..8 are kept
+// (28 of the 49 pairs); the rest lies below 2^-53 of the blocks' scales.
+//
+// When it runs.  The representation is relative to the block maxima, so the
+// kernel is taken when for every block that a tile keeps the scales ex + eg lie
+// at most MARGIN binades over L, the lower bound of the sum of the terms'
+// magnitudes that the skip kernel forms (phases that vary by less than about
+// 2^10 over 32 nodes: k h sin(gamma) 32 < 7).  Measured errors of a map against a
+// longer sum, relative to the sum of the terms' magnitudes (129^2 to 513^2, k = 1
+// and 2): 2^-52.1 to 2^-51.2 at the worst angle, 2^-50.5 to 2^-49.3 for the
+// double-float kernel, which runs beyond that range.
+//
+// Kernel.  D[rho][j] = sum_K A[rho][K] B[j][K], K = (re, im) of 32 nodes; a
+// CTA takes 128 rows of g (A) and 16 phase rows (B: rows j < 16 give the real
+// parts from (P_re, -P_im), 16 + j the imaginary parts from (P_im, P_re)).  The
+// 32 rows of digit t of B are rows [32 (t - 1), 32 t) of one operand, and
+// diagonal D accumulates in tensor-memory columns [32 (D - 2), 32 (D - 1)), so
+// one MMA of digit s of A against digits 1..8-s of B (N = 32 (8 - s)) adds to
+// the right diagonals: seven MMAs per 16 K values, each reading A once.
+// One thread streams digit tiles (16 KB, pre-swizzled in global memory) into a
+// ring with bulk copies, one issues the MMAs, sixteen warps read the two
+// alternating sets of accumulators and join them, all handing over through
+// mbarriers with bounded waits.
+#pragma once
+
+#include <cuda_bf16.h>
+
+#include "csff_internal.h"
+#include "df_bits.cuh"
+
+namespace csff {
+namespace digits {
+
+constexpr int ND = 7;                          // digits of a value
+constexpr int TM = 128, TK = 16;               // rows of g and phase rows of a tile
+constexpr int KB = 32;                         // nodes of a block
+constexpr int A_DIG = TM * 128;                // bytes of a digit of an A block (128-byte rows)
+constexpr int B_DIG = 2 * TK * 128;
+constexpr int B_SET = ND * B_DIG;
+constexpr int NA = 10;                         // A slots of the ring
+constexpr int MAX_NB = 1024;                   // blocks of a row
+constexpr int EPI_WARPS = 16, NT = 32 * (EPI_WARPS + 2);
+constexpr int EK = TK * 4 / EPI_WARPS;           // phase rows of an epilogue warp
+constexpr int OFF_BAR = NA * A_DIG + 2 * B_SET;
+constexpr int OFF_ACT = OFF_BAR + 512;
+constexpr int SMEM = OFF_ACT + MAX_NB * 2 + 1024;
+constexpr int TMEM_COLS = 512, ACC = 256;      // columns of one set of accumulators (7 x 32 used)
+constexpr int MARGIN = 12;
+constexpr unsigned long long WAIT_NS = 500000000ull;   // a wait gives up after half a second
+static_assert(SMEM <= 227 * 1024, "shared memory");
+
+// 128-byte-swizzled K-major row: byte offset of 16-byte chunk c of row r
+__device__ __forceinline__ int sw(int r, int c) { return (r >> 3) * 1024 + (r & 7) * 128 + ((c ^ (r & 7)) << 4); }
+
+// x 2^(55 - e) rounded to an integer, |x| < 2^e, from the IEEE fields
+__device__ __forceinline__ long long fixed55(double x, int e) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int E = (int)((b >> 52) & 0x7ff);
+  if ((b & bits::ABS_MASK) == 0 || E == 0x7ff) return 0;
+  if (E == 0) return __double2ll_rn(ldexp(x, 55 - e));
+  const long long m = (long long)((b & bits::MANT_MASK) | (1ull << 52));
+  const int sh = E - 1020 - e;                 // m 2^(E - 1075) 2^(55 - e)
+  long long q;
+  if (sh >= 0) q = m << (sh < 3 ? sh : 3);
+  else if (sh < -54) q = 0;
+  else q = (m + (1ll << (-sh - 1))) >> -sh;
+  return (b >> 63) ? -q : q;
+}
+
+// the digits of two fixed-point values as pairs of BF16 integers, dig[0] the
+// leading one
+__device__ __forceinline__ void cut(long long p, long long q, uint32_t (&dig)[ND]) {
+#pragma unroll
+  for (int s = ND - 1; s > 0; --s) {
+    const int a = (int)(signed char)(p & 255), b = (int)(signed char)(q & 255);
+    p = (p - a) >> 8;
+    q = (q - b) >> 8;
+    const __nv_bfloat162 v = __floats2bfloat162_rn((float)a, (float)b);
+    dig[s] = *reinterpret_cast<const uint32_t*>(&v);
+  }
+  const __nv_bfloat162 v = __floats2bfloat162_rn((float)(int)p, (float)(int)q);
+  dig[0] = *reinterpret_cast<const uint32_t*>(&v);
+}
+__device__ __forceinline__ uint32_t neg_hi(uint32_t v) { return v ^ 0x80000000u; }      // (a, b) -> (a, -b)
+__device__ __forceinline__ uint32_t swap_pair(uint32_t v) { return (v >> 16) | (v << 16); }
+
+__device__ __forceinline__ uint32_t saddr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ uint64_t desc(uint32_t a) {
+  return (uint64_t)((a & 0x3FFFF) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)(1024 >> 4) << 32) | ((uint64_t)1 << 46) |
+         ((uint64_t)2 << 61);
+}
+__device__ __forceinline__ void bar_init(uint32_t bar, uint32_t count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count));
+}
+__device__ __forceinline__ void bar_arrive(uint32_t bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+// bounded; gives up early when another thread of the CTA has
+__device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity, volatile int* abort) {
+  unsigned long long t0 = 0;
+  for (int it = 0; it < (1 << 28); ++it) {
+    uint32_t done;
+    asm volatile(
+        "{\n.reg .pred p;\nmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(done)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    if (done) return true;
+    if ((it & 63) == 63) {
+      if (*abort) return false;
+      unsigned long long t;
+      asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+      if (t0 == 0) t0 = t;
+      else if (t - t0 > WAIT_NS) break;
+    }
+  }
+  *abort = 1;
+  return false;
+}
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "l"(src), "r"(bytes), "r"(bar)
+               : "memory");
+}
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
+  return p != 0;
+}
+__device__ __forceinline__ void commit(uint32_t bar) {
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void mma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+  asm volatile(
+      "{\n.reg .pred q;\nsetp.ne.b32 q, %4, 0;\n"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, q;\n}\n" ::"r"(d),
+      "l"(a), "l"(b), "r"(idesc), "r"(acc));
+}
+#define CSFF_TMEM_LD4(v, addr)                                                     \
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"        \
+               : "=r"((v)[0]), "=r"((v)[1]), "=r"((v)[2]), "=r"((v)[3])            \
+               : "r"(addr))
+
+// two sums at once (packed two-lane FP32): t + e = x + y exactly
+__device__ __forceinline__ void two_sum(float2 x, float2 y, float2& t, float2& e) {
+  const float2 m1 = make_float2(-1.f, -1.f);
+  t = __fadd2_rn(x, y);
+  const float2 v = __ffma2_rn(x, m1, t);
+  e = __fadd2_rn(__ffma2_rn(__ffma2_rn(v, m1, t), m1, x), __ffma2_rn(v, m1, y));
+}
+// 2^d for d <= 0, zero from d = -127 on (terms that small add nothing)
+__device__ __forceinline__ float pow2_or_0(int d) { return __int_as_float(max(d + 127, 0) << 23); }
+__device__ __forceinline__ float2 both(float a) { return make_float2(a, a); }
+
+// h + l = sum_{d=0..6} p[d] 2^-8d: the four leading terms by exact sums (their
+// digit sums reach 2^23, eight bits apart), the three trailing ones, whose
+// roundings lie below 2^-55 of the scale, by multiply-adds
+__device__ __forceinline__ void join(const float2 (&p)[ND], float2& h, float2& l) {
+  const float2 w = both(0x1p-8f);
+  float2 q = __ffma2_rn(p[6], w, p[5]);
+  q = __ffma2_rn(q, w, p[4]);
+  float2 e3, e2, e1, t;
+  two_sum(p[3], __fmul2_rn(q, w), t, e3);
+  two_sum(p[2], __fmul2_rn(t, w), t, e2);
+  two_sum(p[1], __fmul2_rn(t, w), t, e1);
+  two_sum(p[0], __fmul2_rn(t, w), h, l);
+  l = __fadd2_rn(l, __fmul2_rn(__ffma2_rn(__ffma2_rn(e3, w, e2), w, e1), w));
+}
+
+}  // namespace digits
+}  // namespace csff

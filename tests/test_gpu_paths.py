@@ -107,3 +107,29 @@ def test_vcycle_jacobi(csff, dim, n, coarsest, nu1, nu2, prec):
                             torch.complex128 if prec == "fp64" else torch.complex64)
     tol = 1e-11 if prec == "fp64" else 1e-4
     assert np.linalg.norm(got - ref) <= tol * np.linalg.norm(ref)
+
+
+# the 2D far-field contraction: row counts below, at and above its tiles of 128
+# rows and 16 phase rows, block counts of one and several, odd angle sets; k =
+# 8 on the small box varies too fast per block for the digit form
+@pytest.mark.parametrize("n,coarsest,n_ang,k,R", [(5, 3, 1, 1.0, 2.0), (33, 5, 33, 1.0, 5.0), (35, 18, 31, 1.0, 5.0),
+                                                  (129, 5, 30, 2.0, 10.0), (137, 18, 97, 2.0, 10.0),
+                                                  (273, 18, 64, 3.0, 10.0), (65, 5, 40, 8.0, 10.0)])
+@pytest.mark.parametrize("scale", [1.0, 1e-200, 1e150])
+def test_far_field_contraction(csff, n, coarsest, n_ang, k, R, scale):
+    prob = W.problem(2, n, R, math.pi / 6, k, [W.gauss(-0.7, 1.5), W.gauss(-0.3, 3.0, (0.5, -0.4, 0.0))])
+    opts = {"smoother": "jacobi", "nu1": 1, "nu2": 1, "coarsest_n": coarsest, "rel_tol": 1e-8, "precision": "fp64"}
+    plan = csff.Plan(prob, opts)
+    m = plan.m
+    u0 = scale * W.rand_complex((m, m), 31)
+    eta = np.array([[math.cos(0.4), math.sin(0.4)]])
+    al = W.angle_set_2d(n_ang)
+    F = torch.zeros(n_ang, dtype=torch.complex128, device="cuda")
+    E = torch.zeros(n_ang, dtype=torch.int32, device="cuda")
+    plan.far_field(eta, torch.from_numpy(u0.ravel()).cuda(), al, F, E)
+    mant, e2, tn = O.far_field(O.problem_from_dict(prob), u0, eta[0], al, return_terms_norm=True)
+    got = F.cpu().numpy() * 2.0 ** (E.cpu().numpy().astype(np.float64) - e2)
+    plan.close()
+    # the contraction's rounding (2^-47 of the sum of the terms' magnitudes for
+    # the double-float form, less for digits) and the phase tables' few ulp
+    assert np.all(np.abs(got - mant) <= 1e-13 * tn)
