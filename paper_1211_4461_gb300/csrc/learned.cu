@@ -1004,7 +1004,7 @@ struct csff_net {
   double* sums = nullptr;        // behind grad, in its allocation
   int cap_b = 0;
   float2* cpatch = nullptr;
-  int* tcerr = nullptr;          // set when a tensor-core layer's wait ran out
+  int* tcerr = nullptr;          // set when a tensor-core layer's wait ran out (pinned: read after a sync)
 };
 
 namespace {
@@ -1248,11 +1248,11 @@ static csff_status net_create(int dim, const float* w_host, csff_net** out) {
       (e = cudaMalloc((void**)&N->v, sizeof(float) * np)) != cudaSuccess ||
       (e = cudaMalloc((void**)&N->grad, sizeof(float) * np)) != cudaSuccess ||
       (e = cudaMalloc((void**)&N->wb, sizeof(__nv_bfloat16) * np)) != cudaSuccess ||
-      (e = cudaMalloc((void**)&N->tcerr, sizeof(int))) != cudaSuccess ||
-      (e = cudaMemset(N->tcerr, 0, sizeof(int))) != cudaSuccess ||
+      (e = cudaMallocHost((void**)&N->tcerr, sizeof(int))) != cudaSuccess ||
       (e = cudaMemset(N->m, 0, sizeof(float) * np)) != cudaSuccess ||
       (e = cudaMemset(N->v, 0, sizeof(float) * np)) != cudaSuccess)
     return fail(csff::cuda_fail(e, "net allocation"));
+  *N->tcerr = 0;
   csff_status s = csff_net_set_weights(N, w_host);
   if (s != CSFF_OK) return fail(s);
   *out = N;
@@ -1263,8 +1263,9 @@ void csff_net_destroy(csff_net* N) {
   if (!N) return;
   for (void* p : {(void*)N->w, (void*)N->m, (void*)N->v, (void*)N->grad, (void*)N->wb, (void*)N->h1, (void*)N->h2,
                   (void*)N->dh1, (void*)N->dh2, (void*)N->y, (void*)N->E, (void*)N->G, (void*)N->dy,
-                  (void*)N->cpatch, (void*)N->tcerr})
+                  (void*)N->cpatch})
     if (p) cudaFree(p);
+  if (N->tcerr) cudaFreeHost(N->tcerr);
   delete N;
 }
 
@@ -1389,12 +1390,11 @@ csff_status net_reserve(csff_net* N, long long npix) {
 }
 
 // status of the tensor-core layers since the last check (synchronises)
+// the network's kernels have completed (the caller has synchronised with them)
 csff_status net_check(csff_net* N) {
-  int err = 0;
-  cudaError_t e = cudaMemcpy(&err, N->tcerr, sizeof(int), cudaMemcpyDeviceToHost);
-  if (e != cudaSuccess) return cuda_fail(e, "net status");
-  if (err) {
-    cudaMemset(N->tcerr, 0, sizeof(int));
+  volatile int* err = N->tcerr;
+  if (*err) {
+    *err = 0;
     set_error("learned smoother: a tensor-core wait ran out");
     return CSFF_ERR_TIMEOUT;
   }
