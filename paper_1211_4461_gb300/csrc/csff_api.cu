@@ -309,14 +309,15 @@ csff_status smooth(csff_plan* P, int l, cx<T>* u, const cx<T>* b, int sweeps, bo
   return CSFF_OK;
 }
 
-template <typename T> csff_status coarsest_solve(csff_plan* P, const cx<T>* b, cx<T>* u) {
+template <typename T>
+csff_status coarsest_solve(csff_plan* P, const cx<T>* b, cx<T>* u, int ring_m = 0, int ring_pitch = 0) {
   if constexpr (sizeof(T) == 4) {
     if (coarse_fp64(P)) {
-      CK(csff::launch_coarse_solve_f64(P->coarse_inv, P->coarse_N, b, u, P->stream), "coarse solve");
+      CK(csff::launch_coarse_solve_f64(P->coarse_inv, P->coarse_N, b, u, P->stream, ring_m, ring_pitch), "coarse solve");
       return CSFF_OK;
     }
   }
-  CK(csff::launch_coarse_solve<T>(cinv<T>(P), P->coarse_N, b, u, P->stream), "coarse solve");
+  CK(csff::launch_coarse_solve<T>(cinv<T>(P), P->coarse_N, b, u, P->stream, ring_m, ring_pitch), "coarse solve");
   return CSFF_OK;
 }
 
@@ -438,16 +439,20 @@ csff_status run_vcycle_learned(csff_plan* P, float2* u, const float2* b, bool ze
   return CSFF_OK;
 }
 
+template <typename T> csff::Split3<T>& split_of(Level& L);
+template <> csff::Split3<float>& split_of<float>(Level& L) { return L.s32; }
+template <> csff::Split3<double>& split_of<double>(Level& L) { return L.s64; }
+
 // The 3D V(1,1) RB-GS cycle on colour-split arrays.  first/last: of the cycles
 // run on one right-hand side (the iterate stays split in between).
 template <typename T>
 csff_status run_split3(csff_plan* P, cx<T>* u, const cx<T>* b, bool zero_init, bool first, bool last) {
   const cx<T>* none = nullptr;
   cx<T>* no = nullptr;
-  CK(csff::launch_split3_down<T>(P->lv, first && !zero_init ? u : none, b, zero_init, first, P->stream), "split down");
+  CK(csff::launch_split3_down<T>(P->lv, first && !zero_init ? u : none, b, zero_init, P->stream), "split down");
   Level& C = P->lv.back();
-  CS(coarsest_solve<T>(P, bbuf<T>(C), ubuf<T>(C)));
-  CK(csff::launch_split3_up<T>(P->lv, last ? u : no, false, P->stream), "split up");
+  CS(coarsest_solve<T>(P, bbuf<T>(C), split_of<T>(C).e, C.m, csff::split3_ring_pitch(C.m)));
+  CK(csff::launch_split3_up<T>(P->lv, last ? u : no, P->stream), "split up");
   return CSFF_OK;
 }
 
@@ -684,23 +689,26 @@ csff_status solve_mixed(csff_plan* P, int eb, double nb, csff_info* info, const 
   return result;
 }
 
-template <typename T> csff::Split3<T>& split_of(Level& L);
-template <> csff::Split3<float>& split_of<float>(Level& L) { return L.s32; }
-template <> csff::Split3<double>& split_of<double>(Level& L) { return L.s64; }
-
-// The colour-split arrays of every level above the coarsest: one allocation a
-// level, and 1/d by colour.  Slots outside the domain hold zero: on the finest
-// level every pass writes whole rows, below it the full weighting does not.
+// The colour-split arrays, one allocation a level, and 1/d by colour.  Slots
+// outside the domain hold zero: on the finest level every pass writes whole
+// rows, below it the full weighting does not, and the ring of a correction is
+// never written.
 template <typename T> csff_status alloc_split3(csff_plan* P) {
-  for (size_t l = 0; l + 1 < P->lv.size(); ++l) {
+  const size_t nl = P->lv.size();
+  for (size_t l = 0; l < nl; ++l) {
     Level& L = P->lv[l];
     csff::Split3<T>& S = split_of<T>(L);
     const size_t half = (size_t)L.m * L.m * csff::split3_pitch(L.m);
-    const size_t total = (l == 0 ? 7 : 8) * half;
+    const size_t ring = l == 0 ? 0 : (size_t)(L.m + 2) * (L.m + 2) * csff::split3_ring_pitch(L.m) + 8;
+    const size_t total = (l + 1 < nl ? (l == 0 ? 7 : 6) * half : 0) + ring;
     cx<T>* base = nullptr;
     CS(dev_alloc(P, &base, total));
     S.base = base;
-    if (l > 0) CK(cudaMemsetAsync(base, 0, total * sizeof(cx<T>), P->stream), "zero split arrays");
+    if (l > 0) {
+      CK(cudaMemsetAsync(base, 0, total * sizeof(cx<T>), P->stream), "zero split arrays");
+      S.e = base + (total - ring);
+    }
+    if (l + 1 == nl) break;
     S.ur = base;
     S.ub = base + half;
     S.br = base + 2 * half;
@@ -708,7 +716,6 @@ template <typename T> csff_status alloc_split3(csff_plan* P) {
     S.dr = base + 4 * half;
     S.db = base + 5 * half;
     if (l == 0) S.delta = base + 6 * half;
-    else S.e = base + 6 * half;
     CK(csff::split3_coefs<T>(L, P->prob.k * P->prob.k, P->stream), "split coefficients");
   }
   return CSFF_OK;

@@ -71,7 +71,7 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
 // ---------------------------------------------------------------------------
 // Colour-split arrays of a 3D level (mg_split3.cu): iterate, right-hand side
 // and 1/d by colour (red, black), the black change of a sweep (finest level),
-// and the level's correction in natural order, rows 2 split3_pitch apart.
+// and the level's correction in natural order with a ring of zeros (mg_split3.cu).
 template <typename T> struct Split3 {
   cx<T> *ur = nullptr, *ub = nullptr, *br = nullptr, *bb = nullptr, *dr = nullptr, *db = nullptr;
   cx<T> *delta = nullptr, *e = nullptr;
@@ -266,10 +266,14 @@ cudaError_t launch_resid_norm(int dim, const Level& L, const double2* u, const d
 template <typename T>
 cudaError_t launch_prolong_add(int dim, const Level& F, const Level& C, const cx<T>* ec, cx<T>* u,
                                cudaStream_t s);
+// ring_m > 0: u is a 3D correction of ring_m points a side in a ring of zeros,
+// rows ring_pitch apart (mg_split3.cu)
 template <typename T>
-cudaError_t launch_coarse_solve(const cx<T>* inv, int N, const cx<T>* b, cx<T>* u, cudaStream_t s);
+cudaError_t launch_coarse_solve(const cx<T>* inv, int N, const cx<T>* b, cx<T>* u, cudaStream_t s, int ring_m = 0,
+                                int ring_pitch = 0);
 // FP32 vectors, FP64 inverse and product, one rounding of the result to FP32
-cudaError_t launch_coarse_solve_f64(const double2* inv, int N, const float2* b, float2* u, cudaStream_t s);
+cudaError_t launch_coarse_solve_f64(const double2* inv, int N, const float2* b, float2* u, cudaStream_t s,
+                                    int ring_m = 0, int ring_pitch = 0);
 // ||v||_2 * 2^{-e_scale}... computed as sqrt(sum |v 2^-e|^2) * 2^e; result to out (device)
 template <typename T>
 cudaError_t launch_norm2(const cx<T>* v, long long N, int exp_scale, double* partial, int nblk,
@@ -324,17 +328,16 @@ cudaError_t launch_scale_to32(const double2* v, long long N, int s_exp, float2* 
 int split3_pitch(int m);                       // slots of a row of one colour
 // 1/d by colour from dinv64 (k2: the wavenumber's square, without potential)
 template <typename T> cudaError_t split3_coefs(Level& L, double k2, cudaStream_t s);
-// the levels down to the coarsest right-hand side (b32/b64 of the last level);
-// new_b: b differs from the last call's; u: the natural iterate, or null when it
-// is still in the split arrays (or zero_init)
-template <typename T>
-cudaError_t launch_split3_down(std::vector<Level>& lv, const cx<T>* u, const cx<T>* b, bool zero_init, bool new_b,
-                               cudaStream_t s);
-// and back from the coarsest solution (u32/u64 of the last level); the iterate
-// goes to u_nat (may be null) and, without u_nat or with keep_split, stays in
+int split3_ring_pitch(int mc);                 // row pitch of a level's correction
+// the levels down to the coarsest right-hand side (b32/b64 of the last level):
+// b and the iterate u in natural order, or zero_init, or (u null) both still in
 // the split arrays
 template <typename T>
-cudaError_t launch_split3_up(std::vector<Level>& lv, cx<T>* u_nat, bool keep_split, cudaStream_t s);
+cudaError_t launch_split3_down(std::vector<Level>& lv, const cx<T>* u, const cx<T>* b, bool zero_init, cudaStream_t s);
+// and back from the coarsest solution (the last level's e); the iterate goes to
+// u_nat in natural order or (null) stays in the split arrays
+template <typename T>
+cudaError_t launch_split3_up(std::vector<Level>& lv, cx<T>* u_nat, cudaStream_t s);
 
 // ---- GMRES(m) smoothing step (gmres.cu) ----------------------------------------
 // u += V y for the GMRES(m) minimiser from u; V holds m+1 vectors of L.N

@@ -232,7 +232,8 @@ __global__ void k_prolong_cells(const cx<T>* __restrict__ ec, int mc, cx<T>* __r
 // of fused multiply-adds joined by shuffles: FP64 work is scarce on this part.
 template <typename T, typename TI, int LPR>
 __global__ void __launch_bounds__(256) k_coarse_solve(const cx<TI>* __restrict__ inv, int N,
-                                                      const cx<T>* __restrict__ b, cx<T>* __restrict__ u) {
+                                                      const cx<T>* __restrict__ b, cx<T>* __restrict__ u, int ring_m,
+                                                      int ring_pitch) {
   pdl_start();
   const int t = blockIdx.x * 256 + threadIdx.x, i = t / LPR, part = t % LPR;
   TI re = (TI)0, im = (TI)0;
@@ -252,7 +253,14 @@ __global__ void __launch_bounds__(256) k_coarse_solve(const cx<TI>* __restrict__
     re += __shfl_xor_sync(0xffffffffu, re, o);
     im += __shfl_xor_sync(0xffffffffu, im, o);
   }
-  if (i < N && part == 0) u[i] = mk<cx<T>>((T)re, (T)im);
+  if (i < N && part == 0) {
+    long long o = i;
+    if (ring_m > 0) {
+      const int r = i / ring_m, y = r % ring_m, z = r / ring_m;
+      o = ((long long)(z + 1) * (ring_m + 2) + y + 1) * ring_pitch + (i - r * ring_m) + 2;
+    }
+    u[o] = mk<cx<T>>((T)re, (T)im);
+  }
 }
 
 // ---- reductions ------------------------------------------------------------
@@ -675,21 +683,24 @@ cudaError_t launch_prolong_add(int dim, const Level& F, const Level& C, const cx
 }
 
 template <typename T, typename TI>
-static cudaError_t coarse_solve(const cx<TI>* inv, int N, const cx<T>* b, cx<T>* u, cudaStream_t s) {
+static cudaError_t coarse_solve(const cx<TI>* inv, int N, const cx<T>* b, cx<T>* u, cudaStream_t s, int rm, int rp) {
   ProfScope ps(mg_family<T>(), s, sizeof(cx<T>) * 2.0 * N + sizeof(cx<TI>) * (double)N * N, 8.0 * N * N);
-  cudaError_t e = N <= 128 ? launch_pdl(k_coarse_solve<T, TI, 4>, dim3((4 * N + 255) / 256), dim3(256), 0, s, inv, N, b, u)
-                           : launch_pdl(k_coarse_solve<T, TI, 32>, dim3((32 * N + 255) / 256), dim3(256), 0, s, inv, N, b, u);
+  cudaError_t e = N <= 128 ? launch_pdl(k_coarse_solve<T, TI, 4>, dim3((4 * N + 255) / 256), dim3(256), 0, s, inv, N, b, u, rm, rp)
+                           : launch_pdl(k_coarse_solve<T, TI, 32>, dim3((32 * N + 255) / 256), dim3(256), 0, s, inv, N, b, u,
+                                        rm, rp);
   count_launch();
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 template <typename T>
-cudaError_t launch_coarse_solve(const cx<T>* inv, int N, const cx<T>* b, cx<T>* u, cudaStream_t s) {
-  return coarse_solve<T, T>(inv, N, b, u, s);
+cudaError_t launch_coarse_solve(const cx<T>* inv, int N, const cx<T>* b, cx<T>* u, cudaStream_t s, int ring_m,
+                                int ring_pitch) {
+  return coarse_solve<T, T>(inv, N, b, u, s, ring_m, ring_pitch);
 }
 
-cudaError_t launch_coarse_solve_f64(const double2* inv, int N, const float2* b, float2* u, cudaStream_t s) {
-  return coarse_solve<float, double>(inv, N, b, u, s);
+cudaError_t launch_coarse_solve_f64(const double2* inv, int N, const float2* b, float2* u, cudaStream_t s, int ring_m,
+                                    int ring_pitch) {
+  return coarse_solve<float, double>(inv, N, b, u, s, ring_m, ring_pitch);
 }
 
 cudaError_t launch_resid_norm(int dim, const Level& L, const double2* u, const double2* b, int exp_scale,
@@ -846,7 +857,7 @@ cudaError_t launch_zero(cx<T>* v, long long N, cudaStream_t s) {
                                           cudaStream_t);                                               \
   template cudaError_t launch_prolong_add<T>(int, const Level&, const Level&, const cx<T>*, cx<T>*,    \
                                              cudaStream_t);                                            \
-  template cudaError_t launch_coarse_solve<T>(const cx<T>*, int, const cx<T>*, cx<T>*, cudaStream_t);     \
+  template cudaError_t launch_coarse_solve<T>(const cx<T>*, int, const cx<T>*, cx<T>*, cudaStream_t, int, int);     \
   template cudaError_t launch_norm2<T>(const cx<T>*, long long, int, double*, int, double*,            \
                                        cudaStream_t);                                                  \
   template cudaError_t launch_zero<T>(cx<T>*, long long, cudaStream_t);

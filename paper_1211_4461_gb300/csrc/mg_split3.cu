@@ -72,35 +72,50 @@ __device__ __forceinline__ bool at(int m, int HP, At& p) {
   return p.j < HP && p.iy < m;
 }
 
-// b (both colours) and, when u_nat, the black points of u from natural order;
-// with dr (the iterate enters as zero) the red half sweep u = d^{-1} b
-template <typename T>
-__global__ void k3s_import(const cx<T>* __restrict__ b_nat, const cx<T>* __restrict__ u_nat,
-                           const cx<T>* __restrict__ dr, cx<T> d0, int m, int HP, cx<T>* __restrict__ br,
-                           cx<T>* __restrict__ bb, cx<T>* __restrict__ ub, cx<T>* __restrict__ ur) {
+// Natural order in: b by colour and the red half sweep, from zero (u = d^{-1} b,
+// NAT_U false) or from a natural iterate, whose black points go to ub.
+template <typename T, bool NAT_U>
+__global__ void k3s_first(const cx<T>* __restrict__ b_nat, const cx<T>* __restrict__ u_nat,
+                          const cx<T>* __restrict__ dr, cx<T> c, cx<T> d0, int m, int HP, cx<T>* __restrict__ br,
+                          cx<T>* __restrict__ bb, cx<T>* __restrict__ ub, cx<T>* __restrict__ ur) {
   using C = cx<T>;
   pdl_prologue();
   At p;
   if (!at(m, HP, p)) return;
   const int o = (p.iy + p.iz + 1) & 1;                 // red parity of the row
   const C* row = b_nat + p.row * m;
-  const int x = 2 * p.j;
+  const int x = 2 * p.j, x0 = x + o, x1 = x0 + 2;
   C v[4];
 #pragma unroll
   for (int k = 0; k < 4; ++k) v[k] = x + k < m ? row[x + k] : zc<T>();
   const long long s = p.row * HP + p.j;
+  const Pair<T> d = ld2(dr + s);
+  C s0 = zc<T>(), s1 = zc<T>();
+  if constexpr (NAT_U) {
+    const C* u = u_nat + p.row * m;
+    const long long pl = (long long)m * m;
+    const bool i0 = x0 < m, i1 = x1 < m;
+    const C xl = (x0 > 0 && x0 - 1 < m) ? u[x0 - 1] : zc<T>(), xm = x0 + 1 < m ? u[x0 + 1] : zc<T>(),
+            xr = x1 + 1 < m ? u[x1 + 1] : zc<T>();
+    auto at_row = [&](bool in, long long off, C& q0, C& q1) {
+      q0 = in && i0 ? u[x0 + off] : zc<T>();
+      q1 = in && i1 ? u[x1 + off] : zc<T>();
+    };
+    C yl0, yl1, yr0, yr1, zl0, zl1, zr0, zr1;
+    at_row(p.iy > 0, -m, yl0, yl1);
+    at_row(p.iy < m - 1, m, yr0, yr1);
+    at_row(p.iz > 0, -pl, zl0, zl1);
+    at_row(p.iz < m - 1, pl, zr0, zr1);
+    s0 = cadd(cadd(cadd(xl, xm), cadd(yl0, yr0)), cadd(zl0, zr0));
+    s1 = cadd(cadd(cadd(xm, xr), cadd(yl1, yr1)), cadd(zl1, zr1));
+    // black slots: x = 2 j + 1 - o
+    st2(ub + s, o ? xl : xm, o ? xm : xr);
+  }
   const C r0 = o ? v[1] : v[0], r1 = o ? v[3] : v[2];
   st2(br + s, r0, r1);
   st2(bb + s, o ? v[0] : v[1], o ? v[2] : v[3]);
-  if (dr) {
-    const Pair<T> d = ld2(dr + s);
-    st2(ur + s, dinv_mul(d0, d.a, r0), dinv_mul(d0, d.b, r1));
-  }
-  if (u_nat) {
-    const C* ru = u_nat + p.row * m;
-    const int x0 = x + 1 - o, x1 = x0 + 2;
-    st2(ub + s, x0 < m ? ru[x0] : zc<T>(), x1 < m ? ru[x1] : zc<T>());
-  }
+  st2(ur + s, x0 < m ? dinv_mul(d0, d.a, NAT_U ? cfma(r0, c, s0) : r0) : zc<T>(),
+      x1 < m ? dinv_mul(d0, d.b, NAT_U ? cfma(r1, c, s1) : r1) : zc<T>());
 }
 
 // a level's d^{-1} by colour: FP64 as stored; FP32 as the difference to d0 of
@@ -134,56 +149,51 @@ __global__ void k3s_split(const double2* __restrict__ dinv, float2 dc, cx<T> d0,
   st2(black + s, o ? v[0] : v[1], o ? v[2] : v[3]);
 }
 
+// The coarse correction e is kept with a ring of zeros: node (X, Y, Z), X, Y, Z
+// in [0, mc + 1], at (Z (mc + 2) + Y) pe + X + 1, so that the columns X = j + 1,
+// j + 2 of an even slot j are one aligned access and no load is tested.
+//
 // Neighbour sum of the interpolated correction P e at the red slots j, j + 1 of
 // row (iy, iz).  Node indices: a red node has an even number of odd indices.
 // All even (a coarse node K): 3 e_K + 1/2 sum of its six coarse neighbours.
 // Two odd: with S4 the sum of the four coarse corners around the point in the
 // plane of its odd axes, 5/4 S4 + 1/8 (S4 one coarse plane up and one down the
-// even axis).  e: coarse values, x first, rows pe elements apart, mc a side.
+// even axis).
 template <typename T>
 __device__ __forceinline__ Pair<T> prolong_nbr(const cx<T>* __restrict__ e, int pe, int mc, int j, int iy, int iz) {
   using C = cx<T>;
   const bool oy = !(iy & 1), oz = !(iz & 1);           // odd node indices
   const int Y = (iy + 1) >> 1, Z = (iz + 1) >> 1;      // coarse node at or below
-  auto rowp = [&](int y, int z) -> const C* {
-    return (y >= 1 && y <= mc && z >= 1 && z <= mc) ? e + ((long long)(z - 1) * mc + (y - 1)) * pe - 1 : nullptr;
-  };
-  auto val = [&](const C* r, int X) -> C { return (r && X >= 1 && X <= mc) ? r[X] : zc<T>(); };
+  const long long pz = (long long)(mc + 2) * pe;
+  const C* r = e + Z * pz + (long long)Y * pe + j;     // r[k]: column X = j - 1 + k
   Pair<T> out;
   if (oy == oz) {                                      // x even: coarse columns j + 1 and j + 2
-    const int X = j + 1;
     if (!oy) {
-      const C* r = rowp(Y, Z);
-      const C e0 = val(r, X - 1), e1 = val(r, X), e2 = val(r, X + 1), e3 = val(r, X + 2);
-      C a = cadd(e0, e2), b = cadd(e1, e3);
-      const C *r1 = rowp(Y - 1, Z), *r2 = rowp(Y + 1, Z), *r3 = rowp(Y, Z - 1), *r4 = rowp(Y, Z + 1);
-      a = cadd(a, cadd(cadd(val(r1, X), val(r2, X)), cadd(val(r3, X), val(r4, X))));
-      b = cadd(b, cadd(cadd(val(r1, X + 1), val(r2, X + 1)), cadd(val(r3, X + 1), val(r4, X + 1))));
-      out.a = cadd(cscale(e1, (T)3), cscale(a, (T)0.5));
-      out.b = cadd(cscale(e2, (T)3), cscale(b, (T)0.5));
+      const C e0 = r[1], e3 = r[4];
+      const Pair<T> m = ld2(r + 2), a = ld2(r + 2 - pe), b = ld2(r + 2 + pe), f = ld2(r + 2 - pz), g = ld2(r + 2 + pz);
+      const C s0 = cadd(cadd(e0, m.b), cadd(cadd(a.a, b.a), cadd(f.a, g.a)));
+      const C s1 = cadd(cadd(m.a, e3), cadd(cadd(a.b, b.b), cadd(f.b, g.b)));
+      out.a = cadd(cscale(m.a, (T)3), cscale(s0, (T)0.5));
+      out.b = cadd(cscale(m.b, (T)3), cscale(s1, (T)0.5));
     } else {
-      const C *r1 = rowp(Y, Z), *r2 = rowp(Y + 1, Z), *r3 = rowp(Y, Z + 1), *r4 = rowp(Y + 1, Z + 1);
       C s[4];
-#pragma unroll
-      for (int k = 0; k < 4; ++k)
-        s[k] = cadd(cadd(val(r1, X - 1 + k), val(r2, X - 1 + k)), cadd(val(r3, X - 1 + k), val(r4, X - 1 + k)));
+      const C *r2 = r + pe, *r3 = r + pz, *r4 = r3 + pe;
+      const Pair<T> m1 = ld2(r + 2), m2 = ld2(r2 + 2), m3 = ld2(r3 + 2), m4 = ld2(r4 + 2);
+      s[0] = cadd(cadd(r[1], r2[1]), cadd(r3[1], r4[1]));
+      s[1] = cadd(cadd(m1.a, m2.a), cadd(m3.a, m4.a));
+      s[2] = cadd(cadd(m1.b, m2.b), cadd(m3.b, m4.b));
+      s[3] = cadd(cadd(r[4], r2[4]), cadd(r3[4], r4[4]));
       out.a = cadd(cscale(s[1], (T)1.25), cscale(cadd(s[0], s[2]), (T)0.125));
       out.b = cadd(cscale(s[2], (T)1.25), cscale(cadd(s[1], s[3]), (T)0.125));
     }
   } else {                                             // x odd: between coarse columns j and j + 1 (j + 1 and j + 2)
     C t0[3], t1[3];                                    // S4 at the even axis' plane below, at, above
+    const long long step = oy ? pz : pe, pair = oy ? pe : pz;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-      const C *r1, *r2;
-      if (oy) {
-        r1 = rowp(Y, Z - 1 + k);
-        r2 = rowp(Y + 1, Z - 1 + k);
-      } else {
-        r1 = rowp(Y - 1 + k, Z);
-        r2 = rowp(Y - 1 + k, Z + 1);
-      }
-      const C c0 = cadd(val(r1, j), val(r2, j)), c1 = cadd(val(r1, j + 1), val(r2, j + 1)),
-              c2 = cadd(val(r1, j + 2), val(r2, j + 2));
+      const C* q = r + (k - 1) * step;
+      const Pair<T> a = ld2(q + 2), b = ld2(q + pair + 2);
+      const C c0 = cadd(q[1], q[pair + 1]), c1 = cadd(a.a, b.a), c2 = cadd(a.b, b.b);
       t0[k] = cadd(c0, c1);
       t1[k] = cadd(c1, c2);
     }
@@ -197,9 +207,9 @@ __device__ __forceinline__ Pair<T> prolong_nbr(const cx<T>* __restrict__ e, int 
 //  PLAIN: u
 //  PROLONG (red): the neighbours are u + P e
 //  DELTA (black): also delta = u_new - u_old
-//  NAT (black): both colours to nat in natural order (rows nat_pitch apart); the
-//  split black values too when u
-enum Mode { PLAIN, PROLONG, DELTA, NAT };
+//  NAT (black): both colours to nat in natural order
+//  RING (black): both colours to nat as the ringed correction, rows nat_pitch apart
+enum Mode { PLAIN, PROLONG, DELTA, NAT, RING };
 template <typename T, int COLOUR, int MODE>
 __global__ void k3s_sweep(const cx<T>* __restrict__ uo, const cx<T>* __restrict__ b, const cx<T>* __restrict__ dinv,
                           cx<T> c, cx<T> d0, int m, int HP, cx<T>* u, cx<T>* __restrict__ delta,
@@ -233,19 +243,20 @@ __global__ void k3s_sweep(const cx<T>* __restrict__ uo, const cx<T>* __restrict_
   const int x0 = 2 * p.j + o, x1 = x0 + 2;
   const C v0 = x0 < m ? dinv_mul(d0, dv.a, cfma(bv.a, c, s0)) : zc<T>();
   const C v1 = x1 < m ? dinv_mul(d0, dv.b, cfma(bv.b, c, s1)) : zc<T>();
-  if (MODE != NAT || u) st2(u + s, v0, v1);
+  if constexpr (MODE != NAT && MODE != RING) st2(u + s, v0, v1);
   if constexpr (MODE == DELTA) st2(delta + s, csub(v0, old.a), csub(v1, old.b));
+  if constexpr (MODE == RING) {
+    // slots outside the domain are zero, as the ring has to stay
+    C* n = nat + ((long long)(p.iz + 1) * (m + 2) + p.iy + 1) * nat_pitch + 2 * p.j + 2;
+    st2(n, o ? mid.a : v0, o ? v0 : mid.a);
+    if (2 * p.j + 2 < m) st2(n + 2, o ? mid.b : v1, o ? v1 : mid.b);
+  }
   if constexpr (MODE == NAT) {
-    C* n = nat + p.row * nat_pitch + 2 * p.j;
+    C* n = nat + p.row * m + 2 * p.j;
     const C w[4] = {o ? mid.a : v0, o ? v0 : mid.a, o ? mid.b : v1, o ? v1 : mid.b};
-    if (nat_pitch == 2 * HP) {
-      st2(n, w[0], w[1]);
-      st2(n + 2, w[2], w[3]);
-    } else {
 #pragma unroll
-      for (int k = 0; k < 4; ++k)
-        if (2 * p.j + k < m) n[k] = w[k];
-    }
+    for (int k = 0; k < 4; ++k)
+      if (2 * p.j + k < m) n[k] = w[k];
   }
 }
 
@@ -337,9 +348,6 @@ Shape shape(int pairs, int m) {
 template <typename T> Split3<T>& sp(Level& L);
 template <> Split3<float>& sp<float>(Level& L) { return L.s32; }
 template <> Split3<double>& sp<double>(Level& L) { return L.s64; }
-template <typename T> cx<T>* nat_u(Level& L);
-template <> float2* nat_u<float>(Level& L) { return L.u32; }
-template <> double2* nat_u<double>(Level& L) { return L.u64; }
 template <typename T> cx<T>* nat_b(Level& L);
 template <> float2* nat_b<float>(Level& L) { return L.b32; }
 template <> double2* nat_b<double>(Level& L) { return L.b64; }
@@ -347,6 +355,8 @@ template <> double2* nat_b<double>(Level& L) { return L.b64; }
 }  // namespace
 
 int split3_pitch(int m) { return ((m + 1) / 2 + 3) / 4 * 4; }
+// the finer level's slots j < HP read columns up to j + 4
+int split3_ring_pitch(int mc) { return split3_pitch(2 * mc + 1) + 4; }
 
 template <typename T>
 cudaError_t split3_coefs(Level& L, double k2, cudaStream_t s) {
@@ -363,8 +373,7 @@ cudaError_t split3_coefs(Level& L, double k2, cudaStream_t s) {
 }
 
 template <typename T>
-cudaError_t launch_split3_down(std::vector<Level>& lv, const cx<T>* u, const cx<T>* b, bool zero_init, bool new_b,
-                               cudaStream_t s) {
+cudaError_t launch_split3_down(std::vector<Level>& lv, const cx<T>* u, const cx<T>* b, bool zero_init, cudaStream_t s) {
   cudaError_t e = cudaSuccess;
   int launches = 0;
   auto ok = [&](cudaError_t r) { ++launches; if (e == cudaSuccess) e = r; };
@@ -381,10 +390,13 @@ cudaError_t launch_split3_down(std::vector<Level>& lv, const cx<T>* u, const cx<
     const bool zero = zero_init || l > 0;
     ProfScope ps(mg_family<T>(), s, (zero ? 3.5 : 6.0) * S * L.N + S * C.N, 0);
     if (l == 0) {
-      if (new_b || u)
-        ok(launch_pdl(k3s_import<T>, h.g, h.b, 0, s, b, zero ? none : u, zero ? (const cx<T>*)F.dr : none, F.d0, m, HP, F.br,
-                      F.bb, F.ub, F.ur));
-      if (!zero)
+      if (zero)
+        ok(launch_pdl(k3s_first<T, false>, h.g, h.b, 0, s, b, none, (const cx<T>*)F.dr, c, F.d0, m, HP, F.br, F.bb, no,
+                      F.ur));
+      else if (u)
+        ok(launch_pdl(k3s_first<T, true>, h.g, h.b, 0, s, b, u, (const cx<T>*)F.dr, c, F.d0, m, HP, F.br, F.bb, F.ub,
+                      F.ur));
+      else
         ok(launch_pdl(k3s_sweep<T, 0, PLAIN>, h.g, h.b, 0, s, (const cx<T>*)F.ub, (const cx<T>*)F.br,
                       (const cx<T>*)F.dr, c, F.d0, m, HP, F.ur, no, none, 0, 0, no, 0));
     }
@@ -402,7 +414,7 @@ cudaError_t launch_split3_down(std::vector<Level>& lv, const cx<T>* u, const cx<
 }
 
 template <typename T>
-cudaError_t launch_split3_up(std::vector<Level>& lv, cx<T>* u_nat, bool keep_split, cudaStream_t s) {
+cudaError_t launch_split3_up(std::vector<Level>& lv, cx<T>* u_nat, cudaStream_t s) {
   cudaError_t e = cudaSuccess;
   int launches = 0;
   auto ok = [&](cudaError_t r) { ++launches; if (e == cudaSuccess) e = r; };
@@ -414,20 +426,20 @@ cudaError_t launch_split3_up(std::vector<Level>& lv, cx<T>* u_nat, bool keep_spl
     const int m = L.m, HP = split3_pitch(m);
     const cx<T> c = mk<cx<T>>((T)L.c.x, (T)L.c.y);
     const Shape h = shape(HP / 2, m);
-    const bool last = l + 2 == nl;
-    const cx<T>* ev = last ? nat_u<T>(C) : G.e;
     const cx<T>* none = nullptr;
     cx<T>* no = nullptr;
     ProfScope ps(mg_family<T>(), s, 5.0 * S * L.N + S * C.N, 0);
     ok(launch_pdl(k3s_sweep<T, 0, PROLONG>, h.g, h.b, 0, s, (const cx<T>*)F.ub, (const cx<T>*)F.br,
-                  (const cx<T>*)F.dr, c, F.d0, m, HP, F.ur, no, ev, last ? C.m : 2 * split3_pitch(C.m), C.m, no, 0));
-    if (l == 0 && !u_nat)
+                  (const cx<T>*)F.dr, c, F.d0, m, HP, F.ur, no, (const cx<T>*)G.e, split3_ring_pitch(C.m), C.m, no, 0));
+    if (l > 0)
+      ok(launch_pdl(k3s_sweep<T, 1, RING>, h.g, h.b, 0, s, (const cx<T>*)F.ur, (const cx<T>*)F.bb, (const cx<T>*)F.db,
+                    c, F.d0, m, HP, no, no, none, 0, 0, F.e, split3_ring_pitch(m)));
+    else if (u_nat)
+      ok(launch_pdl(k3s_sweep<T, 1, NAT>, h.g, h.b, 0, s, (const cx<T>*)F.ur, (const cx<T>*)F.bb, (const cx<T>*)F.db,
+                    c, F.d0, m, HP, no, no, none, 0, 0, u_nat, 0));
+    else
       ok(launch_pdl(k3s_sweep<T, 1, PLAIN>, h.g, h.b, 0, s, (const cx<T>*)F.ur, (const cx<T>*)F.bb, (const cx<T>*)F.db,
                     c, F.d0, m, HP, F.ub, no, none, 0, 0, no, 0));
-    else
-      ok(launch_pdl(k3s_sweep<T, 1, NAT>, h.g, h.b, 0, s, (const cx<T>*)F.ur, (const cx<T>*)F.bb, (const cx<T>*)F.db,
-                    c, F.d0, m, HP, l == 0 && keep_split ? F.ub : no, no, none, 0, 0, l == 0 ? u_nat : F.e,
-                    l == 0 ? m : 2 * HP));
   }
   count_launch(launches);
   return e != cudaSuccess ? e : cudaGetLastError();
@@ -435,9 +447,8 @@ cudaError_t launch_split3_up(std::vector<Level>& lv, cx<T>* u_nat, bool keep_spl
 
 #define CSFF_SPLIT3_INST(T)                                                                                      \
   template cudaError_t split3_coefs<T>(Level&, double, cudaStream_t);                                                 \
-  template cudaError_t launch_split3_down<T>(std::vector<Level>&, const cx<T>*, const cx<T>*, bool, bool,        \
-                                             cudaStream_t);                                                     \
-  template cudaError_t launch_split3_up<T>(std::vector<Level>&, cx<T>*, bool, cudaStream_t);
+  template cudaError_t launch_split3_down<T>(std::vector<Level>&, const cx<T>*, const cx<T>*, bool, cudaStream_t); \
+  template cudaError_t launch_split3_up<T>(std::vector<Level>&, cx<T>*, cudaStream_t);
 CSFF_SPLIT3_INST(float)
 CSFF_SPLIT3_INST(double)
 
