@@ -30,6 +30,7 @@
 #include <cstring>
 #include <vector>
 
+#include "df_bits.cuh"
 #include "mg_tiles.cuh"
 #include "net_tile.cuh"
 
@@ -37,7 +38,7 @@ namespace csff {
 namespace {
 
 constexpr int MAXL = 12;            // levels per instance
-constexpr int PT = 2048;            // points per FP64 tile (256 threads x 8)
+constexpr int PY = 8;               // rows of a tile of the point phases (256 columns, one a thread)
 constexpr long long BAR_SPIN_LIMIT = 1ll << 26;
 
 struct BLevel {
@@ -55,8 +56,7 @@ struct BInst {
   const double2* inv64;             // coarsest inverse, applied in FP64 to the FP32 right-hand side
   double2 c64;
   const double2* q64;
-  double2* u64[2];                  // current iterate alternates between these
-  double2 *b64, *r64;
+  double2 *u64, *b64;
   const double2* chi;               // [n_gauss][2][m]
   const double2* uinc;              // [2][m]
   double k2;
@@ -64,8 +64,8 @@ struct BInst {
 };
 
 struct BState {
-  int done, status, cycles, refinements, e, eb, cur, rises, n_hist;
-  int n_step;                       // FP32 cycles of the current refinement step
+  int done, status, cycles, refinements, eb, rises, n_hist;
+  int n_step;                       // FP32 cycles of the current refinement step, 0 once done
   int lrn, lflags;                  // learned step on; bit 0 a network is set, bit 1 it was switched off
   double lref;                      // reference reduction factor of the learned steps
   double prev, nb, rel;
@@ -136,9 +136,7 @@ __device__ __forceinline__ bool inst_done(const BState* st, int i) {
 }
 
 // instance i still runs FP32 cycle c of the current refinement step
-__device__ __forceinline__ bool in_cycle(const BState* st, int i, int c) {
-  return !inst_done(st, i) && c < __ldcg(&st[i].n_step);
-}
+__device__ __forceinline__ bool in_cycle(const BState* st, int i, int c) { return c < __ldcg(&st[i].n_step); }
 
 // ... and ends it with the learned step
 __device__ __forceinline__ bool learned_now(const BState* st, int i, int c) {
@@ -157,95 +155,132 @@ __device__ __forceinline__ V block_sum(V v, V* sh) {
   return s;
 }
 
-__device__ __forceinline__ int frexp_e(double a) {
-  int e = 0;
-  frexp(a, &e);
-  return e;
+// A tile of the point phases: column x (one a thread), rows [y0, y1) of the grid.
+// Marching over rows, a thread has the values above and below in registers.
+struct PTile { int x, y0, y1; };
+__host__ __device__ inline int point_tiles(int m) { return ((m + 255) / 256) * ((m + PY - 1) / PY); }
+__device__ __forceinline__ PTile point_tile(int m, int t) {
+  const int nbx = (m + 255) / 256, by = t / nbx;
+  return PTile{(t - by * nbx) * 256 + (int)threadIdx.x, by * PY, min(by * PY + PY, m)};
+}
+
+// the norms' prescale 2^-eb: needed only where squares could leave FP64's range
+__device__ __forceinline__ double norm_scale(int eb) {
+  return abs(eb) <= 400 ? 1.0 : ldexp(1.0, -min(max(eb, -1000), 1000));
+}
+__device__ __forceinline__ double sq_add(double2 r, double sc, double acc) {
+  if (sc != 1.0) r = cscale(r, sc);
+  return fma(r.x, r.x, fma(r.y, r.y, acc));
 }
 
 // ---- FP64 point phases --------------------------------------------------------
-// rhs: b = k^2 chi u_in, u = 0, r = b; max exponent of |b| into eb
+// Bound by the FP64 pipe (a warp instruction in 19 clocks an SM), so scalings,
+// exponents and conversions work on the bit fields and the iterate is updated
+// in a phase of its own: a refinement step takes 20 FP64 operations a point
+// (2 update, 16 residual, 2 norm).  Formed on the fly at the five points of
+// the stencil, with the conversions in FP64 and the next right-hand side's
+// rounding in another phase, it took 52.
+
+// rhs: b = k^2 chi u_in, u = 0; max exponent of |b| into eb
 __device__ void ph_rhs(const BInst& I, BState* st, int i, int t) {
   __shared__ int smax;
   if (threadIdx.x == 0) smax = -2000;
   __syncthreads();
   const int m = I.m;
+  const PTile p = point_tile(m, t);
   int mx = -2000;
-  for (long long j = (long long)t * PT + threadIdx.x; j < min((long long)(t + 1) * PT, I.N); j += blockDim.x) {
-    int ix = (int)(j % m), iy = (int)(j / m);
-    double2 cu = make_double2(0, 0);      // chi u_in, axis factors paired first
+  if (p.x < m) {
+    // chi u_in by Gaussians, axis factors paired first (the sum of several
+    // passes through b, which only this thread touches)
     for (int g = 0; g < I.n_gauss; ++g) {
       const double2* tb = I.chi + (size_t)g * 2 * m;
-      cu = cadd(cu, cmul(cmul(tb[ix], I.uinc[ix]), cmul(tb[m + iy], I.uinc[m + iy])));
+      const double2 fx = cmul(tb[p.x], I.uinc[p.x]);
+      for (int iy = p.y0; iy < p.y1; ++iy) {
+        const long long j = (long long)iy * m + p.x;
+        double2 v = cmul(fx, cmul(tb[m + iy], I.uinc[m + iy]));
+        if (g > 0) v = cadd(I.b64[j], v);
+        I.b64[j] = v;
+      }
     }
-    double2 bj = cscale(cu, I.k2);
-    I.b64[j] = bj;
-    I.r64[j] = bj;
-    I.u64[0][j] = make_double2(0, 0);
-    double a = fmax(fabs(bj.x), fabs(bj.y));
-    int e = (a == 0.0) ? -2000 : (isfinite(a) ? frexp_e(a) : 4000);
-    mx = max(mx, e);
+    for (int iy = p.y0; iy < p.y1; ++iy) {
+      const long long j = (long long)iy * m + p.x;
+      const double2 v = I.n_gauss > 0 ? cscale(I.b64[j], I.k2) : make_double2(0, 0);
+      I.b64[j] = v;
+      I.u64[j] = make_double2(0, 0);
+      const unsigned long long ax = (unsigned long long)__double_as_longlong(v.x) & bits::ABS_MASK,
+                               ay = (unsigned long long)__double_as_longlong(v.y) & bits::ABS_MASK;
+      const double a = __longlong_as_double((long long)max(ax, ay));
+      mx = max(mx, max(ax, ay) == 0 ? -2000 : (bits::exp_field(a) == 0x7ff ? 4000 : bits::frexp_exp(a)));
+    }
   }
-  atomicMax(&smax, mx);
+  mx = __reduce_max_sync(0xffffffffu, mx);
+  if ((threadIdx.x & 31) == 0) atomicMax(&smax, mx);
   __syncthreads();
   if (threadIdx.x == 0) atomicMax(&st[i].eb, smax);
 }
 
-// norm partial of r (or b) with the prescale 2^-eb
-__device__ void ph_norm(const BInst& I, const BState* st, int i, int t, double* partial, double* shd) {
-  const int eb = __ldcg(&st[i].eb);
-  const double sc = ldexp(1.0, -min(max(eb, -1000), 1000));
+// the first residual, b: its rounding 2^-eb b to FP32 and its norm partial
+__device__ void ph_first(const BInst& I, const BState* st, int i, int t, double* partial, double* shd) {
+  const int eb = __ldcg(&st[i].eb), m = I.m;
+  const double sc = norm_scale(eb);
+  const PTile p = point_tile(m, t);
   double acc = 0;
-  for (long long j = (long long)t * PT + threadIdx.x; j < min((long long)(t + 1) * PT, I.N); j += blockDim.x) {
-    double2 v = __ldcg(I.r64 + j);
-    double a = v.x * sc, b = v.y * sc;
-    acc = fma(a, a, fma(b, b, acc));
-  }
+  if (p.x < m)
+    for (int iy = p.y0; iy < p.y1; ++iy) {
+      const long long j = (long long)iy * m + p.x;
+      const double2 v = __ldcg(I.b64 + j);
+      I.L[0].b[j] = make_float2(bits::narrow(v.x, eb), bits::narrow(v.y, eb));
+      acc = sq_add(v, sc, acc);
+    }
   acc = block_sum(acc, shd);
   if (threadIdx.x == 0) *partial = acc;
 }
 
-// r32 = r64 2^-e into the level-0 FP32 right-hand side
-__device__ void ph_to32(const BInst& I, const BState* st, int i, int t) {
-  const double s = ldexp(1.0, -__ldcg(&st[i].e));
-  for (long long j = (long long)t * PT + threadIdx.x; j < min((long long)(t + 1) * PT, I.N); j += blockDim.x) {
-    double2 r = __ldcg(I.r64 + j);
-    I.L[0].b[j] = make_float2((float)(r.x * s), (float)(r.y * s));
-  }
+// u += 2^eb e32
+__device__ void ph_update(const BInst& I, const BState* st, int i, int t) {
+  const int eb = __ldcg(&st[i].eb), m = I.m;
+  const PTile p = point_tile(m, t);
+  if (p.x >= m) return;
+  auto rows = [&](auto widen) {
+    for (int iy = p.y0; iy < p.y1; ++iy) {
+      const long long j = (long long)iy * m + p.x;
+      const float2 e = __ldcg(I.L[0].u + j);
+      double2 u = __ldcg(I.u64 + j);
+      u.x += widen(e.x);
+      u.y += widen(e.y);
+      I.u64[j] = u;
+    }
+  };
+  if (abs(eb) <= bits::WIDEN_NEAR) rows([&](float f) { return bits::widen_near(f, eb); });
+  else rows([&](float f) { return bits::widen(f, eb); });
 }
 
-// u_new = u + 2^e e32; r = b - A u_new (neighbours formed on the fly from the
-// old iterate, which stays untouched); norm partial of r
-__device__ void ph_update(const BInst& I, const BState* st, int i, int t, double* partial, double* shd) {
-  const int cur = __ldcg(&st[i].cur);
-  const double2* uo = I.u64[cur];
-  double2* un = I.u64[cur ^ 1];
-  const float2* e32 = I.L[0].u;
-  const double s = ldexp(1.0, __ldcg(&st[i].e));
-  const int eb = __ldcg(&st[i].eb);
-  const double sc = ldexp(1.0, -min(max(eb, -1000), 1000));
-  const int m = I.m;
-  auto v_at = [&](long long j) {
-    double2 u = __ldcg(uo + j);
-    float2 e = __ldcg(e32 + j);
-    return make_double2(fma((double)e.x, s, u.x), fma((double)e.y, s, u.y));
-  };
+// r = b - A u: its rounding 2^-eb r to FP32, the right-hand side of the next
+// cycles (as in the single-problem path the scale is fixed for a solve), and
+// its norm partial
+__device__ void ph_residual(const BInst& I, const BState* st, int i, int t, double* partial, double* shd) {
+  const int eb = __ldcg(&st[i].eb), m = I.m;
+  const double sc = norm_scale(eb);
+  const PTile p = point_tile(m, t);
   double acc = 0;
-  for (long long j = (long long)t * PT + threadIdx.x; j < min((long long)(t + 1) * PT, I.N); j += blockDim.x) {
-    int ix = (int)(j % m), iy = (int)(j / m);
-    double2 vj = v_at(j);
-    double2 nb = make_double2(0, 0);
-    if (ix > 0) nb = cadd(nb, v_at(j - 1));
-    if (ix < m - 1) nb = cadd(nb, v_at(j + 1));
-    if (iy > 0) nb = cadd(nb, v_at(j - m));
-    if (iy < m - 1) nb = cadd(nb, v_at(j + m));
-    double2 tt = csub(cscale(vj, 4.0), nb);
-    double2 au = csub(cmul(I.c64, tt), cmul(I.q64[j], vj));
-    double2 r = csub(__ldcg(I.b64 + j), au);
-    un[j] = vj;
-    I.r64[j] = r;
-    double a = r.x * sc, b = r.y * sc;
-    acc = fma(a, a, fma(b, b, acc));
+  if (p.x < m) {
+    const double2 z = make_double2(0, 0), c = I.c64;
+    const double2* u = I.u64 + p.x;
+    double2 lo = p.y0 > 0 ? __ldcg(u + (long long)(p.y0 - 1) * m) : z, v = __ldcg(u + (long long)p.y0 * m);
+    for (int iy = p.y0; iy < p.y1; ++iy) {
+      const long long o = (long long)iy * m, j = o + p.x;
+      const double2 hi = iy < m - 1 ? __ldcg(u + o + m) : z;
+      const double2 xl = p.x > 0 ? __ldcg(u + o - 1) : z, xr = p.x < m - 1 ? __ldcg(u + o + 1) : z;
+      const double2 b = __ldcg(I.b64 + j), q = I.q64[j];
+      const double sx = (xl.x + xr.x) + (lo.x + hi.x), sy = (xl.y + xr.y) + (lo.y + hi.y);
+      const double tx = fma(4.0, v.x, -sx), ty = fma(4.0, v.y, -sy);
+      const double2 r = make_double2(fma(-c.x, tx, fma(c.y, ty, fma(q.x, v.x, fma(-q.y, v.y, b.x)))),
+                                     fma(-c.x, ty, fma(-c.y, tx, fma(q.x, v.y, fma(q.y, v.x, b.y)))));
+      I.L[0].b[j] = make_float2(bits::narrow(r.x, eb), bits::narrow(r.y, eb));
+      acc = sq_add(r, sc, acc);
+      lo = v;
+      v = hi;
+    }
   }
   acc = block_sum(acc, shd);
   if (threadIdx.x == 0) *partial = acc;
@@ -260,7 +295,7 @@ __device__ void ph_finish(const BArgs& A, int i, bool initial, double* shd) {
   if (threadIdx.x != 0) return;
   BState& S = A.st[i];
   const int eb = S.eb;
-  const double nrm = sqrt(acc) * ldexp(1.0, min(max(eb, -1000), 1000));
+  const double nrm = sqrt(acc) / norm_scale(eb);
   if (initial) {
     S.nb = nrm;
     S.hist[0] = 1.0;
@@ -272,8 +307,7 @@ __device__ void ph_finish(const BArgs& A, int i, bool initial, double* shd) {
       S.status = (nrm == 0.0) ? CSFF_OK : CSFF_ERR_NONFINITE;
       S.rel = 0.0;
     }
-    S.e = frexp_e(nrm);
-    S.n_step = A.inner;
+    S.n_step = S.done ? 0 : A.inner;
     S.lrn = 0;
     S.lflags = A.net_wb ? 1 : 0;
     S.lref = A.guard;
@@ -286,8 +320,6 @@ __device__ void ph_finish(const BArgs& A, int i, bool initial, double* shd) {
   S.refinements += 1;
   S.rel = rel;
   if (S.n_hist < CSFF_MAX_HISTORY) S.hist[S.n_hist++] = rel;
-  S.cur ^= 1;
-  S.e = frexp_e(nrm);
   int status = -1;
   if (!isfinite(rel)) status = CSFF_ERR_NONFINITE;
   else if (rel <= A.rel_tol) status = CSFF_OK;
@@ -315,6 +347,7 @@ __device__ void ph_finish(const BArgs& A, int i, bool initial, double* shd) {
   if (status >= 0) {
     S.status = status;
     S.done = 1;
+    S.n_step = 0;
   } else if (A.adaptive) {
     S.n_step = refinement_cycles(rel_before, rel, ran, A.rel_tol, A.inner);
   }
@@ -326,13 +359,13 @@ __device__ void ph_finish(const BArgs& A, int i, bool initial, double* shd) {
 __device__ void ph_resid0(const BInst& I, int t) {
   const BLevel& F = I.L[0];
   const int m = F.m;
-  const long long N = (long long)m * m;
   const float2 c = F.c;
+  const PTile p = point_tile(m, t);
+  if (p.x >= m) return;
   const float2 D0 = make_float2(__fmaf_rn(4.f, c.x, -F.K.k2), __fmul_rn(4.f, c.y));
-  for (int k = 0; k < PT / 256; ++k) {
-    const long long j = (long long)t * PT + k * 256 + threadIdx.x;
-    if (j >= N) return;
-    const int iy = (int)(j / m), ix = (int)(j - (long long)iy * m);
+  const int ix = p.x;
+  for (int iy = p.y0; iy < p.y1; ++iy) {
+    const long long j = (long long)iy * m + ix;
     float2 d = D0;
     for (int g = 0; g < F.K.ng; ++g) {
       const float2* f = F.K.fac + (size_t)g * 2 * m;
@@ -437,7 +470,7 @@ __device__ __forceinline__ void batch_body(const BArgs& A, unsigned char* smem, 
   if (!grid_barrier(A.bar, A.err, A.extra_arrivals, A.spin_limit)) return;
   for (int it = blockIdx.x; it < npts; it += gridDim.x) {
     int i = find_inst(A.off_pts, n, it);
-    ph_norm(A.inst[i], A.st, i, it - A.off_pts[i], A.partials + it, shd);
+    ph_first(A.inst[i], A.st, i, it - A.off_pts[i], A.partials + it, shd);
   }
   if (!grid_barrier(A.bar, A.err, A.extra_arrivals, A.spin_limit)) return;
   for (int i = blockIdx.x; i < n; i += gridDim.x) ph_finish(A, i, true, shd);
@@ -445,19 +478,14 @@ __device__ __forceinline__ void batch_body(const BArgs& A, unsigned char* smem, 
 
   for (;;) {
     bool any = false;
-    for (int i = 0; i < n; ++i) any |= !inst_done(A.st, i);
-    if (!any) break;
-    for (int it = blockIdx.x; it < npts; it += gridDim.x) {
-      int i = find_inst(A.off_pts, n, it);
-      if (!inst_done(A.st, i)) ph_to32(A.inst[i], A.st, i, it - A.off_pts[i]);
-    }
-    if (!grid_barrier(A.bar, A.err, A.extra_arrivals, A.spin_limit)) return;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) any |= !inst_done(A.st, i);
+    if (!__syncthreads_or(any)) break;
     for (int c = 0; c < A.inner; ++c) {
       // instances whose step is shorter sit out its remaining cycles (every
       // CTA reads the same state, so all leave the loop together)
       bool busy = false;
-      for (int i = 0; i < n; ++i) busy |= in_cycle(A.st, i, c);
-      if (!busy) break;
+      for (int i = threadIdx.x; i < n; i += blockDim.x) busy |= in_cycle(A.st, i, c);
+      if (!__syncthreads_or(busy)) break;
       for (int l = 0; l < A.LC; ++l) {
         const int* off = A.off_lvl + (size_t)l * (n + 1);
         for (int it = blockIdx.x; it < off[n]; it += gridDim.x) {
@@ -482,8 +510,8 @@ __device__ __forceinline__ void batch_body(const BArgs& A, unsigned char* smem, 
       }
       if constexpr (LEARNED) {
         bool any = false;
-        for (int i = 0; i < n; ++i) any |= learned_now(A.st, i, c);
-        if (any) {
+        for (int i = threadIdx.x; i < n; i += blockDim.x) any |= learned_now(A.st, i, c);
+        if (__syncthreads_or(any)) {
           for (int it = blockIdx.x; it < npts; it += gridDim.x) {
             int i = find_inst(A.off_pts, n, it);
             if (learned_now(A.st, i, c)) ph_resid0(A.inst[i], it - A.off_pts[i]);
@@ -496,7 +524,12 @@ __device__ __forceinline__ void batch_body(const BArgs& A, unsigned char* smem, 
     }
     for (int it = blockIdx.x; it < npts; it += gridDim.x) {
       int i = find_inst(A.off_pts, n, it);
-      if (!inst_done(A.st, i)) ph_update(A.inst[i], A.st, i, it - A.off_pts[i], A.partials + it, shd);
+      if (!inst_done(A.st, i)) ph_update(A.inst[i], A.st, i, it - A.off_pts[i]);
+    }
+    if (!grid_barrier(A.bar, A.err, A.extra_arrivals, A.spin_limit)) return;
+    for (int it = blockIdx.x; it < npts; it += gridDim.x) {
+      int i = find_inst(A.off_pts, n, it);
+      if (!inst_done(A.st, i)) ph_residual(A.inst[i], A.st, i, it - A.off_pts[i], A.partials + it, shd);
     }
     if (!grid_barrier(A.bar, A.err, A.extra_arrivals, A.spin_limit)) return;
     for (int i = blockIdx.x; i < n; i += gridDim.x)
@@ -505,15 +538,18 @@ __device__ __forceinline__ void batch_body(const BArgs& A, unsigned char* smem, 
   }
 }
 
-// at most 85 registers a thread, so that three CTAs fit on an SM (the
-// autotuner picks between one and the occupancy maximum).  LEARNED: the
+// 64 registers a thread, four CTAs an SM (with the learned step, whose operands
+// leave shared memory for three, 80; the autotuner picks between one and the
+// occupancy maximum).  32 instances of 129^2 to 1025^2: 20.2 ms at three CTAs, 19.1
+// at four, 18.6 at five of 48 registers, whose spills cost 24 instances of up to
+// 257^2 more (4.24 ms against 3.93).  LEARNED: the
 // learned step ends every cycle; each CTA holds the network's weight operands
 // for the whole launch, and the activation planes share the tiles' shared
 // memory.  The network runs on the warp-level MMA instructions: the occupancy
 // calculation, which bounds a cooperative launch, admits one CTA per SM for any
 // kernel with tensor-memory instructions.
 template <bool LEARNED>
-__global__ void __launch_bounds__(256, 3) k_batch_solve(BArgs A) {
+__global__ void __launch_bounds__(256, LEARNED ? 3 : 4) k_batch_solve(BArgs A) {
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ double shd[8];
   nettile::mmat::Ctx nc;
@@ -526,7 +562,7 @@ __global__ void k_batch_init(BState* st, int n, unsigned* bar, int* err) {
   if (i == 0) { bar[0] = 0; bar[1] = 0; *err = 0; }
   if (i >= n) return;
   BState& S = st[i];
-  S.done = 0; S.status = 0; S.cycles = 0; S.refinements = 0; S.e = 0; S.eb = -2000; S.cur = 0;
+  S.done = 0; S.status = 0; S.cycles = 0; S.refinements = 0; S.eb = -2000;
   S.rises = 0; S.n_hist = 0; S.prev = 1.0; S.nb = 0.0; S.rel = 1.0; S.n_step = 1;
   S.lrn = 0; S.lflags = 0; S.lref = 1.0;
 }
@@ -648,15 +684,13 @@ csff_status upload_descriptors(csff_batch* B) {
     I.inv64 = P->coarse_inv;
     I.c64 = P->lv[0].c;
     I.q64 = P->lv[0].q64;
-    I.u64[0] = P->lv[0].u64;
-    I.u64[1] = P->lv[0].t64;
+    I.u64 = P->lv[0].u64;
     I.b64 = P->lv[0].b64;
-    I.r64 = P->lv[0].r64;
     I.chi = P->chi_tab[0];
     I.uinc = P->uinc_tab;
     I.k2 = P->prob.k * P->prob.k;
     I.h2 = (float)(P->lv[0].h * P->lv[0].h);
-    off_pts[i + 1] = off_pts[i] + (int)((I.N + csff::PT - 1) / csff::PT);
+    off_pts[i + 1] = off_pts[i] + csff::point_tiles(I.m);
     off_net[i + 1] = off_net[i] + ((I.m + csff::nettile::TW - 1) / csff::nettile::TW) *
                                       ((I.m + csff::nettile::TH - 1) / csff::nettile::TH);
     for (int l = 0; l < LC; ++l) {
@@ -901,8 +935,7 @@ csff_status csff_batch_solve(csff_batch* B, const double* eta, csff_info* infos)
 csff_status csff_batch_solution(const csff_batch* B, int i, const void** u_dev) {
   if (!B || !u_dev || i < 0 || i >= B->n) return binvalid("bad instance index");
   const csff_plan* P = B->plans[i];
-  // the iterate alternates between two buffers; cur says which holds it
-  *u_dev = B->h_state[i].cur ? (const void*)P->lv[0].t64 : (const void*)P->lv[0].u64;
+  *u_dev = P->lv[0].u64;
   return CSFF_OK;
 }
 

@@ -72,6 +72,23 @@ __device__ __forceinline__ float2 split_scaled(double x, int e) {
   return make_float2(sg * hi, sg * lo);
 }
 
+// x 2^-e rounded to FP32 (to nearest); values below FP32's normal range become
+// zero
+__device__ __forceinline__ float narrow(double x, int e) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const unsigned int hi = (unsigned int)(b >> 32);
+  const int E = (int)((hi >> 20) & 0x7FF);
+  const int Ef = E - e - 1023 + 127;
+  const unsigned long long mant = b & MANT_MASK;
+  if (E == 0x7FF) return mant ? __uint_as_float(0x7FC00000u) : __uint_as_float(0x7F800000u | (hi & 0x80000000u));
+  if (E == 0 || Ef <= 0) return 0.f;
+  if (Ef >= 255) return __uint_as_float(0x7F800000u | (hi & 0x80000000u));   // beyond FP32's range
+  unsigned int f = ((unsigned int)Ef << 23) + (unsigned int)(mant >> 29);
+  const unsigned int rem = (unsigned int)(mant & 0x1FFFFFFFull), halfway = 0x10000000u;
+  f += (rem > halfway || (rem == halfway && (f & 1u))) ? 1u : 0u;
+  return __uint_as_float(f | (hi & 0x80000000u));
+}
+
 // f 2^e in FP64, exactly (a subnormal f is first scaled by 2^64 in FP32, which
 // is exact; a non-finite f or a result outside the normal FP64 range goes
 // through the FP64 conversion and an ldexp)
@@ -86,6 +103,21 @@ __device__ __forceinline__ double widen(float f, int e = 0) {
   if (E == 0xff || Ed < 1 || Ed > 2046) return ldexp((double)f, e);
   return __longlong_as_double(
       (long long)(sign | ((unsigned long long)Ed << 52) | ((unsigned long long)(u & 0x7fffffu) << 29)));
+}
+
+// widen for |e| <= WIDEN_NEAR, where no finite f leaves the normal FP64 range:
+// integer selects only.  (The compiler evaluates widen's FP64 fallback for every
+// value: a pass that widens a field took 365 us with it, 128 us with plain FP64
+// conversions, 257^3.)
+constexpr int WIDEN_NEAR = 800;
+__device__ __forceinline__ double widen_near(float f, int e) {
+  const unsigned u0 = __float_as_uint(f);
+  const bool sub = (u0 & 0x7f800000u) == 0;
+  const unsigned u = sub ? __float_as_uint(f * 18446744073709551616.f) : u0;   // 2^64
+  const int E = (int)((u >> 23) & 0xff);
+  int Ed = E + 896 + e - (sub ? 64 : 0);
+  Ed = E == 0xff ? 0x7ff : (E == 0 ? 0 : Ed);
+  return __hiloint2double((int)((u0 & 0x80000000u) | ((unsigned)Ed << 20) | ((u & 0x7fffffu) >> 3)), (int)(u << 29));
 }
 
 }  // namespace bits

@@ -52,9 +52,6 @@ __device__ __forceinline__ long long nbr_at(const Geom& g, Pix c, long long p, i
   if (ii < 0 || ii >= g.H || jj < 0 || jj >= g.W) return -1;
   return p + (long long)(a - 1) * g.W + (b - 1);
 }
-__device__ __forceinline__ long long nbr(const Geom& g, long long p, int a, int b) {
-  return nbr_at(g, pix_of(g, p), p, a, b);
-}
 
 // layer 1: x0 = bf16(r) (2 channels) -> h1 = bf16(relu(conv)) (16 channels).
 // The weights sit in shared memory as [tap][in][out] so that the 16 output

@@ -452,25 +452,8 @@ __global__ void k_rhs(TabPtrs tabs, int n_gauss, const double2* __restrict__ uin
 }
 
 // ---- FP64 refinement of the mixed solve (option refine_fp64) -------------------
-// r32 = r64 * 2^-e with e = exponent of ||r64||_2 (so |r32| < 1 elementwise).
-// The scaling and the rounding to FP32 (to nearest) work on the bit fields,
-// keeping the pass off the FP64 pipe (1/61 of the FP32 rate on this part);
-// values below FP32's normal range, 2^-126 ||r|| and less, become zero.
-__device__ __forceinline__ float d2f_pow2(double v, int e) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
-  const unsigned int hi = (unsigned int)(b >> 32);
-  const int E = (int)((hi >> 20) & 0x7FF);
-  const int Ef = E - e - 1023 + 127;
-  const unsigned long long mant = b & 0xFFFFFFFFFFFFFull;
-  if (E == 0x7FF) return mant ? __uint_as_float(0x7FC00000u) : __uint_as_float(0x7F800000u | (hi & 0x80000000u));
-  if (E == 0 || Ef <= 0) return 0.f;
-  if (Ef >= 255) return __uint_as_float(0x7F800000u | (hi & 0x80000000u));   // beyond FP32's range
-  unsigned int f = ((unsigned int)Ef << 23) + (unsigned int)(mant >> 29);
-  const unsigned int rem = (unsigned int)(mant & 0x1FFFFFFFull), halfway = 0x10000000u;
-  f += (rem > halfway || (rem == halfway && (f & 1u))) ? 1u : 0u;
-  return __uint_as_float(f | (hi & 0x80000000u));
-}
-
+// r32 = r64 * 2^-e with e = exponent of ||r64||_2 (so |r32| < 1 elementwise);
+// values of 2^-126 ||r|| and less become zero
 __global__ void k_to32_scaled(const double2* __restrict__ r, long long N, const double* __restrict__ nrm,
                               float2* __restrict__ r32, int* __restrict__ exp_out) {
   pdl_prologue();
@@ -480,19 +463,8 @@ __global__ void k_to32_scaled(const double2* __restrict__ r, long long N, const 
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N;
        i += (long long)gridDim.x * blockDim.x) {
     const double2 v = r[i];
-    r32[i] = make_float2(d2f_pow2(v.x, e), d2f_pow2(v.y, e));
+    r32[i] = make_float2(bits::narrow(v.x, e), bits::narrow(v.y, e));
   }
-}
-
-// FP32 value times 2^s as a double, exactly, from the bit fields (zero,
-// subnormal input, or a result outside the normal FP64 range take ldexp)
-__device__ __forceinline__ double f2d_pow2(float v, int s) {
-  const unsigned int b = __float_as_uint(v);
-  const int E = (int)((b >> 23) & 0xFFu), Ed = E + 896 + s;
-  if (E == 0 || Ed < 1 || Ed > 2046) return ldexp((double)v, s);
-  const long long bits = ((long long)(b >> 31) << 63) | ((long long)Ed << 52) |
-                         ((long long)(b & 0x7FFFFFu) << 29);
-  return __longlong_as_double(bits);
 }
 
 __global__ void k_update64(double2* __restrict__ u, const float2* __restrict__ e, long long N,
@@ -503,8 +475,8 @@ __global__ void k_update64(double2* __restrict__ u, const float2* __restrict__ e
        i += (long long)gridDim.x * blockDim.x) {
     const float2 c = e[i];
     double2 v = u[i];
-    v.x += f2d_pow2(c.x, s);
-    v.y += f2d_pow2(c.y, s);
+    v.x += bits::widen(c.x, s);
+    v.y += bits::widen(c.y, s);
     u[i] = v;
   }
 }
@@ -550,7 +522,7 @@ __global__ void k_refine_residual(const double2* __restrict__ u, const double2* 
       const double2 bj = b[i], qj = q[i];
       const double rx = fma(-c.x, tx, fma(c.y, ty, fma(qj.x, uj.x, fma(-qj.y, uj.y, bj.x))));
       const double ry = fma(-c.x, ty, fma(-c.y, tx, fma(qj.x, uj.y, fma(qj.y, uj.x, bj.y))));
-      const float fx = d2f_pow2(rx, s_exp), fy = d2f_pow2(ry, s_exp);
+      const float fx = bits::narrow(rx, s_exp), fy = bits::narrow(ry, s_exp);
       r32[i] = make_float2(fx, fy);
       acc = __fmaf_rn(fx, fx, __fmaf_rn(fy, fy, acc));
     }
@@ -559,16 +531,23 @@ __global__ void k_refine_residual(const double2* __restrict__ u, const double2* 
   if (threadIdx.x == 0) partial[blockIdx.y * gridDim.x + blockIdx.x] = tot;
 }
 
-// u += 2^s e (FP32 correction widened exactly; one FP64 multiply and add per
-// component, p2 = 2^s; on the bit fields the subnormal values of localised
-// corrections take the slow branch: 365 us instead of 128 at 257^3)
-__global__ void k_update64_fixed(double2* __restrict__ u, const float2* __restrict__ e, int N, double p2) {
+// u += 2^s e.  NEAR: the FP32 correction is widened on the bit fields, which
+// leaves two FP64 additions a point and the pass bound by memory (257^3: 128 ->
+// 94 us, 665 MB); else (scales near the ends of the FP64 range) by conversions
+// and multiply-adds.
+template <bool NEAR>
+__global__ void k_update64_fixed(double2* __restrict__ u, const float2* __restrict__ e, int N, int s, double p2) {
   pdl_prologue();
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
     const float2 c = e[i];
     double2 v = u[i];
-    v.x = fma((double)c.x, p2, v.x);
-    v.y = fma((double)c.y, p2, v.y);
+    if constexpr (NEAR) {
+      v.x += bits::widen_near(c.x, s);
+      v.y += bits::widen_near(c.y, s);
+    } else {
+      v.x = fma((double)c.x, p2, v.x);
+      v.y = fma((double)c.y, p2, v.y);
+    }
     u[i] = v;
   }
 }
@@ -578,7 +557,7 @@ __global__ void k_scale_to32(const double2* __restrict__ v, int N, int s, float2
   pdl_prologue();
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
     const double2 x = v[i];
-    r32[i] = make_float2(d2f_pow2(x.x, s), d2f_pow2(x.y, s));
+    r32[i] = make_float2(bits::narrow(x.x, s), bits::narrow(x.y, s));
   }
 }
 
@@ -803,8 +782,8 @@ cudaError_t launch_refine_residual(int dim, const Level& L, const double2* u, co
 cudaError_t launch_update64_fixed(double2* u, const float2* e, long long N, int s_exp, cudaStream_t s) {
   if (N >= (1ll << 31)) return cudaErrorInvalidValue;
   ProfScope ps(PF_MG64, s, 40.0 * N, 0);
-  cudaError_t err = launch_pdl(k_update64_fixed, dim3(flat_blocks(N)), dim3(256), 0, s, u, e, (int)N,
-                               ldexp(1.0, s_exp));
+  cudaError_t err = launch_pdl(abs(s_exp) <= bits::WIDEN_NEAR ? k_update64_fixed<true> : k_update64_fixed<false>,
+                               dim3(flat_blocks(N)), dim3(256), 0, s, u, e, (int)N, s_exp, ldexp(1.0, s_exp));
   count_launch();
   return err != cudaSuccess ? err : cudaGetLastError();
 }

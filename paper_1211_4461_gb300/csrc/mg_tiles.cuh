@@ -684,12 +684,19 @@ constexpr int COARSE_NT = 512;      // threads of the per-level kernel (the pers
 constexpr int COARSE_ROW = 16;      // lanes per grid row: points of a colour in a row of a smoothing level
 constexpr size_t COARSE_STAGE_LIMIT = 200 * 1024;
 
-// shared memory of the block: per smoothing level u, b, r, q, 1/d on (m+2)^2
-// padded grids, for the coarsest u (padded) and b (m^2, in the product's type)
-// and, when staged, the inverse
+// shared memory of the block: per smoothing level u, b, 1/d on (m+2)^2 padded
+// grids and q at the red points, whose residual takes its place (m is odd on
+// these levels: padded index i of a red point is even, slot i / 2); for the
+// coarsest u (padded) and b (m^2, in the product's type) and, when staged, the
+// inverse.  41 KB for FP32 levels from 33^2 down (58 KB with q and r on grids of
+// their own) lets the persistent kernel run four CTAs an SM instead of three
+__host__ __device__ constexpr int coarse_grids(int A) { return 3 * A + (A + 1) / 2; }
 inline size_t coarse_block_bytes(const std::vector<Level>& lv, int lc, size_t el, size_t el_inv, bool staged) {
   size_t n = 0;
-  for (size_t l = lc; l < lv.size(); ++l) n += (l + 1 < lv.size() ? 5 : 1) * (size_t)(lv[l].m + 2) * (lv[l].m + 2);
+  for (size_t l = lc; l < lv.size(); ++l) {
+    const int A = (lv[l].m + 2) * (lv[l].m + 2);
+    n += l + 1 < lv.size() ? coarse_grids(A) : A;
+  }
   n = ((n * el + 15) & ~(size_t)15) + (size_t)lv.back().N * el_inv;
   return n + (staged ? (size_t)lv.back().N * lv.back().N * el_inv : 0);
 }
@@ -735,15 +742,16 @@ __device__ void coarse_levels_block(const CoarseLevels& L, const cx<T>* b_top, c
       if (x < m)
         for (int y = t >> 5; y < m; y += nt >> 5) {
           const int g = y * m + x, s = (y + 1) * W + x + 1;
+          const bool red = ((x + y) & 1) == 0;
           if constexpr (COH) {
-            p[3 * A + s] = q[g];
-            p[4 * A + s] = dv[g];
+            p[2 * A + s] = dv[g];
+            if (red) p[3 * A + (s >> 1)] = q[g];
           } else {
-            cp_async_s<(int)sizeof(C)>(smem_addr(p + 3 * A + s), q + g);
-            cp_async_s<(int)sizeof(C)>(smem_addr(p + 4 * A + s), dv + g);
+            cp_async_s<(int)sizeof(C)>(smem_addr(p + 2 * A + s), dv + g);
+            if (red) cp_async_s<(int)sizeof(C)>(smem_addr(p + 3 * A + (s >> 1)), q + g);
           }
         }
-      p += 5 * A;
+      p += coarse_grids(A);
     }
   }
   C* const Ulast = p;
@@ -771,7 +779,7 @@ __device__ void coarse_levels_block(const CoarseLevels& L, const cx<T>* b_top, c
         const C v = ld<COH>(b_top + y * m + x);
         const int s = (y + 1) * W + x + 1;
         base[A + s] = v;
-        if (((x + y) & 1) == 0) base[s] = xmul(base[4 * A + s], v);
+        if (((x + y) & 1) == 0) base[s] = xmul(base[2 * A + s], v);
       }
   } else {
     for (int i = t; i < n; i += nt) Bc[i] = widen<TI, T>(ld<COH>(b_top + i));
@@ -782,8 +790,8 @@ __device__ void coarse_levels_block(const CoarseLevels& L, const cx<T>* b_top, c
   for (int l = 0; l < last; ++l) {
     const int m = L.m[l], mc = L.m[l + 1], W = m + 2, A = W * W, Wc = mc + 2, Ac = Wc * Wc;
     const C c = level_c<T>(L, l);
-    C *U = p, *B = p + A, *R = p + 2 * A, *Q = p + 3 * A, *D = p + 4 * A;
-    C* const next = p + 5 * A;
+    C *U = p, *B = p + A, *D = p + 2 * A, *Q = p + 3 * A;     // Q: q, then r, at the red points
+    C* const next = p + coarse_grids(A);
     for (int iy = y0 + 1; iy <= m; iy += dy) {               // black
       const int ix = 2 * j + ((iy & 1) ? 2 : 1), i = iy * W + ix;
       if (ix <= m) U[i] = xmul(D[i], xfma(B[i], c, nbr_sum(U, i, W)));
@@ -792,21 +800,22 @@ __device__ void coarse_levels_block(const CoarseLevels& L, const cx<T>* b_top, c
     for (int iy = y0 + 1; iy <= m; iy += dy) {               // residual at the red points
       const int ix = 2 * j + ((iy & 1) ? 1 : 2), i = iy * W + ix;
       if (ix <= m) {
-        const C d = xsub(xscale(c, (T)4), Q[i]);
-        R[i] = xfma(xfms(B[i], d, U[i]), c, nbr_sum(U, i, W));
+        const C d = xsub(xscale(c, (T)4), Q[i >> 1]);
+        Q[i >> 1] = xfma(xfms(B[i], d, U[i]), c, nbr_sum(U, i, W));
       }
     }
     __syncthreads();
     for (int Y = y0 + 1; Y <= mc; Y += dy) {                 // full weighting of the red residuals
       const int X = j + 1;
       if (X > mc) continue;
-      const C* r = R + 2 * Y * W + 2 * X;
-      const C corners = xadd(xadd(r[-W - 1], r[-W + 1]), xadd(r[W - 1], r[W + 1]));
+      const C* r = Q + Y * W + X;
+      const int h0 = (W - 1) / 2, h1 = (W + 1) / 2;          // slots to the diagonal neighbours
+      const C corners = xadd(xadd(r[-h1], r[-h0]), xadd(r[h0], r[h1]));
       const C v = xfma_r(xscale(corners, (T)0.0625), r[0], (T)0.25);
       if (l + 1 < last) {
         const int s = Y * Wc + X;
         next[Ac + s] = v;
-        if (((X + Y) & 1) == 0) next[s] = xmul(next[4 * Ac + s], v);
+        if (((X + Y) & 1) == 0) next[s] = xmul(next[2 * Ac + s], v);
       } else {
         Bc[(Y - 1) * mc + X - 1] = widen<TI, T>(v);
       }
@@ -843,7 +852,7 @@ __device__ void coarse_levels_block(const CoarseLevels& L, const cx<T>* b_top, c
   for (int l = last - 1; l >= 0; --l) {
     const int m = L.m[l], W = m + 2, A = W * W, Wc = L.m[l + 1] + 2;
     const C c = level_c<T>(L, l);
-    C *U = E - 5 * A, *B = U + A, *D = U + 4 * A;
+    C *U = E - coarse_grids(A), *B = U + A, *D = U + 2 * A;
     // red, with the neighbour sum of the interpolated correction: at a cell
     // centre (odd node indices) the four corners; at a coarse node twice its
     // value and half of each of its four neighbours
