@@ -455,6 +455,8 @@ template <bool PHASE>
 __global__ void k_cut_rows(const double2* __restrict__ v, int m, int nrows, const int* __restrict__ ev,
                            const int* __restrict__ spread, unsigned char* __restrict__ out) {
   using namespace digits;
+  using F = Form2;
+  constexpr int ND = F::ND, B_SET = F::B_SET;
   if (!digits_selected(spread)) return;
   constexpr int TR = PHASE ? TK : TM;
   const int lane = threadIdx.x & 31, nb = (m + KB - 1) / KB, total = (nrows + TR - 1) / TR * TR * nb;
@@ -465,10 +467,10 @@ __global__ void k_cut_rows(const double2* __restrict__ v, int m, int nrows, cons
     if (row < nrows && i < m) {
       const double2 x = v[(long long)row * m + i];
       const int e = ev[(long long)row * nb + b];
-      p = fixed55(x.x, e);
-      q = fixed55(x.y, e);
+      p = fixed<F::BITS>(x.x, e);
+      q = fixed<F::BITS>(x.y, e);
     }
-    cut(p, q, dig);
+    cut<ND>(p, q, dig);
     const int r = row % TR;
     unsigned char* tile = out + ((long long)(row / TR) * nb + b) * (PHASE ? B_SET : ND * A_DIG);
     const int o = (lane & 3) * 4;
@@ -495,24 +497,6 @@ __device__ __forceinline__ float pow2f_neg(int d) {
 // value = (hi + lo) 2^E; merging a block sum s 2^Es rescales the smaller of the
 // two exactly (powers of two) and adds with TwoSum, all in FP32
 struct dfacc { float hi, lo; int E; };
-
-__device__ __forceinline__ void dfacc_merge2(dfacc& re, dfacc& im, df sr, df si, int Es) {
-  if (sr.hi == 0.f && si.hi == 0.f && sr.lo == 0.f && si.lo == 0.f) return;
-  const int En = max(re.E, Es);                    // re.E == im.E always
-  const float fa = pow2f_neg(re.E - En), fs = pow2f_neg(Es - En);
-  auto add = [&](dfacc& a, df x) {
-    float ah = a.hi * fa, al = a.lo * fa, xh = x.hi * fs, xl = x.lo * fs;
-    float t = ah + xh, v = t - ah;
-    float err = (ah - (t - v)) + (xh - v);
-    float lo = al + xl + err;
-    float h = t + lo;                              // renormalise (fast TwoSum)
-    a.lo = lo - (h - t);
-    a.hi = h;
-    a.E = En;
-  };
-  add(re, sr);
-  add(im, si);
-}
 
 __device__ __forceinline__ void dfacc_merge3(dfacc& a1, dfacc& a2, dfacc& a3, df s1, df s2, df s3, int Es) {
   if (s1.hi == 0.f && s2.hi == 0.f && s3.hi == 0.f && s1.lo == 0.f && s2.lo == 0.f && s3.lo == 0.f) return;
@@ -740,6 +724,71 @@ __global__ void __launch_bounds__(DF_NT, 5) k_ff_stage1_df(const float4* __restr
   }
 }
 
+// Operands of the 3D form, whose scale blocks have 16 nodes.  Phases: one warp
+// per (row, 32 nodes); ev[row][block of 16].  map: the phase row behind each
+// operand row (negative: none).
+__global__ void k_cut_phase3(const double2* __restrict__ v, const int* __restrict__ map, int m, int nrows,
+                             int* __restrict__ ev, unsigned char* __restrict__ out) {
+  using namespace digits;
+  using F = Form3;
+  const int lane = threadIdx.x & 31, nb = (m + KB - 1) / KB, warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int row = warp / nb, b = warp - row * nb, i = b * KB + lane;
+  if (row >= (nrows + TK - 1) / TK * TK) return;
+  const int src = row >= nrows ? -1 : map ? map[row] : row;
+  const double2 x = src >= 0 && i < m ? v[(long long)src * m + i] : make_double2(0, 0);
+  int e = scale_exp(x);
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
+  if (row < nrows && (lane & 15) == 0) ev[((long long)row * nb + b) * F::SUB + (lane >> 4)] = e;
+  uint32_t dig[F::ND];
+  cut<F::ND>(fixed<F::BITS>(x.x, e), fixed<F::BITS>(x.y, e), dig);
+  const int r = row % TK, o = (lane & 3) * 4;
+  unsigned char* tile = out + ((long long)(row / TK) * nb + b) * F::B_SET;
+#pragma unroll
+  for (int s = 0; s < F::ND; ++s) {
+    *reinterpret_cast<uint32_t*>(tile + s * B_DIG + sw(r, lane >> 2) + o) = neg_hi(dig[s]);
+    *reinterpret_cast<uint32_t*>(tile + s * B_DIG + sw(TK + r, lane >> 2) + o) = swap_pair(dig[s]);
+  }
+}
+
+// The field: a thread takes 16 nodes along z of one column (neighbouring threads
+// neighbouring columns), a block a tile of 128 columns from column tile0 TM on;
+// the 32 bytes of eight nodes' digits are whole sectors.  eg[column of the
+// chunk][block of 16].  blockIdx.z: one of several fields of m rows.
+__global__ void __launch_bounds__(digits::TM) k_cut_field3(const double2* __restrict__ g, int m, long long ncol,
+                                                           int tile0, int* __restrict__ eg,
+                                                           unsigned char* __restrict__ out) {
+  using namespace digits;
+  using F = Form3;
+  const int nbs = gridDim.y, sb = blockIdx.y, r = threadIdx.x;
+  const long long col = (long long)(tile0 + blockIdx.x) * TM + r;
+  const long long xt = (long long)blockIdx.z * gridDim.x + blockIdx.x;        // column tile of the operand
+  const double2* p = g + ((long long)blockIdx.z * m + sb * 16) * ncol + col;
+  const int nz = col < ncol ? min(16, m - sb * 16) : 0;        // nodes of the block inside the grid
+  int e = -1022;
+#pragma unroll
+  for (int k = 0; k < 16; ++k)
+    if (k < nz) e = max(e, scale_exp(p[(long long)k * ncol]));
+  eg[(xt * TM + r) * nbs + sb] = e;
+  unsigned char* tile = out + (xt * nbs + sb) * (F::A_SLOTS * A_DIG);
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    uint32_t d[8][F::ND];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const double2 x = 8 * h + k < nz ? p[(long long)(8 * h + k) * ncol] : make_double2(0, 0);
+      cut<F::ND>(fixed<F::BITS>(x.x, e), fixed<F::BITS>(x.y, e), d[k]);
+    }
+#pragma unroll
+    for (int s = 0; s < F::ND; ++s) {
+      unsigned char* slot = tile + (s >> 1) * A_DIG;
+      const int c = 4 * (s & 1) + 2 * h;
+      *reinterpret_cast<uint4*>(slot + sw(r, c)) = make_uint4(d[0][s], d[1][s], d[2][s], d[3][s]);
+      *reinterpret_cast<uint4*>(slot + sw(r, c + 1)) = make_uint4(d[4][s], d[5][s], d[6][s], d[7][s]);
+    }
+  }
+}
+
 // T[k][rho] from the digit operands (ff_digits.cuh): a tile of 128 rho x 16 k a
 // CTA, its kept blocks in order.  Warps 0-15 join the accumulators (TMEM lanes
 // 32 (w mod 4), phase rows [4 (w / 4), +4)), warp 16 loads, warp 17 issues MMAs.
@@ -748,12 +797,25 @@ __global__ void __launch_bounds__(DF_NT, 5) k_ff_stage1_df(const float4* __restr
 // 64; 150 from one thread in a divergent branch) and by the last wave: 184 tiles
 // on 152 SMs at 1025^2.  361 phase rows x 1023 x 1023, every block kept: 125 us,
 // 18 us for cutting the operands; the double-float contraction takes 538.
+//
+// 3D form: T1[t][col] of the z contraction, every block kept (skip and spread
+// null), columns from tile0 TM on, in chunks whose operands stay in L2.  A block
+// of 16 nodes' diagonals join to one 63-bit integer, rounded once to FP64 and
+// added in FP64 (128 FP64 additions a block and CTA at 19 clocks, beside 16
+// MMAs).  257^3, 32 z components, 2048 angles: z contraction 247 us and 266 us for
+// cutting the field (FP64 kernel: 4080), y contraction 68 and 44 us (FP64: 866);
+// the error of a map against a 113-bit sum is the FP64 kernels', 2^-53.4 to
+// 2^-54.7 of the sum of the terms' magnitudes at the worst angle (65^3 to 161^3).  With several fields (the y contraction) field[tile of phase
+// rows] says which one its rows multiply and map where they go in T.
+template <class F>
 __global__ void __launch_bounds__(digits::NT, 1)
     k_ff_digits(const unsigned char* __restrict__ Ad, const unsigned char* __restrict__ Bd, const int* __restrict__ ex,
                 int M, const int* __restrict__ eg, int N, int nb, const int* __restrict__ spread,
-                const unsigned char* __restrict__ skip, int skip_tiles, double2* __restrict__ T, int* __restrict__ err) {
+                const unsigned char* __restrict__ skip, int skip_tiles, double2* __restrict__ T, int* __restrict__ err,
+                int tile0, const int* __restrict__ field, const int* __restrict__ map) {
   using namespace digits;
-  if (!digits_selected(spread)) return;      // another kernel takes this launch
+  constexpr int ND = F::ND, NA = F::NA, SUB = F::SUB, B_SET = F::B_SET, OFF_BAR = F::OFF_BAR, OFF_ACT = F::OFF_ACT;
+  if (spread && !digits_selected(spread)) return;      // another kernel takes this launch
   extern __shared__ __align__(1024) unsigned char dsm_raw[];
   unsigned char* base = dsm_raw + ((1024 - (saddr(dsm_raw) & 1023)) & 1023);
   const uint32_t sbase = saddr(base), bars = sbase + OFF_BAR;
@@ -765,7 +827,7 @@ __global__ void __launch_bounds__(digits::NT, 1)
   unsigned short* act = reinterpret_cast<unsigned short*>(base + OFF_ACT);
   static_assert(8 * (2 * NA + 9) <= 480, "barriers");
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int n0 = blockIdx.x * TM, m0 = blockIdx.y * TK;
+  const int m0 = blockIdx.y * TK, xt = (field ? field[blockIdx.y] * (int)gridDim.x : 0) + (int)blockIdx.x;
   if (threadIdx.x == 0) {
     for (int i = 0; i < NA; ++i) {
       bar_init(a_full + 8 * i, 1);
@@ -793,7 +855,10 @@ __global__ void __launch_bounds__(digits::NT, 1)
       const int b = b0 + lane;
       bool keep = false;
       if (b < nb)
-        for (int t = t0; t < t1; ++t) keep |= skip[((long long)blockIdx.y * skip_tiles + t) * nb + b] == 0;
+        for (int t = t0; t < t1 || !skip; ++t) {
+          keep |= !skip || skip[((long long)blockIdx.y * skip_tiles + t) * nb + b] == 0;
+          if (!skip) break;
+        }
       const unsigned mask = __ballot_sync(0xffffffffu, keep);
       if (keep) act[n + __popc(mask & ((1u << lane) - 1u))] = (unsigned short)b;
       n += __popc(mask);
@@ -808,20 +873,21 @@ __global__ void __launch_bounds__(digits::NT, 1)
   static_assert(DF_BM == TK && TM % DF_BN == 0, "skip tiles");
   if (warp == EPI_WARPS) {
     // uniform as the MMA warp: one elected lane issues the copies
-    const int n = __reduce_max_sync(0xffffffffu, n_act);
+    const int n = SUB * __reduce_max_sync(0xffffffffu, n_act);
     int ia = 0, slot = 0;
     uint32_t eph = 1;                                  // parity of the slot's last release (first round: none awaited)
     bool ok = true;
     for (int idx = 0; idx < n; ++idx) {
-      const int p = idx & 1, b = __reduce_max_sync(0xffffffffu, (int)act[idx]);
-      if (idx >= 2) ok = bar_wait(b_empty + 8 * p, (uint32_t)((idx >> 1) - 1) & 1u, abort);
+      const int kb = idx / SUB, p = kb & 1, b = __reduce_max_sync(0xffffffffu, (int)act[kb]);
+      const bool first = idx % SUB == 0;
+      if (first && kb >= 2) ok = bar_wait(b_empty + 8 * p, (uint32_t)((kb >> 1) - 1) & 1u, abort);
       if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
-      const unsigned char* src = Ad + ((long long)blockIdx.x * nb + b) * (ND * A_DIG);
-      if (elect_one())
+      const unsigned char* src = Ad + (((long long)xt * nb + b) * SUB + idx % SUB) * (F::A_SLOTS * A_DIG);
+      if (first && elect_one())
         bulk_load(sbase + NA * A_DIG + p * B_SET, Bd + ((long long)blockIdx.y * nb + b) * B_SET, B_SET, b_full + 8 * p);
       __syncwarp();
 #pragma unroll
-      for (int s = 0; s < ND; ++s) {
+      for (int s = 0; s < F::A_SLOTS; ++s) {
         if (ia >= NA) ok = ok && bar_wait(a_empty + 8 * slot, eph, abort);
         if (__all_sync(0xffffffffu, ok)) {
           if (elect_one()) bulk_load(sbase + slot * A_DIG, src + s * A_DIG, A_DIG, a_full + 8 * slot);
@@ -848,7 +914,7 @@ __global__ void __launch_bounds__(digits::NT, 1)
     // uniform (reductions and votes across the warp), one elected lane issues:
     // the MMAs' operands then stay in uniform registers.  With a single thread
     // in a divergent branch each MMA cost 150 clocks in register moves.
-    const int n = __reduce_max_sync(0xffffffffu, n_act);
+    const int n = SUB * __reduce_max_sync(0xffffffffu, n_act);
     const uint32_t tm = __reduce_max_sync(0xffffffffu, tmem);
     // FP32 accumulator, BF16 A and B, both K-major, M = 128; N per digit of A
     constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TM >> 4) << 24);
@@ -858,31 +924,32 @@ __global__ void __launch_bounds__(digits::NT, 1)
     for (int idx = 0; idx < n; ++idx) {
       const int p = idx & 1;
       if (idx >= 2) ok = bar_wait(acc_empty + 8 * p, (uint32_t)((idx >> 1) - 1) & 1u, abort);
-      ok = ok && bar_wait(b_full + 8 * p, (uint32_t)(idx >> 1) & 1u, abort);
+      const int kb = idx / SUB, pb = kb & 1;             // B's buffer
+      ok = ok && bar_wait(b_full + 8 * pb, (uint32_t)(kb >> 1) & 1u, abort);
       if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
-      const uint32_t sB = sbase + NA * A_DIG + p * B_SET;
+      const uint32_t sB = sbase + NA * A_DIG + pb * B_SET + (SUB - 1) * 64 * (idx & 1);
 #pragma unroll
       for (int s = 0; s < ND; ++s) {
-        ok = ok && bar_wait(a_full + 8 * slot, aph, abort);
+        if (s % SUB == 0) ok = ok && bar_wait(a_full + 8 * slot, aph, abort);
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         constexpr int TKK = 2 * TK;
         const uint32_t nd = (uint32_t)(TKK * (ND - s));
-        const uint32_t d = tm + (uint32_t)(p * ACC + TKK * s), sA = sbase + slot * A_DIG;
+        const uint32_t d = tm + (uint32_t)(p * ACC + TKK * s), sA = sbase + slot * A_DIG + 64 * (s % SUB);
         if (__all_sync(0xffffffffu, ok) && elect_one()) {
 #pragma unroll
-          for (int kk = 0; kk < 4; ++kk)
+          for (int kk = 0; kk < 4 / SUB; ++kk)
             mma(d, desc(sA + 32 * kk), desc(sB + 32 * kk), idesc | ((nd >> 3) << 17), (s > 0 || kk > 0) ? 1u : 0u);
-          commit(a_empty + 8 * slot);
+          if (s % SUB == SUB - 1) commit(a_empty + 8 * slot);
         }
         __syncwarp();
-        if (++slot == NA) {
+        if (s % SUB == SUB - 1 && ++slot == NA) {
           slot = 0;
           aph ^= 1u;
         }
       }
       if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
       if (elect_one()) {
-        commit(b_empty + 8 * p);
+        if (idx % SUB == SUB - 1) commit(b_empty + 8 * pb);
         commit(acc_full + 8 * p);
       }
       __syncwarp();
@@ -897,65 +964,95 @@ __global__ void __launch_bounds__(digits::NT, 1)
   } else {
     static_assert(EK == 4, "two packed pairs of phase rows a warp");
     const int lg = warp & 3, kq = EK * (warp >> 2);
-    const int rho = n0 + 32 * lg + lane;
+    const int rho = (tile0 + blockIdx.x) * TM + 32 * lg + lane;
+    const long long rl = (long long)xt * TM + 32 * lg + lane;
     const int k0 = m0 + kq;
     const uint32_t tl = tmem + ((uint32_t)(32 * lg) << 16) + (uint32_t)kq;
-    float2 H[2][2], L[2][2];
+    float2 H[2][2], L[2][2];                           // 2D: running double-float sums, exponents E
     int E[EK];
+    double S[2][EK];                                   // 3D: running sums
+#pragma unroll
+    for (int j = 0; j < EK; ++j) S[0][j] = S[1][j] = 0.0;
 #pragma unroll
     for (int j = 0; j < 2; ++j) H[0][j] = L[0][j] = H[1][j] = L[1][j] = make_float2(0.f, 0.f);
 #pragma unroll
     for (int j = 0; j < EK; ++j) E[j] = -100000;
     bool ok = true;
-    // scale exponents, loaded a block ahead; digit 1 times digit 1 weighs 2^-14
+    // scale exponents, loaded a block ahead; 2D: digit 1 times digit 1 weighs
+    // 2^-14, 3D: the joined integer's unit 2^-57
     int eg1 = 0, ex1[EK];
-    auto scales = [&](int b) {
-      eg1 = (rho < N ? eg[(long long)rho * nb + b] : 0) - 14;
+    auto scales = [&](int idx) {
+      const int b = act[idx / SUB] * SUB + idx % SUB;
+      eg1 = (rho < N ? eg[rl * nb * SUB + b] : 0) - (SUB == 1 ? 14 : 57);
 #pragma unroll
-      for (int j = 0; j < EK; ++j) ex1[j] = k0 + j < M ? ex[(long long)(k0 + j) * nb + b] : 0;
+      for (int j = 0; j < EK; ++j) ex1[j] = k0 + j < M ? ex[(long long)(k0 + j) * nb * SUB + b] : 0;
     };
-    if (n_act > 0) scales(act[0]);
-    for (int idx = 0; idx < n_act; ++idx) {
+    const int n = SUB * n_act;
+    if (n > 0) scales(0);
+    for (int idx = 0; idx < n; ++idx) {
       const int p = idx & 1;
       int es[EK];
 #pragma unroll
       for (int j = 0; j < EK; ++j) es[j] = eg1 + ex1[j];
-      if (idx + 1 < n_act) scales(act[idx + 1]);
+      if (idx + 1 < n) scales(idx + 1);
       // one lane polls: the waits of 512 threads would crowd out the barrier
       // operations of the two threads that feed the tensor core
       if (lane == 0) ok = bar_wait(acc_full + 8 * p, (uint32_t)(idx >> 1) & 1u, abort);
       ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
       if (!ok) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      uint32_t v[2][ND][EK];
-#pragma unroll
-      for (int c = 0; c < 2; ++c)
-#pragma unroll
-        for (int d = 0; d < ND; ++d) CSFF_TMEM_LD4(v[c][d], tl + (uint32_t)(p * ACC + 2 * TK * d + TK * c));
-      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      __syncwarp();
-      if (lane == 0) bar_arrive(acc_empty + 8 * p);
-#pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        // merge into the running sums at the larger of the two exponents
-        const int En0 = max(E[2 * j], es[2 * j]), En1 = max(E[2 * j + 1], es[2 * j + 1]);
-        const float2 fa = make_float2(pow2_or_0(E[2 * j] - En0), pow2_or_0(E[2 * j + 1] - En1));
-        const float2 fs = make_float2(pow2_or_0(es[2 * j] - En0), pow2_or_0(es[2 * j + 1] - En1));
-        E[2 * j] = En0;
-        E[2 * j + 1] = En1;
+      if constexpr (SUB == 2) {
+        // one part at a time: both take more registers than 18 warps have
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
-          float2 q[ND], h, l, t, e;
+          uint32_t v[ND][EK];
 #pragma unroll
-          for (int d = 0; d < ND; ++d)
-            q[d] = make_float2(__uint_as_float(v[c][d][2 * j]), __uint_as_float(v[c][d][2 * j + 1]));
-          join(q, h, l);
-          two_sum(__fmul2_rn(H[c][j], fa), __fmul2_rn(h, fs), t, e);
-          e = __fadd2_rn(e, __ffma2_rn(l, fs, __fmul2_rn(L[c][j], fa)));
-          const float2 hn = __fadd2_rn(t, e);
-          L[c][j] = __ffma2_rn(__ffma2_rn(t, both(-1.f), hn), both(-1.f), e);
-          H[c][j] = hn;
+          for (int d = 0; d < ND; ++d) CSFF_TMEM_LD4(v[d], tl + (uint32_t)(p * ACC + 2 * TK * d + TK * c));
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+          if (c == 1) {
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) bar_arrive(acc_empty + 8 * p);
+          }
+#pragma unroll
+          for (int j = 0; j < EK; ++j) {
+            float q[ND];
+#pragma unroll
+            for (int d = 0; d < ND; ++d) q[d] = __uint_as_float(v[d][j]);
+            S[c][j] += fixed_to_double(join_fixed(q), es[j]);
+          }
+        }
+      } else {
+        uint32_t v[2][ND][EK];
+#pragma unroll
+        for (int c = 0; c < 2; ++c)
+#pragma unroll
+          for (int d = 0; d < ND; ++d) CSFF_TMEM_LD4(v[c][d], tl + (uint32_t)(p * ACC + 2 * TK * d + TK * c));
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) bar_arrive(acc_empty + 8 * p);
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          // merge into the running sums at the larger of the two exponents
+          const int En0 = max(E[2 * j], es[2 * j]), En1 = max(E[2 * j + 1], es[2 * j + 1]);
+          const float2 fa = make_float2(pow2_or_0(E[2 * j] - En0), pow2_or_0(E[2 * j + 1] - En1));
+          const float2 fs = make_float2(pow2_or_0(es[2 * j] - En0), pow2_or_0(es[2 * j + 1] - En1));
+          E[2 * j] = En0;
+          E[2 * j + 1] = En1;
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {
+            float2 q[7], h, l, t, e;
+#pragma unroll
+            for (int d = 0; d < 7; ++d)
+              q[d] = make_float2(__uint_as_float(v[c][d][2 * j]), __uint_as_float(v[c][d][2 * j + 1]));
+            join(q, h, l);
+            two_sum(__fmul2_rn(H[c][j], fa), __fmul2_rn(h, fs), t, e);
+            e = __fadd2_rn(e, __ffma2_rn(l, fs, __fmul2_rn(L[c][j], fa)));
+            const float2 hn = __fadd2_rn(t, e);
+            L[c][j] = __ffma2_rn(__ffma2_rn(t, both(-1.f), hn), both(-1.f), e);
+            H[c][j] = hn;
+          }
         }
       }
     }
@@ -963,11 +1060,13 @@ __global__ void __launch_bounds__(digits::NT, 1)
     if (rho < N)
 #pragma unroll
       for (int j = 0; j < EK; ++j) {
-        if (k0 + j >= M) continue;
+        const int row = k0 + j >= M ? -1 : map ? map[k0 + j] : k0 + j;
+        if (row < 0) continue;
         const float hr = (j & 1) ? H[0][j >> 1].y : H[0][j >> 1].x, lr = (j & 1) ? L[0][j >> 1].y : L[0][j >> 1].x;
         const float hi = (j & 1) ? H[1][j >> 1].y : H[1][j >> 1].x, li = (j & 1) ? L[1][j >> 1].y : L[1][j >> 1].x;
-        T[(long long)(k0 + j) * N + rho] =
+        T[(long long)row * N + rho] =
             !ok ? make_double2(__longlong_as_double(0x7ff8000000000000ll), __longlong_as_double(0x7ff8000000000000ll))
+                : SUB == 2 ? make_double2(S[0][j], S[1][j])
                 : E[j] == -100000 ? make_double2(0.0, 0.0)
                                   : make_double2(bits::widen(hr, E[j]) + bits::widen(lr, E[j]),
                                                  bits::widen(hi, E[j]) + bits::widen(li, E[j]));
@@ -1036,22 +1135,6 @@ __device__ __forceinline__ void split3(float v, __nv_bfloat16& a, __nv_bfloat16&
 __device__ __forceinline__ int exp_bound(double v) {
   const int E = (__double2hiint(v) >> 20) & 0x7FF;
   return (E == 0 ? 1 : E) - 1022;
-}
-
-// float(v * 2^-e), round to nearest even, from the bit fields alone (no FP64
-// arithmetic: this part runs FP64 at 1/61 of the FP32 rate).  Results below
-// FP32's normal range become zero; v must be finite with |v| 2^-e < 2^127.
-__device__ __forceinline__ float d2f_scaled(double v, int e) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
-  const unsigned int hi = (unsigned int)(b >> 32);
-  const int E = (int)((hi >> 20) & 0x7FF);
-  const int Ef = E - e - 1023 + 127;
-  if (E == 0 || Ef <= 0) return 0.f;
-  const unsigned long long mant = b & 0xFFFFFFFFFFFFFull;
-  unsigned int f = ((unsigned int)Ef << 23) + (unsigned int)(mant >> 29);
-  const unsigned int rem = (unsigned int)(mant & 0x1FFFFFFFull), halfway = 0x10000000u;
-  f += (rem > halfway || (rem == halfway && (f & 1u))) ? 1u : 0u;   // a carry into the exponent is exact
-  return __uint_as_float(f | (hi & 0x80000000u));
 }
 
 // v * 2^-e (|v| 2^-e < 1) as four BF16 terms with 32 significant bits: the
@@ -1456,6 +1539,98 @@ static cudaError_t ensure(void** p, size_t& cap, size_t need, csff_plan* P) {
   return e;
 }
 
+// ---- the z contraction of the 3D far field in digits ----------------------------
+// The line to the FP64 kernel.  An operand's error is 2^-64 of its block's scale
+// and a product's dropped diagonals 2^-61, so phases that vary by 6 binades over a
+// block (k h sin(gamma) 15 = 4.2) leave both below FP64's own roundings of the terms.
+constexpr double DIG3_BITS = 6.0, DIG3_WORK = 8e6;
+// column tiles of a chunk: at most 96 MB of operands (the L2 cache holds 129), a
+// whole number of waves of one CTA an SM
+static int dig3_chunk(int m, int T) {
+  const long long tile = 2ll * ((m + digits::KB - 1) / digits::KB) * digits::Form3::A_SLOTS * digits::A_DIG;
+  const int kt = (T + digits::TK - 1) / digits::TK;
+  long long c = std::max(1ll, (96ll << 20) / tile);
+  if (c * kt >= 152) c = std::max(1ll, c * kt / 152 * 152 / kt);
+  return (int)std::min<long long>(c, ((long long)m * m + digits::TM - 1) / digits::TM);
+}
+static cudaError_t dig3_ensure(FFBuffers& B, int m, int T, int chunk, csff_plan* P) {
+  using F = digits::Form3;
+  const size_t nb = (m + digits::KB - 1) / digits::KB, kt = (T + digits::TK - 1) / digits::TK;
+  cudaError_t e = ensure((void**)&B.dxdig, B.xdig, kt * nb * F::B_SET, P);
+  if (e == cudaSuccess)
+    e = ensure((void**)&B.dgdig, B.gdig, (size_t)chunk * nb * F::SUB * F::A_SLOTS * digits::A_DIG, P);
+  if (e == cudaSuccess)
+    e = ensure((void**)&B.dtce, B.tce, sizeof(int) * nb * F::SUB * ((size_t)T + (size_t)chunk * digits::TM), P);
+  return e;
+}
+static cudaError_t stage_a_digits(FFBuffers& B, const double2* zt, int T, const double2* g, int m, int chunk, double2* T1,
+                                  cudaStream_t s) {
+  using namespace digits;
+  using F = Form3;
+  cudaError_t e = cudaFuncSetAttribute(k_ff_digits<F>, cudaFuncAttributeMaxDynamicSharedMemorySize, F::SMEM);
+  if (e != cudaSuccess) return e;
+  const long long ncol = (long long)m * m;
+  const int nb = (m + KB - 1) / KB, kt = (T + TK - 1) / TK, tiles = (int)((ncol + TM - 1) / TM);
+  int *ex = B.dtce, *eg = B.dtce + (size_t)T * nb * F::SUB;
+  k_cut_phase3<<<(unsigned)(((long long)kt * TK * nb * 32 + 255) / 256), 256, 0, s>>>(zt, nullptr, m, T, ex, B.dxdig);
+  count_launch();
+  for (int t0 = 0; t0 < tiles; t0 += chunk) {
+    const int n = std::min(chunk, tiles - t0);
+    k_cut_field3<<<dim3(n, nb * F::SUB), TM, 0, s>>>(g, m, ncol, t0, eg, B.dgdig);
+    k_ff_digits<F><<<dim3(n, kt), NT, F::SMEM, s>>>(B.dgdig, B.dxdig, ex, T, eg, (int)ncol, nb, nullptr, nullptr, 0, T1,
+                                                    B.dmisc + 2, t0, nullptr, nullptr);
+    count_launch(2);
+  }
+  return cudaGetLastError();
+}
+
+// The y contraction T2[a][ix] = sum_iy Py[a][iy] T1[z(a)][iy][ix]: the angles of
+// each distinct z component, padded to tiles of 16 phase rows, against that
+// component's m x m field.
+struct YTiles { std::vector<int> map, field; };
+static YTiles y_tiles(const std::vector<int>& z_of, int T) {
+  std::vector<std::vector<int>> by(T);
+  for (int a = 0; a < (int)z_of.size(); ++a) by[z_of[a]].push_back(a);
+  YTiles y;
+  for (int t = 0; t < T; ++t)
+    for (size_t i = 0; i < by[t].size(); i += digits::TK) {
+      for (size_t j = i; j < i + digits::TK; ++j) y.map.push_back(j < by[t].size() ? by[t][j] : -1);
+      y.field.push_back(t);
+    }
+  return y;
+}
+static size_t dig3_b_ints(const YTiles& y, int m, int T) {
+  const size_t nbs = 2 * (size_t)((m + digits::KB - 1) / digits::KB), tiles = (m + digits::TM - 1) / digits::TM;
+  return y.map.size() * (nbs + 1) + y.field.size() + T * tiles * digits::TM * nbs;
+}
+static cudaError_t dig3_ensure_b(FFBuffers& B, const YTiles& y, int m, int T, csff_plan* P) {
+  using F = digits::Form3;
+  const size_t nb = (m + digits::KB - 1) / digits::KB, tiles = (m + digits::TM - 1) / digits::TM;
+  cudaError_t e = ensure((void**)&B.dxdig, B.xdig, y.field.size() * nb * F::B_SET, P);
+  if (e == cudaSuccess)
+    e = ensure((void**)&B.dgdig, B.gdig, T * tiles * nb * F::SUB * F::A_SLOTS * digits::A_DIG, P);
+  if (e == cudaSuccess) e = ensure((void**)&B.dtce, B.tce, sizeof(int) * dig3_b_ints(y, m, T), P);
+  return e;
+}
+static cudaError_t stage_b_digits(FFBuffers& B, const double2* yt, const YTiles& y, const double2* T1, int T, int m,
+                                  double2* T2, cudaStream_t s) {
+  using namespace digits;
+  using F = Form3;
+  const int nb = (m + KB - 1) / KB, nbs = nb * F::SUB, tiles = (m + TM - 1) / TM;
+  const int rows = (int)y.map.size(), kt = (int)y.field.size();
+  int *map = B.dtce, *field = map + rows, *ex = field + kt, *eg = ex + (size_t)rows * nbs;
+  cudaError_t e;
+  if ((e = cudaMemcpyAsync(map, y.map.data(), sizeof(int) * rows, cudaMemcpyHostToDevice, s)) != cudaSuccess ||
+      (e = cudaMemcpyAsync(field, y.field.data(), sizeof(int) * kt, cudaMemcpyHostToDevice, s)) != cudaSuccess)
+    return e;
+  k_cut_phase3<<<(unsigned)(((long long)rows * nb * 32 + 255) / 256), 256, 0, s>>>(yt, map, m, rows, ex, B.dxdig);
+  k_cut_field3<<<dim3(tiles, nbs, T), TM, 0, s>>>(T1, m, m, 0, eg, B.dgdig);
+  k_ff_digits<F><<<dim3(tiles, kt), NT, F::SMEM, s>>>(B.dgdig, B.dxdig, ex, rows, eg, m, nb, nullptr, nullptr, 0, T2,
+                                                      B.dmisc + 2, 0, field, map);
+  count_launch(3);
+  return cudaGetLastError();
+}
+
 // fraction of the double-float contraction's (tile, block) pairs that the last
 // 2D far field computed (1 when the FP64 kernel ran or nothing was skipped)
 csff_status far_field_executed(csff_plan* P, double* executed) {
@@ -1598,6 +1773,16 @@ csff_status far_field_one(csff_plan* P, const double* eta_host, const double2* u
       double2* T1 = B.dT;
       double2* T2 = B.dT + (size_t)n_uz * ncol;
       const bool use_tc = P->ff_mode == CSFF_FF_TC_BF16X4;
+      // The digit contraction (FP64's accuracy) where the phases vary by at most
+      // DIG3_BITS binades over a block of 16 nodes (g is finite: gmax), its
+      // operands fit, and the work outweighs its fixed cost.
+      double uz_max = 0;
+      for (double v : uz) uz_max = std::max(uz_max, std::fabs(v));
+      const int chunk = dig3_chunk(m, n_uz);
+      bool dig3 = !use_tc && 15.0 * std::fabs(P->prob.k * sg * L.h) * uz_max <= DIG3_BITS * std::log(2.0) &&
+                  (double)n_uz * (double)ncol * m >= DIG3_WORK && (m + digits::KB - 1) / digits::KB <= digits::MAX_NB &&
+                  dig3_ensure(B, m, n_uz, chunk, P) == cudaSuccess;
+      if (!dig3) cudaGetLastError();
       const int nkc = (m + tc::KZ - 1) / tc::KZ;
       if (use_tc) {
         if ((e = ensure((void**)&B.dtcb, B.tcb, (size_t)nkc * tc::NSPLIT * tc::B_SPLIT, P)) != cudaSuccess ||
@@ -1634,6 +1819,9 @@ csff_status far_field_one(csff_plan* P, const double* eta_host, const double2* u
                                                                               B.dtcflag);
             count_launch(3 + (std::min(n_uz, t0 + tc::TT) - t0 + 15) / 16);
           }
+        } else if (dig3) {
+          if ((e = stage_a_digits(B, B.dxt, n_uz, B.dg, m, chunk, T1, s)) != cudaSuccess)
+            return cuda_fail(e, "far field z contraction");
         } else {
           for (int t0 = 0; t0 < n_uz; t0 += 16)
             k_ff3_stageA<16><<<(unsigned)((ncol + 255) / 256), 256, 0, s>>>(B.dxt, n_uz, t0, B.dg, m, ncol, T1,
@@ -1641,7 +1829,27 @@ csff_status far_field_one(csff_plan* P, const double* eta_host, const double2* u
           count_launch((n_uz + 15) / 16);
         }
       }
-      k_ff3_stageB<<<dim3((m + 127) / 128, n_ang), 128, sizeof(double2) * m, s>>>(B.dyt, B.dxr, T1, m, T2);
+      // the y contraction in digits under the same rule, where the angles share
+      // z components (padding at most doubles the phase rows) and the fields'
+      // operands stay below 1 GB
+      double uy_max = 0;
+      for (int a = 0; a < n_ang; ++a) uy_max = std::max(uy_max, std::fabs(alpha_host[(size_t)a * 3 + 1]));
+      bool dig3b = dig3 && 15.0 * std::fabs(P->prob.k * sg * L.h) * uy_max <= DIG3_BITS * std::log(2.0) &&
+                   (double)n_ang * (double)ncol >= DIG3_WORK && n_uz <= 65535;
+      YTiles yt;
+      if (dig3b) {
+        yt = y_tiles(tr, n_uz);
+        dig3b = yt.map.size() <= 2 * (size_t)n_ang && (double)n_uz * ((m + 127) / 128) * ((m + 31) / 32) * 131072.0 <= 1e9 &&
+                dig3_ensure_b(B, yt, m, n_uz, P) == cudaSuccess;
+        if (!dig3b) cudaGetLastError();
+      }
+      if (dig3b) {
+        if ((e = stage_b_digits(B, B.dyt, yt, T1, n_uz, m, T2, s)) != cudaSuccess)
+          return cuda_fail(e, "far field y contraction");
+      } else {
+        k_ff3_stageB<<<dim3((m + 127) / 128, n_ang), 128, sizeof(double2) * m, s>>>(B.dyt, B.dxr, T1, m, T2);
+        count_launch();
+      }
       // stage C: F[a] = pref sum_ix Px[a][ix] T2[a][ix]  (the 2D stage-2 kernel on rows a)
       if ((e = cudaMemcpyAsync(B.dxr, ident.data(), sizeof(int) * n_ang, cudaMemcpyHostToDevice, s)) != cudaSuccess)
         return cuda_fail(e, "far field rows");
@@ -1650,7 +1858,7 @@ csff_status far_field_one(csff_plan* P, const double* eta_host, const double2* u
       double2 pref = make_double2(k2 * hd * std::cos(3 * P->prob.gamma), k2 * hd * std::sin(3 * P->prob.gamma));
       k_ff_stage2<2><<<n_ang, 256, 0, s>>>(T2, B.dxr, B.ds1, B.dzt, B.dzt, m, pref, F, F_exp, F_exp != nullptr,
                                            B.dmisc + 1);
-      count_launch(3);
+      count_launch(2);
       if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "far field 3D kernels");
       if (use_tc) {
         int fl[3] = {0, 0, 0};
@@ -1663,11 +1871,15 @@ csff_status far_field_one(csff_plan* P, const double* eta_host, const double2* u
         }
       }
       if (scaled) {
-        int flag = 0;
-        if ((e = cudaMemcpyAsync(&flag, B.dmisc + 1, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
+        int flag[2] = {0, 0};
+        if ((e = cudaMemcpyAsync(flag, B.dmisc + 1, sizeof(flag), cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
             (e = cudaStreamSynchronize(s)) != cudaSuccess)
           return cuda_fail(e, "far field flag");
-        *scaled = flag != 0;
+        *scaled = flag[0] != 0;
+        if (flag[1]) {
+          set_error("far-field contraction: an mbarrier wait ran out");
+          return CSFF_ERR_TIMEOUT;
+        }
       }
       return CSFF_OK;
     }
@@ -1695,8 +1907,8 @@ csff_status far_field_one(csff_plan* P, const double* eta_host, const double2* u
   // double-float one runs)
   const int gxt = (int)((R + digits::TM - 1) / digits::TM), gkt = (n_ux + digits::TK - 1) / digits::TK;
   bool dig = d == 2 && nbk <= digits::MAX_NB &&
-             ensure((void**)&B.dxdig, B.xdig, (size_t)gkt * nbk * digits::B_SET, P) == cudaSuccess &&
-             ensure((void**)&B.dgdig, B.gdig, (size_t)gxt * nbk * digits::ND * digits::A_DIG, P) == cudaSuccess;
+             ensure((void**)&B.dxdig, B.xdig, (size_t)gkt * nbk * digits::Form2::B_SET, P) == cudaSuccess &&
+             ensure((void**)&B.dgdig, B.gdig, (size_t)gxt * nbk * digits::Form2::ND * digits::A_DIG, P) == cudaSuccess;
   if (!dig) cudaGetLastError();
   // [2] starts far over the margin where the digit form may not run
   if ((e = cudaMemsetAsync(B.dspread, 0, 3 * sizeof(int), s)) != cudaSuccess ||
@@ -1721,7 +1933,8 @@ csff_status far_field_one(csff_plan* P, const double* eta_host, const double2* u
   k_split_rows<<<warps(R), 256, 0, s>>>(B.dg, m, (int)R, B.deg, B.dspread, B.dgdf, B.dgsm);
   count_launch(2);
   if (dig) {
-    if ((e = cudaFuncSetAttribute(k_ff_digits, cudaFuncAttributeMaxDynamicSharedMemorySize, digits::SMEM)) != cudaSuccess)
+    if ((e = cudaFuncSetAttribute(k_ff_digits<digits::Form2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  digits::Form2::SMEM)) != cudaSuccess)
       return cuda_fail(e, "far-field contraction attribute");
     k_cut_rows<true><<<warps((long long)gkt * digits::TK), 256, 0, s>>>(B.dxt, m, n_ux, B.dex, B.dspread, B.dxdig);
     k_cut_rows<false><<<warps((long long)gxt * digits::TM), 256, 0, s>>>(B.dg, m, (int)R, B.deg, B.dspread, B.dgdig);
@@ -1734,8 +1947,9 @@ csff_status far_field_one(csff_plan* P, const double* eta_host, const double2* u
                  8.0 * (double)n_ux * (double)R * m);
     // exactly one of them writes T (device-side checks on the spreads and margin)
     if (dig) {
-      k_ff_digits<<<dim3(gxt, gkt), digits::NT, digits::SMEM, s>>>(B.dgdig, B.dxdig, B.dex, n_ux, B.deg, (int)R, nbk, B.dspread, B.dskip, (int)gdf.x, B.dT,
-                                                                    B.dmisc + 2);
+      k_ff_digits<digits::Form2><<<dim3(gxt, gkt), digits::NT, digits::Form2::SMEM, s>>>(
+          B.dgdig, B.dxdig, B.dex, n_ux, B.deg, (int)R, nbk, B.dspread, B.dskip, (int)gdf.x, B.dT, B.dmisc + 2, 0,
+          nullptr, nullptr);
       count_launch();
     }
     k_ff_stage1_df<<<gdf, DF_NT, 0, s>>>(B.dxdf, B.dxsm, B.dex, n_ux, B.dgdf, B.dgsm, B.deg, (int)R, nbk, B.dspread,

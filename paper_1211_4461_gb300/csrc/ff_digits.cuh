@@ -42,55 +42,75 @@
 namespace csff {
 namespace digits {
 
-constexpr int ND = 7;                          // digits of a value
 constexpr int TM = 128, TK = 16;               // rows of g and phase rows of a tile
 constexpr int KB = 32;                         // nodes of a block
 constexpr int A_DIG = TM * 128;                // bytes of a digit of an A block (128-byte rows)
 constexpr int B_DIG = 2 * TK * 128;
-constexpr int B_SET = ND * B_DIG;
-constexpr int NA = 10;                         // A slots of the ring
 constexpr int MAX_NB = 1024;                   // blocks of a row
 constexpr int EPI_WARPS = 16, NT = 32 * (EPI_WARPS + 2);
 constexpr int EK = TK * 4 / EPI_WARPS;           // phase rows of an epilogue warp
-constexpr int OFF_BAR = NA * A_DIG + 2 * B_SET;
-constexpr int OFF_ACT = OFF_BAR + 512;
-constexpr int SMEM = OFF_ACT + MAX_NB * 2 + 1024;
 constexpr int TMEM_COLS = 512, ACC = 256;      // columns of one set of accumulators (7 x 32 used)
 constexpr int MARGIN = 12;
 constexpr unsigned long long WAIT_NS = 500000000ull;   // a wait gives up after half a second
-static_assert(SMEM <= 227 * 1024, "shared memory");
+
+// A form of the contraction: ND digits a value, NA A slots in the ring, SUB
+// scale blocks in the 32 nodes of a row of B.
+//  2D: seven digits, one block, an A slot one digit of 32 nodes.
+//  3D (the z contraction): eight digits, two blocks, an A slot two digits of 16
+//  nodes; each block's diagonals fill a set of accumulators.
+template <int ND_, int NA_, int SUB_> struct Form {
+  static constexpr int ND = ND_, NA = NA_, SUB = SUB_;
+  static constexpr int BITS = 8 * ND - 1;      // fixed-point bits below the scale
+  static constexpr int A_SLOTS = ND / SUB;     // slots of a block
+  static constexpr int B_SET = ND * B_DIG;
+  static constexpr int OFF_BAR = NA * A_DIG + 2 * B_SET, OFF_ACT = OFF_BAR + 512;
+  static constexpr int SMEM = OFF_ACT + MAX_NB * 2 + 1024;
+  static_assert(SMEM <= 227 * 1024 && ND % SUB == 0 && 2 * TK * ND <= ACC, "shared and tensor memory");
+};
+using Form2 = Form<7, 10, 1>;
+using Form3 = Form<8, 9, 2>;
 
 // 128-byte-swizzled K-major row: byte offset of 16-byte chunk c of row r
 __device__ __forceinline__ int sw(int r, int c) { return (r >> 3) * 1024 + (r & 7) * 128 + ((c ^ (r & 7)) << 4); }
 
-// x 2^(55 - e) rounded to an integer, |x| < 2^e, from the IEEE fields
-__device__ __forceinline__ long long fixed55(double x, int e) {
+// x 2^(BITS - e) rounded to an integer, |x| < 2^e, from the IEEE fields
+template <int BITS> __device__ __forceinline__ long long fixed(double x, int e) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
   const int E = (int)((b >> 52) & 0x7ff);
-  if ((b & bits::ABS_MASK) == 0 || E == 0x7ff) return 0;
-  if (E == 0) return __double2ll_rn(ldexp(x, 55 - e));
-  const long long m = (long long)((b & bits::MANT_MASK) | (1ull << 52));
-  const int sh = E - 1020 - e;                 // m 2^(E - 1075) 2^(55 - e)
+  const long long m = (long long)((b & bits::MANT_MASK) | (E ? 1ull << 52 : 0));
+  const int sh = max(E, 1) - 1075 + BITS - e;  // m 2^(max(E, 1) - 1075) 2^(BITS - e)
   long long q;
-  if (sh >= 0) q = m << (sh < 3 ? sh : 3);
+  if (sh >= 0) q = m << min(sh, 62);
   else if (sh < -54) q = 0;
   else q = (m + (1ll << (-sh - 1))) >> -sh;
-  return (b >> 63) ? -q : q;
+  return E == 0x7ff ? 0 : (b >> 63) ? -q : q;
 }
+// e with |x| < 2^e from the exponent fields (zero and subnormal values: -1022)
+__device__ __forceinline__ int scale_exp(double2 x) { return max(bits::exp_field(x.x), bits::exp_field(x.y)) - 1022; }
 
 // the digits of two fixed-point values as pairs of BF16 integers, dig[0] the
-// leading one
-__device__ __forceinline__ void cut(long long p, long long q, uint32_t (&dig)[ND]) {
+// leading one.  Balanced digits are the bytes after adding 128 to every byte
+// below the leading one, less 128; a byte becomes a float in the mantissa of
+// 2^23 (a full-rate subtraction where a conversion runs at a quarter), whose
+// upper half is the BF16 value.
+__device__ __forceinline__ float byte_digit(unsigned v, int byte) {
+  return __uint_as_float(__byte_perm(v, 0x4B000000u, 0x7440 | byte)) - 8388736.f;      // 2^23 + 128
+}
+template <int ND> __device__ __forceinline__ void cut(long long p, long long q, uint32_t (&dig)[ND]) {
+  constexpr int SH = 8 * (ND - 1);
+  constexpr unsigned long long LOW = (1ull << SH) - 1, HALF = 0x8080808080808080ull & LOW;
+  const unsigned long long lp = ((unsigned long long)p & LOW) + HALF, lq = ((unsigned long long)q & LOW) + HALF;
+  auto pack = [](float a, float b) { return __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x7632); };
 #pragma unroll
-  for (int s = ND - 1; s > 0; --s) {
-    const int a = (int)(signed char)(p & 255), b = (int)(signed char)(q & 255);
-    p = (p - a) >> 8;
-    q = (q - b) >> 8;
-    const __nv_bfloat162 v = __floats2bfloat162_rn((float)a, (float)b);
-    dig[s] = *reinterpret_cast<const uint32_t*>(&v);
+  for (int s = 1; s < ND; ++s) {
+    const int byte = ND - 1 - s;
+    const unsigned a = (unsigned)(byte < 4 ? lp : lp >> 32), b = (unsigned)(byte < 4 ? lq : lq >> 32);
+    dig[s] = pack(byte_digit(a, byte & 3), byte_digit(b, byte & 3));
   }
-  const __nv_bfloat162 v = __floats2bfloat162_rn((float)(int)p, (float)(int)q);
-  dig[0] = *reinterpret_cast<const uint32_t*>(&v);
+  auto top = [&](long long v, unsigned long long low) {
+    return __int_as_float(0x4B400000 + (int)(v >> SH) + (int)(low >> SH)) - 12582912.f;
+  };
+  dig[0] = pack(top(p, lp), top(q, lq));
 }
 __device__ __forceinline__ uint32_t neg_hi(uint32_t v) { return v ^ 0x80000000u; }      // (a, b) -> (a, -b)
 __device__ __forceinline__ uint32_t swap_pair(uint32_t v) { return (v >> 16) | (v << 16); }
@@ -167,7 +187,7 @@ __device__ __forceinline__ float2 both(float a) { return make_float2(a, a); }
 // h + l = sum_{d=0..6} p[d] 2^-8d: the four leading terms by exact sums (their
 // digit sums reach 2^23, eight bits apart), the three trailing ones, whose
 // roundings lie below 2^-55 of the scale, by multiply-adds
-__device__ __forceinline__ void join(const float2 (&p)[ND], float2& h, float2& l) {
+__device__ __forceinline__ void join(const float2 (&p)[7], float2& h, float2& l) {
   const float2 w = both(0x1p-8f);
   float2 q = __ffma2_rn(p[6], w, p[5]);
   q = __ffma2_rn(q, w, p[4]);
@@ -177,6 +197,27 @@ __device__ __forceinline__ void join(const float2 (&p)[ND], float2& h, float2& l
   two_sum(p[1], __fmul2_rn(t, w), t, e1);
   two_sum(p[0], __fmul2_rn(t, w), h, l);
   l = __fadd2_rn(l, __fmul2_rn(__ffma2_rn(__ffma2_rn(e3, w, e2), w, e1), w));
+}
+
+// 3D form: sum_{d=0..7} p[d] 2^(43 - 8 d) as an integer (the block's sum times
+// 2^57; its magnitude, at most 32, leaves a bit).  The digit sums are integers of
+// at most 2^22 and pair up in 32 bits; the last two, below the integer, round.
+__device__ __forceinline__ int exact_int(float x) { return __float_as_int(x + 12582912.f) - 0x4B400000; }
+__device__ __forceinline__ long long join_fixed(const float (&p)[8]) {
+  const int t0 = (exact_int(p[0]) << 8) + exact_int(p[1]), t1 = (exact_int(p[2]) << 8) + exact_int(p[3]);
+  const int t2 = (exact_int(p[4]) << 8) + exact_int(p[5]);
+  const int t3 = exact_int(__fmaf_rn(p[6], 256.f, p[7]) * 0x1p-13f);
+  return (long long)t0 * (1ll << 35) + (long long)t1 * (1ll << 19) + (long long)t2 * 8 + t3;
+}
+// v 2^e rounded to FP64 (a subnormal result truncated), integer operations only
+__device__ __forceinline__ double fixed_to_double(long long v, int e) {
+  const unsigned long long u = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
+  const int lz = __clzll((long long)u), ef = 1086 - lz + e;
+  const unsigned long long n = u << min(lz, 63), mant = (n >> 11) + ((n >> 10) & 1);
+  unsigned long long r = ((unsigned long long)(unsigned)(ef - 1) << 52) + mant;
+  if (ef < 1) r = n >> min(12 - ef, 63);
+  if (ef > 2045) r = 0x7ff0000000000000ull;
+  return __longlong_as_double((long long)(u == 0 ? 0ull : r | ((unsigned long long)(v < 0) << 63)));
 }
 
 }  // namespace digits

@@ -133,3 +133,30 @@ def test_far_field_contraction(csff, n, coarsest, n_ang, k, R, scale):
     # the contraction's rounding (2^-47 of the sum of the terms' magnitudes for
     # the double-float form, less for digits) and the phase tables' few ulp
     assert np.all(np.abs(got - mant) <= 1e-13 * tn)
+
+
+# the z contraction of the 3D far field: distinct z components below, at and
+# above its tiles of 16, last rows of 32 nodes whose second scale block of 16 is
+# empty (m = 71, 79) or short (63, 95), several column chunks (159) and phases
+# too steep for its digits (k = 3 on the wide box: the FP64 kernel)
+@pytest.mark.parametrize("n,coarsest,n_z,k,R", [(65, 5, 33, 1.0, 5.0), (73, 10, 48, 2.0, 5.0), (81, 6, 17, 2.0, 5.0),
+                                                (97, 7, 16, 3.0, 10.0), (161, 6, 7, 2.0, 15.0), (65, 5, 40, 3.0, 10.0)])
+@pytest.mark.parametrize("scale", [1.0, 1e-150])
+def test_far_field_3d_contraction(csff, n, coarsest, n_z, k, R, scale):
+    prob = W.problem(3, n, R, math.pi / 6, k, [W.gauss(-0.7, 1.5), W.gauss(-0.3, 3.0, (0.5, -0.4, 0.2))])
+    opts = {"smoother": "jacobi", "nu1": 1, "nu2": 1, "coarsest_n": coarsest, "rel_tol": 1e-8, "precision": "fp64"}
+    plan = csff.Plan(prob, opts)
+    m = plan.m
+    u0 = scale * W.rand_complex((m, m, m), 31)
+    eta = np.array([[0.6, 0.0, 0.8]])
+    th, ph = np.pi * (np.arange(n_z) + 0.5) / n_z, 0.7 * np.arange(n_z)
+    al = np.ascontiguousarray(np.stack([np.sin(th) * np.cos(ph), np.sin(th) * np.sin(ph), np.cos(th)], axis=1))
+    F = torch.zeros(n_z, dtype=torch.complex128, device="cuda")
+    E = torch.zeros(n_z, dtype=torch.int32, device="cuda")
+    plan.far_field(eta, torch.from_numpy(u0.ravel()).cuda(), al, F, E)
+    plan.close()
+    sel = np.unique(np.array([0, n_z // 2, n_z - 1]))
+    mant, e2, tn = O.far_field(O.problem_from_dict(prob), u0, eta[0], al[sel], return_terms_norm=True)
+    got = F.cpu().numpy()[sel] * 2.0 ** (E.cpu().numpy()[sel].astype(np.float64) - e2)
+    # each stage's rounding is below 2^-48 of the sum of the terms' magnitudes
+    assert np.all(np.abs(got - mant) <= 1e-13 * tn)
