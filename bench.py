@@ -526,10 +526,11 @@ def run_ours(args, rank, world, local_rank):
                                                    alg_note + "; these launches last about one CTA's lifetime"),
                        "all": tiles_roofline(allt, TILES_DRAM_BYTES, "k_down2 / k_up2, every fused level",
                                              alg_note)}
-    roofline_ff = {"kernel": "k_ff_stage1_df (double-float far-field contraction)", "bound": "alu",
+    roofline_ff = {"kernel": "2D far-field contraction: k_ff_digits (exact digits on the tensor cores) for maps whose "
+                             "phases vary slowly over a block, k_ff_stage1_df (double-float) for the others", "bound": "alu",
                 "achieved": achieved_tf, "peak": DF_PEAK_TFLOPS, "unit": "TFLOP/s",
-                "frac": achieved_tf / DF_PEAK_TFLOPS, "traffic": FF_DF_DRAM_BYTES,
-                "peak_source": "derived: 152 SMs x 128 FP32 lanes x 2.07 GHz / 4.5 FP32 operations per "
+                "frac": achieved_tf / DF_PEAK_TFLOPS, "traffic": None,
+                "peak_source": "the double-float kernel's: 152 SMs x 128 FP32 lanes x 2.07 GHz / 4.5 FP32 operations per "
                                "FP64-equivalent flop (36 per complex multiply-add: three double-float "
                                "multiply-adds, Gauss's product; a packed two-lane instruction counts two)",
                 "avg_launch_ms": ff_avg_ms, "launches": ff["launches"],
