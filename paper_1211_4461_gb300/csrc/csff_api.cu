@@ -449,10 +449,16 @@ template <typename T>
 csff_status run_split3(csff_plan* P, cx<T>* u, const cx<T>* b, bool zero_init, bool first, bool last) {
   const cx<T>* none = nullptr;
   cx<T>* no = nullptr;
-  CK(csff::launch_split3_down<T>(P->lv, first && !zero_init ? u : none, b, zero_init, P->stream), "split down");
-  Level& C = P->lv.back();
-  CS(coarsest_solve<T>(P, bbuf<T>(C), split_of<T>(C).e, C.m, csff::split3_ring_pitch(C.m)));
-  CK(csff::launch_split3_up<T>(P->lv, last ? u : no, P->stream), "split up");
+  const int lb = sizeof(T) == 4 ? P->split_block : 0, stop = lb > 0 ? lb : (int)P->lv.size() - 1;
+  CK(csff::launch_split3_down<T>(P->lv, stop, first && !zero_init ? u : none, b, zero_init, P->stream), "split down");
+  if (lb > 0) {
+    CK(csff::launch_split3_block(P->lv, lb, cinv<float>(P), coarse_fp64(P) ? P->coarse_inv : nullptr, P->stream),
+       "coarse block");
+  } else {
+    Level& C = P->lv.back();
+    CS(coarsest_solve<T>(P, bbuf<T>(C), split_of<T>(C).e, C.m, csff::split3_ring_pitch(C.m)));
+  }
+  CK(csff::launch_split3_up<T>(P->lv, stop, last ? u : no, P->stream), "split up");
   return CSFF_OK;
 }
 
@@ -956,6 +962,10 @@ csff_status csff_plan_create(const csff_problem* prob, const csff_opts* opts, vo
     csff_status s = mixed ? alloc_split3<float>(P) : alloc_split3<double>(P);
     if (s != CSFF_OK) return fail(s);
     (mixed ? P->split32 : P->split64) = true;
+    if (mixed && (P->split_block = csff::split3_block_level(P->lv)) > 0) {
+      cudaError_t e = csff::prepare_split3_block();
+      if (e != cudaSuccess) return fail(csff::cuda_fail(e, "coarse block attributes"));
+    }
   }
   // fused V(1,1) RB-GS path (2D): the levels from the first with n <= 33 run in
   // one CTA; at least one fused fine level is needed

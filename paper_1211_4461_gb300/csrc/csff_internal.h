@@ -166,8 +166,10 @@ struct csff_plan {
   double log_rhs_max = 0, log_ff_max = 0;
   // fused V(1,1) RB-GS path (2D): levels >= fused_lc run in one CTA; -1 = unfused
   int fused_lc = -1;
-  // colour-split 3D V(1,1) RB-GS cycles: their arrays exist in FP32 / FP64
+  // colour-split 3D V(1,1) RB-GS cycles: their arrays exist in FP32 / FP64; FP32:
+  // the level from which one CTA runs the coarser ones (0: none)
   bool split32 = false, split64 = false;
+  int split_block = 0;
   // CUDA graphs of solver steps (FP64 cycle, or mixed refinement step of a
   // given cycle count), captured on an internal stream and kept by key; the
   // oldest is replaced when all slots are taken
@@ -329,15 +331,22 @@ int split3_pitch(int m);                       // slots of a row of one colour
 // 1/d by colour from dinv64 (k2: the wavenumber's square, without potential)
 template <typename T> cudaError_t split3_coefs(Level& L, double k2, cudaStream_t s);
 int split3_ring_pitch(int mc);                 // row pitch of a level's correction
-// the levels down to the coarsest right-hand side (b32/b64 of the last level):
-// b and the iterate u in natural order, or zero_init, or (u null) both still in
-// the split arrays
+// the levels above `stop` down to its right-hand side (split, with the red half
+// sweep from zero; of the last level b32/b64 in natural order): b and the
+// iterate u in natural order, or zero_init, or (u null) both still in the split
+// arrays
 template <typename T>
-cudaError_t launch_split3_down(std::vector<Level>& lv, const cx<T>* u, const cx<T>* b, bool zero_init, cudaStream_t s);
-// and back from the coarsest solution (the last level's e); the iterate goes to
-// u_nat in natural order or (null) stays in the split arrays
+cudaError_t launch_split3_down(std::vector<Level>& lv, int stop, const cx<T>* u, const cx<T>* b, bool zero_init,
+                               cudaStream_t s);
+// and back from level stop's correction e; the iterate goes to u_nat in natural
+// order or (null) stays in the split arrays
 template <typename T>
-cudaError_t launch_split3_up(std::vector<Level>& lv, cx<T>* u_nat, cudaStream_t s);
+cudaError_t launch_split3_up(std::vector<Level>& lv, int stop, cx<T>* u_nat, cudaStream_t s);
+// FP32 cycles: the level from which one CTA runs all coarser ones (0: none), its
+// set-up and launch (inv64: the coarsest product in FP64)
+int split3_block_level(const std::vector<Level>& lv);
+cudaError_t prepare_split3_block();
+cudaError_t launch_split3_block(std::vector<Level>& lv, int lb, const float2* inv, const double2* inv64, cudaStream_t s);
 
 // ---- GMRES(m) smoothing step (gmres.cu) ----------------------------------------
 // u += V y for the GMRES(m) minimiser from u; V holds m+1 vectors of L.N

@@ -62,6 +62,14 @@ template <typename C> __device__ __forceinline__ C cfma(C a, C b, C c) {
 __device__ __forceinline__ float2 dinv_mul(float2 d0, float2 dv, float2 t) { return cfma(cmul(d0, t), dv, t); }
 __device__ __forceinline__ double2 dinv_mul(double2, double2 dv, double2 t) { return cmul(dv, t); }
 
+// Launches of at most one CTA an SM (the small levels) let their dependent be set
+// up as soon as they have passed their own wait; a sweep's and a full weighting's
+// 1/d, which no pass writes, is loaded before that wait.
+__device__ __forceinline__ void wait_and_trigger() {
+  pdl_prologue();
+  if (gridDim.x * gridDim.y * gridDim.z <= 152u) pdl_trigger();
+}
+
 // coordinates of a thread: slot pair, row, plane
 struct At { int j, iy, iz; long long row; };
 __device__ __forceinline__ bool at(int m, int HP, At& p) {
@@ -79,7 +87,7 @@ __global__ void k3s_first(const cx<T>* __restrict__ b_nat, const cx<T>* __restri
                           const cx<T>* __restrict__ dr, cx<T> c, cx<T> d0, int m, int HP, cx<T>* __restrict__ br,
                           cx<T>* __restrict__ bb, cx<T>* __restrict__ ub, cx<T>* __restrict__ ur) {
   using C = cx<T>;
-  pdl_prologue();
+  wait_and_trigger();
   At p;
   if (!at(m, HP, p)) return;
   const int o = (p.iy + p.iz + 1) & 1;                 // red parity of the row
@@ -215,11 +223,12 @@ __global__ void k3s_sweep(const cx<T>* __restrict__ uo, const cx<T>* __restrict_
                           cx<T> c, cx<T> d0, int m, int HP, cx<T>* u, cx<T>* __restrict__ delta,
                           const cx<T>* __restrict__ e, int pe, int mc, cx<T>* __restrict__ nat, int nat_pitch) {
   using C = cx<T>;
-  pdl_prologue();
   At p;
   if (!at(m, HP, p)) return;
   const int o = (p.iy + p.iz + 1 + COLOUR) & 1;
   const long long s = p.row * HP + p.j;
+  const Pair<T> dv = ld2(dinv + s);
+  wait_and_trigger();
   const long long plane = (long long)m * HP;
   const Pair<T> zero{zc<T>(), zc<T>()};
   const Pair<T> mid = ld2(uo + s);
@@ -227,7 +236,7 @@ __global__ void k3s_sweep(const cx<T>* __restrict__ uo, const cx<T>* __restrict_
   const C edge = (je >= 0 && je < HP) ? uo[s + (je - p.j)] : zc<T>();
   const Pair<T> yl = p.iy > 0 ? ld2(uo + s - HP) : zero, yr = p.iy < m - 1 ? ld2(uo + s + HP) : zero;
   const Pair<T> zl = p.iz > 0 ? ld2(uo + s - plane) : zero, zr = p.iz < m - 1 ? ld2(uo + s + plane) : zero;
-  const Pair<T> bv = ld2(b + s), dv = ld2(dinv + s);
+  const Pair<T> bv = ld2(b + s);
   Pair<T> old = zero;
   if constexpr (MODE == DELTA) old = ld2(u + s);
   // x - 1 and x + 1 of both slots
@@ -269,10 +278,12 @@ __global__ void k3s_restrict(const cx<T>* __restrict__ delta, int m, int HP, cx<
                              cx<T>* __restrict__ br, cx<T>* __restrict__ bb, const cx<T>* __restrict__ dr,
                              cx<T> d0, cx<T>* __restrict__ ur, cx<T>* __restrict__ nat) {
   using C = cx<T>;
-  pdl_prologue();
   const int P = 2 * (int)(blockIdx.x * blockDim.x + threadIdx.x);
   const int Yc = blockIdx.y * blockDim.y + threadIdx.y, Zc = blockIdx.z;
   if (P >= mc || Yc >= mc) return;
+  const long long row = (long long)Zc * mc + Yc, s = row * HPc + (P >> 1);
+  const C dc = nat ? zc<T>() : dr[s];
+  wait_and_trigger();
   const int fy = 2 * Yc + 1, fz = 2 * Zc + 1;          // rows one unit off lie inside the grid (m is odd)
   const C* const own = delta + ((long long)fz * m + fy) * HP + P;
   auto rowp = [&](int dy, int dz) {
@@ -328,18 +339,175 @@ __global__ void k3s_restrict(const cx<T>* __restrict__ delta, int m, int HP, cx<
   const C w0 = cadd(cadd(cscale(f0, (T)0.25), cscale(g0, (T)0.09375)), cscale(h0, (T)0.03125));
   const C w1 = cadd(cadd(cscale(f1, (T)0.25), cscale(g1, (T)0.09375)), cscale(h1, (T)0.03125));
   const C v0 = cmul(c, w0), v1 = P + 1 < mc ? cmul(c, w1) : zc<T>();
-  const long long row = (long long)Zc * mc + Yc;
   if (nat) {
     nat[row * mc + P] = v0;
     if (P + 1 < mc) nat[row * mc + P + 1] = v1;
     return;
   }
   const int o = (Yc + Zc + 1) & 1;                     // red parity of the coarse row
-  const long long s = row * HPc + (P >> 1);
   const C vr = o ? v1 : v0;
   br[s] = vr;
   bb[s] = o ? v0 : v1;
-  ur[s] = dinv_mul(d0, dr[s], vr);
+  ur[s] = dinv_mul(d0, dc, vr);
+}
+
+// All levels from one of at most 15 points a side down to the coarsest and back
+// in one CTA (FP32 cycles; FP64 ones would be bound by the one SM's FP64 pipe).
+//
+// Bound by latency: a chain of short phases on grids in shared memory, natural
+// order with a ring of zeros (u, b, 1/d of the smoothing levels; 137 KB from 17^3
+// down).  A row of a colour takes eight lanes; phases as above.  17^3, 9^3 and 5^3:
+// 20.9 us alone, where the ten passes took 42 one by one; in the dependent
+// launches of a cycle 4 us of that difference are left (257^3 cycle 367 -> 363).
+constexpr int BLOCK_M = 15, BLOCK_NT = 1024, BLOCK_LEVELS = 6, BLOCK_LAST = 64;
+struct BlockLevels {
+  int nl, m[BLOCK_LEVELS], HP[BLOCK_LEVELS];            // the last is the coarsest
+  const float2 *dr[BLOCK_LEVELS], *db[BLOCK_LEVELS];
+  float2 c[BLOCK_LEVELS], d0[BLOCK_LEVELS];
+};
+__host__ __device__ inline int ringed(int m) { return (m + 2) * (m + 2) * (m + 2); }
+
+// neighbour sum of the interpolated correction at a red point (node indices
+// nx, ny, nz), e ringed with W values a row: the cases of prolong_nbr
+__device__ __forceinline__ float2 prolong_nbr_ringed(const float2* e, int W, int nx, int ny, int nz) {
+  const float2* p = e + ((nz >> 1) * W + (ny >> 1)) * W + (nx >> 1);
+  const int W2 = W * W;
+  if (!((nx | ny | nz) & 1)) {
+    const float2 s = cadd(cadd(cadd(p[-1], p[1]), cadd(p[-W], p[W])), cadd(p[-W2], p[W2]));
+    return cadd(cscale(p[0], 3.f), cscale(s, 0.5f));
+  }
+  const int se = !(nx & 1) ? 1 : !(ny & 1) ? W : W2, s1 = (nx & 1) ? 1 : W, s2 = (nz & 1) ? W2 : W;
+  auto s4 = [&](const float2* q) { return cadd(cadd(q[0], q[s1]), cadd(q[s2], q[s1 + s2])); };
+  return cadd(cscale(s4(p), 1.25f), cscale(cadd(s4(p - se), s4(p + se)), 0.125f));
+}
+
+template <typename TI>
+__global__ void __launch_bounds__(BLOCK_NT, 1)
+    k3s_block(BlockLevels L, const float2* __restrict__ br, const float2* __restrict__ bb, const float2* __restrict__ ur,
+              const cx<TI>* __restrict__ inv, float2* __restrict__ e_out, int pe) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ __align__(16) cx<TI> Bc[BLOCK_LAST];
+  float2* const base = reinterpret_cast<float2*>(smem_raw);
+  const int t = threadIdx.x, last = L.nl - 1, j = t & 7, r0 = t >> 3;
+  constexpr int RS = BLOCK_NT / 8;
+  int total = ringed(L.m[last]);
+  for (int l = 0; l < last; ++l) total += 3 * ringed(L.m[l]);
+  for (int i = t; i < total; i += BLOCK_NT) base[i] = make_float2(0.f, 0.f);
+  __syncthreads();
+  float2* p = base;
+  for (int l = 0; l < last; ++l) {                     // 1/d in natural order
+    const int m = L.m[l], W = m + 2, A = ringed(m);
+    for (int row = r0; row < m * m; row += RS) {
+      const int iz = row / m, iy = row - iz * m, o = (iy + iz + 1) & 1, i = ((iz + 1) * W + iy + 1) * W + 2 * j + 1;
+      const long long s = (long long)row * L.HP[l] + j;
+      if (2 * j + o < m) p[2 * A + i + o] = L.dr[l][s];
+      if (2 * j + 1 - o < m) p[2 * A + i + 1 - o] = L.db[l][s];
+    }
+    p += 3 * A;
+  }
+  pdl_prologue();
+  pdl_trigger();
+  {
+    const int m = L.m[0], W = m + 2, A = ringed(m);
+    for (int row = r0; row < m * m; row += RS) {
+      const int iz = row / m, iy = row - iz * m, o = (iy + iz + 1) & 1, i = ((iz + 1) * W + iy + 1) * W + 2 * j + 1;
+      const long long s = (long long)row * L.HP[0] + j;
+      if (2 * j + o < m) {
+        base[i + o] = ur[s];
+        base[A + i + o] = br[s];
+      }
+      if (2 * j + 1 - o < m) base[A + i + 1 - o] = bb[s];
+    }
+  }
+  __syncthreads();
+  auto nbr = [](const float2* u, int W) {
+    const int W2 = W * W;
+    return cadd(cadd(cadd(u[-1], u[1]), cadd(u[-W], u[W])), cadd(u[-W2], u[W2]));
+  };
+  p = base;
+  for (int l = 0; l < last; ++l) {
+    const int m = L.m[l], W = m + 2, A = ringed(m), mc = L.m[l + 1], Wc = mc + 2, Ac = ringed(mc);
+    float2 *U = p, *B = p + A, *D = p + 2 * A, *next = p + 3 * A;
+    const float2 c = L.c[l], d0 = L.d0[l];
+    for (int row = r0; row < m * m; row += RS) {       // black
+      const int iz = row / m, iy = row - iz * m, x = 2 * j + ((iy + iz) & 1);
+      const int i = ((iz + 1) * W + iy + 1) * W + x + 1;
+      if (x < m) U[i] = dinv_mul(d0, D[i], cfma(B[i], c, nbr(U + i, W)));
+    }
+    __syncthreads();
+    for (int q = t; q < mc * mc * mc; q += BLOCK_NT) { // full weighting of the red residuals
+      const int Z = q / (mc * mc), Y = q / mc - Z * mc, X = q - (Z * mc + Y) * mc, W2 = W * W;
+      const float2* u = U + ((2 * Z + 2) * W + 2 * Y + 2) * W + 2 * X + 2;
+      auto pair = [&](int a) { return cadd(u[-a], u[a]); };
+      const float2 f = cadd(cadd(pair(1), pair(W)), pair(W2));
+      const float2 g = cadd(cadd(pair(1 + W + W2), pair(1 + W - W2)), cadd(pair(1 - W + W2), pair(1 - W - W2)));
+      auto edge = [&](int a, int b) { return cadd(cadd(pair(2 * a + b), pair(2 * a - b)), cadd(pair(a + 2 * b), pair(a - 2 * b))); };
+      const float2 h = cadd(cadd(edge(1, W), edge(1, W2)), edge(W, W2));
+      const float2 v = cmul(c, cadd(cadd(cscale(f, 0.25f), cscale(g, 0.09375f)), cscale(h, 0.03125f)));
+      if (l + 1 < last) {
+        const int s = ((Z + 1) * Wc + Y + 1) * Wc + X + 1;
+        next[Ac + s] = v;
+        if ((X + Y + Z) & 1) next[s] = dinv_mul(L.d0[l + 1], next[2 * Ac + s], v);
+      } else {
+        Bc[q] = mk<cx<TI>>((TI)v.x, (TI)v.y);
+      }
+    }
+    __syncthreads();
+    p = next;
+  }
+  {                                                    // coarsest: inv b, 16 lanes a row
+    const int ml = L.m[last], n = ml * ml * ml, i = t >> 4, part = t & 15;
+    TI re = (TI)0, im = (TI)0;
+    if (i < n)
+      for (int k = part; k < n; k += 16) {
+        const cx<TI> a = inv[i * n + k], b = Bc[k];
+        re = fma(a.x, b.x, fma(-a.y, b.y, re));
+        im = fma(a.x, b.y, fma(a.y, b.x, im));
+      }
+#pragma unroll
+    for (int o = 1; o < 16; o <<= 1) {
+      re += __shfl_xor_sync(0xffffffffu, re, o);
+      im += __shfl_xor_sync(0xffffffffu, im, o);
+    }
+    if (i < n && part == 0) {
+      const int z = i / (ml * ml), y = i / ml - z * ml, x = i - (z * ml + y) * ml;
+      p[((z + 1) * (ml + 2) + y + 1) * (ml + 2) + x + 1] = make_float2((float)re, (float)im);
+    }
+    __syncthreads();
+  }
+  const float2* E = p;
+  for (int l = last - 1; l >= 0; --l) {
+    const int m = L.m[l], W = m + 2, A = ringed(m), Wc = L.m[l + 1] + 2;
+    p -= 3 * A;
+    float2 *U = p, *B = p + A, *D = p + 2 * A;
+    const float2 c = L.c[l], d0 = L.d0[l];
+    for (int row = r0; row < m * m; row += RS) {       // red, with the correction's neighbour sum
+      const int iz = row / m, iy = row - iz * m, x = 2 * j + ((iy + iz + 1) & 1);
+      const int i = ((iz + 1) * W + iy + 1) * W + x + 1;
+      if (x < m)
+        U[i] = dinv_mul(d0, D[i], cfma(B[i], c, cadd(nbr(U + i, W), prolong_nbr_ringed(E, Wc, x + 1, iy + 1, iz + 1))));
+    }
+    __syncthreads();
+    for (int row = r0; row < m * m; row += RS) {       // black; the top level's correction goes out
+      const int iz = row / m, iy = row - iz * m, o = (iy + iz) & 1, x = 2 * j + o;
+      const int i = ((iz + 1) * W + iy + 1) * W + x + 1;
+      float2* out = e_out + ((long long)(iz + 1) * W + iy + 1) * pe + 2 * j + 2;
+      if (x < m) {
+        const float2 v = dinv_mul(d0, D[i], cfma(B[i], c, nbr(U + i, W)));
+        if (l > 0) U[i] = v;
+        else out[o] = v;
+      }
+      if (l == 0 && 2 * j + 1 - o < m) out[1 - o] = U[i + 1 - 2 * o];
+    }
+    __syncthreads();
+    E = U;
+  }
+}
+
+size_t block_bytes(const std::vector<Level>& lv, int lb) {
+  size_t n = ringed(lv.back().m);
+  for (size_t l = lb; l + 1 < lv.size(); ++l) n += 3 * (size_t)ringed(lv[l].m);
+  return n * sizeof(float2);
 }
 
 struct Shape { dim3 g, b; };
@@ -380,14 +548,53 @@ cudaError_t split3_coefs(Level& L, double k2, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+// the line lies at 15 points a side, where a level's passes last one CTA's
+// lifetime each and its grids fit the block; the coarsest product has 16 lanes
+// a row
+int split3_block_level(const std::vector<Level>& lv) {
+  const int nl = (int)lv.size();
+  if (lv.back().N > BLOCK_LAST) return 0;
+  for (int l = 1; l + 1 < nl; ++l)
+    if (lv[l].m <= BLOCK_M) return nl - l <= BLOCK_LEVELS ? l : 0;
+  return 0;
+}
+cudaError_t prepare_split3_block() {
+  const int bytes = 160 * 1024;
+  cudaError_t e = cudaFuncSetAttribute(k3s_block<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  return e != cudaSuccess ? e : cudaFuncSetAttribute(k3s_block<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+}
+cudaError_t launch_split3_block(std::vector<Level>& lv, int lb, const float2* inv, const double2* inv64, cudaStream_t s) {
+  BlockLevels L{};
+  L.nl = (int)lv.size() - lb;
+  for (int i = 0; i < L.nl; ++i) {
+    const Level& v = lv[lb + i];
+    L.m[i] = v.m;
+    L.HP[i] = split3_pitch(v.m);
+    L.dr[i] = v.s32.dr;
+    L.db[i] = v.s32.db;
+    L.c[i] = make_float2((float)v.c.x, (float)v.c.y);
+    L.d0[i] = v.s32.d0;
+  }
+  const Split3<float>& F = lv[lb].s32;
+  const size_t sm = block_bytes(lv, lb);
+  const int pe = split3_ring_pitch(lv[lb].m);
+  ProfScope ps(mg_family<float>(), s, 2.0 * sizeof(float2) * lv[lb].N, 0);
+  const float2 *br = F.br, *bb = F.bb, *ur = F.ur;
+  const cudaError_t e = inv64 ? launch_pdl(k3s_block<double>, dim3(1), dim3(BLOCK_NT), sm, s, L, br, bb, ur, inv64, F.e, pe)
+                              : launch_pdl(k3s_block<float>, dim3(1), dim3(BLOCK_NT), sm, s, L, br, bb, ur, inv, F.e, pe);
+  count_launch();
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+
 template <typename T>
-cudaError_t launch_split3_down(std::vector<Level>& lv, const cx<T>* u, const cx<T>* b, bool zero_init, cudaStream_t s) {
+cudaError_t launch_split3_down(std::vector<Level>& lv, int stop, const cx<T>* u, const cx<T>* b, bool zero_init,
+                               cudaStream_t s) {
   cudaError_t e = cudaSuccess;
   int launches = 0;
   auto ok = [&](cudaError_t r) { ++launches; if (e == cudaSuccess) e = r; };
   const int nl = (int)lv.size();
   const double S = sizeof(cx<T>);
-  for (int l = 0; l + 1 < nl && e == cudaSuccess; ++l) {
+  for (int l = 0; l < stop && e == cudaSuccess; ++l) {
     Level &L = lv[l], &C = lv[l + 1];
     Split3<T>&F = sp<T>(L), &G = sp<T>(C);
     const int m = L.m, HP = split3_pitch(m), HPc = split3_pitch(C.m);
@@ -422,13 +629,12 @@ cudaError_t launch_split3_down(std::vector<Level>& lv, const cx<T>* u, const cx<
 }
 
 template <typename T>
-cudaError_t launch_split3_up(std::vector<Level>& lv, cx<T>* u_nat, cudaStream_t s) {
+cudaError_t launch_split3_up(std::vector<Level>& lv, int stop, cx<T>* u_nat, cudaStream_t s) {
   cudaError_t e = cudaSuccess;
   int launches = 0;
   auto ok = [&](cudaError_t r) { ++launches; if (e == cudaSuccess) e = r; };
-  const int nl = (int)lv.size();
   const double S = sizeof(cx<T>);
-  for (int l = nl - 2; l >= 0 && e == cudaSuccess; --l) {
+  for (int l = stop - 1; l >= 0 && e == cudaSuccess; --l) {
     Level &L = lv[l], &C = lv[l + 1];
     Split3<T>&F = sp<T>(L), &G = sp<T>(C);
     const int m = L.m, HP = split3_pitch(m);
@@ -455,8 +661,8 @@ cudaError_t launch_split3_up(std::vector<Level>& lv, cx<T>* u_nat, cudaStream_t 
 
 #define CSFF_SPLIT3_INST(T)                                                                                      \
   template cudaError_t split3_coefs<T>(Level&, double, cudaStream_t);                                                 \
-  template cudaError_t launch_split3_down<T>(std::vector<Level>&, const cx<T>*, const cx<T>*, bool, cudaStream_t); \
-  template cudaError_t launch_split3_up<T>(std::vector<Level>&, cx<T>*, cudaStream_t);
+  template cudaError_t launch_split3_down<T>(std::vector<Level>&, int, const cx<T>*, const cx<T>*, bool, cudaStream_t); \
+  template cudaError_t launch_split3_up<T>(std::vector<Level>&, int, cx<T>*, cudaStream_t);
 CSFF_SPLIT3_INST(float)
 CSFF_SPLIT3_INST(double)
 
