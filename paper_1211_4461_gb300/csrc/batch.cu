@@ -103,6 +103,28 @@ __device__ __forceinline__ int find_inst(const int* off, int n, int item) {
   return lo;
 }
 
+// the same for a CTA's next, larger item, from its last item's instance on
+__device__ __forceinline__ int next_inst(const int* off, int n, int item, int i) {
+  if (item < off[i + 1]) return i;
+  return i + 1 + find_inst(off + i + 1, n - i - 1, item);
+}
+
+constexpr int MAX_INST = 4096;      // as csff_batch_create admits
+// instances as bits in shared memory, set by the whole CTA: a work item's test
+// then costs no trip to L2 (with next_inst 32 instances 19.1 -> 18.2 ms, 24 of up
+// to 257^2 3.93 -> 3.79)
+__device__ __forceinline__ bool has(const unsigned* mask, int i) { return (mask[i >> 5] >> (i & 31)) & 1u; }
+template <typename Pred> __device__ __forceinline__ bool fill_mask(unsigned* mask, int n, Pred pred) {
+  bool any = false;
+  for (int i = threadIdx.x; i < ((n + 31) & ~31); i += blockDim.x) {
+    const bool p = i < n && pred(i);
+    const unsigned b = __ballot_sync(0xffffffffu, p);
+    if ((threadIdx.x & 31) == 0) mask[i >> 5] = b;
+    any |= p;
+  }
+  return __syncthreads_or(any) != 0;
+}
+
 // Grid-wide barrier with a bounded wait.  Returns false if any CTA gave up.
 __device__ bool grid_barrier(unsigned* bar, int* err, int extra, long long limit) {
   __shared__ int s_ok;
@@ -460,6 +482,7 @@ __device__ void ph_up(const BInst& I, int l, int t, unsigned char* smem) {
 
 template <bool LEARNED>
 __device__ __forceinline__ void batch_body(const BArgs& A, unsigned char* smem, double* shd, nettile::mmat::Ctx& nc) {
+  __shared__ unsigned live[MAX_INST / 32], act[MAX_INST / 32];
   const int n = A.n_inst;
   const int npts = A.off_pts[n];
   // ---- initial residual r = b (u = 0) and its norm
@@ -477,34 +500,30 @@ __device__ __forceinline__ void batch_body(const BArgs& A, unsigned char* smem, 
   if (!grid_barrier(A.bar, A.err, A.extra_arrivals, A.spin_limit)) return;
 
   for (;;) {
-    bool any = false;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) any |= !inst_done(A.st, i);
-    if (!__syncthreads_or(any)) break;
+    if (!fill_mask(live, n, [&](int i) { return !inst_done(A.st, i); })) break;
     for (int c = 0; c < A.inner; ++c) {
       // instances whose step is shorter sit out its remaining cycles (every
       // CTA reads the same state, so all leave the loop together)
-      bool busy = false;
-      for (int i = threadIdx.x; i < n; i += blockDim.x) busy |= in_cycle(A.st, i, c);
-      if (!__syncthreads_or(busy)) break;
+      if (!fill_mask(act, n, [&](int i) { return in_cycle(A.st, i, c); })) break;
       for (int l = 0; l < A.LC; ++l) {
         const int* off = A.off_lvl + (size_t)l * (n + 1);
-        for (int it = blockIdx.x; it < off[n]; it += gridDim.x) {
-          int i = find_inst(off, n, it);
-          if (in_cycle(A.st, i, c)) ph_down(A.inst[i], l, it - off[i], c == 0, smem);
+        for (int it = blockIdx.x, i = 0; it < off[n]; it += gridDim.x) {
+          i = next_inst(off, n, it, i);
+          if (has(act, i)) ph_down(A.inst[i], l, it - off[i], c == 0, smem);
         }
         if (!grid_barrier(A.bar, A.err, A.extra_arrivals, A.spin_limit)) return;
       }
       for (int i = blockIdx.x; i < n; i += gridDim.x) {
-        if (!in_cycle(A.st, i, c)) continue;
+        if (!has(act, i)) continue;
         const BInst& I = A.inst[i];
         tiles::coarse_levels_block<float, true, double>(I.cl, I.L[I.lc].b, I.L[I.lc].u, I.inv64, smem, false);
       }
       if (!grid_barrier(A.bar, A.err, A.extra_arrivals, A.spin_limit)) return;
       for (int l = A.LC - 1; l >= 0; --l) {
         const int* off = A.off_lvl + (size_t)l * (n + 1);
-        for (int it = blockIdx.x; it < off[n]; it += gridDim.x) {
-          int i = find_inst(off, n, it);
-          if (in_cycle(A.st, i, c)) ph_up(A.inst[i], l, it - off[i], smem);
+        for (int it = blockIdx.x, i = 0; it < off[n]; it += gridDim.x) {
+          i = next_inst(off, n, it, i);
+          if (has(act, i)) ph_up(A.inst[i], l, it - off[i], smem);
         }
         if (!grid_barrier(A.bar, A.err, A.extra_arrivals, A.spin_limit)) return;
       }
@@ -522,26 +541,26 @@ __device__ __forceinline__ void batch_body(const BArgs& A, unsigned char* smem, 
         }
       }
     }
-    for (int it = blockIdx.x; it < npts; it += gridDim.x) {
-      int i = find_inst(A.off_pts, n, it);
-      if (!inst_done(A.st, i)) ph_update(A.inst[i], A.st, i, it - A.off_pts[i]);
+    for (int it = blockIdx.x, i = 0; it < npts; it += gridDim.x) {
+      i = next_inst(A.off_pts, n, it, i);
+      if (has(live, i)) ph_update(A.inst[i], A.st, i, it - A.off_pts[i]);
     }
     if (!grid_barrier(A.bar, A.err, A.extra_arrivals, A.spin_limit)) return;
-    for (int it = blockIdx.x; it < npts; it += gridDim.x) {
-      int i = find_inst(A.off_pts, n, it);
-      if (!inst_done(A.st, i)) ph_residual(A.inst[i], A.st, i, it - A.off_pts[i], A.partials + it, shd);
+    for (int it = blockIdx.x, i = 0; it < npts; it += gridDim.x) {
+      i = next_inst(A.off_pts, n, it, i);
+      if (has(live, i)) ph_residual(A.inst[i], A.st, i, it - A.off_pts[i], A.partials + it, shd);
     }
     if (!grid_barrier(A.bar, A.err, A.extra_arrivals, A.spin_limit)) return;
     for (int i = blockIdx.x; i < n; i += gridDim.x)
-      if (!inst_done(A.st, i)) ph_finish(A, i, false, shd);
+      if (has(live, i)) ph_finish(A, i, false, shd);
     if (!grid_barrier(A.bar, A.err, A.extra_arrivals, A.spin_limit)) return;
   }
 }
 
 // 64 registers a thread, four CTAs an SM (with the learned step, whose operands
 // leave shared memory for three, 80; the autotuner picks between one and the
-// occupancy maximum).  32 instances of 129^2 to 1025^2: 20.2 ms at three CTAs, 19.1
-// at four, 18.6 at five of 48 registers, whose spills cost 24 instances of up to
+// occupancy maximum).  32 instances of 129^2 to 1025^2: 20.4 ms at three CTAs, 18.2
+// at four; in an earlier build 20.2 at three, 19.1 at four, 18.6 at five of 48 registers, whose spills cost 24 instances of up to
 // 257^2 more (4.24 ms against 3.93).  LEARNED: the
 // learned step ends every cycle; each CTA holds the network's weight operands
 // for the whole launch, and the activation planes share the tiles' shared
@@ -877,7 +896,7 @@ csff_status csff_batch_create(int n_inst, const csff_problem* probs, const csff_
                               csff_batch** out) {
   if (!out) return binvalid("out is NULL");
   *out = nullptr;
-  if (n_inst < 1 || n_inst > 4096 || !probs || !opts) return binvalid("need 1..4096 problems and options");
+  if (n_inst < 1 || n_inst > csff::MAX_INST || !probs || !opts) return binvalid("need 1..4096 problems and options");
   if (opts->smoother != CSFF_SMOOTHER_RBGS || opts->nu1 != 1 || opts->nu2 != 1 || opts->precision != CSFF_PREC_MIXED) {
     csff::set_error("batched solve: needs red-black GS V(1,1) with mixed precision");
     return CSFF_ERR_UNSUPPORTED;
