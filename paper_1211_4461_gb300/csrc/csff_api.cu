@@ -632,8 +632,8 @@ csff_status solve_mixed(csff_plan* P, int eb, double nb, csff_info* info, const 
   // 2^-eb u (guess or zero).  FP64: u in L.u64, its residual and norm.
   cudaStream_t s = P->stream;
   if (r64) {
-    // the first right-hand side of the FP32 cycles: 2^-eb r for the guess, or
-    // 2^-eb b from zero
+    // the first right-hand side of the FP32 cycles: 2^-eb r for the guess (from
+    // zero it is 2^-eb b, which came with the norm)
     P->refine_eb = eb;
     if (guess) {
       CK(cudaMemcpyAsync(L.u64, guess, sizeof(double2) * (size_t)L.N, cudaMemcpyDeviceToDevice, s), "copy guess");
@@ -641,7 +641,6 @@ csff_status solve_mixed(csff_plan* P, int eb, double nb, csff_info* info, const 
          "residual");
     } else {
       CK(csff::launch_zero<double>(L.u64, L.N, s), "zero");
-      CK(csff::launch_scale_to32(L.b64, L.N, eb, L.b32, s), "scale b");
     }
   } else if (guess) {
     CK(csff::launch_df_split(guess, L.N, -eb, P->dfu, nullptr, nullptr, nullptr, s), "split u");
@@ -1066,21 +1065,27 @@ csff_status csff_plan_describe(const csff_plan* P, csff_plan_desc* d) {
   return CSFF_OK;
 }
 
-csff_status csff_rhs(csff_plan* P, int n_rhs, const double* eta, void* b_dev) {
-  if (!P || !eta || !b_dev || n_rhs < 0) return invalid("bad rhs arguments");
+// one right-hand side; emax: where its exponent goes, or null
+static csff_status rhs_into(csff_plan* P, const double* eta, double2* b, int* emax) {
   Level& L = P->lv[0];
   std::vector<const double2*> per_g(P->prob.n_gauss);
   for (int g = 0; g < P->prob.n_gauss; ++g) per_g[g] = P->chi_tab[0] + (size_t)g * P->dim * L.m;
-  for (int r = 0; r < n_rhs; ++r) {
-    CS(upload_uinc(P, eta + (size_t)r * P->dim));
-    CK(csff::launch_rhs(P->dim, L.m, per_g.data(), P->prob.n_gauss, P->uinc_tab, P->prob.k * P->prob.k,
-                        (double2*)b_dev + (size_t)r * L.N, P->stream),
-       "rhs");
-  }
+  CS(upload_uinc(P, eta));
+  CK(csff::launch_rhs(P->dim, L.m, per_g.data(), P->prob.n_gauss, P->uinc_tab, P->prob.k * P->prob.k, b, P->stream, emax),
+     "rhs");
   return CSFF_OK;
 }
 
-static csff_status solve_loaded(csff_plan* P, double2* u, int use_guess, csff_info* in);
+csff_status csff_rhs(csff_plan* P, int n_rhs, const double* eta, void* b_dev) {
+  if (!P || !eta || !b_dev || n_rhs < 0) return invalid("bad rhs arguments");
+  for (int r = 0; r < n_rhs; ++r)
+    CS(rhs_into(P, eta + (size_t)r * P->dim, (double2*)b_dev + (size_t)r * P->lv[0].N, nullptr));
+  return CSFF_OK;
+}
+
+// where the exponent of max |b| goes
+static int* rhs_exp(csff_plan* P) { return reinterpret_cast<int*>(P->red_out + 4); }
+static csff_status solve_loaded(csff_plan* P, double2* u, int use_guess, csff_info* in, bool have_exp = false);
 
 csff_status csff_solve(csff_plan* P, int n_rhs, const double* eta, void* u_dev, int use_guess, csff_info* info) {
   if (!P || !eta || !u_dev || n_rhs < 0) return invalid("bad solve arguments");
@@ -1089,8 +1094,8 @@ csff_status csff_solve(csff_plan* P, int n_rhs, const double* eta, void* u_dev, 
   for (int r = 0; r < n_rhs; ++r) {
     double2* u = (double2*)u_dev + (size_t)r * L.N;
     csff_info* in = info ? info + r : nullptr;
-    CS(csff_rhs(P, 1, eta + (size_t)r * P->dim, L.b64));
-    const csff_status st = solve_loaded(P, u, use_guess, in);
+    CS(rhs_into(P, eta + (size_t)r * P->dim, L.b64, rhs_exp(P)));
+    const csff_status st = solve_loaded(P, u, use_guess, in, true);
     if (st == CSFF_ERR_CUDA || st == CSFF_ERR_OOM || st == CSFF_ERR_INVALID_ARG) return st;
     worst = worse(worst, st);
   }
@@ -1161,16 +1166,16 @@ static csff_status fmg_loaded(csff_plan* P, double2* u_out, int* level_cycles, c
   return result;
 }
 
-static csff_status solve_loaded(csff_plan* P, double2* u, int use_guess, csff_info* in) {
+static csff_status solve_loaded(csff_plan* P, double2* u, int use_guess, csff_info* in, bool have_exp) {
   Level& L = P->lv[0];
-  if (!use_guess) CK(csff::launch_zero<double>(u, L.N, P->stream), "zero");
   // ||b|| with a power-of-two prescale taken from max |b|
-  int* ex = reinterpret_cast<int*>(P->red_out + 4);
-  CK(csff::launch_max_exp(L.b64, L.N, ex, P->stream), "max exponent");
+  int* ex = rhs_exp(P);
+  if (!have_exp) CK(csff::launch_max_exp(L.b64, L.N, ex, P->stream), "max exponent");
   int eb = 0;
   CK(cudaMemcpyAsync(&eb, ex, sizeof(int), cudaMemcpyDeviceToHost, P->stream), "read exponent");
   CK(cudaStreamSynchronize(P->stream), "sync");
   if (eb >= 4000) {
+    if (!use_guess) CK(csff::launch_zero<double>(u, L.N, P->stream), "zero");
     csff::set_error("right-hand side is not finite");
     if (in) { std::memset(in, 0, sizeof(*in)); in->status = CSFF_ERR_NONFINITE; }
     return CSFF_ERR_NONFINITE;
@@ -1178,7 +1183,10 @@ static csff_status solve_loaded(csff_plan* P, double2* u, int use_guess, csff_in
   if (eb <= -2000) eb = 0;
   const bool fp64 = P->opts.precision == CSFF_PREC_FP64;
   const bool df = !fp64 && P->opts.refine_fp64 == 0;
-  if (!df) {
+  if (!df && !fp64 && !use_guess) {
+    // with it the first right-hand side of the FP32 cycles, 2^-eb b
+    CK(csff::launch_first_residual(L.b64, L.N, eb, L.b32, P->red, P->red_blocks, P->red_out + 1, P->stream), "norm b");
+  } else if (!df) {
     CS(norm64(P, L.b64, eb, 1));
   } else {
     // the mixed solve's operands: q (once per coefficient set) and b' = 2^-eb b as

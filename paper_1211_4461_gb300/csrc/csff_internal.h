@@ -284,8 +284,9 @@ cudaError_t launch_norm2(const cx<T>* v, long long N, int exp_scale, double* par
 cudaError_t launch_max_exp(const double2* v, long long N, int* out, cudaStream_t s);
 cudaError_t launch_coefs(int dim, const Level& L, const double2* const* chi_tab, int n_gauss,
                          double k2, cudaStream_t s);
+// emax: also the exponent of max |b| (as launch_max_exp)
 cudaError_t launch_rhs(int dim, int m, const double2* const* chi_tab, int n_gauss,
-                       const double2* uinc_tab, double k2, double2* b, cudaStream_t s);
+                       const double2* uinc_tab, double k2, double2* b, cudaStream_t s, int* emax = nullptr);
 template <typename T>
 cudaError_t launch_zero(cx<T>* v, long long N, cudaStream_t s);
 
@@ -324,7 +325,9 @@ cudaError_t launch_update64(double2* u, const float2* e, long long N, const int*
 cudaError_t launch_refine_residual(int dim, const Level& L, const double2* u, const double2* b, int s_exp,
                                    float2* r32, double* partial, int nblk, double* out, cudaStream_t s);
 cudaError_t launch_update64_fixed(double2* u, const float2* e, long long N, int s_exp, cudaStream_t s);
-cudaError_t launch_scale_to32(const double2* v, long long N, int s_exp, float2* r32, cudaStream_t s);
+// ||b|| into *out and the first FP32 right-hand side 2^-s_exp b of a solve from zero
+cudaError_t launch_first_residual(const double2* b, long long N, int s_exp, float2* r32, double* partial, int nblk,
+                                  double* out, cudaStream_t s);
 
 // ---- 3D V(1,1) cycles on colour-split arrays (mg_split3.cu) ----------------------
 int split3_pitch(int m);                       // slots of a row of one colour

@@ -292,8 +292,29 @@ __global__ void k_norm_partial(const cx<T>* __restrict__ v, long long N, double 
   double acc = 0;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N;
        i += (long long)gridDim.x * blockDim.x) {
-    double a = (double)v[i].x * scale, b = (double)v[i].y * scale;
+    double a = (double)v[i].x, b = (double)v[i].y;
+    if (scale != 1.0) {
+      a *= scale;
+      b *= scale;
+    }
     acc = fma(a, a, fma(b, b, acc));
+  }
+  acc = block_reduce(acc, AddOp(), sh, 0.0);
+  if (threadIdx.x == 0) partial[blockIdx.x] = acc;
+}
+
+// the same for a solve's right-hand side, with its rounding r32 = 2^-s v to FP32,
+// the first right-hand side of the cycles from zero
+__global__ void k_first_residual(const double2* __restrict__ v, int N, double scale, int s, float2* __restrict__ r32,
+                                 double* __restrict__ partial) {
+  pdl_prologue();
+  __shared__ double sh[32];
+  double acc = 0;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
+    double2 x = v[i];
+    r32[i] = make_float2(bits::narrow(x.x, s), bits::narrow(x.y, s));
+    if (scale != 1.0) x = cscale(x, scale);
+    acc = fma(x.x, x.x, fma(x.y, x.y, acc));
   }
   acc = block_reduce(acc, AddOp(), sh, 0.0);
   if (threadIdx.x == 0) partial[blockIdx.x] = acc;
@@ -333,23 +354,22 @@ __global__ void __launch_bounds__(RED_THREADS) k_resid_norm(const double2* __res
   if (threadIdx.x == 0) partial[blockIdx.x] = acc;
 }
 
+// frexp's exponent of max(|re|, |im|) from the IEEE fields: -2000 for zero, 4000
+// when a component is not finite
+__device__ __forceinline__ int max_exp(double2 x) {
+  const int Ex = bits::exp_field(x.x), Ey = bits::exp_field(x.y);
+  if (Ex == 0x7ff || Ey == 0x7ff) return 4000;
+  const bool nzx = ((unsigned long long)__double_as_longlong(x.x) & bits::ABS_MASK) != 0;
+  const bool nzy = ((unsigned long long)__double_as_longlong(x.y) & bits::ABS_MASK) != 0;
+  return max(nzx ? bits::frexp_exp(x.x) : -2000, nzy ? bits::frexp_exp(x.y) : -2000);
+}
+
 __global__ void k_max_exp(const double2* __restrict__ v, long long N, int* __restrict__ out) {
   __shared__ int sh[32];
   int mx = -2000;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N;
        i += (long long)gridDim.x * blockDim.x) {
-    // frexp's exponent of max(|re|, |im|) from the IEEE fields: -2000 for zero,
-    // 4000 when a component is not finite
-    const double2 x = v[i];
-    const int Ex = bits::exp_field(x.x), Ey = bits::exp_field(x.y);
-    int e;
-    if (Ex == 0x7ff || Ey == 0x7ff) e = 4000;
-    else {
-      const bool nzx = ((unsigned long long)__double_as_longlong(x.x) & bits::ABS_MASK) != 0;
-      const bool nzy = ((unsigned long long)__double_as_longlong(x.y) & bits::ABS_MASK) != 0;
-      e = max(nzx ? bits::frexp_exp(x.x) : -2000, nzy ? bits::frexp_exp(x.y) : -2000);
-    }
-    mx = e > mx ? e : mx;
+    mx = max(mx, max_exp(v[i]));
   }
   mx = block_reduce(mx, MaxIOp(), sh, -2000);
   if (threadIdx.x == 0) atomicMax(out, mx);
@@ -415,7 +435,7 @@ __global__ void k_coefs_from_q(const double2* __restrict__ q64, int m, double2 c
 
 template <int D>
 __global__ void k_rhs(TabPtrs tabs, int n_gauss, const double2* __restrict__ uinc, int m, double k2,
-                      double2* __restrict__ b) {
+                      double2* __restrict__ b, int* __restrict__ emax) {
   // chi u_in = sum_g prod_c (E_{g,c} U_c): each axis' Gaussian factor is paired
   // with its incident-wave factor first, so no partial product leaves the
   // FP64 range when chi u_in itself does not.  The pairs for the block's 32
@@ -445,10 +465,16 @@ __global__ void k_rhs(TabPtrs tabs, int n_gauss, const double2* __restrict__ uin
   }
   __syncthreads();
   int ix, iy, iz; long long idx;
-  if (!thread_point<D>(m, ix, iy, iz, idx)) return;
+  const bool in = thread_point<D>(m, ix, iy, iz, idx);
   double2 acc = n_gauss > 0 ? cmul(px[0][threadIdx.x], py[0][threadIdx.y]) : make_double2(0, 0);
   for (int g = 1; g < n_gauss; ++g) acc = cadd(acc, cmul(px[g][threadIdx.x], py[g][threadIdx.y]));
-  b[idx] = acc;
+  if (in) b[idx] = acc;
+  // a solve's exponent of max |b|, while the values are at hand (a pass of its
+  // own reads b again: 70 us at 257^3)
+  if (emax) {
+    const int e = __reduce_max_sync(0xffffffffu, in ? max_exp(acc) : -2000);
+    if ((t & 31) == 0 && e > *(volatile int*)emax) atomicMax(emax, e);
+  }
 }
 
 // ---- FP64 refinement of the mixed solve (option refine_fp64) -------------------
@@ -549,15 +575,6 @@ __global__ void k_update64_fixed(double2* __restrict__ u, const float2* __restri
       v.y = fma((double)c.y, p2, v.y);
     }
     u[i] = v;
-  }
-}
-
-// r32 = 2^-s v rounded to FP32 (the first right-hand side of a solve from zero)
-__global__ void k_scale_to32(const double2* __restrict__ v, int N, int s, float2* __restrict__ r32) {
-  pdl_prologue();
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
-    const double2 x = v[i];
-    r32[i] = make_float2(bits::narrow(x.x, s), bits::narrow(x.y, s));
   }
 }
 
@@ -709,6 +726,7 @@ cudaError_t launch_norm2(const cx<T>* v, long long N, int exp_scale, double* par
                          double* out, cudaStream_t s) {
   long long need = (N + RED_THREADS - 1) / RED_THREADS;
   int nb = (int)(need < nblk ? (need < 1 ? 1 : need) : nblk);
+  if (abs(exp_scale) <= 400) exp_scale = 0;      // squares stay inside the FP64 range
   ProfScope ps(mg_family<T>(), s, (double)sizeof(cx<T>) * N, 0);
   cudaError_t e = launch_pdl(k_norm_partial<T>, dim3(nb), dim3(RED_THREADS), 0, s, v, N, ldexp(1.0, -exp_scale),
                              partial);
@@ -740,12 +758,16 @@ cudaError_t launch_coefs(int dim, const Level& L, const double2* const* chi_tab,
 }
 
 cudaError_t launch_rhs(int dim, int m, const double2* const* chi_tab, int n_gauss,
-                       const double2* uinc_tab, double k2, double2* b, cudaStream_t s) {
+                       const double2* uinc_tab, double k2, double2* b, cudaStream_t s, int* emax) {
   TabPtrs t{};
   for (int i = 0; i < n_gauss; ++i) t.p[i] = chi_tab[i];
   dim3 g = grid_of(dim, m), blk(BX, BY);
-  if (dim == 2) k_rhs<2><<<g, blk, 0, s>>>(t, n_gauss, uinc_tab, m, k2, b);
-  else k_rhs<3><<<g, blk, 0, s>>>(t, n_gauss, uinc_tab, m, k2, b);
+  if (emax) {
+    k_set_int<<<1, 1, 0, s>>>(emax, -2000);
+    count_launch();
+  }
+  if (dim == 2) k_rhs<2><<<g, blk, 0, s>>>(t, n_gauss, uinc_tab, m, k2, b, emax);
+  else k_rhs<3><<<g, blk, 0, s>>>(t, n_gauss, uinc_tab, m, k2, b, emax);
   count_launch();
   return cudaGetLastError();
 }
@@ -788,12 +810,18 @@ cudaError_t launch_update64_fixed(double2* u, const float2* e, long long N, int 
   return err != cudaSuccess ? err : cudaGetLastError();
 }
 
-cudaError_t launch_scale_to32(const double2* v, long long N, int s_exp, float2* r32, cudaStream_t s) {
+cudaError_t launch_first_residual(const double2* b, long long N, int s_exp, float2* r32, double* partial, int nblk,
+                                  double* out, cudaStream_t s) {
   if (N >= (1ll << 31)) return cudaErrorInvalidValue;
+  const long long need = (N + RED_THREADS - 1) / RED_THREADS;
+  const int nb = (int)(need < nblk ? (need < 1 ? 1 : need) : nblk), ex = abs(s_exp) <= 400 ? 0 : s_exp;
   ProfScope ps(PF_MG64, s, 24.0 * N, 0);
-  cudaError_t err = launch_pdl(k_scale_to32, dim3(flat_blocks(N)), dim3(256), 0, s, v, (int)N, s_exp, r32);
-  count_launch();
-  return err != cudaSuccess ? err : cudaGetLastError();
+  cudaError_t e = launch_pdl(k_first_residual, dim3(nb), dim3(RED_THREADS), 0, s, b, (int)N, ldexp(1.0, -ex), s_exp, r32,
+                             partial);
+  if (e == cudaSuccess)
+    e = launch_pdl(k_norm_finish, dim3(1), dim3(RED_THREADS), 0, s, (const double*)partial, nb, ldexp(1.0, ex), out);
+  count_launch(2);
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 cudaError_t launch_update64(double2* u, const float2* e, long long N, const int* exp_in,
