@@ -60,9 +60,8 @@ DF_INSTR_PER_FLOP = 36.0 / 8.0
 DF_PEAK_TFLOPS = FP32_INSTR_PER_S / DF_INSTR_PER_FLOP / 1e12
 # DRAM bytes (read + write) per launch of the dominant kernels, from one ncu
 # capture of the current kernels on this workload (None when no capture of
-# the current kernels exists): the double-float far-field contraction and the
-# fused FP32 V(1,1) tiles (all levels, and those of the 1025^2 level).
-FF_DF_DRAM_BYTES = 10.67e6
+# the current kernels exists): the fused FP32 V(1,1) tiles (all levels, and those
+# of the 1025^2 level).
 TILES_DRAM_BYTES = 0.223e6
 TILES_FINE_DRAM_BYTES = 0.771e6
 

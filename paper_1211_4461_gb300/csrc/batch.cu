@@ -58,8 +58,8 @@ struct BInst {
   const double2* q64;
   double2 *u64, *b64;
   const double2* chi;               // [n_gauss][2][m]
-  const double2* uinc;              // [2][m]
-  double k2;
+  double2* uinc;                    // [2][m], from the solve's direction
+  double k2, k, lo, h, cg, sg;
   float h2;                         // h^2 of the finest level (the learned step's input scale)
 };
 
@@ -576,6 +576,16 @@ __global__ void __launch_bounds__(256, LEARNED ? 3 : 4) k_batch_solve(BArgs A) {
   batch_body<LEARNED>(A, smem, shd, nc);
 }
 
+// incident-wave tables of every instance for its direction (eta: [instance][2])
+__global__ void k_batch_incident(const BInst* __restrict__ inst, const double* __restrict__ eta) {
+  const BInst& I = inst[blockIdx.z];
+  const int c = blockIdx.y;
+  const double ke = __dmul_rn(I.k, eta[2 * blockIdx.z + c]);
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < I.m; i += gridDim.x * blockDim.x)
+    I.uinc[(long long)c * I.m + i] =
+        incident(__dmul_rn(ke, __dadd_rn(I.lo, __dmul_rn((double)(i + 1), I.h))), I.cg, I.sg);
+}
+
 __global__ void k_batch_init(BState* st, int n, unsigned* bar, int* err) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i == 0) { bar[0] = 0; bar[1] = 0; *err = 0; }
@@ -618,7 +628,7 @@ struct csff_batch {
   double* d_partials = nullptr;
   unsigned* d_bar = nullptr;
   int* d_err = nullptr;
-  double2* h_uinc = nullptr;      // pinned staging of incident tables
+  double *h_eta = nullptr, *d_eta = nullptr;     // directions: pinned staging, device
   int h_err = 0;
   int* h_err_p = nullptr;         // pinned error word mirror
   cudaStream_t gstream = nullptr; // capture/replay stream
@@ -708,6 +718,11 @@ csff_status upload_descriptors(csff_batch* B) {
     I.chi = P->chi_tab[0];
     I.uinc = P->uinc_tab;
     I.k2 = P->prob.k * P->prob.k;
+    I.k = P->prob.k;
+    I.lo = P->prob.box_lo;
+    I.h = P->lv[0].h;
+    I.cg = std::cos(P->prob.gamma);
+    I.sg = std::sin(P->prob.gamma);
     I.h2 = (float)(P->lv[0].h * P->lv[0].h);
     off_pts[i + 1] = off_pts[i] + csff::point_tiles(I.m);
     off_net[i + 1] = off_net[i] + ((I.m + csff::nettile::TW - 1) / csff::nettile::TW) *
@@ -772,34 +787,15 @@ csff_status launch_batch(csff_batch* B, cudaStream_t s) {
   return CSFF_OK;
 }
 
-// incident-wave tables of every instance into the pinned staging buffer
-void fill_incident(csff_batch* B, const double* eta) {
-  size_t off = 0;
-  for (int i = 0; i < B->n; ++i) {
-    csff_plan* P = B->plans[i];
-    const int m = P->lv[0].m;
-    const std::complex<double> ik(0.0, P->prob.k), rot = std::polar(1.0, P->prob.gamma);
-    for (int c = 0; c < 2; ++c)
-      for (int j = 0; j < m; ++j) {
-        double x = P->prob.box_lo + (j + 1) * P->lv[0].h;
-        std::complex<double> v = std::exp(ik * eta[2 * i + c] * x * rot);
-        B->h_uinc[off + (size_t)c * m + j] = make_double2(v.real(), v.imag());
-      }
-    off += 2 * (size_t)m;
-  }
-}
-
-// the device work of one batched solve: staged uploads, state init, the
+// the device work of one batched solve: directions and incident tables (by the
+// host 3 ms of a 32-instance solve), state init, the
 // persistent kernel, state readback (capturable: pinned buffers only)
 csff_status enqueue_solve(csff_batch* B, cudaStream_t s) {
-  size_t off = 0;
-  for (int i = 0; i < B->n; ++i) {
-    csff_plan* P = B->plans[i];
-    const int m = P->lv[0].m;
-    BK(cudaMemcpyAsync(P->uinc_tab, B->h_uinc + off, sizeof(double2) * 2 * m, cudaMemcpyHostToDevice, s),
-       "upload incident tables");
-    off += 2 * (size_t)m;
-  }
+  int m = 0;
+  for (const csff_plan* P : B->plans) m = std::max(m, P->lv[0].m);
+  BK(cudaMemcpyAsync(B->d_eta, B->h_eta, sizeof(double) * 2 * B->n, cudaMemcpyHostToDevice, s), "upload directions");
+  csff::k_batch_incident<<<dim3((m + 127) / 128, 2, B->n), 128, 0, s>>>(B->d_inst, B->d_eta);
+  csff::count_launch();
   csff_status st = launch_batch(B, s);
   if (st != CSFF_OK) return st;
   BK(cudaMemcpyAsync(B->h_state, B->d_state, sizeof(BState) * B->n, cudaMemcpyDeviceToHost, s), "states");
@@ -881,10 +877,10 @@ void csff_batch_destroy(csff_batch* B) {
   if (!B) return;
   for (csff_plan* P : B->plans) csff_plan_destroy(P);
   for (void* p : {(void*)B->d_inst, (void*)B->d_state, (void*)B->d_off, (void*)B->d_partials, (void*)B->d_bar,
-                  (void*)B->d_err})
+                  (void*)B->d_err, (void*)B->d_eta})
     if (p) cudaFree(p);
   if (B->h_state) cudaFreeHost(B->h_state);
-  if (B->h_uinc) cudaFreeHost(B->h_uinc);
+  if (B->h_eta) cudaFreeHost(B->h_eta);
   if (B->h_err_p) cudaFreeHost(B->h_err_p);
   if (B->gexec) cudaGraphExecDestroy(B->gexec);
   if (B->gstream) cudaStreamDestroy(B->gstream);
@@ -909,7 +905,6 @@ csff_status csff_batch_create(int n_inst, const csff_problem* probs, const csff_
     csff_batch_destroy(B);
     return s;
   };
-  size_t uinc_total = 0;
   for (int i = 0; i < n_inst; ++i) {
     if (probs[i].dim != 2) return fail(binvalid("batched solve: 2D problems only"));
     csff_plan* P = nullptr;
@@ -920,7 +915,6 @@ csff_status csff_batch_create(int n_inst, const csff_problem* probs, const csff_
       csff::set_error("batched solve: each grid needs n >= 65 and at most 12 levels");
       return fail(CSFF_ERR_UNSUPPORTED);
     }
-    uinc_total += 2 * (size_t)P->lv[0].m;
   }
   cudaError_t e;
   if ((e = cudaMalloc((void**)&B->d_inst, sizeof(BInst) * n_inst)) != cudaSuccess ||
@@ -928,7 +922,8 @@ csff_status csff_batch_create(int n_inst, const csff_problem* probs, const csff_
       (e = cudaMalloc((void**)&B->d_bar, 2 * sizeof(unsigned))) != cudaSuccess ||
       (e = cudaMalloc((void**)&B->d_err, sizeof(int))) != cudaSuccess ||
       (e = cudaMallocHost((void**)&B->h_state, sizeof(BState) * n_inst)) != cudaSuccess ||
-      (e = cudaMallocHost((void**)&B->h_uinc, sizeof(double2) * uinc_total)) != cudaSuccess ||
+      (e = cudaMallocHost((void**)&B->h_eta, sizeof(double) * 2 * n_inst)) != cudaSuccess ||
+      (e = cudaMalloc((void**)&B->d_eta, sizeof(double) * 2 * n_inst)) != cudaSuccess ||
       (e = cudaMallocHost((void**)&B->h_err_p, sizeof(int))) != cudaSuccess ||
       (e = cudaStreamCreateWithFlags(&B->gstream, cudaStreamNonBlocking)) != cudaSuccess ||
       (e = cudaEventCreateWithFlags(&B->gev, cudaEventDisableTiming)) != cudaSuccess)
@@ -943,7 +938,7 @@ csff_status csff_batch_create(int n_inst, const csff_problem* probs, const csff_
 
 csff_status csff_batch_solve(csff_batch* B, const double* eta, csff_info* infos) {
   if (!B || !eta) return binvalid("NULL argument");
-  fill_incident(B, eta);
+  std::memcpy(B->h_eta, eta, sizeof(double) * 2 * B->n);
   csff_status s = run_solve(B);
   if (s != CSFF_OK) return s;
   int worst = CSFF_OK;
@@ -1042,7 +1037,7 @@ csff_status csff_batch_autotune(csff_batch* B, const double* eta, int* tc_big_ou
   BK(cudaEventCreate(&e1), "event");
   float best = 1e30f;
   int best_tc = B->tc_big, best_per = B->ctas_per_sm;
-  fill_incident(B, eta);
+  std::memcpy(B->h_eta, eta, sizeof(double) * 2 * B->n);
   if (B->gexec) { cudaGraphExecDestroy(B->gexec); B->gexec = nullptr; }
   csff_status s = CSFF_OK;
   for (int tc : {16, 8}) {

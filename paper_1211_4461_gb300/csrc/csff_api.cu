@@ -232,22 +232,6 @@ bool coarse_inverse(const csff_plan* P, const Level& L, std::vector<double2>& ou
   return true;
 }
 
-// Incident-wave tables U_c(i) = exp(i k eta_c x_i e^{i gamma}) on the finest grid.
-csff_status upload_uinc(csff_plan* P, const double* eta) {
-  const Level& L = P->lv[0];
-  const int d = P->dim, m = L.m;
-  std::vector<double2> ut((size_t)d * m);
-  const cd ik(0.0, P->prob.k), rot = std::polar(1.0, P->prob.gamma);
-  for (int c = 0; c < d; ++c)
-    for (int i = 0; i < m; ++i) {
-      double x = P->prob.box_lo + (i + 1) * L.h;
-      cd v = std::exp(ik * eta[c] * x * rot);
-      ut[(size_t)c * m + i] = make_double2(v.real(), v.imag());
-    }
-  CK(cudaMemcpyAsync(P->uinc_tab, ut.data(), sizeof(double2) * ut.size(), cudaMemcpyHostToDevice, P->stream),
-     "upload incident tables");
-  return CSFF_OK;
-}
 
 // ---- per-precision buffer access ------------------------------------------------
 template <typename T> cx<T>* ubuf(Level& L);
@@ -1070,7 +1054,8 @@ static csff_status rhs_into(csff_plan* P, const double* eta, double2* b, int* em
   Level& L = P->lv[0];
   std::vector<const double2*> per_g(P->prob.n_gauss);
   for (int g = 0; g < P->prob.n_gauss; ++g) per_g[g] = P->chi_tab[0] + (size_t)g * P->dim * L.m;
-  CS(upload_uinc(P, eta));
+  CK(csff::launch_incident(P->uinc_tab, P->dim, L.m, P->prob.box_lo, L.h, P->prob.k, P->prob.gamma, eta, P->stream),
+     "incident tables");
   CK(csff::launch_rhs(P->dim, L.m, per_g.data(), P->prob.n_gauss, P->uinc_tab, P->prob.k * P->prob.k, b, P->stream, emax),
      "rhs");
   return CSFF_OK;

@@ -284,6 +284,9 @@ cudaError_t launch_norm2(const cx<T>* v, long long N, int exp_scale, double* par
 cudaError_t launch_max_exp(const double2* v, long long N, int* out, cudaStream_t s);
 cudaError_t launch_coefs(int dim, const Level& L, const double2* const* chi_tab, int n_gauss,
                          double k2, cudaStream_t s);
+// incident-wave tables U_c[i] = exp(i k eta_c z_i) of the finest level, [dim][m]
+cudaError_t launch_incident(double2* tab, int dim, int m, double lo, double h, double k, double gamma, const double* eta,
+                            cudaStream_t s);
 // emax: also the exponent of max |b| (as launch_max_exp)
 cudaError_t launch_rhs(int dim, int m, const double2* const* chi_tab, int n_gauss,
                        const double2* uinc_tab, double k2, double2* b, cudaStream_t s, int* emax = nullptr);

@@ -121,4 +121,19 @@ __device__ __forceinline__ double widen_near(float f, int e) {
 }
 
 }  // namespace bits
+
+// exp(i t e^{i gamma}), t = k eta x, (cg, sg) = (cos, sin) gamma: one factor of the
+// incident wave.  The magnitude is applied in halves where it alone may leave the
+// FP64 range.
+__device__ __forceinline__ double2 incident(double t, double cg, double sg) {
+  const double a = __dmul_rn(-sg, t);
+  double sn, cs;
+  sincos(__dmul_rn(cg, t), &sn, &cs);
+  if (fabs(a) > 700.0) {
+    const double h = exp(0.5 * a);
+    return make_double2((h * cs) * h, (h * sn) * h);
+  }
+  const double e = exp(a);
+  return make_double2(e * cs, e * sn);
+}
 }  // namespace csff

@@ -1699,21 +1699,8 @@ csff_status far_field_one(csff_plan* P, const double* eta_host, const double2* u
   if (!B.dmisc) {
     if ((e = cudaMalloc((void**)&B.dmisc, 4 * sizeof(int))) != cudaSuccess) return cuda_fail(e, "malloc");
   }
-  // incident-wave tables for eta: U_c[i] = exp(i k eta_c z_i)
-  {
-    std::vector<double2> ut((size_t)d * m);
-    const double cg = std::cos(P->prob.gamma), sg = std::sin(P->prob.gamma);
-    for (int c = 0; c < d; ++c)
-      for (int i = 0; i < m; ++i) {
-        double x = P->prob.box_lo + (double)(i + 1) * L.h;
-        double t = P->prob.k * eta_host[c] * x;   // i k eta_c x e^{i g} = -k sg t + i k cg t
-        double mag = std::exp(-sg * t);
-        ut[(size_t)c * m + i] = make_double2(mag * std::cos(cg * t), mag * std::sin(cg * t));
-      }
-    if ((e = cudaMemcpyAsync(P->uinc_tab, ut.data(), sizeof(double2) * ut.size(), cudaMemcpyHostToDevice, s)) !=
-        cudaSuccess)
-      return cuda_fail(e, "upload incident tables");
-  }
+  if ((e = launch_incident(P->uinc_tab, d, m, P->prob.box_lo, L.h, P->prob.k, P->prob.gamma, eta_host, s)) != cudaSuccess)
+    return cuda_fail(e, "incident tables");
   if ((e = cudaMemcpyAsync(B.dal, alpha_host, sizeof(double) * (size_t)n_ang * d, cudaMemcpyHostToDevice, s)) !=
           cudaSuccess ||
       (e = cudaMemcpyAsync(B.dux, ux.data(), sizeof(double) * n_ux, cudaMemcpyHostToDevice, s)) != cudaSuccess ||

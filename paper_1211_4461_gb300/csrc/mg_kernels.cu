@@ -433,6 +433,18 @@ __global__ void k_coefs_from_q(const double2* __restrict__ q64, int m, double2 c
   dinv32[idx] = make_float2((float)di.x, (float)di.y);
 }
 
+// The incident wave's tables, on the device: the 2 x 1023 exponentials of a
+// 1025^2 map took the host longer than a V-cycle takes the GPU, before the first
+// kernel of a solve and again of a far field.
+__global__ void k_incident(double2* __restrict__ tab, int m, double lo, double h, double k, double eta0, double eta1,
+                           double eta2, double cg, double sg) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x, c = blockIdx.y;
+  if (i >= m) return;
+  const double eta = c == 0 ? eta0 : c == 1 ? eta1 : eta2;
+  const double x = __dadd_rn(lo, __dmul_rn((double)(i + 1), h));
+  tab[(long long)c * m + i] = incident(__dmul_rn(__dmul_rn(k, eta), x), cg, sg);
+}
+
 template <int D>
 __global__ void k_rhs(TabPtrs tabs, int n_gauss, const double2* __restrict__ uinc, int m, double k2,
                       double2* __restrict__ b, int* __restrict__ emax) {
@@ -753,6 +765,14 @@ cudaError_t launch_coefs(int dim, const Level& L, const double2* const* chi_tab,
     k_coefs<2><<<g, blk, 0, s>>>(t, n_gauss, L.m, k2, L.c, L.q64, L.dinv64, L.q32, L.dinv32);
   else
     k_coefs<3><<<g, blk, 0, s>>>(t, n_gauss, L.m, k2, L.c, L.q64, L.dinv64, L.q32, L.dinv32);
+  count_launch();
+  return cudaGetLastError();
+}
+
+cudaError_t launch_incident(double2* tab, int dim, int m, double lo, double h, double k, double gamma, const double* eta,
+                            cudaStream_t s) {
+  k_incident<<<dim3((m + 127) / 128, dim), 128, 0, s>>>(tab, m, lo, h, k, eta[0], eta[1], dim == 3 ? eta[2] : 0.0,
+                                                        cos(gamma), sin(gamma));
   count_launch();
   return cudaGetLastError();
 }

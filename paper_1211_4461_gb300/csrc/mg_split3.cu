@@ -27,10 +27,11 @@
 //    adds the interpolated correction's neighbour sum, formed from the coarse
 //    values directly;
 //  - the last black half sweep writes both colours in natural order.
-// 257^3 FP32 cycle through the public call (natural order in and out): 411 us,
-// 670 with interleaved colours; a half sweep of 255^3 48 us, 80 before (copy
-// rate: 39), the 38-point full weighting 39 us, residual and full weighting
-// 123 before, the prolonging half sweep 74, both passes 125 before.
+// 257^3 FP32 cycle through the public call (natural order in and out): 362 us,
+// 670 with interleaved colours.  A half sweep of 255^3 39 us (the copy rate), 53
+// with the black change, 61 prolonging, 59 into natural order (80 before, 125 with
+// the prolongation's pass); the 38-point full weighting 32 us, residual and full
+// weighting 123 before.
 #include "csff_internal.h"
 
 namespace csff {
@@ -358,7 +359,9 @@ __global__ void k3s_restrict(const cx<T>* __restrict__ delta, int m, int HP, cx<
 // order with a ring of zeros (u, b, 1/d of the smoothing levels; 137 KB from 17^3
 // down).  A row of a colour takes eight lanes; phases as above.  17^3, 9^3 and 5^3:
 // 20.9 us alone, where the ten passes took 42 one by one; in the dependent
-// launches of a cycle 4 us of that difference are left (257^3 cycle 367 -> 363).
+// launches of a cycle 4 us of that difference are left (257^3 cycle 367 -> 363;
+// with the early triggers and the full weighting's loads 129^3 89.5 -> 75.9, 33^3
+// 33.3 -> 27.2).
 constexpr int BLOCK_M = 15, BLOCK_NT = 1024, BLOCK_LEVELS = 6, BLOCK_LAST = 64;
 struct BlockLevels {
   int nl, m[BLOCK_LEVELS], HP[BLOCK_LEVELS];            // the last is the coarsest
