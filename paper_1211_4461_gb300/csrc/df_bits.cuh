@@ -12,8 +12,8 @@
 //     range; |x 2^-e| < 2^-69 there and the pair stays within 2^-149 of it.
 //     Below -150 the pair is zero, as RN_24 gives;
 //   - the exact widening of an FP32 value to FP64, times a power of two.
-// Zero, subnormal and non-finite FP64 inputs, and scaled exponents above 100,
-// take the FP64 conversions instead.
+// In the splits zero, subnormal and non-finite FP64 inputs, and scaled exponents
+// above 100, take the FP64 conversions instead.
 #pragma once
 
 namespace csff {
@@ -27,13 +27,12 @@ __device__ __forceinline__ int exp_field(double x) {
   return (int)(((unsigned long long)__double_as_longlong(x) >> 52) & 0x7ff);
 }
 
-// e with |x| = f 2^e, f in [1/2, 1) (frexp's exponent); x finite and nonzero
+// e with |x| = f 2^e, f in [1/2, 1) (frexp's exponent); x finite and nonzero.
+// Integer operations only, for subnormal values too.
 __device__ __forceinline__ int frexp_exp(double x) {
-  const int E = exp_field(x);
-  if (E != 0) return E - 1022;
-  int e;
-  frexp(x, &e);                 // subnormal
-  return e;
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int E = (int)((b >> 52) & 0x7ff);
+  return E != 0 ? E - 1022 : -1010 - __clzll((long long)(b & MANT_MASK));
 }
 
 // (hi, lo) with hi = RN_24(x 2^-e), lo = RN_24(x 2^-e - hi)

@@ -451,42 +451,50 @@ __global__ void k_rhs(TabPtrs tabs, int n_gauss, const double2* __restrict__ uin
   // chi u_in = sum_g prod_c (E_{g,c} U_c): each axis' Gaussian factor is paired
   // with its incident-wave factor first, so no partial product leaves the
   // FP64 range when chi u_in itself does not.  The pairs for the block's 32
-  // columns, 8 rows (and plane) are formed once per block, and so are the
-  // row factors k^2 (E_y U_y)(E_z U_z): a node costs one complex product per
-  // Gaussian (this pass runs on the FP64 pipe, 1/61 of the FP32 rate here).
-  __shared__ double2 px[8][BX], py[8][BY], pz[8];
+  // columns and 8 rows are formed once per block (in 3D for its 8 planes), the row
+  // factors k^2 (E_y U_y)(E_z U_z) once per plane: a node costs one complex
+  // product per Gaussian (this pass runs on the FP64 pipe, 1/61 of the FP32 rate
+  // here).  257^3 with the exponent 238 us; one plane a block 290, or 213 and a pass of
+  // its own for the exponent, 70.
+  __shared__ double2 px[8][BX], py[8][BY], pyz[2][8][BY];
+  __shared__ int wmax;
   const int t = threadIdx.y * BX + threadIdx.x;
-  for (int i = t; i < n_gauss * (BX + BY + 1); i += BX * BY) {
-    const int g = i / (BX + BY + 1), r = i % (BX + BY + 1);
+  if (t == 0) wmax = -2000;
+  for (int i = t; i < n_gauss * (BX + BY); i += BX * BY) {
+    const int g = i / (BX + BY), r = i % (BX + BY);
     const double2* E = tabs.p[g];
     if (r < BX) {
       const int x = blockIdx.x * BX + r;
       px[g][r] = x < m ? cmul(E[x], uinc[x]) : make_double2(0, 0);
-    } else if (r < BX + BY) {
+    } else {
       const int y = blockIdx.y * BY + (r - BX);
       py[g][r - BX] = y < m ? cmul(E[m + y], uinc[m + y]) : make_double2(0, 0);
-    } else if (D == 3) {
-      pz[g] = cmul(E[2 * m + blockIdx.z], uinc[2 * m + blockIdx.z]);
     }
   }
   __syncthreads();
-  for (int i = t; i < n_gauss * BY; i += BX * BY) {
-    const int g = i / BY, r = i % BY;
-    const double2 v = (D == 3) ? cmul(py[g][r], pz[g]) : py[g][r];
-    py[g][r] = cscale(v, k2);
+  const int ix = blockIdx.x * BX + threadIdx.x, iy = blockIdx.y * BY + threadIdx.y;
+  const int z0 = (D == 3) ? 8 * (int)blockIdx.z : 0, z1 = (D == 3) ? min(z0 + 8, m) : 1;
+  int e = -2000;
+  for (int iz = z0; iz < z1; ++iz) {
+    const int buf = iz & 1;              // the other one may still be read
+    for (int i = t; i < n_gauss * BY; i += BX * BY) {
+      const int g = i / BY, r = i % BY;
+      const double2 v = (D == 3) ? cmul(py[g][r], cmul(tabs.p[g][2 * m + iz], uinc[2 * m + iz])) : py[g][r];
+      pyz[buf][g][r] = cscale(v, k2);
+    }
+    __syncthreads();
+    if (ix >= m || iy >= m) continue;
+    double2 acc = n_gauss > 0 ? cmul(px[0][threadIdx.x], pyz[buf][0][threadIdx.y]) : make_double2(0, 0);
+    for (int g = 1; g < n_gauss; ++g) acc = cadd(acc, cmul(px[g][threadIdx.x], pyz[buf][g][threadIdx.y]));
+    b[((long long)iz * m + iy) * m + ix] = acc;
+    // a solve's exponent of max |b|, while the values are at hand
+    if (emax) e = max(e, max_exp(acc));
   }
+  if (!emax) return;
+  e = __reduce_max_sync(0xffffffffu, e);
+  if ((t & 31) == 0) atomicMax(&wmax, e);
   __syncthreads();
-  int ix, iy, iz; long long idx;
-  const bool in = thread_point<D>(m, ix, iy, iz, idx);
-  double2 acc = n_gauss > 0 ? cmul(px[0][threadIdx.x], py[0][threadIdx.y]) : make_double2(0, 0);
-  for (int g = 1; g < n_gauss; ++g) acc = cadd(acc, cmul(px[g][threadIdx.x], py[g][threadIdx.y]));
-  if (in) b[idx] = acc;
-  // a solve's exponent of max |b|, while the values are at hand (a pass of its
-  // own reads b again: 70 us at 257^3)
-  if (emax) {
-    const int e = __reduce_max_sync(0xffffffffu, in ? max_exp(acc) : -2000);
-    if ((t & 31) == 0 && e > *(volatile int*)emax) atomicMax(emax, e);
-  }
+  if (t == 0 && wmax > *(volatile int*)emax) atomicMax(emax, wmax);
 }
 
 // ---- FP64 refinement of the mixed solve (option refine_fp64) -------------------
@@ -781,7 +789,7 @@ cudaError_t launch_rhs(int dim, int m, const double2* const* chi_tab, int n_gaus
                        const double2* uinc_tab, double k2, double2* b, cudaStream_t s, int* emax) {
   TabPtrs t{};
   for (int i = 0; i < n_gauss; ++i) t.p[i] = chi_tab[i];
-  dim3 g = grid_of(dim, m), blk(BX, BY);
+  dim3 g((m + BX - 1) / BX, (m + BY - 1) / BY, dim == 3 ? (m + 7) / 8 : 1), blk(BX, BY);
   if (emax) {
     k_set_int<<<1, 1, 0, s>>>(emax, -2000);
     count_launch();
