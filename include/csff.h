@@ -239,6 +239,14 @@ csff_status csff_plan_set_far_field_mode(csff_plan* plan, int mode);
    Synchronises the plan's stream.  Errors: CSFF_ERR_INVALID_ARG, CSFF_ERR_CUDA. */
 csff_status csff_far_field_work(csff_plan* plan, double* executed);
 
+/* Test hook for the bounded waits of the tensor-core digit contraction:
+   extra_arrivals = 1 makes the next far fields' contraction wait for an arrival
+   that never comes, so its waits run out after wait_ms milliseconds (0 = the
+   default limit of 500); 0 restores normal runs.  *gave_up (host, may be NULL)
+   receives 1 if a wait of the plan's last far field ran out, else 0, which
+   synchronises the plan's stream.  Errors: CSFF_ERR_INVALID_ARG, CSFF_ERR_CUDA. */
+csff_status csff_far_field_debug_waits(csff_plan* plan, int extra_arrivals, int wait_ms, int* gave_up);
+
 /* ---- user coefficients and right-hand sides (Sec. 5.2-5.3) ---------------
    The partial-wave Schroedinger problem (-1/2 Delta + V - E) u = phi along the
    rotated contour is, times 2, the plan's operator A u = c (2d u - sum_nbr u)

@@ -139,6 +139,7 @@ _SIGS = {
     "csff_prof_end": (_i, [C.POINTER(ProfStatsC)]),
     "csff_plan_set_potential": (_i, [_vp, _vp]),
     "csff_far_field_work": (_i, [_vp, _dp]),
+    "csff_far_field_debug_waits": (_i, [_vp, _i, _i, C.POINTER(_i)]),
     "csff_solve_rhs": (_i, [_vp, _vp, _vp, _i, C.POINTER(InfoC)]),
     "csff_plan_set_schroedinger": (_i, [_vp, _d, _vp]),
     "csff_solve_schroedinger": (_i, [_vp, _vp, _vp, _i, C.POINTER(InfoC)]),
@@ -605,6 +606,15 @@ class Plan:
         out = C.c_double()
         _check(_lib.csff_far_field_work(self._h, C.byref(out)), "far_field_work")
         return out.value
+
+    def debug_far_field_waits(self, extra_arrivals, wait_ms=0) -> bool:
+        """Test hook of the digit contraction's bounded waits
+        (csff_far_field_debug_waits); returns whether a wait of the last far
+        field ran out."""
+        out = _i()
+        _check(_lib.csff_far_field_debug_waits(self._h, int(extra_arrivals), int(wait_ms), C.byref(out)),
+               "far_field_debug_waits")
+        return bool(out.value)
 
     def set_potential(self, q):
         """q: complex128 CUDA tensor of m^d samples of q (csff_plan_set_potential)."""

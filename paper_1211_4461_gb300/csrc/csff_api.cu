@@ -1315,6 +1315,13 @@ csff_status csff_far_field_work(csff_plan* P, double* executed) {
   return csff::far_field_executed(P, executed);
 }
 
+csff_status csff_far_field_debug_waits(csff_plan* P, int extra_arrivals, int wait_ms, int* gave_up) {
+  if (!P || extra_arrivals < 0 || extra_arrivals > 1 || wait_ms < 0) return invalid("bad debug settings");
+  P->ff.waits.extra = extra_arrivals;
+  P->ff.waits.ns = wait_ms > 0 ? 1000000ull * (unsigned long long)wait_ms : csff::FF_WAIT_NS;
+  return gave_up ? csff::far_field_gave_up(P, gave_up) : CSFF_OK;
+}
+
 csff_status csff_plan_set_far_field_mode(csff_plan* P, int mode) {
   if (!P || (mode != CSFF_FF_FP64 && mode != CSFF_FF_TC_BF16X4)) return invalid("bad far-field mode");
   P->ff_mode = mode;

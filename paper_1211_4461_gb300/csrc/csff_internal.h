@@ -104,6 +104,15 @@ struct Level {
   Split3<double> s64;
 };
 
+// Waits of the digit contraction (ff_digits.cuh): a wait gives up after ns; a free
+// set of accumulators asks for extra arrivals beyond the epilogue's (0; with one
+// more than ever comes the waits run out, csff_far_field_debug_waits).
+constexpr unsigned long long FF_WAIT_NS = 500000000ull;
+struct FFWaits {
+  unsigned long long ns = FF_WAIT_NS;
+  int extra = 0;
+};
+
 // Far-field scratch (grown on demand): g = chi (u_in + u); x/y/z phase
 // tables; stage-1 sums T; angle data; per-row exponents; misc[0] = max
 // exponent of |g|, misc[1] = "a scale was applied" flag, misc[2] = a wait of
@@ -126,6 +135,7 @@ struct FFBuffers {
   // digit operands of the tensor-core contraction (ff_digits.cuh)
   size_t xdig = 0, gdig = 0;
   unsigned char *dxdig = nullptr, *dgdig = nullptr;
+  FFWaits waits;
   // tensor-core 3D stage A: pre-swizzled split phase operand, per-column and
   // per-row exponents, [spread_g, spread_P, error word]
   size_t tcb = 0, tce = 0;
@@ -393,6 +403,7 @@ int net_dim(const csff_net* N);                    // 2 or 3
 
 // ---- far field (farfield.cu) -----------------------------------------------
 void free_ff_buffers(csff_plan* P);
+csff_status far_field_gave_up(csff_plan* P, int* gave_up);
 csff_status far_field_executed(csff_plan* P, double* executed);
 csff_status far_field_one(csff_plan* P, const double* eta_host, const double2* u, int n_ang,
                           const double* alpha_host, double2* F, int32_t* F_exp, bool* scaled);

@@ -821,7 +821,7 @@ __global__ void __launch_bounds__(digits::NT, 1)
     k_ff_digits(const unsigned char* __restrict__ Ad, const unsigned char* __restrict__ Bd, const int* __restrict__ ex,
                 int M, const int* __restrict__ eg, int N, int nb, const int* __restrict__ spread,
                 const unsigned char* __restrict__ skip, int skip_tiles, double2* __restrict__ T, int* __restrict__ err,
-                int tile0, const int* __restrict__ field, const int* __restrict__ map) {
+                int tile0, const int* __restrict__ field, const int* __restrict__ map, FFWaits waits) {
   using namespace digits;
   constexpr int ND = F::ND, NA = F::NA, SUB = F::SUB, B_SET = F::B_SET, OFF_BAR = F::OFF_BAR, OFF_ACT = F::OFF_ACT;
   if (spread && !digits_selected(spread)) return;      // another kernel takes this launch
@@ -846,7 +846,7 @@ __global__ void __launch_bounds__(digits::NT, 1)
       bar_init(b_full + 8 * i, 1);
       bar_init(b_empty + 8 * i, 1);
       bar_init(acc_full + 8 * i, 1);
-      bar_init(acc_empty + 8 * i, EPI_WARPS);
+      bar_init(acc_empty + 8 * i, EPI_WARPS + waits.extra);
     }
     bar_init(fin, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -883,21 +883,24 @@ __global__ void __launch_bounds__(digits::NT, 1)
   if (warp == EPI_WARPS) {
     // uniform as the MMA warp: one elected lane issues the copies
     const int n = SUB * __reduce_max_sync(0xffffffffu, n_act);
-    int ia = 0, slot = 0;
+    int ia = 0, ib = 0, slot = 0;                      // A slots and B sets issued
     uint32_t eph = 1;                                  // parity of the slot's last release (first round: none awaited)
     bool ok = true;
     for (int idx = 0; idx < n; ++idx) {
       const int kb = idx / SUB, p = kb & 1, b = __reduce_max_sync(0xffffffffu, (int)act[kb]);
       const bool first = idx % SUB == 0;
-      if (first && kb >= 2) ok = bar_wait(b_empty + 8 * p, (uint32_t)((kb >> 1) - 1) & 1u, abort);
+      if (first && kb >= 2) ok = bar_wait(b_empty + 8 * p, (uint32_t)((kb >> 1) - 1) & 1u, abort, waits.ns);
       if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
       const unsigned char* src = Ad + (((long long)xt * nb + b) * SUB + idx % SUB) * (F::A_SLOTS * A_DIG);
-      if (first && elect_one())
-        bulk_load(sbase + NA * A_DIG + p * B_SET, Bd + ((long long)blockIdx.y * nb + b) * B_SET, B_SET, b_full + 8 * p);
+      if (first) {
+        if (elect_one())
+          bulk_load(sbase + NA * A_DIG + p * B_SET, Bd + ((long long)blockIdx.y * nb + b) * B_SET, B_SET, b_full + 8 * p);
+        ++ib;
+      }
       __syncwarp();
 #pragma unroll
       for (int s = 0; s < F::A_SLOTS; ++s) {
-        if (ia >= NA) ok = ok && bar_wait(a_empty + 8 * slot, eph, abort);
+        if (ia >= NA) ok = ok && bar_wait(a_empty + 8 * slot, eph, abort, waits.ns);
         if (__all_sync(0xffffffffu, ok)) {
           if (elect_one()) bulk_load(sbase + slot * A_DIG, src + s * A_DIG, A_DIG, a_full + 8 * slot);
           ++ia;
@@ -911,11 +914,11 @@ __global__ void __launch_bounds__(digits::NT, 1)
       if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
     }
     if (!ok) {
-      // the CTA gives up: its copies land before it ends
+      // the CTA gives up: its copies, the last of every slot and set, land before
+      // it ends
       int never = 0;
       for (int i = ia > NA ? ia - NA : 0; i < ia; ++i) bar_wait(a_full + 8 * (i % NA), (uint32_t)(i / NA) & 1u, &never);
-      bar_wait(b_full, 0, &never);
-      bar_wait(b_full + 8, 0, &never);
+      for (int i = ib > 2 ? ib - 2 : 0; i < ib; ++i) bar_wait(b_full + 8 * (i & 1), (uint32_t)(i >> 1) & 1u, &never);
     }
     __syncwarp();
   } else if (warp == EPI_WARPS + 1) {
@@ -932,14 +935,14 @@ __global__ void __launch_bounds__(digits::NT, 1)
     bool ok = true;
     for (int idx = 0; idx < n; ++idx) {
       const int p = idx & 1;
-      if (idx >= 2) ok = bar_wait(acc_empty + 8 * p, (uint32_t)((idx >> 1) - 1) & 1u, abort);
+      if (idx >= 2) ok = bar_wait(acc_empty + 8 * p, (uint32_t)((idx >> 1) - 1) & 1u, abort, waits.ns);
       const int kb = idx / SUB, pb = kb & 1;             // B's buffer
-      ok = ok && bar_wait(b_full + 8 * pb, (uint32_t)(kb >> 1) & 1u, abort);
+      ok = ok && bar_wait(b_full + 8 * pb, (uint32_t)(kb >> 1) & 1u, abort, waits.ns);
       if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
       const uint32_t sB = sbase + NA * A_DIG + pb * B_SET + (SUB - 1) * 64 * (idx & 1);
 #pragma unroll
       for (int s = 0; s < ND; ++s) {
-        if (s % SUB == 0) ok = ok && bar_wait(a_full + 8 * slot, aph, abort);
+        if (s % SUB == 0) ok = ok && bar_wait(a_full + 8 * slot, aph, abort, waits.ns);
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         constexpr int TKK = 2 * TK;
         const uint32_t nd = (uint32_t)(TKK * (ND - s));
@@ -1006,7 +1009,7 @@ __global__ void __launch_bounds__(digits::NT, 1)
       if (idx + 1 < n) scales(idx + 1);
       // one lane polls: the waits of 512 threads would crowd out the barrier
       // operations of the two threads that feed the tensor core
-      if (lane == 0) ok = bar_wait(acc_full + 8 * p, (uint32_t)(idx >> 1) & 1u, abort);
+      if (lane == 0) ok = bar_wait(acc_full + 8 * p, (uint32_t)(idx >> 1) & 1u, abort, waits.ns);
       ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
       if (!ok) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -1587,7 +1590,7 @@ static cudaError_t stage_a_digits(FFBuffers& B, const double2* zt, int T, const 
     const int n = std::min(chunk, tiles - t0);
     k_cut_field3<<<dim3(n, nb * F::SUB), TM, 0, s>>>(g, m, ncol, t0, eg, B.dgdig);
     k_ff_digits<F><<<dim3(n, kt), NT, F::SMEM, s>>>(B.dgdig, B.dxdig, ex, T, eg, (int)ncol, nb, nullptr, nullptr, 0, T1,
-                                                    B.dmisc + 2, t0, nullptr, nullptr);
+                                                    B.dmisc + 2, t0, nullptr, nullptr, B.waits);
     count_launch(2);
   }
   return cudaGetLastError();
@@ -1635,7 +1638,7 @@ static cudaError_t stage_b_digits(FFBuffers& B, const double2* yt, const YTiles&
   k_cut_phase3<<<(unsigned)(((long long)rows * nb * 32 + 255) / 256), 256, 0, s>>>(yt, map, m, rows, ex, B.dxdig);
   k_cut_field3<<<dim3(tiles, nbs, T), TM, 0, s>>>(T1, m, m, 0, eg, B.dgdig);
   k_ff_digits<F><<<dim3(tiles, kt), NT, F::SMEM, s>>>(B.dgdig, B.dxdig, ex, rows, eg, m, nb, nullptr, nullptr, 0, T2,
-                                                      B.dmisc + 2, 0, field, map);
+                                                      B.dmisc + 2, 0, field, map, B.waits);
   count_launch(3);
   return cudaGetLastError();
 }
@@ -1658,6 +1661,15 @@ csff_status far_field_executed(csff_plan* P, double* executed) {
   for (unsigned char c : h) run += c == 0;
   *executed = (double)run / (double)h.size();
   return CSFF_OK;
+}
+
+// whether a wait of the last far field's digit contraction ran out
+csff_status far_field_gave_up(csff_plan* P, int* gave_up) {
+  *gave_up = 0;
+  if (!P->ff.dmisc) return CSFF_OK;
+  cudaError_t e = cudaMemcpyAsync(gave_up, P->ff.dmisc + 2, sizeof(int), cudaMemcpyDeviceToHost, P->stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(P->stream);
+  return e == cudaSuccess ? CSFF_OK : cuda_fail(e, "far-field waits");
 }
 
 void free_ff_buffers(csff_plan* P) {
@@ -1945,7 +1957,7 @@ csff_status far_field_one(csff_plan* P, const double* eta_host, const double2* u
     if (dig) {
       k_ff_digits<digits::Form2><<<dim3(gxt, gkt), digits::NT, digits::Form2::SMEM, s>>>(
           B.dgdig, B.dxdig, B.dex, n_ux, B.deg, (int)R, nbk, B.dspread, B.dskip, (int)gdf.x, B.dT, B.dmisc + 2, 0,
-          nullptr, nullptr);
+          nullptr, nullptr, B.waits);
       count_launch();
     }
     k_ff_stage1_df<<<gdf, DF_NT, 0, s>>>(B.dxdf, B.dxsm, B.dex, n_ux, B.dgdf, B.dgsm, B.deg, (int)R, nbk, B.dspread,

@@ -51,7 +51,6 @@ constexpr int EPI_WARPS = 16, NT = 32 * (EPI_WARPS + 2);
 constexpr int EK = TK * 4 / EPI_WARPS;           // phase rows of an epilogue warp
 constexpr int TMEM_COLS = 512, ACC = 256;      // columns of one set of accumulators (7 x 32 used)
 constexpr int MARGIN = 12;
-constexpr unsigned long long WAIT_NS = 500000000ull;   // a wait gives up after half a second
 
 // A form of the contraction: ND digits a value, NA A slots in the ring, SUB
 // scale blocks in the 32 nodes of a row of B.
@@ -127,7 +126,8 @@ __device__ __forceinline__ void bar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 // bounded; gives up early when another thread of the CTA has
-__device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity, volatile int* abort) {
+__device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity, volatile int* abort,
+                                         unsigned long long limit = FF_WAIT_NS) {
   unsigned long long t0 = 0;
   for (int it = 0; it < (1 << 28); ++it) {
     uint32_t done;
@@ -142,7 +142,7 @@ __device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity, volatile
       unsigned long long t;
       asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
       if (t0 == 0) t0 = t;
-      else if (t - t0 > WAIT_NS) break;
+      else if (t - t0 > limit) break;
     }
   }
   *abort = 1;
