@@ -242,7 +242,8 @@ csff_status csff_far_field_work(csff_plan* plan, double* executed);
 /* Test hook for the bounded waits of the tensor-core digit contraction:
    extra_arrivals = 1 makes the next far fields' contraction wait for an arrival
    that never comes, so its waits run out after wait_ms milliseconds (0 = the
-   default limit of 500); 0 restores normal runs.  *gave_up (host, may be NULL)
+   default limit of 500) and the FP64 kernels form the map instead; 0 restores
+   normal runs.  *gave_up (host, may be NULL)
    receives 1 if a wait of the plan's last far field ran out, else 0, which
    synchronises the plan's stream.  Errors: CSFF_ERR_INVALID_ARG, CSFF_ERR_CUDA. */
 csff_status csff_far_field_debug_waits(csff_plan* plan, int extra_arrivals, int wait_ms, int* gave_up);

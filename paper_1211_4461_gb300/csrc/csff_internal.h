@@ -116,7 +116,7 @@ struct FFWaits {
 // Far-field scratch (grown on demand): g = chi (u_in + u); x/y/z phase
 // tables; stage-1 sums T; angle data; per-row exponents; misc[0] = max
 // exponent of |g|, misc[1] = "a scale was applied" flag, misc[2] = a wait of
-// the digit contraction ran out.
+// the digit contraction ran out (the FP64 kernels then run behind it).
 struct FFBuffers {
   size_t g = 0, xt = 0, yt = 0, zt = 0, T = 0, al = 0, ux = 0, xr = 0, s1 = 0;
   double2 *dg = nullptr, *dxt = nullptr, *dyt = nullptr, *dzt = nullptr, *dT = nullptr;

@@ -225,8 +225,10 @@ __device__ __forceinline__ bool digits_selected(const int* __restrict__ spread) 
 
 __global__ void __launch_bounds__(256) k_ff_stage1(const double2* __restrict__ X, int M,
                                                    const double2* __restrict__ G, int N, int K,
-                                                   double2* __restrict__ T, const int* __restrict__ skip_if_df) {
-  if (skip_if_df && (digits_selected(skip_if_df) || df_selected(skip_if_df))) return;   // another kernel ran
+                                                   double2* __restrict__ T, const int* __restrict__ skip_if_df,
+                                                   const int* __restrict__ gave_up) {
+  // another kernel ran, and no wait of the digit contraction ran out
+  if (*gave_up == 0 && (digits_selected(skip_if_df) || df_selected(skip_if_df))) return;
   __shared__ double2 As[S1_BK][S1_BM];
   __shared__ double2 Bs[S1_BK][S1_BN + 1];
   const int tid = threadIdx.x;
@@ -801,7 +803,9 @@ __global__ void __launch_bounds__(digits::TM) k_cut_field3(const double2* __rest
 // T[k][rho] from the digit operands (ff_digits.cuh): a tile of 128 rho x 16 k a
 // CTA, its kept blocks in order.  Warps 0-15 join the accumulators (TMEM lanes
 // 32 (w mod 4), phase rows [4 (w / 4), +4)), warp 16 loads, warp 17 issues MMAs.
-// A wait that runs out (none should) leaves NaN in the tile and sets *err.
+// A wait that runs out (none should; half a second, which a preempted CTA can
+// reach) leaves NaN in the tile and sets *err: the FP64 kernel launched behind,
+// which else returns at once, then forms T again.
 // Bound by the issue of the MMAs (114 clocks each where the tensor core needs
 // 64; 150 from one thread in a divergent branch) and by the last wave: 184 tiles
 // on 152 SMs at 1025^2.  361 phase rows x 1023 x 1023, every block kept: 125 us,
@@ -1068,7 +1072,7 @@ __global__ void __launch_bounds__(digits::NT, 1)
         }
       }
     }
-    if (!ok && lane == 0) atomicOr(err, 1);
+    if (!ok && lane == 0) atomicOr(err, 1);            // the FP64 kernel behind takes the launch over
     if (rho < N)
 #pragma unroll
       for (int j = 0; j < EK; ++j) {
@@ -1463,8 +1467,10 @@ __global__ void __launch_bounds__(tc::NTHR, 1)
 template <int TB>
 __global__ void __launch_bounds__(256) k_ff3_stageA(const double2* __restrict__ zt, int T, int t0,
                                                     const double2* __restrict__ g, int m, long long ncol,
-                                                    double2* __restrict__ T1, const int* __restrict__ skip_if_tc) {
+                                                    double2* __restrict__ T1, const int* __restrict__ skip_if_tc,
+                                                    const int* __restrict__ only_if) {
   if (skip_if_tc && tc_selected(skip_if_tc)) return;   // the tensor-core kernel wrote T1
+  if (only_if && *only_if == 0) return;                // the digit contraction did
   __shared__ double2 zs[TB][32];
   const long long col = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   double2 acc[TB];
@@ -1499,7 +1505,8 @@ __global__ void __launch_bounds__(256) k_ff3_stageA(const double2* __restrict__ 
 // stage B: T2[a][ix] = sum_iy Py[a][iy] T1[t(a)][iy m + ix]
 __global__ void __launch_bounds__(128) k_ff3_stageB(const double2* __restrict__ yt, const int* __restrict__ trow,
                                                     const double2* __restrict__ T1, int m,
-                                                    double2* __restrict__ T2) {
+                                                    double2* __restrict__ T2, const int* __restrict__ only_if) {
+  if (only_if && *only_if == 0) return;                // the digit contraction wrote T2
   extern __shared__ double2 ys[];
   const int a = blockIdx.y;
   for (int i = threadIdx.x; i < m; i += blockDim.x) ys[i] = yt[(long long)a * m + i];
@@ -1824,16 +1831,17 @@ csff_status far_field_one(csff_plan* P, const double* eta_host, const double2* u
                 B.dg, m, ncol, n_uz, t0, nkc, B.dtcb, B.dtce, erow, B.dtcflag, T1);
             for (int tb = t0; tb < std::min(n_uz, t0 + tc::TT); tb += 16)
               k_ff3_stageA<16><<<(unsigned)((ncol + 255) / 256), 256, 0, s>>>(B.dxt, n_uz, tb, B.dg, m, ncol, T1,
-                                                                              B.dtcflag);
+                                                                              B.dtcflag, nullptr);
             count_launch(3 + (std::min(n_uz, t0 + tc::TT) - t0 + 15) / 16);
           }
-        } else if (dig3) {
-          if ((e = stage_a_digits(B, B.dxt, n_uz, B.dg, m, chunk, T1, s)) != cudaSuccess)
-            return cuda_fail(e, "far field z contraction");
         } else {
+          if (dig3 && (e = stage_a_digits(B, B.dxt, n_uz, B.dg, m, chunk, T1, s)) != cudaSuccess)
+            return cuda_fail(e, "far field z contraction");
+          // in FP64: without the digits, and (else they return at once) where one of
+          // their waits ran out
           for (int t0 = 0; t0 < n_uz; t0 += 16)
             k_ff3_stageA<16><<<(unsigned)((ncol + 255) / 256), 256, 0, s>>>(B.dxt, n_uz, t0, B.dg, m, ncol, T1,
-                                                                            nullptr);
+                                                                            nullptr, dig3 ? B.dmisc + 2 : nullptr);
           count_launch((n_uz + 15) / 16);
         }
       }
@@ -1851,13 +1859,11 @@ csff_status far_field_one(csff_plan* P, const double* eta_host, const double2* u
                 dig3_ensure_b(B, yt, m, n_uz, P) == cudaSuccess;
         if (!dig3b) cudaGetLastError();
       }
-      if (dig3b) {
-        if ((e = stage_b_digits(B, B.dyt, yt, T1, n_uz, m, T2, s)) != cudaSuccess)
-          return cuda_fail(e, "far field y contraction");
-      } else {
-        k_ff3_stageB<<<dim3((m + 127) / 128, n_ang), 128, sizeof(double2) * m, s>>>(B.dyt, B.dxr, T1, m, T2);
-        count_launch();
-      }
+      if (dig3b && (e = stage_b_digits(B, B.dyt, yt, T1, n_uz, m, T2, s)) != cudaSuccess)
+        return cuda_fail(e, "far field y contraction");
+      k_ff3_stageB<<<dim3((m + 127) / 128, n_ang), 128, sizeof(double2) * m, s>>>(B.dyt, B.dxr, T1, m, T2,
+                                                                                  dig3b ? B.dmisc + 2 : nullptr);
+      count_launch();
       // stage C: F[a] = pref sum_ix Px[a][ix] T2[a][ix]  (the 2D stage-2 kernel on rows a)
       if ((e = cudaMemcpyAsync(B.dxr, ident.data(), sizeof(int) * n_ang, cudaMemcpyHostToDevice, s)) != cudaSuccess)
         return cuda_fail(e, "far field rows");
@@ -1879,15 +1885,11 @@ csff_status far_field_one(csff_plan* P, const double* eta_host, const double2* u
         }
       }
       if (scaled) {
-        int flag[2] = {0, 0};
-        if ((e = cudaMemcpyAsync(flag, B.dmisc + 1, sizeof(flag), cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
+        int flag = 0;
+        if ((e = cudaMemcpyAsync(&flag, B.dmisc + 1, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
             (e = cudaStreamSynchronize(s)) != cudaSuccess)
           return cuda_fail(e, "far field flag");
-        *scaled = flag[0] != 0;
-        if (flag[1]) {
-          set_error("far-field contraction: an mbarrier wait ran out");
-          return CSFF_ERR_TIMEOUT;
-        }
+        *scaled = flag != 0;
       }
       return CSFF_OK;
     }
@@ -1962,7 +1964,7 @@ csff_status far_field_one(csff_plan* P, const double* eta_host, const double2* u
     }
     k_ff_stage1_df<<<gdf, DF_NT, 0, s>>>(B.dxdf, B.dxsm, B.dex, n_ux, B.dgdf, B.dgsm, B.deg, (int)R, nbk, B.dspread,
                                          B.dskip, B.dT);
-    k_ff_stage1<<<g1, 256, 0, s>>>(B.dxt, n_ux, B.dg, (int)R, m, B.dT, B.dspread);
+    k_ff_stage1<<<g1, 256, 0, s>>>(B.dxt, n_ux, B.dg, (int)R, m, B.dT, B.dspread, B.dmisc + 2);
   }
   count_launch(2);
   const double hd = std::pow(L.h, d);
@@ -1977,15 +1979,11 @@ csff_status far_field_one(csff_plan* P, const double* eta_host, const double2* u
   count_launch();
   if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "far field kernels");
   if (scaled) {
-    int flag[2] = {0, 0};
-    if ((e = cudaMemcpyAsync(flag, B.dmisc + 1, sizeof(flag), cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
+    int flag = 0;
+    if ((e = cudaMemcpyAsync(&flag, B.dmisc + 1, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
         (e = cudaStreamSynchronize(s)) != cudaSuccess)
       return cuda_fail(e, "far field flag");
-    *scaled = flag[0] != 0;
-    if (flag[1]) {
-      set_error("far-field contraction: an mbarrier wait ran out");
-      return CSFF_ERR_TIMEOUT;
-    }
+    *scaled = flag != 0;
   }
   return CSFF_OK;
 }

@@ -63,3 +63,17 @@ def test_contraction_whose_waits_run_out_ends_and_leaves_the_next_call_whole(csf
     assert st == csff.OK and c.plan.debug_far_field_waits(0) is False
     c.check(got)
     c.plan.close()
+
+
+@pytest.mark.parametrize("with_exp", [True, False])
+@pytest.mark.parametrize("dim", [2, 3])
+def test_contraction_whose_waits_run_out_is_repeated_in_fp64(csff, dim, with_exp):
+    """The map of the call itself is right, with and without exponents: both
+    contractions of the 3D case (its angles share z components) give up."""
+    c = Case(csff, dim)
+    c.plan.debug_far_field_waits(1, wait_ms=20)
+    st, got = c.run(with_exp)
+    assert c.plan.debug_far_field_waits(0) is True
+    assert st == csff.OK
+    c.check(got)
+    c.plan.close()
