@@ -750,7 +750,7 @@ __global__ void k_cut_phase3(const double2* __restrict__ v, const int* __restric
   int e = scale_exp(x);
 #pragma unroll
   for (int o = 8; o > 0; o >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
-  if (row < nrows && (lane & 15) == 0) ev[((long long)row * nb + b) * F::SUB + (lane >> 4)] = e;
+  if (row < nrows && (lane & 15) == 0) ev[((long long)row * nb + b) * F::SUB + (lane >> 4)] = block_scale(e);
   uint32_t dig[F::ND];
   cut<F::ND>(fixed<F::BITS>(x.x, e), fixed<F::BITS>(x.y, e), dig);
   const int r = row % TK, o = (lane & 3) * 4;
@@ -780,7 +780,7 @@ __global__ void __launch_bounds__(digits::TM) k_cut_field3(const double2* __rest
 #pragma unroll
   for (int k = 0; k < 16; ++k)
     if (k < nz) e = max(e, scale_exp(p[(long long)k * ncol]));
-  eg[(xt * TM + r) * nbs + sb] = e;
+  eg[(xt * TM + r) * nbs + sb] = block_scale(e);
   unsigned char* tile = out + (xt * nbs + sb) * (F::A_SLOTS * A_DIG);
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
@@ -986,7 +986,8 @@ __global__ void __launch_bounds__(digits::NT, 1)
     const uint32_t tl = tmem + ((uint32_t)(32 * lg) << 16) + (uint32_t)kq;
     float2 H[2][2], L[2][2];                           // 2D: running double-float sums, exponents E
     int E[EK];
-    double S[2][EK];                                   // 3D: running sums
+    double S[2][EK];                                   // 3D: running sums; bit j of bad: NaN
+    unsigned bad = 0;
 #pragma unroll
     for (int j = 0; j < EK; ++j) S[0][j] = S[1][j] = 0.0;
 #pragma unroll
@@ -1009,7 +1010,10 @@ __global__ void __launch_bounds__(digits::NT, 1)
       const int p = idx & 1;
       int es[EK];
 #pragma unroll
-      for (int j = 0; j < EK; ++j) es[j] = eg1 + ex1[j];
+      for (int j = 0; j < EK; ++j) {
+        es[j] = eg1 + ex1[j];
+        if (SUB == 2 && es[j] > NONFINITE / 2) bad |= 1u << j;
+      }
       if (idx + 1 < n) scales(idx + 1);
       // one lane polls: the waits of 512 threads would crowd out the barrier
       // operations of the two threads that feed the tensor core
@@ -1081,7 +1085,7 @@ __global__ void __launch_bounds__(digits::NT, 1)
         const float hr = (j & 1) ? H[0][j >> 1].y : H[0][j >> 1].x, lr = (j & 1) ? L[0][j >> 1].y : L[0][j >> 1].x;
         const float hi = (j & 1) ? H[1][j >> 1].y : H[1][j >> 1].x, li = (j & 1) ? L[1][j >> 1].y : L[1][j >> 1].x;
         T[(long long)row * N + rho] =
-            !ok ? make_double2(__longlong_as_double(0x7ff8000000000000ll), __longlong_as_double(0x7ff8000000000000ll))
+            !ok || (bad >> j & 1u) ? make_double2(__longlong_as_double(0x7ff8000000000000ll), __longlong_as_double(0x7ff8000000000000ll))
                 : SUB == 2 ? make_double2(S[0][j], S[1][j])
                 : E[j] == -100000 ? make_double2(0.0, 0.0)
                                   : make_double2(bits::widen(hr, E[j]) + bits::widen(lr, E[j]),

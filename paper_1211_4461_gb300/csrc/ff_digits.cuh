@@ -84,8 +84,14 @@ template <int BITS> __device__ __forceinline__ long long fixed(double x, int e) 
   else q = (m + (1ll << (-sh - 1))) >> -sh;
   return E == 0x7ff ? 0 : (b >> 63) ? -q : q;
 }
-// e with |x| < 2^e from the exponent fields (zero and subnormal values: -1022)
+// e with |x| < 2^e from the exponent fields (zero and subnormal values: -1022;
+// infinities and NaN, whose digits are zero: 1025)
 __device__ __forceinline__ int scale_exp(double2 x) { return max(bits::exp_field(x.x), bits::exp_field(x.y)) - 1022; }
+
+// the scale of a block of the 3D form that holds an infinity or a NaN: what it
+// enters becomes NaN
+constexpr int NONFINITE = 1 << 24;
+__device__ __forceinline__ int block_scale(int e) { return e > 1024 ? NONFINITE : e; }
 
 // the digits of two fixed-point values as pairs of BF16 integers, dig[0] the
 // leading one.  Balanced digits are the bytes after adding 128 to every byte
