@@ -710,6 +710,19 @@ template <typename T> csff_status alloc_split3(csff_plan* P) {
   return CSFF_OK;
 }
 
+// the kernel's CTAs read b while others write u: b is copied first where the two
+// share memory (a solve in place)
+template <typename T> csff_status coarse_solve_any(csff_plan* P, const cx<T>* b, cx<T>* u, const cx<T>* inv) {
+  const uintptr_t pb = (uintptr_t)b, pu = (uintptr_t)u, bytes = sizeof(cx<T>) * (size_t)P->coarse_N;
+  if (pb < pu + bytes && pu < pb + bytes) {
+    cx<T>* t = tbuf<T>(P->lv.back());
+    CK(cudaMemcpyAsync(t, b, bytes, cudaMemcpyDeviceToDevice, P->stream), "copy rhs");
+    b = t;
+  }
+  CK(csff::launch_coarse_solve<T>(inv, P->coarse_N, b, u, P->stream), "coarse");
+  return CSFF_OK;
+}
+
 csff_status check_level(const csff_plan* P, int level, int arith) {
   if (!P) return invalid("plan is NULL");
   if (level < 0 || level >= (int)P->lv.size()) return invalid("level out of range");
@@ -1375,13 +1388,8 @@ csff_status csff_prolong_add(csff_plan* P, int level, int arith, const void* ec,
 csff_status csff_coarse_solve(csff_plan* P, int arith, const void* b, void* u) {
   CS(check_level(P, 0, arith));
   if (!b || !u) return invalid("NULL buffer");
-  if (arith == CSFF_ARITH_FP64)
-    CK(csff::launch_coarse_solve<double>(P->coarse_inv, P->coarse_N, (const double2*)b, (double2*)u, P->stream),
-       "coarse");
-  else
-    CK(csff::launch_coarse_solve<float>(P->coarse_inv32, P->coarse_N, (const float2*)b, (float2*)u, P->stream),
-       "coarse");
-  return CSFF_OK;
+  if (arith == CSFF_ARITH_FP64) return coarse_solve_any<double>(P, (const double2*)b, (double2*)u, P->coarse_inv);
+  return coarse_solve_any<float>(P, (const float2*)b, (float2*)u, P->coarse_inv32);
 }
 
 csff_status csff_norm2(csff_plan* P, int level, int arith, const void* v, double* out) {
