@@ -423,26 +423,19 @@ csff_status run_vcycle_learned(csff_plan* P, float2* u, const float2* b, bool ze
   return CSFF_OK;
 }
 
-template <typename T> csff::Split3<T>& split_of(Level& L);
-template <> csff::Split3<float>& split_of<float>(Level& L) { return L.s32; }
-template <> csff::Split3<double>& split_of<double>(Level& L) { return L.s64; }
-
-// The 3D V(1,1) RB-GS cycle on colour-split arrays.  first/last: of the cycles
-// run on one right-hand side (the iterate stays split in between).
-template <typename T>
-csff_status run_split3(csff_plan* P, cx<T>* u, const cx<T>* b, bool zero_init, bool first, bool last) {
-  const cx<T>* none = nullptr;
-  cx<T>* no = nullptr;
-  const int lb = sizeof(T) == 4 ? P->split_block : 0, stop = lb > 0 ? lb : (int)P->lv.size() - 1;
-  CK(csff::launch_split3_down<T>(P->lv, stop, first && !zero_init ? u : none, b, zero_init, P->stream), "split down");
+// The 3D FP32 V(1,1) RB-GS cycle on colour-split arrays.  first/last: of the
+// cycles run on one right-hand side (the iterate stays split in between).
+csff_status run_split3(csff_plan* P, float2* u, const float2* b, bool zero_init, bool first, bool last) {
+  const int lb = P->split_block, stop = lb > 0 ? lb : (int)P->lv.size() - 1;
+  CK(csff::launch_split3_down(P->lv, stop, first && !zero_init ? u : nullptr, b, zero_init, P->stream), "split down");
   if (lb > 0) {
     CK(csff::launch_split3_block(P->lv, lb, cinv<float>(P), coarse_fp64(P) ? P->coarse_inv : nullptr, P->stream),
        "coarse block");
   } else {
     Level& C = P->lv.back();
-    CS(coarsest_solve<T>(P, bbuf<T>(C), split_of<T>(C).e, C.m, csff::split3_ring_pitch(C.m)));
+    CS(coarsest_solve<float>(P, C.b32, C.s32.e, C.m, csff::split3_ring_pitch(C.m)));
   }
-  CK(csff::launch_split3_up<T>(P->lv, stop, last ? u : no, P->stream), "split up");
+  CK(csff::launch_split3_up(P->lv, stop, last ? u : nullptr, P->stream), "split up");
   return CSFF_OK;
 }
 
@@ -454,10 +447,10 @@ csff_status run_split3(csff_plan* P, cx<T>* u, const cx<T>* b, bool zero_init, b
 template <typename T>
 csff_status run_vcycle(csff_plan* P, cx<T>* u, const cx<T>* b, bool zero_init, bool first = true, bool last = true) {
   const int lc = P->fused_lc;
-  const bool learned = sizeof(T) == 4 && P->net && !P->learned_off;
-  if ((sizeof(T) == 4 ? P->split32 : P->split64) && !learned) return run_split3<T>(P, u, b, zero_init, first, last);
   if constexpr (sizeof(T) == 4) {
-    if (P->net && !P->learned_off) {
+    const bool learned = P->net && !P->learned_off;
+    if (P->split32 && !learned) return run_split3(P, u, b, zero_init, first, last);
+    if (learned) {
       if (lc > P->learned_levels) return run_vcycle_learned(P, u, b, zero_init);
       return vcycle<T>(P, 0, u, b, zero_init);
     }
@@ -682,19 +675,19 @@ csff_status solve_mixed(csff_plan* P, int eb, double nb, csff_info* info, const 
 // outside the domain hold zero: on the finest level every pass writes whole
 // rows, below it the full weighting does not, and the ring of a correction is
 // never written.
-template <typename T> csff_status alloc_split3(csff_plan* P) {
+csff_status alloc_split3(csff_plan* P) {
   const size_t nl = P->lv.size();
   for (size_t l = 0; l < nl; ++l) {
     Level& L = P->lv[l];
-    csff::Split3<T>& S = split_of<T>(L);
+    csff::Split3& S = L.s32;
     const size_t half = (size_t)L.m * L.m * csff::split3_pitch(L.m);
     const size_t ring = l == 0 ? 0 : (size_t)(L.m + 2) * (L.m + 2) * csff::split3_ring_pitch(L.m) + 8;
     const size_t total = (l + 1 < nl ? (l == 0 ? 7 : 6) * half : 0) + ring;
-    cx<T>* base = nullptr;
+    float2* base = nullptr;
     CS(dev_alloc(P, &base, total));
     S.base = base;
     if (l > 0) {
-      CK(cudaMemsetAsync(base, 0, total * sizeof(cx<T>), P->stream), "zero split arrays");
+      CK(cudaMemsetAsync(base, 0, total * sizeof(float2), P->stream), "zero split arrays");
       S.e = base + (total - ring);
     }
     if (l + 1 == nl) break;
@@ -705,7 +698,7 @@ template <typename T> csff_status alloc_split3(csff_plan* P) {
     S.dr = base + 4 * half;
     S.db = base + 5 * half;
     if (l == 0) S.delta = base + 6 * half;
-    CK(csff::split3_coefs<T>(L, P->prob.k * P->prob.k, P->stream), "split coefficients");
+    CK(csff::split3_coefs(L, P->prob.k * P->prob.k, P->stream), "split coefficients");
   }
   return CSFF_OK;
 }
@@ -800,7 +793,7 @@ void csff_plan_destroy(csff_plan* P) {
   for (Level& L : P->lv)
     for (void* p : {(void*)L.q64, (void*)L.dinv64, (void*)L.q32, (void*)L.dinv32, (void*)L.u64, (void*)L.t64,
                     (void*)L.b64, (void*)L.r64, (void*)L.u32, (void*)L.t32, (void*)L.b32, (void*)L.r32,
-                    (void*)L.fac32, (void*)L.kq64, (void*)L.kq32, L.s32.base, L.s64.base})
+                    (void*)L.fac32, (void*)L.kq64, (void*)L.kq32, L.s32.base})
       if (p) cudaFree(p);
   for (double2* p : P->chi_tab)
     if (p) cudaFree(p);
@@ -952,13 +945,16 @@ csff_status csff_plan_create(const csff_problem* prob, const csff_opts* opts, vo
       }
     }
   }
-  // colour-split V(1,1) RB-GS path (3D), in the precision of the plan's cycles
-  if (d == 3 && opts->smoother == CSFF_SMOOTHER_RBGS && opts->nu1 == 1 && opts->nu2 == 1 && P->lv.size() > 1) {
-    const bool mixed = P->opts.precision == CSFF_PREC_MIXED;
-    csff_status s = mixed ? alloc_split3<float>(P) : alloc_split3<double>(P);
+  // colour-split V(1,1) RB-GS path (3D, FP32 cycles).  FP64 cycles take the per-level
+  // kernels: the split ones hand no rounding of 1/d and of the values on to the
+  // coarse levels, so a cycle from an iterate was 9 to 33 units of 2^-53 off, the
+  // per-level ones 1.8 to 2.4 (65^3, k = 1; 257^3: 2.14 ms against 2.86)
+  if (d == 3 && opts->smoother == CSFF_SMOOTHER_RBGS && opts->nu1 == 1 && opts->nu2 == 1 && P->lv.size() > 1 &&
+      P->opts.precision == CSFF_PREC_MIXED) {
+    csff_status s = alloc_split3(P);
     if (s != CSFF_OK) return fail(s);
-    (mixed ? P->split32 : P->split64) = true;
-    if (mixed && (P->split_block = csff::split3_block_level(P->lv)) > 0) {
+    P->split32 = true;
+    if ((P->split_block = csff::split3_block_level(P->lv)) > 0) {
       cudaError_t e = csff::prepare_split3_block();
       if (e != cudaSuccess) return fail(csff::cuda_fail(e, "coarse block attributes"));
     }
@@ -1263,8 +1259,7 @@ static csff_status user_q_levels(csff_plan* P) {
   if (P->opts.smoother == CSFF_SMOOTHER_GMRES)
     for (const Level& L : P->lv) CK(csff::launch_gmres_coefs(L, s), "GMRES coefficients");
   for (size_t l = 0; l + 1 < P->lv.size(); ++l) {
-    if (P->split32) CK(csff::split3_coefs<float>(P->lv[l], P->prob.k * P->prob.k, s), "split coefficients");
-    if (P->split64) CK(csff::split3_coefs<double>(P->lv[l], P->prob.k * P->prob.k, s), "split coefficients");
+    if (P->split32) CK(csff::split3_coefs(P->lv[l], P->prob.k * P->prob.k, s), "split coefficients");
   }
   const Level& Lc = P->lv.back();
   std::vector<double2> qc((size_t)Lc.N);

@@ -69,13 +69,13 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
 // ---------------------------------------------------------------------------
 // plan internals
 // ---------------------------------------------------------------------------
-// Colour-split arrays of a 3D level (mg_split3.cu): iterate, right-hand side
+// Colour-split FP32 arrays of a 3D level (mg_split3.cu): iterate, right-hand side
 // and 1/d by colour (red, black), the black change of a sweep (finest level),
-// and the level's correction in natural order with a ring of zeros (mg_split3.cu).
-template <typename T> struct Split3 {
-  cx<T> *ur = nullptr, *ub = nullptr, *br = nullptr, *bb = nullptr, *dr = nullptr, *db = nullptr;
-  cx<T> *delta = nullptr, *e = nullptr;
-  cx<T> d0{};                    // FP32: dr, db hold 1/d - d0
+// and the level's correction in natural order with a ring of zeros.
+struct Split3 {
+  float2 *ur = nullptr, *ub = nullptr, *br = nullptr, *bb = nullptr, *dr = nullptr, *db = nullptr;
+  float2 *delta = nullptr, *e = nullptr;
+  float2 d0{};                   // dr, db hold 1/d - d0
   void* base = nullptr;          // the one allocation behind them
 };
 
@@ -100,8 +100,7 @@ struct Level {
   // work buffers
   double2 *u64 = nullptr, *t64 = nullptr, *b64 = nullptr, *r64 = nullptr;
   float2 *u32 = nullptr, *t32 = nullptr, *b32 = nullptr, *r32 = nullptr;
-  Split3<float> s32;
-  Split3<double> s64;
+  Split3 s32;
 };
 
 // Waits of the digit contraction (ff_digits.cuh): a wait gives up after ns; a free
@@ -176,9 +175,9 @@ struct csff_plan {
   double log_rhs_max = 0, log_ff_max = 0;
   // fused V(1,1) RB-GS path (2D): levels >= fused_lc run in one CTA; -1 = unfused
   int fused_lc = -1;
-  // colour-split 3D V(1,1) RB-GS cycles: their arrays exist in FP32 / FP64; FP32:
-  // the level from which one CTA runs the coarser ones (0: none)
-  bool split32 = false, split64 = false;
+  // colour-split 3D V(1,1) RB-GS cycles in FP32: their arrays exist; the level
+  // from which one CTA runs the coarser ones (0: none)
+  bool split32 = false;
   int split_block = 0;
   // CUDA graphs of solver steps (FP64 cycle, or mixed refinement step of a
   // given cycle count), captured on an internal stream and kept by key; the
@@ -342,23 +341,21 @@ cudaError_t launch_update64_fixed(double2* u, const float2* e, long long N, int 
 cudaError_t launch_first_residual(const double2* b, long long N, int s_exp, float2* r32, double* partial, int nblk,
                                   double* out, cudaStream_t s);
 
-// ---- 3D V(1,1) cycles on colour-split arrays (mg_split3.cu) ----------------------
+// ---- 3D FP32 V(1,1) cycles on colour-split arrays (mg_split3.cu) ----------------------
 int split3_pitch(int m);                       // slots of a row of one colour
 // 1/d by colour from dinv64 (k2: the wavenumber's square, without potential)
-template <typename T> cudaError_t split3_coefs(Level& L, double k2, cudaStream_t s);
+cudaError_t split3_coefs(Level& L, double k2, cudaStream_t s);
 int split3_ring_pitch(int mc);                 // row pitch of a level's correction
 // the levels above `stop` down to its right-hand side (split, with the red half
-// sweep from zero; of the last level b32/b64 in natural order): b and the
+// sweep from zero; of the last level b32 in natural order): b and the
 // iterate u in natural order, or zero_init, or (u null) both still in the split
 // arrays
-template <typename T>
-cudaError_t launch_split3_down(std::vector<Level>& lv, int stop, const cx<T>* u, const cx<T>* b, bool zero_init,
+cudaError_t launch_split3_down(std::vector<Level>& lv, int stop, const float2* u, const float2* b, bool zero_init,
                                cudaStream_t s);
 // and back from level stop's correction e; the iterate goes to u_nat in natural
 // order or (null) stays in the split arrays
-template <typename T>
-cudaError_t launch_split3_up(std::vector<Level>& lv, int stop, cx<T>* u_nat, cudaStream_t s);
-// FP32 cycles: the level from which one CTA runs all coarser ones (0: none), its
+cudaError_t launch_split3_up(std::vector<Level>& lv, int stop, float2* u_nat, cudaStream_t s);
+// the level from which one CTA runs all coarser ones (0: none), its
 // set-up and launch (inv64: the coarsest product in FP64)
 int split3_block_level(const std::vector<Level>& lv);
 cudaError_t prepare_split3_block();

@@ -37,19 +37,14 @@
 namespace csff {
 namespace {
 
-template <typename T> struct Pair { cx<T> a, b; };
-template <typename T> __device__ __forceinline__ cx<T> zc() { return mk<cx<T>>((T)0, (T)0); }
-__device__ __forceinline__ Pair<float> ld2(const float2* p) {
+struct Pair { float2 a, b; };
+__device__ __forceinline__ float2 zc() { return make_float2(0.f, 0.f); }
+__device__ __forceinline__ Pair ld2(const float2* p) {
   const float4 v = *reinterpret_cast<const float4*>(p);
-  return Pair<float>{make_float2(v.x, v.y), make_float2(v.z, v.w)};
+  return Pair{make_float2(v.x, v.y), make_float2(v.z, v.w)};
 }
-__device__ __forceinline__ Pair<double> ld2(const double2* p) { return Pair<double>{p[0], p[1]}; }
 __device__ __forceinline__ void st2(float2* p, float2 a, float2 b) {
   *reinterpret_cast<float4*>(p) = make_float4(a.x, a.y, b.x, b.y);
-}
-__device__ __forceinline__ void st2(double2* p, double2 a, double2 b) {
-  p[0] = a;
-  p[1] = b;
 }
 // a + b c for complex values, a chain of fused multiply-adds
 template <typename C> __device__ __forceinline__ C cfma(C a, C b, C c) {
@@ -61,7 +56,6 @@ template <typename C> __device__ __forceinline__ C cfma(C a, C b, C c) {
 // shifts every equation by the same 2^-25 |d|, which the folded residual (no
 // explicit b - A u) would pass to the coarse levels as a residual.
 __device__ __forceinline__ float2 dinv_mul(float2 d0, float2 dv, float2 t) { return cfma(cmul(d0, t), dv, t); }
-__device__ __forceinline__ double2 dinv_mul(double2, double2 dv, double2 t) { return cmul(dv, t); }
 
 // Launches of at most one CTA an SM (the small levels) let their dependent be set
 // up as soon as they have passed their own wait; a sweep's and a full weighting's
@@ -83,11 +77,11 @@ __device__ __forceinline__ bool at(int m, int HP, At& p) {
 
 // Natural order in: b by colour and the red half sweep, from zero (u = d^{-1} b,
 // NAT_U false) or from a natural iterate, whose black points go to ub.
-template <typename T, bool NAT_U>
-__global__ void k3s_first(const cx<T>* __restrict__ b_nat, const cx<T>* __restrict__ u_nat,
-                          const cx<T>* __restrict__ dr, cx<T> c, cx<T> d0, int m, int HP, cx<T>* __restrict__ br,
-                          cx<T>* __restrict__ bb, cx<T>* __restrict__ ub, cx<T>* __restrict__ ur) {
-  using C = cx<T>;
+template <bool NAT_U>
+__global__ void k3s_first(const float2* __restrict__ b_nat, const float2* __restrict__ u_nat,
+                          const float2* __restrict__ dr, float2 c, float2 d0, int m, int HP, float2* __restrict__ br,
+                          float2* __restrict__ bb, float2* __restrict__ ub, float2* __restrict__ ur) {
+  using C = float2;
   wait_and_trigger();
   At p;
   if (!at(m, HP, p)) return;
@@ -96,19 +90,19 @@ __global__ void k3s_first(const cx<T>* __restrict__ b_nat, const cx<T>* __restri
   const int x = 2 * p.j, x0 = x + o, x1 = x0 + 2;
   C v[4];
 #pragma unroll
-  for (int k = 0; k < 4; ++k) v[k] = x + k < m ? row[x + k] : zc<T>();
+  for (int k = 0; k < 4; ++k) v[k] = x + k < m ? row[x + k] : zc();
   const long long s = p.row * HP + p.j;
-  const Pair<T> d = ld2(dr + s);
-  C s0 = zc<T>(), s1 = zc<T>();
+  const Pair d = ld2(dr + s);
+  C s0 = zc(), s1 = zc();
   if constexpr (NAT_U) {
     const C* u = u_nat + p.row * m;
     const long long pl = (long long)m * m;
     const bool i0 = x0 < m, i1 = x1 < m;
-    const C xl = (x0 > 0 && x0 - 1 < m) ? u[x0 - 1] : zc<T>(), xm = x0 + 1 < m ? u[x0 + 1] : zc<T>(),
-            xr = x1 + 1 < m ? u[x1 + 1] : zc<T>();
+    const C xl = (x0 > 0 && x0 - 1 < m) ? u[x0 - 1] : zc(), xm = x0 + 1 < m ? u[x0 + 1] : zc(),
+            xr = x1 + 1 < m ? u[x1 + 1] : zc();
     auto at_row = [&](bool in, long long off, C& q0, C& q1) {
-      q0 = in && i0 ? u[x0 + off] : zc<T>();
-      q1 = in && i1 ? u[x1 + off] : zc<T>();
+      q0 = in && i0 ? u[x0 + off] : zc();
+      q1 = in && i1 ? u[x1 + off] : zc();
     };
     C yl0, yl1, yr0, yr1, zl0, zl1, zr0, zr1;
     at_row(p.iy > 0, -m, yl0, yl1);
@@ -123,34 +117,28 @@ __global__ void k3s_first(const cx<T>* __restrict__ b_nat, const cx<T>* __restri
   const C r0 = o ? v[1] : v[0], r1 = o ? v[3] : v[2];
   st2(br + s, r0, r1);
   st2(bb + s, o ? v[0] : v[1], o ? v[2] : v[3]);
-  st2(ur + s, x0 < m ? dinv_mul(d0, d.a, NAT_U ? cfma(r0, c, s0) : r0) : zc<T>(),
-      x1 < m ? dinv_mul(d0, d.b, NAT_U ? cfma(r1, c, s1) : r1) : zc<T>());
+  st2(ur + s, x0 < m ? dinv_mul(d0, d.a, NAT_U ? cfma(r0, c, s0) : r0) : zc(),
+      x1 < m ? dinv_mul(d0, d.b, NAT_U ? cfma(r1, c, s1) : r1) : zc());
 }
 
 // a level's d^{-1} by colour: FP64 as stored; FP32 as the difference to d0 of
 // 1 / (6 c - q) with c the FP32 value that the sweeps multiply by, to first
 // order in dc, six times the rounding of c (relative 2^-25: its square and the
 // rounding of this term lie far below the result's)
-template <typename T>
-__global__ void k3s_split(const double2* __restrict__ dinv, float2 dc, cx<T> d0, int m, int HP,
-                          cx<T>* __restrict__ red, cx<T>* __restrict__ black) {
-  using C = cx<T>;
+__global__ void k3s_split(const double2* __restrict__ dinv, float2 dc, float2 d0, int m, int HP,
+                          float2* __restrict__ red, float2* __restrict__ black) {
+  using C = float2;
   At p;
   if (!at(m, HP, p)) return;
   const int o = (p.iy + p.iz + 1) & 1, x = 2 * p.j;
   C v[4];
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
-    v[k] = zc<T>();
+    v[k] = zc();
     if (x + k < m) {
-      const long long i = p.row * m + x + k;
-      if constexpr (sizeof(T) == 8) {
-        v[k] = dinv[i];
-      } else {
-        const double2 di = dinv[i];
-        const float2 f = make_float2((float)di.x, (float)di.y), t = cmul(cmul(f, f), dc);
-        v[k] = make_float2((float)(di.x - (double)d0.x) - t.x, (float)(di.y - (double)d0.y) - t.y);
-      }
+      const double2 di = dinv[p.row * m + x + k];
+      const float2 f = make_float2((float)di.x, (float)di.y), t = cmul(cmul(f, f), dc);
+      v[k] = make_float2((float)(di.x - (double)d0.x) - t.x, (float)(di.y - (double)d0.y) - t.y);
     }
   }
   const long long s = p.row * HP + p.j;
@@ -168,32 +156,31 @@ __global__ void k3s_split(const double2* __restrict__ dinv, float2 dc, cx<T> d0,
 // Two odd: with S4 the sum of the four coarse corners around the point in the
 // plane of its odd axes, 5/4 S4 + 1/8 (S4 one coarse plane up and one down the
 // even axis).
-template <typename T>
-__device__ __forceinline__ Pair<T> prolong_nbr(const cx<T>* __restrict__ e, int pe, int mc, int j, int iy, int iz) {
-  using C = cx<T>;
+__device__ __forceinline__ Pair prolong_nbr(const float2* __restrict__ e, int pe, int mc, int j, int iy, int iz) {
+  using C = float2;
   const bool oy = !(iy & 1), oz = !(iz & 1);           // odd node indices
   const int Y = (iy + 1) >> 1, Z = (iz + 1) >> 1;      // coarse node at or below
   const long long pz = (long long)(mc + 2) * pe;
   const C* r = e + Z * pz + (long long)Y * pe + j;     // r[k]: column X = j - 1 + k
-  Pair<T> out;
+  Pair out;
   if (oy == oz) {                                      // x even: coarse columns j + 1 and j + 2
     if (!oy) {
       const C e0 = r[1], e3 = r[4];
-      const Pair<T> m = ld2(r + 2), a = ld2(r + 2 - pe), b = ld2(r + 2 + pe), f = ld2(r + 2 - pz), g = ld2(r + 2 + pz);
+      const Pair m = ld2(r + 2), a = ld2(r + 2 - pe), b = ld2(r + 2 + pe), f = ld2(r + 2 - pz), g = ld2(r + 2 + pz);
       const C s0 = cadd(cadd(e0, m.b), cadd(cadd(a.a, b.a), cadd(f.a, g.a)));
       const C s1 = cadd(cadd(m.a, e3), cadd(cadd(a.b, b.b), cadd(f.b, g.b)));
-      out.a = cadd(cscale(m.a, (T)3), cscale(s0, (T)0.5));
-      out.b = cadd(cscale(m.b, (T)3), cscale(s1, (T)0.5));
+      out.a = cadd(cscale(m.a, 3.f), cscale(s0, 0.5f));
+      out.b = cadd(cscale(m.b, 3.f), cscale(s1, 0.5f));
     } else {
       C s[4];
       const C *r2 = r + pe, *r3 = r + pz, *r4 = r3 + pe;
-      const Pair<T> m1 = ld2(r + 2), m2 = ld2(r2 + 2), m3 = ld2(r3 + 2), m4 = ld2(r4 + 2);
+      const Pair m1 = ld2(r + 2), m2 = ld2(r2 + 2), m3 = ld2(r3 + 2), m4 = ld2(r4 + 2);
       s[0] = cadd(cadd(r[1], r2[1]), cadd(r3[1], r4[1]));
       s[1] = cadd(cadd(m1.a, m2.a), cadd(m3.a, m4.a));
       s[2] = cadd(cadd(m1.b, m2.b), cadd(m3.b, m4.b));
       s[3] = cadd(cadd(r[4], r2[4]), cadd(r3[4], r4[4]));
-      out.a = cadd(cscale(s[1], (T)1.25), cscale(cadd(s[0], s[2]), (T)0.125));
-      out.b = cadd(cscale(s[2], (T)1.25), cscale(cadd(s[1], s[3]), (T)0.125));
+      out.a = cadd(cscale(s[1], 1.25f), cscale(cadd(s[0], s[2]), 0.125f));
+      out.b = cadd(cscale(s[2], 1.25f), cscale(cadd(s[1], s[3]), 0.125f));
     }
   } else {                                             // x odd: between coarse columns j and j + 1 (j + 1 and j + 2)
     C t0[3], t1[3];                                    // S4 at the even axis' plane below, at, above
@@ -201,13 +188,13 @@ __device__ __forceinline__ Pair<T> prolong_nbr(const cx<T>* __restrict__ e, int 
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
       const C* q = r + (k - 1) * step;
-      const Pair<T> a = ld2(q + 2), b = ld2(q + pair + 2);
+      const Pair a = ld2(q + 2), b = ld2(q + pair + 2);
       const C c0 = cadd(q[1], q[pair + 1]), c1 = cadd(a.a, b.a), c2 = cadd(a.b, b.b);
       t0[k] = cadd(c0, c1);
       t1[k] = cadd(c1, c2);
     }
-    out.a = cadd(cscale(t0[1], (T)1.25), cscale(cadd(t0[0], t0[2]), (T)0.125));
-    out.b = cadd(cscale(t1[1], (T)1.25), cscale(cadd(t1[0], t1[2]), (T)0.125));
+    out.a = cadd(cscale(t0[1], 1.25f), cscale(cadd(t0[0], t0[2]), 0.125f));
+    out.b = cadd(cscale(t1[1], 1.25f), cscale(cadd(t1[0], t1[2]), 0.125f));
   }
   return out;
 }
@@ -219,26 +206,26 @@ __device__ __forceinline__ Pair<T> prolong_nbr(const cx<T>* __restrict__ e, int 
 //  NAT (black): both colours to nat in natural order
 //  RING (black): both colours to nat as the ringed correction, rows nat_pitch apart
 enum Mode { PLAIN, PROLONG, DELTA, NAT, RING };
-template <typename T, int COLOUR, int MODE>
-__global__ void k3s_sweep(const cx<T>* __restrict__ uo, const cx<T>* __restrict__ b, const cx<T>* __restrict__ dinv,
-                          cx<T> c, cx<T> d0, int m, int HP, cx<T>* u, cx<T>* __restrict__ delta,
-                          const cx<T>* __restrict__ e, int pe, int mc, cx<T>* __restrict__ nat, int nat_pitch) {
-  using C = cx<T>;
+template <int COLOUR, int MODE>
+__global__ void k3s_sweep(const float2* __restrict__ uo, const float2* __restrict__ b, const float2* __restrict__ dinv,
+                          float2 c, float2 d0, int m, int HP, float2* u, float2* __restrict__ delta,
+                          const float2* __restrict__ e, int pe, int mc, float2* __restrict__ nat, int nat_pitch) {
+  using C = float2;
   At p;
   if (!at(m, HP, p)) return;
   const int o = (p.iy + p.iz + 1 + COLOUR) & 1;
   const long long s = p.row * HP + p.j;
-  const Pair<T> dv = ld2(dinv + s);
+  const Pair dv = ld2(dinv + s);
   wait_and_trigger();
   const long long plane = (long long)m * HP;
-  const Pair<T> zero{zc<T>(), zc<T>()};
-  const Pair<T> mid = ld2(uo + s);
+  const Pair zero{zc(), zc()};
+  const Pair mid = ld2(uo + s);
   const int je = o ? p.j + 2 : p.j - 1;                 // the row's third neighbour slot
-  const C edge = (je >= 0 && je < HP) ? uo[s + (je - p.j)] : zc<T>();
-  const Pair<T> yl = p.iy > 0 ? ld2(uo + s - HP) : zero, yr = p.iy < m - 1 ? ld2(uo + s + HP) : zero;
-  const Pair<T> zl = p.iz > 0 ? ld2(uo + s - plane) : zero, zr = p.iz < m - 1 ? ld2(uo + s + plane) : zero;
-  const Pair<T> bv = ld2(b + s);
-  Pair<T> old = zero;
+  const C edge = (je >= 0 && je < HP) ? uo[s + (je - p.j)] : zc();
+  const Pair yl = p.iy > 0 ? ld2(uo + s - HP) : zero, yr = p.iy < m - 1 ? ld2(uo + s + HP) : zero;
+  const Pair zl = p.iz > 0 ? ld2(uo + s - plane) : zero, zr = p.iz < m - 1 ? ld2(uo + s + plane) : zero;
+  const Pair bv = ld2(b + s);
+  Pair old = zero;
   if constexpr (MODE == DELTA) old = ld2(u + s);
   // x - 1 and x + 1 of both slots
   const C a0 = o ? mid.a : edge, a1 = o ? mid.b : mid.a, b0 = o ? mid.b : mid.a, b1 = o ? edge : mid.b;
@@ -246,13 +233,13 @@ __global__ void k3s_sweep(const cx<T>* __restrict__ uo, const cx<T>* __restrict_
   C s0 = cadd(cadd(cadd(a0, a1), cadd(yl.a, yr.a)), cadd(zl.a, zr.a));
   C s1 = cadd(cadd(cadd(b0, b1), cadd(yl.b, yr.b)), cadd(zl.b, zr.b));
   if constexpr (MODE == PROLONG) {
-    const Pair<T> q = prolong_nbr<T>(e, pe, mc, p.j, p.iy, p.iz);
+    const Pair q = prolong_nbr(e, pe, mc, p.j, p.iy, p.iz);
     s0 = cadd(s0, q.a);
     s1 = cadd(s1, q.b);
   }
   const int x0 = 2 * p.j + o, x1 = x0 + 2;
-  const C v0 = x0 < m ? dinv_mul(d0, dv.a, cfma(bv.a, c, s0)) : zc<T>();
-  const C v1 = x1 < m ? dinv_mul(d0, dv.b, cfma(bv.b, c, s1)) : zc<T>();
+  const C v0 = x0 < m ? dinv_mul(d0, dv.a, cfma(bv.a, c, s0)) : zc();
+  const C v1 = x1 < m ? dinv_mul(d0, dv.b, cfma(bv.b, c, s1)) : zc();
   if constexpr (MODE != NAT && MODE != RING) st2(u + s, v0, v1);
   if constexpr (MODE == DELTA) st2(delta + s, csub(v0, old.a), csub(v1, old.b));
   if constexpr (MODE == RING) {
@@ -274,16 +261,15 @@ __global__ void k3s_sweep(const cx<T>* __restrict__ uo, const cx<T>* __restrict_
 // its b in both colours and the red half sweep u = d^{-1} b from zero, or (the
 // coarsest level, nat) b in natural order.  A thread takes the coarse points
 // P, P + 1 (P even) of a row: one of them red.
-template <typename T>
-__global__ void k3s_restrict(const cx<T>* __restrict__ delta, int m, int HP, cx<T> c, int mc, int HPc,
-                             cx<T>* __restrict__ br, cx<T>* __restrict__ bb, const cx<T>* __restrict__ dr,
-                             cx<T> d0, cx<T>* __restrict__ ur, cx<T>* __restrict__ nat) {
-  using C = cx<T>;
+__global__ void k3s_restrict(const float2* __restrict__ delta, int m, int HP, float2 c, int mc, int HPc,
+                             float2* __restrict__ br, float2* __restrict__ bb, const float2* __restrict__ dr,
+                             float2 d0, float2* __restrict__ ur, float2* __restrict__ nat) {
+  using C = float2;
   const int P = 2 * (int)(blockIdx.x * blockDim.x + threadIdx.x);
   const int Yc = blockIdx.y * blockDim.y + threadIdx.y, Zc = blockIdx.z;
   if (P >= mc || Yc >= mc) return;
   const long long row = (long long)Zc * mc + Yc, s = row * HPc + (P >> 1);
-  const C dc = nat ? zc<T>() : dr[s];
+  const C dc = nat ? zc() : dr[s];
   wait_and_trigger();
   const int fy = 2 * Yc + 1, fz = 2 * Zc + 1;          // rows one unit off lie inside the grid (m is odd)
   const C* const own = delta + ((long long)fz * m + fy) * HP + P;
@@ -297,49 +283,49 @@ __global__ void k3s_restrict(const cx<T>* __restrict__ delta, int m, int HP, cx<
   // coarse points 35 -> 32 us, 31^3 and 15^3 7.9 and 7.7 -> 6.5 and 6.0)
   auto pair = [&](const C* r) { return ld2(r); };
   auto pair_in = [&](const C* r) {
-    const Pair<T> v = ld2(r);
-    return r != own ? v : Pair<T>{zc<T>(), zc<T>()};
+    const Pair v = ld2(r);
+    return r != own ? v : Pair{zc(), zc()};
   };
   const int ro = P + 2 < HP ? 2 : 0, lo = P > 0 ? -1 : 0;
-  auto right = [&](const C* r) { const C v = r[ro]; return ro ? v : zc<T>(); };
-  auto left = [&](const C* r) { const C v = r[lo]; return lo ? v : zc<T>(); };
-  C f0 = zc<T>(), f1 = f0, g0 = f0, g1 = f0, h0 = f0, h1 = f0;      // distance (1,0,0), (1,1,1), (2,1,0)
+  auto right = [&](const C* r) { const C v = r[ro]; return ro ? v : zc(); };
+  auto left = [&](const C* r) { const C v = r[lo]; return lo ? v : zc(); };
+  C f0 = zc(), f1 = f0, g0 = f0, g1 = f0, h0 = f0, h1 = f0;      // distance (1,0,0), (1,1,1), (2,1,0)
   auto add = [](C& x, C& y, C u, C v) { x = cadd(x, u); y = cadd(y, v); };
   {                                                    // own row: x offsets -1 and +1
     const C* r = rowp(0, 0);
-    const Pair<T> v = ld2(r);
+    const Pair v = ld2(r);
     add(f0, f1, cadd(v.a, v.b), cadd(v.b, right(r)));
   }
 #pragma unroll
   for (int k = 0; k < 4; ++k) {                        // one unit off in y or z: x offset 0, and -2, +2
     const int s = (k & 1) ? 1 : -1;
     const C* r = (k < 2) ? rowp(s, 0) : rowp(0, s);
-    const Pair<T> v = pair(r);
+    const Pair v = pair(r);
     add(f0, f1, v.a, v.b);
     add(h0, h1, cadd(left(r), v.b), cadd(v.a, right(r)));
   }
 #pragma unroll
   for (int k = 0; k < 4; ++k) {                        // one unit off in both: x offsets -1 and +1
     const C* r = rowp((k & 1) ? 1 : -1, (k & 2) ? 1 : -1);
-    const Pair<T> v = pair(r);
+    const Pair v = pair(r);
     add(g0, g1, cadd(v.a, v.b), cadd(v.b, right(r)));
   }
 #pragma unroll
   for (int k = 0; k < 4; ++k) {                        // two units off in one: x offsets -1 and +1
     const int s = (k & 1) ? 2 : -2;
     const C* r = (k < 2) ? rowp(s, 0) : rowp(0, s);
-    const Pair<T> v = pair_in(r);
-    add(h0, h1, cadd(v.a, v.b), cadd(v.b, r != own ? right(r) : zc<T>()));
+    const Pair v = pair_in(r);
+    add(h0, h1, cadd(v.a, v.b), cadd(v.b, r != own ? right(r) : zc()));
   }
 #pragma unroll
   for (int k = 0; k < 8; ++k) {                        // two and one: x offset 0
     const int s = (k & 1) ? 1 : -1, s2 = (k & 2) ? 2 : -2;
-    const Pair<T> v = pair_in((k & 4) ? rowp(s2, s) : rowp(s, s2));
+    const Pair v = pair_in((k & 4) ? rowp(s2, s) : rowp(s, s2));
     add(h0, h1, v.a, v.b);
   }
-  const C w0 = cadd(cadd(cscale(f0, (T)0.25), cscale(g0, (T)0.09375)), cscale(h0, (T)0.03125));
-  const C w1 = cadd(cadd(cscale(f1, (T)0.25), cscale(g1, (T)0.09375)), cscale(h1, (T)0.03125));
-  const C v0 = cmul(c, w0), v1 = P + 1 < mc ? cmul(c, w1) : zc<T>();
+  const C w0 = cadd(cadd(cscale(f0, 0.25f), cscale(g0, 0.09375f)), cscale(h0, 0.03125f));
+  const C w1 = cadd(cadd(cscale(f1, 0.25f), cscale(g1, 0.09375f)), cscale(h1, 0.03125f));
+  const C v0 = cmul(c, w0), v1 = P + 1 < mc ? cmul(c, w1) : zc();
   if (nat) {
     nat[row * mc + P] = v0;
     if (P + 1 < mc) nat[row * mc + P + 1] = v1;
@@ -524,29 +510,21 @@ Shape shape(int pairs, int m) {
   return Shape{dim3((pairs + tx - 1) / tx, (m + ty - 1) / ty, m), dim3(tx, ty)};
 }
 
-template <typename T> Split3<T>& sp(Level& L);
-template <> Split3<float>& sp<float>(Level& L) { return L.s32; }
-template <> Split3<double>& sp<double>(Level& L) { return L.s64; }
-template <typename T> cx<T>* nat_b(Level& L);
-template <> float2* nat_b<float>(Level& L) { return L.b32; }
-template <> double2* nat_b<double>(Level& L) { return L.b64; }
-
 }  // namespace
 
 int split3_pitch(int m) { return ((m + 1) / 2 + 3) / 4 * 4; }
 // the finer level's slots j < HP read columns up to j + 4
 int split3_ring_pitch(int mc) { return split3_pitch(2 * mc + 1) + 4; }
 
-template <typename T>
 cudaError_t split3_coefs(Level& L, double k2, cudaStream_t s) {
   const int HP = split3_pitch(L.m);
   const Shape h = shape(HP / 2, L.m);
-  Split3<T>& S = sp<T>(L);
-  const cx<T> c = mk<cx<T>>((T)L.c.x, (T)L.c.y);
+  Split3& S = L.s32;
+  const float2 c = make_float2((float)L.c.x, (float)L.c.y);
   const double dx = 6.0 * (double)c.x - k2, dy = 6.0 * (double)c.y, den = dx * dx + dy * dy;
-  S.d0 = den > 0.0 ? mk<cx<T>>((T)(dx / den), (T)(-dy / den)) : mk<cx<T>>((T)0, (T)0);
+  S.d0 = den > 0.0 ? make_float2((float)(dx / den), (float)(-dy / den)) : make_float2(0.f, 0.f);
   const float2 dc = make_float2((float)(6.0 * ((double)c.x - L.c.x)), (float)(6.0 * ((double)c.y - L.c.y)));
-  k3s_split<T><<<h.g, h.b, 0, s>>>(L.dinv64, dc, S.d0, L.m, HP, S.dr, S.db);
+  k3s_split<<<h.g, h.b, 0, s>>>(L.dinv64, dc, S.d0, L.m, HP, S.dr, S.db);
   count_launch();
   return cudaGetLastError();
 }
@@ -578,7 +556,7 @@ cudaError_t launch_split3_block(std::vector<Level>& lv, int lb, const float2* in
     L.c[i] = make_float2((float)v.c.x, (float)v.c.y);
     L.d0[i] = v.s32.d0;
   }
-  const Split3<float>& F = lv[lb].s32;
+  const Split3& F = lv[lb].s32;
   const size_t sm = block_bytes(lv, lb);
   const int pe = split3_ring_pitch(lv[lb].m);
   ProfScope ps(mg_family<float>(), s, 2.0 * sizeof(float2) * lv[lb].N, 0);
@@ -589,84 +567,75 @@ cudaError_t launch_split3_block(std::vector<Level>& lv, int lb, const float2* in
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-template <typename T>
-cudaError_t launch_split3_down(std::vector<Level>& lv, int stop, const cx<T>* u, const cx<T>* b, bool zero_init,
+cudaError_t launch_split3_down(std::vector<Level>& lv, int stop, const float2* u, const float2* b, bool zero_init,
                                cudaStream_t s) {
   cudaError_t e = cudaSuccess;
   int launches = 0;
   auto ok = [&](cudaError_t r) { ++launches; if (e == cudaSuccess) e = r; };
   const int nl = (int)lv.size();
-  const double S = sizeof(cx<T>);
+  const double S = sizeof(float2);
   for (int l = 0; l < stop && e == cudaSuccess; ++l) {
     Level &L = lv[l], &C = lv[l + 1];
-    Split3<T>&F = sp<T>(L), &G = sp<T>(C);
+    Split3 &F = L.s32, &G = C.s32;
     const int m = L.m, HP = split3_pitch(m), HPc = split3_pitch(C.m);
-    const cx<T> c = mk<cx<T>>((T)L.c.x, (T)L.c.y);
+    const float2 c = make_float2((float)L.c.x, (float)L.c.y);
     const Shape h = shape(HP / 2, m), hc = shape((C.m + 1) / 2, C.m);
-    const cx<T>* none = nullptr;
-    cx<T>* no = nullptr;
+    const float2* none = nullptr;
+    float2* no = nullptr;
     const bool zero = zero_init || l > 0;
-    ProfScope ps(mg_family<T>(), s, (zero ? 3.5 : 6.0) * S * L.N + S * C.N, 0);
+    ProfScope ps(mg_family<float>(), s, (zero ? 3.5 : 6.0) * S * L.N + S * C.N, 0);
     if (l == 0) {
       if (zero)
-        ok(launch_pdl(k3s_first<T, false>, h.g, h.b, 0, s, b, none, (const cx<T>*)F.dr, c, F.d0, m, HP, F.br, F.bb, no,
+        ok(launch_pdl(k3s_first<false>, h.g, h.b, 0, s, b, none, (const float2*)F.dr, c, F.d0, m, HP, F.br, F.bb, no,
                       F.ur));
       else if (u)
-        ok(launch_pdl(k3s_first<T, true>, h.g, h.b, 0, s, b, u, (const cx<T>*)F.dr, c, F.d0, m, HP, F.br, F.bb, F.ub,
+        ok(launch_pdl(k3s_first<true>, h.g, h.b, 0, s, b, u, (const float2*)F.dr, c, F.d0, m, HP, F.br, F.bb, F.ub,
                       F.ur));
       else
-        ok(launch_pdl(k3s_sweep<T, 0, PLAIN>, h.g, h.b, 0, s, (const cx<T>*)F.ub, (const cx<T>*)F.br,
-                      (const cx<T>*)F.dr, c, F.d0, m, HP, F.ur, no, none, 0, 0, no, 0));
+        ok(launch_pdl(k3s_sweep<0, PLAIN>, h.g, h.b, 0, s, (const float2*)F.ub, (const float2*)F.br,
+                      (const float2*)F.dr, c, F.d0, m, HP, F.ur, no, none, 0, 0, no, 0));
     }
     if (zero)
-      ok(launch_pdl(k3s_sweep<T, 1, PLAIN>, h.g, h.b, 0, s, (const cx<T>*)F.ur, (const cx<T>*)F.bb, (const cx<T>*)F.db,
+      ok(launch_pdl(k3s_sweep<1, PLAIN>, h.g, h.b, 0, s, (const float2*)F.ur, (const float2*)F.bb, (const float2*)F.db,
                     c, F.d0, m, HP, F.ub, no, none, 0, 0, no, 0));
     else
-      ok(launch_pdl(k3s_sweep<T, 1, DELTA>, h.g, h.b, 0, s, (const cx<T>*)F.ur, (const cx<T>*)F.bb, (const cx<T>*)F.db,
+      ok(launch_pdl(k3s_sweep<1, DELTA>, h.g, h.b, 0, s, (const float2*)F.ur, (const float2*)F.bb, (const float2*)F.db,
                     c, F.d0, m, HP, F.ub, F.delta, none, 0, 0, no, 0));
-    ok(launch_pdl(k3s_restrict<T>, hc.g, hc.b, 0, s, (const cx<T>*)(zero ? F.ub : F.delta), m, HP, c, C.m, HPc, G.br,
-                  G.bb, (const cx<T>*)G.dr, G.d0, G.ur, l + 2 == nl ? nat_b<T>(C) : no));
+    ok(launch_pdl(k3s_restrict, hc.g, hc.b, 0, s, (const float2*)(zero ? F.ub : F.delta), m, HP, c, C.m, HPc, G.br,
+                  G.bb, (const float2*)G.dr, G.d0, G.ur, l + 2 == nl ? C.b32 : no));
   }
   count_launch(launches);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-template <typename T>
-cudaError_t launch_split3_up(std::vector<Level>& lv, int stop, cx<T>* u_nat, cudaStream_t s) {
+cudaError_t launch_split3_up(std::vector<Level>& lv, int stop, float2* u_nat, cudaStream_t s) {
   cudaError_t e = cudaSuccess;
   int launches = 0;
   auto ok = [&](cudaError_t r) { ++launches; if (e == cudaSuccess) e = r; };
-  const double S = sizeof(cx<T>);
+  const double S = sizeof(float2);
   for (int l = stop - 1; l >= 0 && e == cudaSuccess; --l) {
     Level &L = lv[l], &C = lv[l + 1];
-    Split3<T>&F = sp<T>(L), &G = sp<T>(C);
+    Split3 &F = L.s32, &G = C.s32;
     const int m = L.m, HP = split3_pitch(m);
-    const cx<T> c = mk<cx<T>>((T)L.c.x, (T)L.c.y);
+    const float2 c = make_float2((float)L.c.x, (float)L.c.y);
     const Shape h = shape(HP / 2, m);
-    const cx<T>* none = nullptr;
-    cx<T>* no = nullptr;
-    ProfScope ps(mg_family<T>(), s, 5.0 * S * L.N + S * C.N, 0);
-    ok(launch_pdl(k3s_sweep<T, 0, PROLONG>, h.g, h.b, 0, s, (const cx<T>*)F.ub, (const cx<T>*)F.br,
-                  (const cx<T>*)F.dr, c, F.d0, m, HP, F.ur, no, (const cx<T>*)G.e, split3_ring_pitch(C.m), C.m, no, 0));
+    const float2* none = nullptr;
+    float2* no = nullptr;
+    ProfScope ps(mg_family<float>(), s, 5.0 * S * L.N + S * C.N, 0);
+    ok(launch_pdl(k3s_sweep<0, PROLONG>, h.g, h.b, 0, s, (const float2*)F.ub, (const float2*)F.br,
+                  (const float2*)F.dr, c, F.d0, m, HP, F.ur, no, (const float2*)G.e, split3_ring_pitch(C.m), C.m, no, 0));
     if (l > 0)
-      ok(launch_pdl(k3s_sweep<T, 1, RING>, h.g, h.b, 0, s, (const cx<T>*)F.ur, (const cx<T>*)F.bb, (const cx<T>*)F.db,
+      ok(launch_pdl(k3s_sweep<1, RING>, h.g, h.b, 0, s, (const float2*)F.ur, (const float2*)F.bb, (const float2*)F.db,
                     c, F.d0, m, HP, no, no, none, 0, 0, F.e, split3_ring_pitch(m)));
     else if (u_nat)
-      ok(launch_pdl(k3s_sweep<T, 1, NAT>, h.g, h.b, 0, s, (const cx<T>*)F.ur, (const cx<T>*)F.bb, (const cx<T>*)F.db,
+      ok(launch_pdl(k3s_sweep<1, NAT>, h.g, h.b, 0, s, (const float2*)F.ur, (const float2*)F.bb, (const float2*)F.db,
                     c, F.d0, m, HP, no, no, none, 0, 0, u_nat, 0));
     else
-      ok(launch_pdl(k3s_sweep<T, 1, PLAIN>, h.g, h.b, 0, s, (const cx<T>*)F.ur, (const cx<T>*)F.bb, (const cx<T>*)F.db,
+      ok(launch_pdl(k3s_sweep<1, PLAIN>, h.g, h.b, 0, s, (const float2*)F.ur, (const float2*)F.bb, (const float2*)F.db,
                     c, F.d0, m, HP, F.ub, no, none, 0, 0, no, 0));
   }
   count_launch(launches);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
-
-#define CSFF_SPLIT3_INST(T)                                                                                      \
-  template cudaError_t split3_coefs<T>(Level&, double, cudaStream_t);                                                 \
-  template cudaError_t launch_split3_down<T>(std::vector<Level>&, int, const cx<T>*, const cx<T>*, bool, cudaStream_t); \
-  template cudaError_t launch_split3_up<T>(std::vector<Level>&, int, cx<T>*, cudaStream_t);
-CSFF_SPLIT3_INST(float)
-CSFF_SPLIT3_INST(double)
 
 }  // namespace csff
