@@ -260,7 +260,7 @@ csff_status csff_far_field_debug_waits(csff_plan* plan, int extra_arrivals, int 
    nodes are fine nodes), 1/d and the FP32 copies are rebuilt and the coarsest
    inverse is formed again (FP64 Gauss-Jordan on the host).  From then on
    V-cycles use the per-level kernels (the fused FP32 tiles form q from the
-   Gaussian factors).  csff_rhs / csff_solve keep forming the Gaussian
+   Gaussian factors, the 3D FP32 cycles hold 1/d relative to k^2's).  csff_rhs / csff_solve keep forming the Gaussian
    right-hand side; use csff_solve_rhs.  Errors: CSFF_ERR_INVALID_ARG for NULL
    arguments or a singular coarsest operator, CSFF_ERR_CUDA. */
 csff_status csff_plan_set_potential(csff_plan* plan, const void* q_dev);

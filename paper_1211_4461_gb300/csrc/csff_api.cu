@@ -675,6 +675,18 @@ csff_status solve_mixed(csff_plan* P, int eb, double nb, csff_info* info, const 
 // outside the domain hold zero: on the finest level every pass writes whole
 // rows, below it the full weighting does not, and the ring of a correction is
 // never written.
+void free_split3(csff_plan* P) {
+  P->split32 = false;
+  P->split_block = 0;
+  for (Level& L : P->lv) {
+    if (L.s32.base) {
+      cudaFree(L.s32.base);
+      P->bytes -= L.s32.bytes;
+    }
+    L.s32 = csff::Split3();
+  }
+}
+
 csff_status alloc_split3(csff_plan* P) {
   const size_t nl = P->lv.size();
   for (size_t l = 0; l < nl; ++l) {
@@ -686,6 +698,7 @@ csff_status alloc_split3(csff_plan* P) {
     float2* base = nullptr;
     CS(dev_alloc(P, &base, total));
     S.base = base;
+    S.bytes = total * sizeof(float2);
     if (l > 0) {
       CK(cudaMemsetAsync(base, 0, total * sizeof(float2), P->stream), "zero split arrays");
       S.e = base + (total - ring);
@@ -951,11 +964,16 @@ csff_status csff_plan_create(const csff_problem* prob, const csff_opts* opts, vo
   // per-level ones 1.8 to 2.4 (65^3, k = 1; 257^3: 2.14 ms against 2.86)
   if (d == 3 && opts->smoother == CSFF_SMOOTHER_RBGS && opts->nu1 == 1 && opts->nu2 == 1 && P->lv.size() > 1 &&
       P->opts.precision == CSFF_PREC_MIXED) {
-    csff_status s = alloc_split3(P);
-    if (s != CSFF_OK) return fail(s);
-    P->split32 = true;
-    if ((P->split_block = csff::split3_block_level(P->lv)) > 0) {
-      cudaError_t e = csff::prepare_split3_block();
+    bool suits = false;
+    cudaError_t e = csff::split3_suits(P->lv, reinterpret_cast<unsigned*>(P->red_out), P->stream, &suits);
+    if (e != cudaSuccess) return fail(csff::cuda_fail(e, "coefficient range"));
+    if (suits) {
+      csff_status s = alloc_split3(P);
+      if (s != CSFF_OK) return fail(s);
+      P->split32 = true;
+    }
+    if (P->split32 && (P->split_block = csff::split3_block_level(P->lv)) > 0) {
+      e = csff::prepare_split3_block();
       if (e != cudaSuccess) return fail(csff::cuda_fail(e, "coarse block attributes"));
     }
   }
@@ -1258,9 +1276,6 @@ static csff_status user_q_levels(csff_plan* P) {
   for (const Level& L : P->lv) CK(csff::launch_coefs_from_q(P->dim, L, s), "coefficients");
   if (P->opts.smoother == CSFF_SMOOTHER_GMRES)
     for (const Level& L : P->lv) CK(csff::launch_gmres_coefs(L, s), "GMRES coefficients");
-  for (size_t l = 0; l + 1 < P->lv.size(); ++l) {
-    if (P->split32) CK(csff::split3_coefs(P->lv[l], P->prob.k * P->prob.k, s), "split coefficients");
-  }
   const Level& Lc = P->lv.back();
   std::vector<double2> qc((size_t)Lc.N);
   CK(cudaMemcpyAsync(qc.data(), Lc.q64, sizeof(double2) * qc.size(), cudaMemcpyDeviceToHost, s), "read q");
@@ -1272,8 +1287,11 @@ static csff_status user_q_levels(csff_plan* P) {
   CK(cudaMemcpy(P->coarse_inv, inv.data(), sizeof(double2) * inv.size(), cudaMemcpyHostToDevice), "upload inverse");
   CK(cudaMemcpy(P->coarse_inv32, inv32.data(), sizeof(float2) * inv32.size(), cudaMemcpyHostToDevice),
      "upload inverse");
-  // the fused FP32 tiles form q from the Gaussian factors: per-level kernels from now on
+  // the fused FP32 tiles form q from the Gaussian factors, and the colour-split 3D
+  // cycles hold 1/d relative to its value for the plan's k: per-level kernels from
+  // now on
   P->fused_lc = -1;
+  free_split3(P);
   P->user_q = true;
   P->dfq_ready = false;
   destroy_graphs(P);

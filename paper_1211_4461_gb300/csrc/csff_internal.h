@@ -77,6 +77,7 @@ struct Split3 {
   float2 *delta = nullptr, *e = nullptr;
   float2 d0{};                   // dr, db hold 1/d - d0
   void* base = nullptr;          // the one allocation behind them
+  size_t bytes = 0;
 };
 
 struct Level {
@@ -345,6 +346,9 @@ cudaError_t launch_first_residual(const double2* b, long long N, int s_exp, floa
 int split3_pitch(int m);                       // slots of a row of one colour
 // 1/d by colour from dinv64 (k2: the wavenumber's square, without potential)
 cudaError_t split3_coefs(Level& L, double k2, cudaStream_t s);
+// whether the smoothing levels' coefficients suit the colour-split cycles (waits
+// for the stream)
+cudaError_t split3_suits(const std::vector<Level>& lv, unsigned* scratch, cudaStream_t s, bool* suits);
 int split3_ring_pitch(int mc);                 // row pitch of a level's correction
 // the levels above `stop` down to its right-hand side (split, with the red half
 // sweep from zero; of the last level b32 in natural order): b and the

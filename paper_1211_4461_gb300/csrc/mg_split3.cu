@@ -34,6 +34,8 @@
 // weighting 123 before.
 #include "csff_internal.h"
 
+#include <cmath>
+
 namespace csff {
 namespace {
 
@@ -144,6 +146,17 @@ __global__ void k3s_split(const double2* __restrict__ dinv, float2 dc, float2 d0
   const long long s = p.row * HP + p.j;
   st2(red + s, o ? v[1] : v[0], o ? v[3] : v[2]);
   st2(black + s, o ? v[0] : v[1], o ? v[2] : v[3]);
+}
+
+// largest |6 c / d| of a level (as bits; a d of zero gives infinity or NaN)
+__global__ void k3s_worst(const double2* __restrict__ dinv, double c6, long long N, unsigned* __restrict__ worst) {
+  unsigned w = 0;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
+    const double2 d = dinv[i];
+    w = max(w, __float_as_uint((float)(c6 * hypot(d.x, d.y))));
+  }
+  w = __reduce_max_sync(0xffffffffu, w);
+  if ((threadIdx.x & 31) == 0) atomicMax(worst, w);
 }
 
 // The coarse correction e is kept with a ring of zeros: node (X, Y, Z), X, Y, Z
@@ -527,6 +540,29 @@ cudaError_t split3_coefs(Level& L, double k2, cudaStream_t s) {
   k3s_split<<<h.g, h.b, 0, s>>>(L.dinv64, dc, S.d0, L.m, HP, S.dr, S.db);
   count_launch();
   return cudaGetLastError();
+}
+
+// The line to the per-level kernels, by the smallest diagonal: 1/d is that of the
+// FP32 value of c (k3s_split), which moves it by |6 c / d| 2^-25 of itself.  One
+// cycle's error from an iterate against the per-level kernels', restated in FP32
+// (33^3, box of 15, Gaussian barriers): 0.9 at |6 c / d| of 3.7 and 4.9, 1.3 at 5.8,
+// 1.9 at 8.3, 3.8 at 10.8.
+constexpr float SPLIT3_WORST = 4.f;
+cudaError_t split3_suits(const std::vector<Level>& lv, unsigned* scratch, cudaStream_t s, bool* suits) {
+  cudaError_t e = cudaMemsetAsync(scratch, 0, sizeof(unsigned), s);
+  for (size_t l = 0; l + 1 < lv.size() && e == cudaSuccess; ++l) {
+    const Level& L = lv[l];
+    const long long blocks = (L.N + 255) / 256;
+    k3s_worst<<<(unsigned)(blocks < 152 * 8 ? blocks : 152 * 8), 256, 0, s>>>(L.dinv64, 6.0 * hypot(L.c.x, L.c.y), L.N,
+                                                                             scratch);
+    count_launch();
+    e = cudaGetLastError();
+  }
+  float worst = 0.f;
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&worst, scratch, sizeof(worst), cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  *suits = worst <= SPLIT3_WORST;                      // false for NaN
+  return e;
 }
 
 // the line lies at 15 points a side, where a level's passes last one CTA's

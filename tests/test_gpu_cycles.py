@@ -127,3 +127,41 @@ def test_vcycle_3d_rounding_from_an_iterate(csff, prec, R):
     plan.close()
     err = np.linalg.norm((ug.cpu().numpy().reshape(ref.shape) - ref).astype(complex)) / np.linalg.norm(ref.astype(complex))
     assert err <= 4 * unit
+
+
+def _cycle_error(csff, plan, n, coarsest, R, k, q, before=4):
+    """Error of one FP32 cycle, in units of 2^-24, from an iterate that `before` cycles left."""
+    m = plan.m
+    b = W.rand_complex((m,) * 3, 4).astype(np.complex64)
+    exact = Cycle3D(n, coarsest, R, k, np.complex128, q)
+    u = np.zeros((m,) * 3, complex)
+    for _ in range(before):
+        u = exact(u, b.astype(complex))
+    u = u.astype(np.complex64)
+    ref = exact(u.astype(complex), b.astype(complex))
+    ug = torch.from_numpy(u.ravel()).cuda()
+    plan.vcycle(ug, torch.from_numpy(b.ravel()).cuda())
+    got = ug.cpu().numpy().reshape(ref.shape)
+    return np.linalg.norm(got - ref) / np.linalg.norm(ref) * 2.0 ** 24
+
+
+OPTS3 = {"smoother": "rbgs", "nu1": 1, "nu2": 1, "coarsest_n": 5, "rel_tol": 1e-8, "precision": "mixed"}
+
+
+# coefficients far from the plan's k^2: an energy of 20 on a plan of k = 1, and
+# barriers whose diagonal 6 c - q comes near zero on a level (|6 c / d| = 10.8),
+# as samples and as a Gaussian plan.  Per-level passes restated: 0.7 to 2.4 units
+@pytest.mark.parametrize("E,V,kind", [(20.0, 2.0, "sampled"), (1.0, 40.0, "sampled"), (1.0, 40.0, "gauss"),
+                                      (1.0, 20.0, "sampled")])
+def test_vcycle_3d_rounding_on_other_coefficients(csff, E, V, kind):
+    n, R, w = 33, 15.0, 1.5
+    g = math.pi / 6
+    k = math.sqrt(2 * E) if kind == "gauss" else 1.0
+    plan = csff.Plan(W.problem(3, n, R, g, k, [W.gauss(-V / E, w)] if kind == "gauss" else []), OPTS3)
+    z = (-R + np.arange(1, n - 1) * 2 * R / (n - 1)) * np.exp(1j * g)
+    ax = np.exp(-z * z / w)
+    q = 2 * E - 2 * V * ax[:, None, None] * ax[None, :, None] * ax[None, None, :]
+    if kind == "sampled":
+        plan.set_potential(torch.from_numpy(q.ravel()).cuda())
+    assert _cycle_error(csff, plan, n, 5, R, k, q) <= 4.0
+    plan.close()
