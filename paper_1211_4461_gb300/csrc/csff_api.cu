@@ -969,8 +969,14 @@ csff_status csff_plan_create(const csff_problem* prob, const csff_opts* opts, vo
     if (e != cudaSuccess) return fail(csff::cuda_fail(e, "coefficient range"));
     if (suits) {
       csff_status s = alloc_split3(P);
-      if (s != CSFF_OK) return fail(s);
-      P->split32 = true;
+      if (s == CSFF_OK) {
+        P->split32 = true;
+      } else {
+        free_split3(P);
+        if (s != CSFF_ERR_OOM) return fail(s);
+        cudaGetLastError();                    // without room for the arrays: the per-level kernels
+        csff::set_error("");
+      }
     }
     if (P->split32 && (P->split_block = csff::split3_block_level(P->lv)) > 0) {
       e = csff::prepare_split3_block();

@@ -165,3 +165,31 @@ def test_vcycle_3d_rounding_on_other_coefficients(csff, E, V, kind):
         plan.set_potential(torch.from_numpy(q.ravel()).cuda())
     assert _cycle_error(csff, plan, n, 5, R, k, q) <= 4.0
     plan.close()
+
+
+def test_plan_3d_without_room_for_the_split_arrays(csff):
+    """A device with room for the plan but not for the colour-split arrays gives
+    a plan that cycles per level."""
+    n, R, k = 257, 15.0, 1.0
+    prob = W.problem(3, n, R, math.pi / 6, k, [])
+    plan = csff.Plan(prob, OPTS3)
+    m, full = plan.m, plan.describe()["device_bytes"]
+    b = torch.from_numpy(W.rand_complex((m,) * 3, 4).astype(np.complex64)).cuda().ravel()
+    want = torch.zeros_like(b)
+    plan.vcycle(want, b)
+    plan.set_potential(torch.full((m ** 3,), k * k, dtype=torch.complex128, device="cuda"))
+    split = full - plan.describe()["device_bytes"]        # what the plan gave back
+    plan.close()
+    assert split > 400 << 20
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    # all but the plan's own arrays and some room for their granules
+    fill = torch.empty(torch.cuda.mem_get_info()[0] - (full - split) - (200 << 20), dtype=torch.uint8, device="cuda")
+    plan = csff.Plan(prob, OPTS3)
+    assert plan.describe()["device_bytes"] == full - split
+    got = torch.zeros_like(b)
+    plan.vcycle(got, b)
+    plan.close()
+    del fill
+    torch.cuda.empty_cache()
+    assert torch.linalg.vector_norm(got - want) <= 1e-5 * torch.linalg.vector_norm(want)
