@@ -53,11 +53,18 @@ template <typename C> __device__ __forceinline__ C cfma(C a, C b, C c) {
   return mk<C>(fma(b.x, c.x, fma(-b.y, c.y, a.x)), fma(b.x, c.y, fma(b.y, c.x, a.y)));
 }
 
-// d^{-1} t.  FP32 cycles hold d^{-1} as d0 + dv, d0 the level's FP32 value
-// without the potential and dv the FP32 difference: rounding d^{-1} itself
-// shifts every equation by the same 2^-25 |d|, which the folded residual (no
-// explicit b - A u) would pass to the coarse levels as a residual.
-__device__ __forceinline__ float2 dinv_mul(float2 d0, float2 dv, float2 t) { return cfma(cmul(d0, t), dv, t); }
+// d^{-1} t.  d^{-1} is held as d0 + dv, d0 the level's FP32 value without the
+// potential and dv the FP32 difference: rounding d^{-1} itself shifts every
+// equation by the same 2^-25 |d|, which the folded residual (no explicit b - A u)
+// would pass to the coarse levels as a residual.  dv's products come first: added
+// to a rounded d0 t, terms below half its last place would be lost at every point
+// alike and leave two thirds of that shift (a cycle from an iterate that cycles
+// left, 65^3, k = 1, no potential: 20.1 units of 2^-24 off on a box of 5, 5.8 on one
+// of 15; in this order 3.0 and 1.9; per-level passes 2.1 and 1.7).
+__device__ __forceinline__ float2 dinv_mul(float2 d0, float2 dv, float2 t) {
+  return make_float2(fmaf(d0.x, t.x, fmaf(-d0.y, t.y, fmaf(dv.x, t.x, -(dv.y * t.y)))),
+                     fmaf(d0.x, t.y, fmaf(d0.y, t.x, fmaf(dv.x, t.y, dv.y * t.x))));
+}
 
 // Launches of at most one CTA an SM (the small levels) let their dependent be set
 // up as soon as they have passed their own wait; a sweep's and a full weighting's
@@ -149,11 +156,11 @@ __global__ void k3s_split(const double2* __restrict__ dinv, float2 dc, float2 d0
 }
 
 // largest |6 c / d| of a level (as bits; a d of zero gives infinity or NaN)
-__global__ void k3s_worst(const double2* __restrict__ dinv, double c6, long long N, unsigned* __restrict__ worst) {
+__global__ void k3s_worst(const float2* __restrict__ dinv, float c6, long long N, unsigned* __restrict__ worst) {
   unsigned w = 0;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
-    const double2 d = dinv[i];
-    w = max(w, __float_as_uint((float)(c6 * hypot(d.x, d.y))));
+    const float2 d = make_float2(c6 * dinv[i].x, c6 * dinv[i].y);
+    w = max(w, __float_as_uint(sqrtf(fmaf(d.x, d.x, d.y * d.y))));
   }
   w = __reduce_max_sync(0xffffffffu, w);
   if ((threadIdx.x & 31) == 0) atomicMax(worst, w);
@@ -553,8 +560,8 @@ cudaError_t split3_suits(const std::vector<Level>& lv, unsigned* scratch, cudaSt
   for (size_t l = 0; l + 1 < lv.size() && e == cudaSuccess; ++l) {
     const Level& L = lv[l];
     const long long blocks = (L.N + 255) / 256;
-    k3s_worst<<<(unsigned)(blocks < 152 * 8 ? blocks : 152 * 8), 256, 0, s>>>(L.dinv64, 6.0 * hypot(L.c.x, L.c.y), L.N,
-                                                                             scratch);
+    k3s_worst<<<(unsigned)(blocks < 152 * 8 ? blocks : 152 * 8), 256, 0, s>>>(
+        L.dinv32, (float)(6.0 * std::hypot(L.c.x, L.c.y)), L.N, scratch);
     count_launch();
     e = cudaGetLastError();
   }

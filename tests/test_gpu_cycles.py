@@ -107,7 +107,7 @@ class Cycle3D:
 # a cycle from an iterate that earlier cycles left.  A few dozen roundings a
 # point, most of them averaged: 1.0 to 2.4 units of the type in the norm for
 # per-level passes restated on the CPU
-@pytest.mark.parametrize("prec,R", [("fp64", 5.0), ("fp64", 15.0)])
+@pytest.mark.parametrize("prec,R", [("fp64", 5.0), ("fp64", 15.0), ("mixed", 5.0), ("mixed", 15.0)])
 def test_vcycle_3d_rounding_from_an_iterate(csff, prec, R):
     n, coarsest, k = 65, 5, 1.0
     unit, ct, nt = (2.0 ** -53, np.clongdouble, np.complex128) if prec == "fp64" else (2.0 ** -24, np.complex128,
@@ -143,6 +143,26 @@ def _cycle_error(csff, plan, n, coarsest, R, k, q, before=4):
     plan.vcycle(ug, torch.from_numpy(b.ravel()).cuda())
     got = ug.cpu().numpy().reshape(ref.shape)
     return np.linalg.norm(got - ref) / np.linalg.norm(ref) * 2.0 ** 24
+
+
+# one level above the direct solve (its right-hand side goes out in natural order)
+# and several, rows of a slot pair up to several blocks' worth
+@pytest.mark.parametrize("n,coarsest,R", [(5, 3, 3.0), (7, 4, 3.0), (13, 4, 3.0), (19, 10, 3.0), (37, 10, 5.0),
+                                          (41, 6, 5.0), (65, 5, 5.0), (73, 10, 5.0)])
+def test_vcycle_3d_from_an_iterate_over_grids(csff, n, coarsest, R):
+    k, opts = 1.0, dict(OPTS3, coarsest_n=coarsest)
+    plan = csff.Plan(W.problem(3, n, R, math.pi / 6, k, []), opts)
+    levels = O.make_hierarchy(O.problem_from_dict(W.problem(3, n, R, math.pi / 6, k, [])), coarsest)
+    lu, o, m = O.coarse_factor(levels[-1]), O.opts_from_dict(opts), plan.m
+    b = W.rand_complex((m,) * 3, 4).astype(np.complex64)
+    u = O.vcycle(levels, lu, 0, np.zeros((m,) * 3, complex), b.astype(complex), o).astype(np.complex64)
+    ref = O.vcycle(levels, lu, 0, u.astype(complex), b.astype(complex), o)
+    ug = torch.from_numpy(u.ravel()).cuda()
+    plan.vcycle(ug, torch.from_numpy(b.ravel()).cuda())
+    plan.close()
+    # rounding as above (at most 4 units), and the coarsest product's in FP32, a
+    # few units of a correction that on two levels is most of the result
+    assert np.linalg.norm(ug.cpu().numpy().reshape(ref.shape) - ref) <= 16 * 2.0 ** -24 * np.linalg.norm(ref)
 
 
 OPTS3 = {"smoother": "rbgs", "nu1": 1, "nu2": 1, "coarsest_n": 5, "rel_tol": 1e-8, "precision": "mixed"}
