@@ -827,7 +827,7 @@ __global__ void __launch_bounds__(digits::NT, 1)
                 const unsigned char* __restrict__ skip, int skip_tiles, double2* __restrict__ T, int* __restrict__ err,
                 int tile0, const int* __restrict__ field, const int* __restrict__ map, FFWaits waits) {
   using namespace digits;
-  constexpr int ND = F::ND, NA = F::NA, SUB = F::SUB, B_SET = F::B_SET, OFF_BAR = F::OFF_BAR, OFF_ACT = F::OFF_ACT;
+  constexpr int ND = F::ND, DG = F::DG, NA = F::NA, SUB = F::SUB, B_SET = F::B_SET, OFF_BAR = F::OFF_BAR, OFF_ACT = F::OFF_ACT;
   if (spread && !digits_selected(spread)) return;      // another kernel takes this launch
   extern __shared__ __align__(1024) unsigned char dsm_raw[];
   unsigned char* base = dsm_raw + ((1024 - (saddr(dsm_raw) & 1023)) & 1023);
@@ -949,12 +949,17 @@ __global__ void __launch_bounds__(digits::NT, 1)
         if (s % SUB == 0) ok = ok && bar_wait(a_full + 8 * slot, aph, abort, waits.ns);
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         constexpr int TKK = 2 * TK;
-        const uint32_t nd = (uint32_t)(TKK * (ND - s));
+        const uint32_t nd = (uint32_t)(TKK * min(ND, DG - s));       // columns: digits of B for the kept diagonals
         const uint32_t d = tm + (uint32_t)(p * ACC + TKK * s), sA = sbase + slot * A_DIG + 64 * (s % SUB);
         if (__all_sync(0xffffffffu, ok) && elect_one()) {
 #pragma unroll
-          for (int kk = 0; kk < 4 / SUB; ++kk)
-            mma(d, desc(sA + 32 * kk), desc(sB + 32 * kk), idesc | ((nd >> 3) << 17), (s > 0 || kk > 0) ? 1u : 0u);
+          for (int kk = 0; kk < 4 / SUB; ++kk) {
+            const bool more = DG > ND && s == DG - ND;             // its last columns start a diagonal
+            const uint32_t n1 = more && kk == 0 ? nd - TKK : nd;
+            mma(d, desc(sA + 32 * kk), desc(sB + 32 * kk), idesc | ((n1 >> 3) << 17), (s > 0 || kk > 0) ? 1u : 0u);
+            if (more && kk == 0)
+              mma(d + n1, desc(sA), desc(sB + (n1 / TKK) * B_DIG), idesc | ((uint32_t)(TKK >> 3) << 17), 0u);
+          }
           if (s % SUB == SUB - 1) commit(a_empty + 8 * slot);
         }
         __syncwarp();
@@ -1025,9 +1030,9 @@ __global__ void __launch_bounds__(digits::NT, 1)
         // one part at a time: both take more registers than 18 warps have
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
-          uint32_t v[ND][EK];
+          uint32_t v[DG][EK];
 #pragma unroll
-          for (int d = 0; d < ND; ++d) CSFF_TMEM_LD4(v[d], tl + (uint32_t)(p * ACC + 2 * TK * d + TK * c));
+          for (int d = 0; d < DG; ++d) CSFF_TMEM_LD4(v[d], tl + (uint32_t)(p * ACC + 2 * TK * d + TK * c));
           asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
           if (c == 1) {
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -1036,18 +1041,18 @@ __global__ void __launch_bounds__(digits::NT, 1)
           }
 #pragma unroll
           for (int j = 0; j < EK; ++j) {
-            float q[ND];
+            float q[DG];
 #pragma unroll
-            for (int d = 0; d < ND; ++d) q[d] = __uint_as_float(v[d][j]);
+            for (int d = 0; d < DG; ++d) q[d] = __uint_as_float(v[d][j]);
             S[c][j] += fixed_to_double(join_fixed(q), es[j]);
           }
         }
       } else {
-        uint32_t v[2][ND][EK];
+        uint32_t v[2][DG][EK];
 #pragma unroll
         for (int c = 0; c < 2; ++c)
 #pragma unroll
-          for (int d = 0; d < ND; ++d) CSFF_TMEM_LD4(v[c][d], tl + (uint32_t)(p * ACC + 2 * TK * d + TK * c));
+          for (int d = 0; d < DG; ++d) CSFF_TMEM_LD4(v[c][d], tl + (uint32_t)(p * ACC + 2 * TK * d + TK * c));
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncwarp();
@@ -1062,9 +1067,9 @@ __global__ void __launch_bounds__(digits::NT, 1)
           E[2 * j + 1] = En1;
 #pragma unroll
           for (int c = 0; c < 2; ++c) {
-            float2 q[7], h, l, t, e;
+            float2 q[DG], h, l, t, e;
 #pragma unroll
-            for (int d = 0; d < 7; ++d)
+            for (int d = 0; d < DG; ++d)
               q[d] = make_float2(__uint_as_float(v[c][d][2 * j]), __uint_as_float(v[c][d][2 * j + 1]));
             join(q, h, l);
             two_sum(__fmul2_rn(H[c][j], fa), __fmul2_rn(h, fs), t, e);

@@ -9,17 +9,32 @@
 // digits balanced (round to nearest), stored as BF16 integers.  A product of two
 // digits is at most 2^14; a block's sum over 64 real terms (32 complex nodes)
 // and the at most 7 digit pairs (s, t) of one diagonal s + t = D stays below
-// 2^23, so the FP32 accumulators hold it exactly.  Diagonals D = 2..8 are kept
-// (28 of the 49 pairs); the rest lies below 2^-53 of the blocks' scales.
+// 2^23, so the FP32 accumulators hold it exactly.  Diagonals D = 2..9 are kept (34
+// of the 49 pairs).  Cutting into slices whose products add up exactly is a
+// published method (Ozaki, Ogita, Oishi and Rump, Numer. Algorithms 59, 2012).
 //
-// When it runs.  The representation is relative to the block maxima, so the
-// kernel is taken when for every block that a tile keeps the scales ex + eg lie
-// at most MARGIN binades over L, the lower bound of the sum of the terms'
-// magnitudes that the skip kernel forms (phases that vary by less than about
-// 2^10 over 32 nodes: k h sin(gamma) 32 < 7).  Measured errors of a map against a
-// longer sum, relative to the sum of the terms' magnitudes (129^2 to 513^2, k = 1
-// and 2): 2^-52.1 to 2^-51.2 at the worst angle, 2^-50.5 to 2^-49.3 for the
-// double-float kernel, which runs beyond that range.
+// Error of a block, relative to the product 2^(ex + eg) of the two scales: five
+// pairs of at most 2^14 at 2^-78 are dropped for each of 64 real products (2^-55.7,
+// 2^-61 for digits of random signs), and the operands' remainders of up to
+// 2^-56 each enter 64 times (2^-49 at most; 2^-54.8 rms for dense blocks, less where
+// few values count).
+//
+// When it runs.  These errors are relative to the block maxima, so the kernel is
+// taken when for every block that a tile keeps the scales ex + eg lie at most
+// MARGIN binades over L, the lower bound of the sum of the terms' magnitudes that
+// the skip kernel forms (2 for constant phases, more as they vary over a block:
+// about k h sin(gamma) 32 < 3.5).  The line is where the error reaches the
+// double-float kernel's, which runs beyond it.  Both restated on the CPU on single
+// blocks against a longer sum, relative to the sum of the terms' magnitudes, by
+// margin, as binades of the rms error over the double-float kernel's (2^-48.5 to
+// 2^-45.7):
+//   fields                                margin 6     8      9     10     11     12
+//   random                                     -3.7  -3.5  -3.4  -3.3  -3.2  -3.8
+//   balanced against the phases                -4.5  -3.6  -2.8  -1.9  -1.1  -0.6
+//   falling three times as fast                -4.6  -2.9  -1.7  -0.9  -0.1  -0.3
+//   three nodes where the phase is smallest    -2.4  -1.5  -0.6  +0.4  +1.1  +1.9
+//   a single node there                        -1.8  -0.2  +0.4  +1.5  +2.3  +3.1
+// (with diagonals up to 8 and a margin of 12, as before, up to 3.9 binades larger.)
 //
 // Kernel.  D[rho][j] = sum_K A[rho][K] B[j][K], K = (re, im) of 32 nodes; a
 // CTA takes 128 rows of g (A) and 16 phase rows (B: rows j < 16 give the real
@@ -49,8 +64,8 @@ constexpr int B_DIG = 2 * TK * 128;
 constexpr int MAX_NB = 1024;                   // blocks of a row
 constexpr int EPI_WARPS = 16, NT = 32 * (EPI_WARPS + 2);
 constexpr int EK = TK * 4 / EPI_WARPS;           // phase rows of an epilogue warp
-constexpr int TMEM_COLS = 512, ACC = 256;      // columns of one set of accumulators (7 x 32 used)
-constexpr int MARGIN = 12;
+constexpr int TMEM_COLS = 512, ACC = 256;      // columns of one set of accumulators, one diagonal in 32
+constexpr int MARGIN = 8;
 
 // A form of the contraction: ND digits a value, NA A slots in the ring, SUB
 // scale blocks in the 32 nodes of a row of B.
@@ -59,12 +74,13 @@ constexpr int MARGIN = 12;
 //  nodes; each block's diagonals fill a set of accumulators.
 template <int ND_, int NA_, int SUB_> struct Form {
   static constexpr int ND = ND_, NA = NA_, SUB = SUB_;
+  static constexpr int DG = 8;                 // diagonals kept
   static constexpr int BITS = 8 * ND - 1;      // fixed-point bits below the scale
   static constexpr int A_SLOTS = ND / SUB;     // slots of a block
   static constexpr int B_SET = ND * B_DIG;
   static constexpr int OFF_BAR = NA * A_DIG + 2 * B_SET, OFF_ACT = OFF_BAR + 512;
   static constexpr int SMEM = OFF_ACT + MAX_NB * 2 + 1024;
-  static_assert(SMEM <= 227 * 1024 && ND % SUB == 0 && 2 * TK * ND <= ACC, "shared and tensor memory");
+  static_assert(SMEM <= 227 * 1024 && ND % SUB == 0 && ND <= DG && 2 * TK * DG <= ACC, "shared and tensor memory");
 };
 using Form2 = Form<7, 10, 1>;
 using Form3 = Form<8, 9, 2>;
@@ -190,12 +206,13 @@ __device__ __forceinline__ void two_sum(float2 x, float2 y, float2& t, float2& e
 __device__ __forceinline__ float pow2_or_0(int d) { return __int_as_float(max(d + 127, 0) << 23); }
 __device__ __forceinline__ float2 both(float a) { return make_float2(a, a); }
 
-// h + l = sum_{d=0..6} p[d] 2^-8d: the four leading terms by exact sums (their
-// digit sums reach 2^23, eight bits apart), the three trailing ones, whose
+// h + l = sum_{d=0..7} p[d] 2^-8d: the four leading terms by exact sums (their
+// digit sums reach 2^23, eight bits apart), the four trailing ones, whose
 // roundings lie below 2^-55 of the scale, by multiply-adds
-__device__ __forceinline__ void join(const float2 (&p)[7], float2& h, float2& l) {
+__device__ __forceinline__ void join(const float2 (&p)[8], float2& h, float2& l) {
   const float2 w = both(0x1p-8f);
-  float2 q = __ffma2_rn(p[6], w, p[5]);
+  float2 q = __ffma2_rn(p[7], w, p[6]);
+  q = __ffma2_rn(q, w, p[5]);
   q = __ffma2_rn(q, w, p[4]);
   float2 e3, e2, e1, t;
   two_sum(p[3], __fmul2_rn(q, w), t, e3);

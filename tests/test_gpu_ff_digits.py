@@ -48,3 +48,36 @@ def test_nan_direction_3d_gives_nan(csff, component):
     others = np.arange(len(al)) != 77
     assert np.isnan(F1[77].real) and np.isnan(F1[77].imag)
     assert np.all(np.isfinite(F0)) and np.array_equal(F0[others], F1[others]) and np.array_equal(E0[others], E1[others])
+
+
+# fields (far over the incident wave's) that live where the phases of a block of
+# 32 nodes are smallest, so that the block's scales lie far over its terms: a
+# single node of a row, three of them, or a fall three times the phases' growth;
+# phases that vary by var binades over the block, below, around and above the
+# digit form's line.  The contraction against the FP64 one of the same call (the
+# waits made to run out), whose rounding is 2^-52: no further apart than the
+# double-float form's rms error of 2^-48
+@pytest.mark.parametrize("var", [2.0, 4.5, 5.5, 6.5, 8.3, 9.5])
+@pytest.mark.parametrize("nodes", [1, 3, 32])
+def test_far_field_2d_of_unbalanced_blocks(csff, var, nodes):
+    n, R, g = 129, 10.0, math.pi / 6
+    h = 2 * R / (n - 1)
+    k = var * math.log(2.0) / (32 * h * math.sin(g))
+    prob = W.problem(2, n, R, g, k, [W.gauss(1.0, 1e6)])
+    plan = csff.Plan(prob, {"smoother": "jacobi", "nu1": 1, "nu2": 1, "coarsest_n": 5, "rel_tol": 1e-8,
+                            "precision": "fp64"})
+    m = plan.m
+    u, i = np.zeros((m, m), dtype=complex), np.arange(nodes)
+    u[60, 32:32 + nodes] = W.rand_complex(nodes, 7) * (1e40 * 2.0 ** (-3 * var * i / 32 * (nodes == 32)))
+    t = np.linspace(-0.3, 0.3, 97)
+    al = np.ascontiguousarray(np.stack([np.cos(t), np.sin(t)], axis=1))
+    eta = np.array([[0.6, 0.8]])
+    F, E = _far(plan, eta, u, al)
+    plan.debug_far_field_waits(1, wait_ms=20)
+    F64, E64 = _far(plan, eta, u, al)
+    digits = plan.debug_far_field_waits(0)
+    plan.close()
+    assert digits or var > 4.5
+    tn, e2 = O.far_field(O.problem_from_dict(prob), u, eta[0], al, return_terms_norm=True)[:0:-1]
+    diff = np.abs(F * 2.0 ** (E.astype(np.float64) - e2) - F64 * 2.0 ** (E64.astype(np.float64) - e2)) / tn
+    assert np.sqrt(np.mean(diff ** 2)) <= 2.0 ** -48
