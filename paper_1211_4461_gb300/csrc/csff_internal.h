@@ -122,20 +122,19 @@ struct FFBuffers {
   double2 *dg = nullptr, *dxt = nullptr, *dyt = nullptr, *dzt = nullptr, *dT = nullptr;
   double *dal = nullptr, *dux = nullptr;
   int *dxr = nullptr, *ds1 = nullptr, *dmisc = nullptr;
-  // double-float stage 1: split operands, block exponents, spread flags [2]
-  size_t xdf = 0, gdf = 0, exs = 0, egs = 0, xsm = 0, gsm = 0;
-  float4 *dxdf = nullptr, *dgdf = nullptr;
-  float2 *dxsm = nullptr, *dgsm = nullptr;   // re + im of the split operands
+  // operands of the contraction that runs, split or (ff_digits.cuh) cut into
+  // digits: the phases' and g's
+  size_t xop = 0, gop = 0;
+  unsigned char *dxop = nullptr, *dgop = nullptr;
+  FFWaits waits;
+  // 2D stage 1: block exponents, spread flags [2] and the digit form's margin
+  size_t exs = 0, egs = 0;
   int *dex = nullptr, *deg = nullptr, *dspread = nullptr;
   // block bounds for skipping negligible blocks and the per-tile skip flags
   size_t xlo = 0, ghi = 0, skip = 0;
   int *dxlo = nullptr, *dghi = nullptr;
   unsigned char* dskip = nullptr;
   size_t skip_used = 0;       // flags written by the last 2D far field
-  // digit operands of the tensor-core contraction (ff_digits.cuh)
-  size_t xdig = 0, gdig = 0;
-  unsigned char *dxdig = nullptr, *dgdig = nullptr;
-  FFWaits waits;
   // tensor-core 3D stage A: pre-swizzled split phase operand, per-column and
   // per-row exponents, [spread_g, spread_P, error word]
   size_t tcb = 0, tce = 0;

@@ -1584,9 +1584,9 @@ static int dig3_chunk(int m, int T) {
 static cudaError_t dig3_ensure(FFBuffers& B, int m, int T, int chunk, csff_plan* P) {
   using F = digits::Form3;
   const size_t nb = (m + digits::KB - 1) / digits::KB, kt = (T + digits::TK - 1) / digits::TK;
-  cudaError_t e = ensure((void**)&B.dxdig, B.xdig, kt * nb * F::B_SET, P);
+  cudaError_t e = ensure((void**)&B.dxop, B.xop, kt * nb * F::B_SET, P);
   if (e == cudaSuccess)
-    e = ensure((void**)&B.dgdig, B.gdig, (size_t)chunk * nb * F::SUB * F::A_SLOTS * digits::A_DIG, P);
+    e = ensure((void**)&B.dgop, B.gop, (size_t)chunk * nb * F::SUB * F::A_SLOTS * digits::A_DIG, P);
   if (e == cudaSuccess)
     e = ensure((void**)&B.dtce, B.tce, sizeof(int) * nb * F::SUB * ((size_t)T + (size_t)chunk * digits::TM), P);
   return e;
@@ -1600,12 +1600,12 @@ static cudaError_t stage_a_digits(FFBuffers& B, const double2* zt, int T, const 
   const long long ncol = (long long)m * m;
   const int nb = (m + KB - 1) / KB, kt = (T + TK - 1) / TK, tiles = (int)((ncol + TM - 1) / TM);
   int *ex = B.dtce, *eg = B.dtce + (size_t)T * nb * F::SUB;
-  k_cut_phase3<<<(unsigned)(((long long)kt * TK * nb * 32 + 255) / 256), 256, 0, s>>>(zt, nullptr, m, T, ex, B.dxdig);
+  k_cut_phase3<<<(unsigned)(((long long)kt * TK * nb * 32 + 255) / 256), 256, 0, s>>>(zt, nullptr, m, T, ex, B.dxop);
   count_launch();
   for (int t0 = 0; t0 < tiles; t0 += chunk) {
     const int n = std::min(chunk, tiles - t0);
-    k_cut_field3<<<dim3(n, nb * F::SUB), TM, 0, s>>>(g, m, ncol, t0, eg, B.dgdig);
-    k_ff_digits<F><<<dim3(n, kt), NT, F::SMEM, s>>>(B.dgdig, B.dxdig, ex, T, eg, (int)ncol, nb, nullptr, nullptr, 0, T1,
+    k_cut_field3<<<dim3(n, nb * F::SUB), TM, 0, s>>>(g, m, ncol, t0, eg, B.dgop);
+    k_ff_digits<F><<<dim3(n, kt), NT, F::SMEM, s>>>(B.dgop, B.dxop, ex, T, eg, (int)ncol, nb, nullptr, nullptr, 0, T1,
                                                     B.dmisc + 2, t0, nullptr, nullptr, B.waits);
     count_launch(2);
   }
@@ -1634,9 +1634,9 @@ static size_t dig3_b_ints(const YTiles& y, int m, int T) {
 static cudaError_t dig3_ensure_b(FFBuffers& B, const YTiles& y, int m, int T, csff_plan* P) {
   using F = digits::Form3;
   const size_t nb = (m + digits::KB - 1) / digits::KB, tiles = (m + digits::TM - 1) / digits::TM;
-  cudaError_t e = ensure((void**)&B.dxdig, B.xdig, y.field.size() * nb * F::B_SET, P);
+  cudaError_t e = ensure((void**)&B.dxop, B.xop, y.field.size() * nb * F::B_SET, P);
   if (e == cudaSuccess)
-    e = ensure((void**)&B.dgdig, B.gdig, T * tiles * nb * F::SUB * F::A_SLOTS * digits::A_DIG, P);
+    e = ensure((void**)&B.dgop, B.gop, T * tiles * nb * F::SUB * F::A_SLOTS * digits::A_DIG, P);
   if (e == cudaSuccess) e = ensure((void**)&B.dtce, B.tce, sizeof(int) * dig3_b_ints(y, m, T), P);
   return e;
 }
@@ -1651,9 +1651,9 @@ static cudaError_t stage_b_digits(FFBuffers& B, const double2* yt, const YTiles&
   if ((e = cudaMemcpyAsync(map, y.map.data(), sizeof(int) * rows, cudaMemcpyHostToDevice, s)) != cudaSuccess ||
       (e = cudaMemcpyAsync(field, y.field.data(), sizeof(int) * kt, cudaMemcpyHostToDevice, s)) != cudaSuccess)
     return e;
-  k_cut_phase3<<<(unsigned)(((long long)rows * nb * 32 + 255) / 256), 256, 0, s>>>(yt, map, m, rows, ex, B.dxdig);
-  k_cut_field3<<<dim3(tiles, nbs, T), TM, 0, s>>>(T1, m, m, 0, eg, B.dgdig);
-  k_ff_digits<F><<<dim3(tiles, kt), NT, F::SMEM, s>>>(B.dgdig, B.dxdig, ex, rows, eg, m, nb, nullptr, nullptr, 0, T2,
+  k_cut_phase3<<<(unsigned)(((long long)rows * nb * 32 + 255) / 256), 256, 0, s>>>(yt, map, m, rows, ex, B.dxop);
+  k_cut_field3<<<dim3(tiles, nbs, T), TM, 0, s>>>(T1, m, m, 0, eg, B.dgop);
+  k_ff_digits<F><<<dim3(tiles, kt), NT, F::SMEM, s>>>(B.dgop, B.dxop, ex, rows, eg, m, nb, nullptr, nullptr, 0, T2,
                                                       B.dmisc + 2, 0, field, map, B.waits);
   count_launch(3);
   return cudaGetLastError();
@@ -1691,9 +1691,9 @@ csff_status far_field_gave_up(csff_plan* P, int* gave_up) {
 void free_ff_buffers(csff_plan* P) {
   FFBuffers& b = P->ff;
   for (void* p : {(void*)b.dg, (void*)b.dxt, (void*)b.dyt, (void*)b.dzt, (void*)b.dT, (void*)b.dal,
-                  (void*)b.dux, (void*)b.dxr, (void*)b.ds1, (void*)b.dmisc, (void*)b.dxdf, (void*)b.dgdf, (void*)b.dxsm, (void*)b.dgsm,
+                  (void*)b.dux, (void*)b.dxr, (void*)b.ds1, (void*)b.dmisc,
                   (void*)b.dex, (void*)b.deg, (void*)b.dspread, (void*)b.dtcb, (void*)b.dtce, (void*)b.dtcflag,
-                  (void*)b.dxlo, (void*)b.dghi, (void*)b.dskip, (void*)b.dxdig, (void*)b.dgdig})
+                  (void*)b.dxlo, (void*)b.dghi, (void*)b.dskip, (void*)b.dxop, (void*)b.dgop})
     if (p) cudaFree(p);
   b = FFBuffers{};
 }
@@ -1909,26 +1909,32 @@ csff_status far_field_one(csff_plan* P, const double* eta_host, const double2* u
                                                                  L.h, P->prob.k, sg, cg, B.dmisc, B.dxt, B.dyt,
                                                                  B.dzt, B.ds1, B.dmisc + 1);
   count_launch();
-  // operands of the double-float contraction
   const int nbk = (m + DKB - 1) / DKB;
-  if ((e = ensure((void**)&B.dxdf, B.xdf, sizeof(float4) * (size_t)n_ux * nbk * DKB, P)) != cudaSuccess ||
-      (e = ensure((void**)&B.dgdf, B.gdf, sizeof(float4) * (size_t)R * nbk * DKB, P)) != cudaSuccess ||
-      (e = ensure((void**)&B.dxsm, B.xsm, sizeof(float2) * (size_t)n_ux * nbk * DKB, P)) != cudaSuccess ||
-      (e = ensure((void**)&B.dgsm, B.gsm, sizeof(float2) * (size_t)R * nbk * DKB, P)) != cudaSuccess ||
-      (e = ensure((void**)&B.dex, B.exs, sizeof(int) * (size_t)n_ux * nbk, P)) != cudaSuccess ||
+  if ((e = ensure((void**)&B.dex, B.exs, sizeof(int) * (size_t)n_ux * nbk, P)) != cudaSuccess ||
       (e = ensure((void**)&B.deg, B.egs, sizeof(int) * (size_t)R * nbk, P)) != cudaSuccess ||
       (e = ensure((void**)&B.dxlo, B.xlo, sizeof(int) * (size_t)n_ux * nbk, P)) != cudaSuccess ||
       (e = ensure((void**)&B.dghi, B.ghi, sizeof(int) * (size_t)R * nbk, P)) != cudaSuccess)
     return cuda_fail(e, "far field scratch");
   if (!B.dspread && (e = cudaMalloc((void**)&B.dspread, 3 * sizeof(int))) != cudaSuccess)
     return cuda_fail(e, "far field scratch");
-  // the digit contraction: 2D, where its operands fit (without room for them the
-  // double-float one runs)
+  // Operands of whichever contraction the device selects, in the same memory: the
+  // digit form (2D), where its larger ones fit, or the double-float form's
+  // (per node 16 bytes of pairs, then 8 of their sums).
   const int gxt = (int)((R + digits::TM - 1) / digits::TM), gkt = (n_ux + digits::TK - 1) / digits::TK;
+  const size_t xn = (size_t)n_ux * nbk * DKB, gn = (size_t)R * nbk * DKB, node = sizeof(float4) + sizeof(float2);
   bool dig = d == 2 && nbk <= digits::MAX_NB &&
-             ensure((void**)&B.dxdig, B.xdig, (size_t)gkt * nbk * digits::Form2::B_SET, P) == cudaSuccess &&
-             ensure((void**)&B.dgdig, B.gdig, (size_t)gxt * nbk * digits::Form2::ND * digits::A_DIG, P) == cudaSuccess;
-  if (!dig) cudaGetLastError();
+             ensure((void**)&B.dxop, B.xop, std::max(node * xn, (size_t)gkt * nbk * digits::Form2::B_SET), P) ==
+                 cudaSuccess &&
+             ensure((void**)&B.dgop, B.gop,
+                    std::max(node * gn, (size_t)gxt * nbk * digits::Form2::ND * digits::A_DIG), P) == cudaSuccess;
+  if (!dig) {
+    cudaGetLastError();
+    if ((e = ensure((void**)&B.dxop, B.xop, node * xn, P)) != cudaSuccess ||
+        (e = ensure((void**)&B.dgop, B.gop, node * gn, P)) != cudaSuccess)
+      return cuda_fail(e, "far field scratch");
+  }
+  float4 *const xdf = (float4*)B.dxop, *const gdfv = (float4*)B.dgop;
+  float2 *const xsum = (float2*)(xdf + xn), *const gsum = (float2*)(gdfv + gn);
   // [2] starts far over the margin where the digit form may not run
   if ((e = cudaMemsetAsync(B.dspread, 0, 3 * sizeof(int), s)) != cudaSuccess ||
       (!dig && (e = cudaMemsetAsync(B.dspread + 2, 1, sizeof(int), s)) != cudaSuccess))
@@ -1948,15 +1954,15 @@ csff_status far_field_one(csff_plan* P, const double* eta_host, const double2* u
   count_launch();
   // the operands of whichever contraction the device selects
   auto warps = [&](long long rows) { return (unsigned)std::min<long long>((rows * nbk * 32 + 255) / 256, 152 * 8); };
-  k_split_rows<<<warps(n_ux), 256, 0, s>>>(B.dxt, m, n_ux, B.dex, B.dspread, B.dxdf, B.dxsm);
-  k_split_rows<<<warps(R), 256, 0, s>>>(B.dg, m, (int)R, B.deg, B.dspread, B.dgdf, B.dgsm);
+  k_split_rows<<<warps(n_ux), 256, 0, s>>>(B.dxt, m, n_ux, B.dex, B.dspread, xdf, xsum);
+  k_split_rows<<<warps(R), 256, 0, s>>>(B.dg, m, (int)R, B.deg, B.dspread, gdfv, gsum);
   count_launch(2);
   if (dig) {
     if ((e = cudaFuncSetAttribute(k_ff_digits<digits::Form2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   digits::Form2::SMEM)) != cudaSuccess)
       return cuda_fail(e, "far-field contraction attribute");
-    k_cut_rows<true><<<warps((long long)gkt * digits::TK), 256, 0, s>>>(B.dxt, m, n_ux, B.dex, B.dspread, B.dxdig);
-    k_cut_rows<false><<<warps((long long)gxt * digits::TM), 256, 0, s>>>(B.dg, m, (int)R, B.deg, B.dspread, B.dgdig);
+    k_cut_rows<true><<<warps((long long)gkt * digits::TK), 256, 0, s>>>(B.dxt, m, n_ux, B.dex, B.dspread, B.dxop);
+    k_cut_rows<false><<<warps((long long)gxt * digits::TM), 256, 0, s>>>(B.dg, m, (int)R, B.deg, B.dspread, B.dgop);
     count_launch(2);
   }
   if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "far-field skip flags");
@@ -1967,11 +1973,11 @@ csff_status far_field_one(csff_plan* P, const double* eta_host, const double2* u
     // exactly one of them writes T (device-side checks on the spreads and margin)
     if (dig) {
       k_ff_digits<digits::Form2><<<dim3(gxt, gkt), digits::NT, digits::Form2::SMEM, s>>>(
-          B.dgdig, B.dxdig, B.dex, n_ux, B.deg, (int)R, nbk, B.dspread, B.dskip, (int)gdf.x, B.dT, B.dmisc + 2, 0,
+          B.dgop, B.dxop, B.dex, n_ux, B.deg, (int)R, nbk, B.dspread, B.dskip, (int)gdf.x, B.dT, B.dmisc + 2, 0,
           nullptr, nullptr, B.waits);
       count_launch();
     }
-    k_ff_stage1_df<<<gdf, DF_NT, 0, s>>>(B.dxdf, B.dxsm, B.dex, n_ux, B.dgdf, B.dgsm, B.deg, (int)R, nbk, B.dspread,
+    k_ff_stage1_df<<<gdf, DF_NT, 0, s>>>(xdf, xsum, B.dex, n_ux, gdfv, gsum, B.deg, (int)R, nbk, B.dspread,
                                          B.dskip, B.dT);
     k_ff_stage1<<<g1, 256, 0, s>>>(B.dxt, n_ux, B.dg, (int)R, m, B.dT, B.dspread, B.dmisc + 2);
   }

@@ -81,3 +81,20 @@ def test_far_field_2d_of_unbalanced_blocks(csff, var, nodes):
     tn, e2 = O.far_field(O.problem_from_dict(prob), u, eta[0], al, return_terms_norm=True)[:0:-1]
     diff = np.abs(F * 2.0 ** (E.astype(np.float64) - e2) - F64 * 2.0 ** (E64.astype(np.float64) - e2)) / tn
     assert np.sqrt(np.mean(diff ** 2)) <= 2.0 ** -48
+
+
+def test_far_field_2d_holds_one_set_of_operands(csff):
+    """The digit and the double-float contraction share their operands' memory."""
+    prob, plan = _plan(csff, 2, 513, 9, 10.0, 1.0)
+    m, ang = plan.m, 300
+    al = W.angle_set_2d(ang)
+    before = plan.describe()["device_bytes"]
+    _far(plan, np.array([[0.6, 0.8]]), np.zeros((m, m), dtype=complex), al)
+    grown = plan.describe()["device_bytes"] - before
+    plan.close()
+    rows, nb = len(np.unique(al[:, 0])), (m + 31) // 32
+    tiles_x, tiles_g = (rows + 15) // 16, (m + 127) // 128
+    field = 16 * m * m + 16 * m * (rows + 2 * ang) + 16 * m * rows           # g, phase tables, sums
+    digits = nb * (tiles_x * 7 * 4096 + tiles_g * 7 * 16384)
+    words = 8 * nb * (rows + m) + tiles_x * ((m + 31) // 32) * nb + 8 * 3 * (rows + ang) + 4 * ang
+    assert grown <= field + digits + words
