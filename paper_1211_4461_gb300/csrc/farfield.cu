@@ -392,16 +392,27 @@ __device__ __forceinline__ void df_mac2(float2& sh, float2& sl, float2 ah, float
 
 // one warp per (row, block): block exponent of |v| (upper bound) and the
 // row-block spread (max - min exponent) into *spread.
-// elo (block bounds for skipping negligible blocks, see k_ff_df_skip):
-// lo_min != 0 writes the smallest exponent of the block's entries inside the
+// elo (block bounds for skipping negligible blocks, see k_ff_df_skip): of the
+// phases the smallest exponent of the block's entries inside the
 // grid (-100000 if one is zero: max(|re|, |im|) >= 2^(e-1) for every entry),
-// else the largest (-100000 for an all-zero block: some entry reaches 2^(e-1)).
-__global__ void k_row_exps(const double2* __restrict__ v, int m, int nrows, int* __restrict__ ev,
-                           int* __restrict__ spread, int* __restrict__ elo, int lo_min) {
+// of g the largest (-100000 for an all-zero block: some entry reaches 2^(e-1)).
+// The phases' rows take the first xblocks CTAs, g's the rest (this pass, the skip
+// flags, the operands and the contractions are launches of a few microseconds on
+// small maps: 257^2, k = 3, 157 us with two launches for the exponents, two for the
+// splits and two for the digits, 140 with one each).
+struct Rows { const double2* v; int n; int *ev, *elo; };
+__global__ void k_row_exps(Rows X, Rows G, int xblocks, int m, int* __restrict__ spread) {
   // the spread is reduced over the CTA before one atomic (a per-warp atomic on
   // the one counter serialises in L2)
   __shared__ int wsp[8];
-  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  const bool lo_min = (int)blockIdx.x < xblocks;
+  const double2* __restrict__ v = lo_min ? X.v : G.v;
+  const int nrows = lo_min ? X.n : G.n;
+  int* __restrict__ ev = lo_min ? X.ev : G.ev;
+  int* __restrict__ elo = lo_min ? X.elo : G.elo;
+  if (!lo_min) ++spread;
+  const int block = (int)blockIdx.x - (lo_min ? 0 : xblocks);
+  const int warp = (block * (int)blockDim.x + (int)threadIdx.x) >> 5, lane = threadIdx.x & 31;
   const int nb = (m + DKB - 1) / DKB;
   if (threadIdx.x < 8) wsp[threadIdx.x] = 0;
   __syncthreads();
@@ -437,62 +448,70 @@ __global__ void k_row_exps(const double2* __restrict__ v, int m, int nrows, int*
   }
 }
 
-// one warp per (row, block), after k_row_exps: the operands of the
-// double-float contraction (rows scaled per block, split into FP32 pairs)
-__global__ void k_split_rows(const double2* __restrict__ v, int m, int nrows, const int* __restrict__ ev,
-                             const int* __restrict__ spread, float4* __restrict__ vdf, float2* __restrict__ vsum) {
-  if (digits_selected(spread) || !df_selected(spread)) return;
-  const int lane = threadIdx.x & 31, nb = (m + DKB - 1) / DKB;
-  for (int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; warp < nrows * nb; warp += gridDim.x * blockDim.x >> 5) {
-    const int row = warp / nb, b = warp % nb, i = b * DKB + lane;
-    const double2 x = i < m ? v[(long long)row * m + i] : make_double2(0, 0);
-    const int eb = ev[(long long)row * nb + b];
-    // the scaled splits of re, im and re + im (Gauss's three-product complex
-    // multiply); the scale applies to the values themselves, since 2^-eb alone
-    // overflows for subnormal blocks
-    const float2 re = bits::split_scaled(x.x, eb), im = bits::split_scaled(x.y, eb);
-    const float2 sm = eb <= 1000 ? bits::split_scaled(x.x + x.y, eb)      // RN(x + y) 2^-eb = RN(x 2^-eb + y 2^-eb)
-                                 : bits::split_scaled(ldexp(x.x, -eb) + ldexp(x.y, -eb), 0);
-    const long long o = (long long)row * nb * DKB + b * DKB + lane;
-    vdf[o] = make_float4(re.x, re.y, im.x, im.y);
-    vsum[o] = sm;
+// one warp: block b of a row as an operand of the double-float contraction, scaled
+// and split into FP32 pairs
+__device__ __forceinline__ void split_row(double2 x, int eb, long long o, float4* __restrict__ vdf,
+                                          float2* __restrict__ vsum) {
+  // the scaled splits of re, im and re + im (Gauss's three-product complex
+  // multiply); the scale applies to the values themselves, since 2^-eb alone
+  // overflows for subnormal blocks
+  const float2 re = bits::split_scaled(x.x, eb), im = bits::split_scaled(x.y, eb);
+  const float2 sm = eb <= 1000 ? bits::split_scaled(x.x + x.y, eb)      // RN(x + y) 2^-eb = RN(x 2^-eb + y 2^-eb)
+                               : bits::split_scaled(ldexp(x.x, -eb) + ldexp(x.y, -eb), 0);
+  vdf[o] = make_float4(re.x, re.y, im.x, im.y);
+  vsum[o] = sm;
+}
+
+// one warp: the digits of a block of a row for k_ff_digits, in its tile.  PHASE:
+// the two rows (P_re, -P_im), (P_im, P_re) of a phase row in tiles of TK; else a row
+// of g, tiles of TM.
+template <bool PHASE>
+__device__ __forceinline__ void cut_row(double2 x, int e, int row, int b, int nb, unsigned char* __restrict__ out) {
+  using namespace digits;
+  using F = Form2;
+  constexpr int ND = F::ND, B_SET = F::B_SET, TR = PHASE ? TK : TM;
+  const int lane = threadIdx.x & 31, r = row % TR, o = (lane & 3) * 4;
+  uint32_t dig[ND];
+  cut<ND>(fixed<F::BITS>(x.x, e), fixed<F::BITS>(x.y, e), dig);
+  unsigned char* tile = out + ((long long)(row / TR) * nb + b) * (PHASE ? B_SET : ND * A_DIG);
+#pragma unroll
+  for (int s = 0; s < ND; ++s) {
+    if (PHASE) {
+      *reinterpret_cast<uint32_t*>(tile + s * B_DIG + sw(r, lane >> 2) + o) = neg_hi(dig[s]);
+      *reinterpret_cast<uint32_t*>(tile + s * B_DIG + sw(TK + r, lane >> 2) + o) = swap_pair(dig[s]);
+    } else {
+      *reinterpret_cast<uint32_t*>(tile + s * A_DIG + sw(r, lane >> 2) + o) = dig[s];
+    }
   }
 }
 
-// one warp per (row, block), after k_row_exps: the digit operands of
-// k_ff_digits, rows padded with zeros to whole tiles.  PHASE: the two rows (P_re,
-// -P_im), (P_im, P_re) of a phase row in tiles of TK; else a row of g, tiles of TM.
-template <bool PHASE>
-__global__ void k_cut_rows(const double2* __restrict__ v, int m, int nrows, const int* __restrict__ ev,
-                           const int* __restrict__ spread, unsigned char* __restrict__ out) {
-  using namespace digits;
-  using F = Form2;
-  constexpr int ND = F::ND, B_SET = F::B_SET;
-  if (!digits_selected(spread)) return;
-  constexpr int TR = PHASE ? TK : TM;
-  const int lane = threadIdx.x & 31, nb = (m + KB - 1) / KB, total = (nrows + TR - 1) / TR * TR * nb;
-  for (int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; warp < total; warp += gridDim.x * blockDim.x >> 5) {
-    const int row = warp / nb, b = warp % nb, i = b * KB + lane;
-    uint32_t dig[ND];
-    long long p = 0, q = 0;
-    if (row < nrows && i < m) {
-      const double2 x = v[(long long)row * m + i];
-      const int e = ev[(long long)row * nb + b];
-      p = fixed<F::BITS>(x.x, e);
-      q = fixed<F::BITS>(x.y, e);
-    }
-    cut<ND>(p, q, dig);
-    const int r = row % TR;
-    unsigned char* tile = out + ((long long)(row / TR) * nb + b) * (PHASE ? B_SET : ND * A_DIG);
-    const int o = (lane & 3) * 4;
-#pragma unroll
-    for (int s = 0; s < ND; ++s) {
-      if (PHASE) {
-        *reinterpret_cast<uint32_t*>(tile + s * B_DIG + sw(r, lane >> 2) + o) = neg_hi(dig[s]);
-        *reinterpret_cast<uint32_t*>(tile + s * B_DIG + sw(TK + r, lane >> 2) + o) = swap_pair(dig[s]);
-      } else {
-        *reinterpret_cast<uint32_t*>(tile + s * A_DIG + sw(r, lane >> 2) + o) = dig[s];
-      }
+// after k_row_exps and the skip flags: the operands of the contraction that will
+// run, one warp per (row, block) of the phases, then of g.  Double-float: xop, gop
+// hold 16 bytes of pairs a node, then 8 of their sums.  Digits: rows padded with zeros
+// to whole tiles.
+__global__ void __launch_bounds__(256) k_operands(Rows X, Rows G, int m, const int* __restrict__ spread,
+                                                  unsigned char* __restrict__ xop, unsigned char* __restrict__ gop) {
+  const bool dig = digits_selected(spread);
+  if (!dig && !df_selected(spread)) return;
+  const int lane = threadIdx.x & 31, nb = (m + DKB - 1) / DKB;
+  auto up = [](int n, int t) { return (n + t - 1) / t * t; };
+  const int xrows = dig ? up(X.n, digits::TK) : X.n, grows = dig ? up(G.n, digits::TM) : G.n;
+  const long long total = (long long)(xrows + grows) * nb;
+  for (long long w = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5; w < total;
+       w += gridDim.x * (long long)blockDim.x >> 5) {
+    const int rb = (int)(w / nb), b = (int)(w - (long long)rb * nb), i = b * DKB + lane;
+    const bool phase = rb < xrows;
+    const int row = phase ? rb : rb - xrows, n = phase ? X.n : G.n;
+    const bool in = row < n;
+    const double2 x = in && i < m ? (phase ? X.v : G.v)[(long long)row * m + i] : make_double2(0, 0);
+    const int e = in ? (phase ? X.ev : G.ev)[(long long)row * nb + b] : 0;
+    if (dig) {
+      if (phase) cut_row<true>(x, e, row, b, nb, xop);
+      else cut_row<false>(x, e, row, b, nb, gop);
+    } else {
+      float4* const vdf = reinterpret_cast<float4*>(phase ? xop : gop);
+      const long long o = ((long long)row * nb + b) * DKB + lane;
+      split_row(x, e, o, vdf, reinterpret_cast<float2*>(vdf + (long long)n * nb * DKB));
     }
   }
 }
@@ -1939,11 +1958,11 @@ csff_status far_field_one(csff_plan* P, const double* eta_host, const double2* u
   if ((e = cudaMemsetAsync(B.dspread, 0, 3 * sizeof(int), s)) != cudaSuccess ||
       (!dig && (e = cudaMemsetAsync(B.dspread + 2, 1, sizeof(int), s)) != cudaSuccess))
     return cuda_fail(e, "memset");
+  const Rows rx{B.dxt, n_ux, B.dex, B.dxlo}, rg{B.dg, (int)R, B.deg, B.dghi};
   {
-    const long long wx = (long long)n_ux * nbk, wg = (long long)R * nbk;
-    k_row_exps<<<(unsigned)((wx * 32 + 255) / 256), 256, 0, s>>>(B.dxt, m, n_ux, B.dex, B.dspread, B.dxlo, 1);
-    k_row_exps<<<(unsigned)((wg * 32 + 255) / 256), 256, 0, s>>>(B.dg, m, (int)R, B.deg, B.dspread + 1, B.dghi, 0);
-    count_launch(2);
+    auto blocks = [&](long long rows) { return (unsigned)((rows * nbk * 32 + 255) / 256); };
+    k_row_exps<<<blocks(n_ux) + blocks(R), 256, 0, s>>>(rx, rg, (int)blocks(n_ux), m, B.dspread);
+    count_launch();
   }
   dim3 g1((unsigned)((R + S1_BN - 1) / S1_BN), (n_ux + S1_BM - 1) / S1_BM);
   dim3 gdf((unsigned)((R + DF_BN - 1) / DF_BN), (n_ux + DF_BM - 1) / DF_BM);
@@ -1952,19 +1971,15 @@ csff_status far_field_one(csff_plan* P, const double* eta_host, const double2* u
   k_ff_df_skip<<<gdf, 256, df_skip_smem(nbk), s>>>(B.dex, B.dxlo, n_ux, B.deg, B.dghi, (int)R, nbk, B.dskip,
                                                    B.dspread + 2);
   count_launch();
-  // the operands of whichever contraction the device selects
-  auto warps = [&](long long rows) { return (unsigned)std::min<long long>((rows * nbk * 32 + 255) / 256, 152 * 8); };
-  k_split_rows<<<warps(n_ux), 256, 0, s>>>(B.dxt, m, n_ux, B.dex, B.dspread, xdf, xsum);
-  k_split_rows<<<warps(R), 256, 0, s>>>(B.dg, m, (int)R, B.deg, B.dspread, gdfv, gsum);
-  count_launch(2);
-  if (dig) {
-    if ((e = cudaFuncSetAttribute(k_ff_digits<digits::Form2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  digits::Form2::SMEM)) != cudaSuccess)
-      return cuda_fail(e, "far-field contraction attribute");
-    k_cut_rows<true><<<warps((long long)gkt * digits::TK), 256, 0, s>>>(B.dxt, m, n_ux, B.dex, B.dspread, B.dxop);
-    k_cut_rows<false><<<warps((long long)gxt * digits::TM), 256, 0, s>>>(B.dg, m, (int)R, B.deg, B.dspread, B.dgop);
-    count_launch(2);
+  {
+    const long long rows = (long long)(dig ? gkt * digits::TK + gxt * digits::TM : n_ux + R);
+    k_operands<<<(unsigned)std::min<long long>((rows * nbk * 32 + 255) / 256, 152 * 8), 256, 0, s>>>(
+        rx, rg, m, B.dspread, B.dxop, B.dgop);
+    count_launch();
   }
+  if (dig && (e = cudaFuncSetAttribute(k_ff_digits<digits::Form2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       digits::Form2::SMEM)) != cudaSuccess)
+    return cuda_fail(e, "far-field contraction attribute");
   if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "far-field skip flags");
   B.skip_used = (size_t)gdf.x * gdf.y * nbk;
   {
