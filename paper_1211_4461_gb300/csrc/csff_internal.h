@@ -134,7 +134,7 @@ struct FFBuffers {
   size_t xlo = 0, ghi = 0, skip = 0;
   int *dxlo = nullptr, *dghi = nullptr;
   unsigned char* dskip = nullptr;
-  size_t skip_used = 0;       // flags written by the last 2D far field
+  int skip_tiles = 0, skip_rows = 0, skip_nb = 0;      // tiles along g and phase rows, blocks of the last far field
   // tensor-core 3D stage A: pre-swizzled split phase operand, per-column and
   // per-row exponents, [spread_g, spread_P, error word]
   size_t tcb = 0, tce = 0;

@@ -1678,23 +1678,34 @@ static cudaError_t stage_b_digits(FFBuffers& B, const double2* yt, const YTiles&
   return cudaGetLastError();
 }
 
-// fraction of the double-float contraction's (tile, block) pairs that the last
-// 2D far field computed (1 when the FP64 kernel ran or nothing was skipped)
+// fraction of the contraction's (tile, block) pairs that the last 2D far field
+// computed: of the double-float form's tiles, or of the digit form's, which span
+// several of them and compute a block that one of these keeps (1 when an FP64 kernel
+// ran or nothing was skipped)
 csff_status far_field_executed(csff_plan* P, double* executed) {
   FFBuffers& B = P->ff;
   *executed = 1.0;
-  if (!B.dskip || !B.dspread || B.skip_used == 0) return CSFF_OK;
-  std::vector<unsigned char> h(B.skip_used);
-  int sp[3] = {0, 0, 0};
+  const int tiles = B.skip_tiles, rows = B.skip_rows, nb = B.skip_nb;
+  if (!B.dskip || !B.dspread || nb == 0) return CSFF_OK;
+  std::vector<unsigned char> h((size_t)tiles * rows * nb);
+  int sp[3] = {0, 0, 0}, gave_up = 0;
   cudaError_t e = cudaMemcpyAsync(h.data(), B.dskip, h.size(), cudaMemcpyDeviceToHost, P->stream);
   if (e == cudaSuccess) e = cudaMemcpyAsync(sp, B.dspread, sizeof(sp), cudaMemcpyDeviceToHost, P->stream);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&gave_up, B.dmisc + 2, sizeof(int), cudaMemcpyDeviceToHost, P->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(P->stream);
   if (e != cudaSuccess) return cuda_fail(e, "far-field work");
-  const bool finite = sp[0] < DF_NONFINITE && sp[1] < DF_NONFINITE;
-  if (!finite || (std::min(sp[0], sp[1]) > DF_SPREAD_LIMIT && sp[2] > digits::MARGIN)) return CSFF_OK;
-  size_t run = 0;
-  for (unsigned char c : h) run += c == 0;
-  *executed = (double)run / (double)h.size();
+  const bool finite = sp[0] < DF_NONFINITE && sp[1] < DF_NONFINITE, dig = sp[2] <= digits::MARGIN;
+  if (!finite || gave_up || (!dig && std::min(sp[0], sp[1]) > DF_SPREAD_LIMIT)) return CSFF_OK;
+  const int group = dig ? digits::TM / DF_BN : 1;
+  size_t run = 0, all = 0;
+  for (int r = 0; r < rows; ++r)
+    for (int t0 = 0; t0 < tiles; t0 += group)
+      for (int b = 0; b < nb; ++b, ++all) {
+        bool keep = false;
+        for (int t = t0; t < std::min(t0 + group, tiles); ++t) keep |= h[((size_t)r * tiles + t) * nb + b] == 0;
+        run += keep;
+      }
+  *executed = (double)run / (double)all;
   return CSFF_OK;
 }
 
@@ -1981,7 +1992,9 @@ csff_status far_field_one(csff_plan* P, const double* eta_host, const double2* u
                                        digits::Form2::SMEM)) != cudaSuccess)
     return cuda_fail(e, "far-field contraction attribute");
   if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "far-field skip flags");
-  B.skip_used = (size_t)gdf.x * gdf.y * nbk;
+  B.skip_tiles = (int)gdf.x;
+  B.skip_rows = (int)gdf.y;
+  B.skip_nb = nbk;
   {
     ProfScope ps(PF_FF_CONTRACT, s, 16.0 * ((double)n_ux * m + (double)R * m + (double)n_ux * R),
                  8.0 * (double)n_ux * (double)R * m);

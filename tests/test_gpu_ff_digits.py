@@ -98,3 +98,19 @@ def test_far_field_2d_holds_one_set_of_operands(csff):
     digits = nb * (tiles_x * 7 * 4096 + tiles_g * 7 * 16384)
     words = 8 * nb * (rows + m) + tiles_x * ((m + 31) // 32) * nb + 8 * 3 * (rows + ang) + 4 * ang
     assert grown <= field + digits + words
+
+
+def test_far_field_work_counts_the_tiles_of_the_contraction_that_ran(csff):
+    """Rows 0-31 live in the first of four blocks, the others in the last: every
+    double-float tile (32 rows) keeps one block of four, the digit form's one tile
+    of 128 rows two.  At k = 3 the phases vary too much over a block for digits."""
+    for k, fraction in ((0.5, 0.5), (3.0, 0.25)):
+        prob = W.problem(2, 129, 10.0, math.pi / 6, k, [W.gauss(1.0, 1e6)])
+        plan = csff.Plan(prob, {"smoother": "jacobi", "nu1": 1, "nu2": 1, "coarsest_n": 5, "rel_tol": 1e-8,
+                                "precision": "fp64"})
+        m = plan.m
+        u = np.zeros((m, m), dtype=complex)
+        u[:32, :32], u[32:, 96:] = 1e60, 1e60
+        _far(plan, np.array([[0.6, 0.8]]), u, W.angle_set_2d(40))
+        assert plan.far_field_work() == fraction
+        plan.close()
