@@ -327,10 +327,6 @@ cudaError_t launch_df_update(float4* u, const float2* e, long long N, cudaStream
 cudaError_t launch_df_to64(const float4* u, long long N, int exp_scale, double2* out, cudaStream_t s);
 
 // ---- FP64 refinement of the mixed solve (option refine_fp64; mg_kernels.cu) ------
-// r32 = 2^-e r with e the exponent of *norm_dev (written to *exp_out); u += 2^e e32
-cudaError_t launch_to32_scaled(const double2* r, long long N, const double* norm_dev, float2* r32,
-                               int* exp_out, cudaStream_t s);
-cudaError_t launch_update64(double2* u, const float2* e, long long N, const int* exp_in, cudaStream_t s);
 // The FP64 refinement step with a fixed scale 2^s: r = b - A u in FP64, r32 =
 // 2^-s r in FP32, ||r|| into *out (device; partial: nblk doubles of scratch);
 // u += 2^s e; r32 = 2^-s v.  N < 2^31.

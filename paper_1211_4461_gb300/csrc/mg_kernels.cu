@@ -498,35 +498,6 @@ __global__ void k_rhs(TabPtrs tabs, int n_gauss, const double2* __restrict__ uin
 }
 
 // ---- FP64 refinement of the mixed solve (option refine_fp64) -------------------
-// r32 = r64 * 2^-e with e = exponent of ||r64||_2 (so |r32| < 1 elementwise);
-// values of 2^-126 ||r|| and less become zero
-__global__ void k_to32_scaled(const double2* __restrict__ r, long long N, const double* __restrict__ nrm,
-                              float2* __restrict__ r32, int* __restrict__ exp_out) {
-  pdl_prologue();
-  int e;
-  frexp(*nrm, &e);
-  if (blockIdx.x == 0 && threadIdx.x == 0) *exp_out = e;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N;
-       i += (long long)gridDim.x * blockDim.x) {
-    const double2 v = r[i];
-    r32[i] = make_float2(bits::narrow(v.x, e), bits::narrow(v.y, e));
-  }
-}
-
-__global__ void k_update64(double2* __restrict__ u, const float2* __restrict__ e, long long N,
-                           const int* __restrict__ exp_in) {
-  pdl_prologue();
-  const int s = *exp_in;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N;
-       i += (long long)gridDim.x * blockDim.x) {
-    const float2 c = e[i];
-    double2 v = u[i];
-    v.x += bits::widen(c.x, s);
-    v.y += bits::widen(c.y, s);
-    u[i] = v;
-  }
-}
-
 // One pass of the FP64 refinement step (option refine_fp64): the residual
 // r = b - A u in FP64 as a chain of fused multiply-adds,
 //   r = b - c (2d u - sum_nbr u) + q u,
@@ -800,14 +771,6 @@ cudaError_t launch_rhs(int dim, int m, const double2* const* chi_tab, int n_gaus
   return cudaGetLastError();
 }
 
-cudaError_t launch_to32_scaled(const double2* r, long long N, const double* norm_dev, float2* r32,
-                               int* exp_out, cudaStream_t s) {
-  ProfScope ps(PF_MG64, s, 24.0 * N, 0);
-  cudaError_t e = launch_pdl(k_to32_scaled, dim3(flat_blocks(N)), dim3(256), 0, s, r, N, norm_dev, r32, exp_out);
-  count_launch();
-  return e != cudaSuccess ? e : cudaGetLastError();
-}
-
 cudaError_t launch_refine_residual(int dim, const Level& L, const double2* u, const double2* b, int s_exp,
                                    float2* r32, double* partial, int nblk, double* out, cudaStream_t s) {
   if (L.N >= (1ll << 31)) return cudaErrorInvalidValue;
@@ -850,14 +813,6 @@ cudaError_t launch_first_residual(const double2* b, long long N, int s_exp, floa
     e = launch_pdl(k_norm_finish, dim3(1), dim3(RED_THREADS), 0, s, (const double*)partial, nb, ldexp(1.0, ex), out);
   count_launch(2);
   return e != cudaSuccess ? e : cudaGetLastError();
-}
-
-cudaError_t launch_update64(double2* u, const float2* e, long long N, const int* exp_in,
-                            cudaStream_t s) {
-  ProfScope ps(PF_MG64, s, 40.0 * N, 0);
-  cudaError_t err = launch_pdl(k_update64, dim3(flat_blocks(N)), dim3(256), 0, s, u, e, N, exp_in);
-  count_launch();
-  return err != cudaSuccess ? err : cudaGetLastError();
 }
 
 cudaError_t launch_inject_q(int dim, const Level& F, const Level& C, cudaStream_t s) {
