@@ -213,3 +213,23 @@ def test_plan_3d_without_room_for_the_split_arrays(csff):
     del fill
     torch.cuda.empty_cache()
     assert torch.linalg.vector_norm(got - want) <= 1e-5 * torch.linalg.vector_norm(want)
+
+
+# amplitudes at which the residual of a converging solve is subnormal in FP64
+# (below 2^-1022 from a relative 1e-8 on): its rounding to FP32 keeps it
+@pytest.mark.parametrize("batch", [False, True])
+def test_refinement_of_tiny_amplitudes(csff, batch):
+    prob = W.problem(2, 65, 5.0, math.pi / 6, 1.0, [W.gauss(1e-300, 1.5)])
+    opts = {"smoother": "rbgs", "nu1": 1, "nu2": 1, "coarsest_n": 5, "rel_tol": 1e-10, "max_cycles": 60,
+            "precision": "mixed", "refine_fp64": 1}
+    eta = np.array([[1.0, 0.0]])
+    if batch:
+        b = csff.Batch([prob], opts)
+        st, infos = b.solve(eta)
+        b.close()
+    else:
+        plan = csff.Plan(prob, opts)
+        u = torch.zeros(plan.N, dtype=torch.complex128, device="cuda")
+        st, infos = plan.solve(eta, u)
+        plan.close()
+    assert st == csff.OK and infos[0]["rel_res"] <= 1e-10
