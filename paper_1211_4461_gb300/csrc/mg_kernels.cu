@@ -229,25 +229,43 @@ __global__ void k_prolong_cells(const cx<T>* __restrict__ ec, int mc, cx<T>* __r
 
 // Coarsest level: u = inv b, the inverse from FP64 Gauss-Jordan, in TI
 // arithmetic, rounded once to T.  LPR lanes a row (4, or 32 for large N), chains
-// of fused multiply-adds joined by shuffles: FP64 work is scarce on this part.
-template <typename T, typename TI, int LPR>
+// of fused multiply-adds joined by shuffles: FP64 work is scarce on this part.  Above
+// 32 unknowns four lanes keep NA = 8 chains each where the product is in the vectors'
+// own precision (121 unknowns: 1.2 units of rounding off, 2.1 with one chain, 1.5
+// with 32 lanes).
+template <typename T, typename TI, int LPR, int NA>
 __global__ void __launch_bounds__(256) k_coarse_solve(const cx<TI>* __restrict__ inv, int N,
                                                       const cx<T>* __restrict__ b, cx<T>* __restrict__ u, int ring_m,
                                                       int ring_pitch) {
   pdl_start();
   const int t = blockIdx.x * 256 + threadIdx.x, i = t / LPR, part = t % LPR;
-  TI re = (TI)0, im = (TI)0;
+  TI rc[NA], ic[NA];
+#pragma unroll
+  for (int a = 0; a < NA; ++a) rc[a] = ic[a] = (TI)0;
   if (i < N) {
     const cx<TI>* row = inv + (long long)i * N;
-#pragma unroll 8
-    for (int j = part; j < N; j += LPR) {
-      const cx<TI> a = row[j];
-      const cx<T> bj = b[j];
-      const TI bx = (TI)bj.x, by = (TI)bj.y;
-      re = fma(a.x, bx, fma(-a.y, by, re));
-      im = fma(a.x, by, fma(a.y, bx, im));
+#pragma unroll(NA == 1 ? 8 : 1)
+    for (int j0 = part; j0 < N; j0 += LPR * NA) {
+#pragma unroll
+      for (int c = 0; c < NA; ++c) {
+        const int j = j0 + LPR * c;
+        if (j >= N) continue;
+        const cx<TI> a = row[j];
+        const cx<T> bj = b[j];
+        const TI bx = (TI)bj.x, by = (TI)bj.y;
+        rc[c] = fma(a.x, bx, fma(-a.y, by, rc[c]));
+        ic[c] = fma(a.x, by, fma(a.y, bx, ic[c]));
+      }
     }
   }
+#pragma unroll
+  for (int h = NA / 2; h > 0; h >>= 1)
+#pragma unroll
+    for (int c = 0; c < h; ++c) {
+      rc[c] += rc[c + h];
+      ic[c] += ic[c + h];
+    }
+  TI re = rc[0], im = ic[0];
 #pragma unroll
   for (int o = 1; o < LPR; o <<= 1) {
     re += __shfl_xor_sync(0xffffffffu, re, o);
@@ -675,9 +693,11 @@ cudaError_t launch_prolong_add(int dim, const Level& F, const Level& C, const cx
 template <typename T, typename TI>
 static cudaError_t coarse_solve(const cx<TI>* inv, int N, const cx<T>* b, cx<T>* u, cudaStream_t s, int rm, int rp) {
   ProfScope ps(mg_family<T>(), s, sizeof(cx<T>) * 2.0 * N + sizeof(cx<TI>) * (double)N * N, 8.0 * N * N);
-  cudaError_t e = N <= 128 ? launch_pdl(k_coarse_solve<T, TI, 4>, dim3((4 * N + 255) / 256), dim3(256), 0, s, inv, N, b, u, rm, rp)
-                           : launch_pdl(k_coarse_solve<T, TI, 32>, dim3((32 * N + 255) / 256), dim3(256), 0, s, inv, N, b, u,
-                                        rm, rp);
+  constexpr int NA = sizeof(T) == sizeof(TI) ? 8 : 1;
+  const int lanes = N <= 128 ? 4 : 32;
+  cudaError_t e = launch_pdl(N <= 32 ? k_coarse_solve<T, TI, 4, 1> : N <= 128 ? k_coarse_solve<T, TI, 4, NA>
+                                                                            : k_coarse_solve<T, TI, 32, 1>,
+                             dim3((lanes * N + 255) / 256), dim3(256), 0, s, inv, N, b, u, rm, rp);
   count_launch();
   return e != cudaSuccess ? e : cudaGetLastError();
 }

@@ -233,3 +233,25 @@ def test_refinement_of_tiny_amplitudes(csff, batch):
         st, infos = plan.solve(eta, u)
         plan.close()
     assert st == csff.OK and infos[0]["rel_res"] <= 1e-10
+
+
+# the coarsest product in FP32: the restated rms error of a row in 32 lanes (or
+# four of eight chains) is 1.2 to 1.5 units of 2^-24 of the result, of four lanes
+# with a chain each 2.1; the rounding of the inverse adds 0.4 in the square
+@pytest.mark.parametrize("coarsest", [11, 12, 13])
+def test_coarse_product_rounding(csff, coarsest):
+    n, R, g = 2 * coarsest - 1, 5.0, math.pi / 6
+    plan = csff.Plan(W.problem(2, n, R, g, 1.0, []), {"smoother": "rbgs", "nu1": 1, "nu2": 1, "coarsest_n": coarsest,
+                                                      "rel_tol": 1e-8, "precision": "fp64"})
+    m, h = coarsest - 2, 2 * R / (coarsest - 1)
+    T = 2 * np.eye(m) - np.eye(m, k=1) - np.eye(m, k=-1)
+    A = np.exp(-2j * g) / h ** 2 * (np.kron(np.eye(m), T) + np.kron(T, np.eye(m))) - np.eye(m * m)
+    err = []
+    for seed in range(8):
+        b = W.rand_real(m * m, seed).astype(np.complex64)
+        u = torch.zeros(m * m, dtype=torch.complex64, device="cuda")
+        plan.coarse_solve(torch.from_numpy(b).cuda(), u)
+        ref = np.linalg.solve(A, b.astype(complex))
+        err.append(np.linalg.norm(u.cpu().numpy() - ref) / np.linalg.norm(ref))
+    plan.close()
+    assert np.sqrt(np.mean(np.square(err))) <= 1.7 * 2.0 ** -24
