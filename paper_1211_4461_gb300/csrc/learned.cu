@@ -1037,7 +1037,7 @@ csff_status ensure_scratch(csff_net* N, long long npix, int B, bool train) {
       NK(cudaMalloc((void**)&N->dh1, sizeof(float) * 16 * cap), "net scratch");
       NK(cudaMalloc((void**)&N->dh2, sizeof(float) * 16 * cap), "net scratch");
       NK(cudaMalloc((void**)&N->E, sizeof(float2) * cap), "net scratch");
-      NK(cudaMalloc((void**)&N->G, sizeof(float2) * cap), "net scratch");
+      if (N->dim == 3) NK(cudaMalloc((void**)&N->G, sizeof(float2) * cap), "net scratch");
       NK(cudaMalloc((void**)&N->dy, sizeof(float2) * cap), "net scratch");
     }
     N->cap = cap;
@@ -1386,8 +1386,8 @@ csff_status net_reserve(csff_net* N, long long npix) {
   return N->dim == 3 ? ensure_scratch(N, npix, 1, false) : CSFF_OK;
 }
 
-// status of the tensor-core layers since the last check (synchronises)
-// the network's kernels have completed (the caller has synchronised with them)
+// status of the tensor-core layers since the last check; their kernels have
+// completed (the caller has synchronised with them)
 csff_status net_check(csff_net* N) {
   volatile int* err = N->tcerr;
   if (*err) {
