@@ -114,3 +114,32 @@ def test_far_field_work_counts_the_tiles_of_the_contraction_that_ran(csff):
         _far(plan, np.array([[0.6, 0.8]]), u, W.angle_set_2d(40))
         assert plan.far_field_work() == fraction
         plan.close()
+
+
+# the y contraction in digits (angles that share z components, in numbers that are
+# no multiple of its tiles of 16; rows of 63 to 127 nodes, whose second scale block
+# of the last 32 is full, empty or short): against the oracle at selected angles.
+# A y component too steep for digits takes its three launches away
+@pytest.mark.parametrize("n,coarsest,per_z,n_z,k,R", [(65, 5, 40, 56, 1.0, 5.0), (73, 10, 24, 67, 2.0, 5.0),
+                                                      (81, 6, 17, 80, 2.0, 5.0), (97, 7, 33, 30, 2.0, 10.0),
+                                                      (129, 5, 9, 60, 2.0, 10.0)])
+def test_far_field_3d_y_contraction(csff, n, coarsest, per_z, n_z, k, R):
+    prob, plan = _plan(csff, 3, n, coarsest, R, k)
+    u = W.rand_complex((plan.m,) * 3, 31)
+    th, ph = np.pi * (np.arange(n_z) + 0.5) / n_z, 2 * np.pi * (np.arange(per_z) + 0.2) / per_z
+    T, P = np.meshgrid(th, ph, indexing="ij")
+    al = np.ascontiguousarray(np.stack([np.sin(T) * np.cos(P), np.sin(T) * np.sin(P), np.cos(T)], -1).reshape(-1, 3))
+    eta = np.array([[0.6, 0.0, 0.8]])
+    before = csff.kernel_launches()
+    F, E = _far(plan, eta, u, al)
+    launches = csff.kernel_launches() - before
+    steep = al.copy()
+    steep[5, 1] = 40.0
+    _far(plan, eta, u, steep)
+    plan.close()
+    assert csff.kernel_launches() - before == 2 * launches - 3
+    sel = np.array([0, per_z // 2, len(al) // 2 + 7, len(al) - 1])
+    mant, e2, tn = O.far_field(O.problem_from_dict(prob), u, eta[0], al[sel], return_terms_norm=True)
+    # each stage's rounding is below 2^-48 of the sum of the terms' magnitudes, the
+    # phases' own k |z| and a few ulp
+    assert np.all(np.abs(F[sel] * 2.0 ** (E[sel].astype(np.float64) - e2) - mant) <= 1e-13 * tn)
