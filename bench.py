@@ -49,15 +49,6 @@ def _peaks():
 # FP64 FMA throughput of this part, measured with an FMA-loop kernel
 # (0.599e12 DFMA/s over 152 SMs; 2 flops per FMA).
 FP64_PEAK_TFLOPS = 1.198
-# FP32 operation rate derived from unit counts and clock: 152 SMs x 128 FP32
-# lanes x 2.07 GHz (a packed two-lane instruction counts two operations).  The
-# double-float contraction spends 36 FP32 operations (three double-float
-# multiply-adds of 12, Gauss's complex product) per complex multiply-add, i.e.
-# 4.5 per FP64-equivalent flop (8 per complex multiply-add), so its arithmetic
-# ceiling in FP64-equivalent flops is that rate / 4.5.
-FP32_INSTR_PER_S = 152 * 128 * 2.07e9
-DF_INSTR_PER_FLOP = 36.0 / 8.0
-DF_PEAK_TFLOPS = FP32_INSTR_PER_S / DF_INSTR_PER_FLOP / 1e12
 # DRAM bytes (read + write) per launch of the dominant kernels, from one ncu
 # capture of the current kernels on this workload (None when no capture of
 # the current kernels exists): the fused FP32 V(1,1) tiles (all levels, and those
@@ -526,17 +517,13 @@ def run_ours(args, rank, world, local_rank):
                        "all": tiles_roofline(allt, TILES_DRAM_BYTES, "k_down2 / k_up2, every fused level",
                                              alg_note)}
     roofline_ff = {"kernel": "2D far-field contraction: k_ff_digits (exact digits on the tensor cores) for maps whose "
-                             "phases vary slowly over a block, k_ff_stage1_df (double-float) for the others", "bound": "alu",
-                "achieved": achieved_tf, "peak": DF_PEAK_TFLOPS, "unit": "TFLOP/s",
-                "frac": achieved_tf / DF_PEAK_TFLOPS, "traffic": None,
-                "peak_source": "the double-float kernel's: 152 SMs x 128 FP32 lanes x 2.07 GHz / 4.5 FP32 operations per "
-                               "FP64-equivalent flop (36 per complex multiply-add: three double-float "
-                               "multiply-adds, Gauss's product; a packed two-lane instruction counts two)",
-                "avg_launch_ms": ff_avg_ms, "launches": ff["launches"],
+                             "phases vary slowly over a block, k_ff_stage1_df (double-float) for the others",
+                "achieved": achieved_tf, "unit": "TFLOP/s", "avg_launch_ms": ff_avg_ms, "launches": ff["launches"],
                 "alg_flops_per_launch": ff_flops_all, "executed_flops_per_launch": ff_flops,
                 "executed_fraction_per_map": ff_work,
                 "note": "achieved counts the executed flops: blocks whose terms stay below 2^-55 of each "
-                        "far-field value's sum of term magnitudes are skipped"}
+                        "far-field value's sum of term magnitudes are skipped; no fraction of a ceiling, since the "
+                        "launches run on two different units"}
     mg32, mg64 = breakdown["mg32"], breakdown["mg64"]
     cycles = sum(infos[i]["cycles"] for i in infos)
     vc = {"fp32_kernels_ms": mg32["ms"], "fp32_alg_bytes": mg32["alg_bytes"],
@@ -568,7 +555,27 @@ def run_ours(args, rank, world, local_rank):
         finally:
             runner.close()
         line["cpu_baseline"] = cpu_baseline_record(r, runner.workers)
-    print(json.dumps(line), flush=True)
+    if args.details:
+        with open(args.details, "w") as f:
+            json.dump(line, f, indent=1)
+    print(json.dumps(compact_line(line, args.details)), flush=True)
+
+
+# keys of a record whose whole contents go to the details file
+DETAIL_KEYS = ("roofline_levels", "roofline_ff_contraction", "vcycle", "solve", "variants")
+
+
+def compact_line(line, details):
+    """The printed record: a few kilobytes, so that whoever keeps only the end of
+    the output still has all of it.  Of the variants their rates alone; the
+    rest is in the details file."""
+    out = {k: v for k, v in line.items() if k not in DETAIL_KEYS}
+    if isinstance(out.get("roofline"), dict):
+        out["roofline"] = {k: v for k, v in out["roofline"].items() if k != "note"}
+    if "variants" in line:
+        out["variants"] = {k: v["value"] for k, v in line["variants"].items() if isinstance(v, dict) and "value" in v}
+    out["details"] = details or None
+    return out
 
 
 def _time_events(torch, stream, fn, flush, reps):
@@ -1278,6 +1285,8 @@ def main():
     ap.add_argument("--no-cpu-baseline", dest="cpu_baseline", action="store_false")
     ap.add_argument("--no-variants", dest="variants", action="store_false",
                     help="skip the plain-FP64 and batched comparison runs")
+    ap.add_argument("--details", default=os.path.join(ROOT, "bench_details.json"),
+                    help="file for the whole record (rooflines, per-map solves, every variant); empty: none")
     ap.add_argument("--ks", default="", help="comma-separated subset of the wavenumbers (profiling runs)")
     ap.add_argument("--inner-cycles", type=int, default=INNER_CYCLES,
                     help="FP32 V-cycles per refinement step of the mixed solve")
