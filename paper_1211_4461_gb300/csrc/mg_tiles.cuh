@@ -839,13 +839,13 @@ __device__ void coarse_levels_block(const CoarseLevels& L, const cx<T>* b_top, c
       for (int a = 0; a < NA; ++a) chain[a] = mk<CI>((TI)0, (TI)0);
       if (i < n) {
         const CI* row = iv + (long long)i * n;
-        for (int c0 = part; c0 < n; c0 += 4 * NA) {
+        int col = part;
+        for (; col + 4 * (NA - 1) < n; col += 4 * NA)
 #pragma unroll
-          for (int a = 0; a < NA; ++a) {
-            const int col = c0 + 4 * a;
-            if (col < n) chain[a] = xfma(chain[a], row[col], Bc[col]);
-          }
-        }
+          for (int a = 0; a < NA; ++a) chain[a] = xfma(chain[a], row[col + 4 * a], Bc[col + 4 * a]);
+#pragma unroll
+        for (int a = 0; a < NA - 1; ++a, col += 4)
+          if (col < n) chain[a] = xfma(chain[a], row[col], Bc[col]);
       }
 #pragma unroll
       for (int h = NA / 2; h > 0; h >>= 1)
