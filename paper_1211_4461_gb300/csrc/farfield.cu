@@ -395,7 +395,8 @@ __device__ __forceinline__ void df_mac2(float2& sh, float2& sl, float2 ah, float
 // elo (block bounds for skipping negligible blocks, see k_ff_df_skip): of the
 // phases the smallest exponent of the block's entries inside the
 // grid (-100000 if one is zero: max(|re|, |im|) >= 2^(e-1) for every entry),
-// of g the largest (-100000 for an all-zero block: some entry reaches 2^(e-1)).
+// of g that of a lower bound of the entries' sum, from their exponents: the sum of
+// max(|re|, |im|) is at least 2^(e-1) (-100000 for an all-zero block).
 // The phases' rows take the first xblocks CTAs, g's the rest (this pass, the skip
 // flags, the operands and the contractions are launches of a few microseconds on
 // small maps: 257^2, k = 3, 157 us with two launches for the exponents, two for the
@@ -427,6 +428,7 @@ __global__ void k_row_exps(Rows X, Rows G, int xblocks, int m, int* __restrict__
   const bool nzy = ((unsigned long long)__double_as_longlong(x.y) & bits::ABS_MASK) != 0;
   const bool pos = fin && (nzx || nzy);
   int e = pos ? max(nzx ? bits::frexp_exp(x.x) : -100000, nzy ? bits::frexp_exp(x.y) : -100000) : -100000;
+  const int own = e;
   int emin = pos ? e : 100000;
   int elow = (i < m) ? e : 100000;               // -100000 for a zero entry; padding lanes ignored
   for (int o = 16; o > 0; o >>= 1) {
@@ -435,9 +437,14 @@ __global__ void k_row_exps(Rows X, Rows G, int xblocks, int m, int* __restrict__
     elow = min(elow, __shfl_xor_sync(0xffffffffu, elow, o));
   }
   const bool bad = __any_sync(0xffffffffu, !fin);   // non-finite: the FP64 kernel runs
+  int esum = e;                                     // floor(log2 sum 2^exponent), terms from 2^-20 of the largest
+  if (!lo_min && e > -100000) {
+    const unsigned part = pos && own - e >= -20 ? 1u << (20 + own - e) : 0u;
+    esum = e + 11 - __clz((int)__reduce_add_sync(0xffffffffu, part));
+  }
   if (active && lane == 0) {
     ev[(long long)row * nb + b] = (e == -100000 || bad) ? 0 : e;
-    elo[(long long)row * nb + b] = lo_min ? elow : e;
+    elo[(long long)row * nb + b] = lo_min ? elow : esum;
     wsp[threadIdx.x >> 5] = bad ? DF_NONFINITE : ((e == -100000) ? 0 : e - emin);
   }
   __syncthreads();
@@ -562,7 +569,7 @@ constexpr int DF_BM = 16, DF_BN = 32, DF_NT = 128;
 // Negligible blocks of the contraction.  For an output T[k][rho] the sum of
 // its terms' magnitudes is at least
 //   2^L,  L = max_b (xlo[k][b] + ghi[rho][b] - 2)
-// (xlo: smallest exponent of X's entries in block b, ghi: largest of g's), and
+// (xlo: smallest exponent of X's entries in block b, ghi: that of the sum of g's), and
 // block b adds at most 32 * 2 * 2^(ex[k][b] + eg[rho][b]) (ex, eg: the block
 // exponents the split scales by).  A block whose bound lies 60 binades under
 // L for every (k, rho) of a contraction tile is skipped by that tile: per

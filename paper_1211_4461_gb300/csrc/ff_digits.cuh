@@ -22,19 +22,20 @@
 // When it runs.  These errors are relative to the block maxima, so the kernel is
 // taken when for every block that a tile keeps the scales ex + eg lie at most
 // MARGIN binades over L, the lower bound of the sum of the terms' magnitudes that
-// the skip kernel forms (2 for constant phases, more as they vary over a block:
-// about k h sin(gamma) 32 < 3.5).  The line is where the error reaches the
+// the skip kernel forms (-3 to 2 for constant phases, more as they vary over a block:
+// up to about k h sin(gamma) 32 = 5).  The line is where the error reaches the
 // double-float kernel's, which runs beyond it.  Both restated on the CPU on single
 // blocks against a longer sum, relative to the sum of the terms' magnitudes, by
 // margin, as binades of the rms error over the double-float kernel's (2^-48.5 to
 // 2^-45.7):
-//   fields                                margin 6     8      9     10     11     12
-//   random                                     -3.7  -3.5  -3.4  -3.3  -3.2  -3.8
-//   balanced against the phases                -4.5  -3.6  -2.8  -1.9  -1.1  -0.6
-//   falling three times as fast                -4.6  -2.9  -1.7  -0.9  -0.1  -0.3
-//   three nodes where the phase is smallest    -2.4  -1.5  -0.6  +0.4  +1.1  +1.9
-//   a single node there                        -1.8  -0.2  +0.4  +1.5  +2.3  +3.1
-// (with diagonals up to 8 and a margin of 12, as before, up to 3.9 binades larger.)
+//   fields                                margin 5     6     7     8     9     10
+//   random                                     -3.5  -3.3  -3.3  -3.2
+//   balanced against the phases                -4.1  -3.7  -3.0  -2.0  -1.4  -0.6
+//   falling three times as fast                -4.4  -3.7  -2.9  -1.9  -1.1  -0.6
+//   three nodes where the phase is smallest    -2.5  -2.2  -1.7  -0.9  +0.1  +0.7
+//   a single node there                        -2.0  -1.8  -1.5  -0.8  +0.1  +1.0
+// (with diagonals up to 8 and the line at 12 binades over a bound from single
+// nodes, as before, up to 3.9 binades larger.)
 //
 // Kernel.  D[rho][j] = sum_K A[rho][K] B[j][K], K = (re, im) of 32 nodes; a
 // CTA takes 128 rows of g (A) and 16 phase rows (B: rows j < 16 give the real
@@ -65,7 +66,7 @@ constexpr int MAX_NB = 1024;                   // blocks of a row
 constexpr int EPI_WARPS = 16, NT = 32 * (EPI_WARPS + 2);
 constexpr int EK = TK * 4 / EPI_WARPS;           // phase rows of an epilogue warp
 constexpr int TMEM_COLS = 512, ACC = 256;      // columns of one set of accumulators, one diagonal in 32
-constexpr int MARGIN = 8;
+constexpr int MARGIN = 9;
 
 // A form of the contraction: ND digits a value, NA A slots in the ring, SUB
 // scale blocks in the 32 nodes of a row of B.

@@ -103,8 +103,8 @@ def test_far_field_2d_holds_one_set_of_operands(csff):
 def test_far_field_work_counts_the_tiles_of_the_contraction_that_ran(csff):
     """Rows 0-31 live in the first of four blocks, the others in the last: every
     double-float tile (32 rows) keeps one block of four, the digit form's one tile
-    of 128 rows two.  At k = 3 the phases vary too much over a block for digits."""
-    for k, fraction in ((0.5, 0.5), (3.0, 0.25)):
+    of 128 rows two.  At k = 6 the phases vary too much over a block for digits."""
+    for k, fraction in ((0.5, 0.5), (6.0, 0.25)):
         prob = W.problem(2, 129, 10.0, math.pi / 6, k, [W.gauss(1.0, 1e6)])
         plan = csff.Plan(prob, {"smoother": "jacobi", "nu1": 1, "nu2": 1, "coarsest_n": 5, "rel_tol": 1e-8,
                                 "precision": "fp64"})
