@@ -214,8 +214,13 @@ csff_status csff_far_field(csff_plan* plan, int n_rhs, const double* eta_host, c
 
 /* Arithmetic of the far-field contraction (eq. FFmap; the paper leaves the
    quadrature's arithmetic open, Sec. 4).
-   CSFF_FF_FP64 (default): FP64-class throughout (2D stage 1 in double-float
-     arithmetic on the FP32 pipes, FP64 where the operand ranges need it).
+   CSFF_FF_FP64 (default): FP64-class throughout.  The contractions run on the
+     tensor cores where the phases vary slowly over a block of nodes: both
+     operands are cut into 8-bit digits whose products add up exactly (2D: the
+     first stage, 3D: z and y).  Elsewhere 2D stage 1 runs in double-float
+     arithmetic on the FP32 pipes, and FP64 kernels where the operands' ranges
+     need them.  A wait inside the digit kernel that runs out makes the FP64
+     kernels form the map, on the device and within the call.
    CSFF_FF_TC_BF16X4: 3D plans evaluate the z-contraction (the largest stage)
      on the tensor cores: each operand split into four BF16 terms (32
      significant bits), the ten products of terms i, j with i + j <= 3
@@ -223,8 +228,8 @@ csff_status csff_far_field(csff_plan* plan, int n_rhs, const double* eta_host, c
      across them; F then carries an absolute error of about 2^-26 times
      sum_j |term_j| per angle.  The library falls back to FP64 on the device
      when an operand is not finite or its exponent range is too wide.  2D plans
-     are unaffected.  A wait inside the tensor-core kernel that runs out makes
-     csff_far_field return CSFF_ERR_TIMEOUT.
+     are unaffected.  In this mode a wait inside the tensor-core kernel that runs
+     out makes csff_far_field return CSFF_ERR_TIMEOUT.
    Errors: CSFF_ERR_INVALID_ARG for an unknown mode. */
 enum { CSFF_FF_FP64 = 0, CSFF_FF_TC_BF16X4 = 1 };
 csff_status csff_plan_set_far_field_mode(csff_plan* plan, int mode);
@@ -243,9 +248,8 @@ csff_status csff_far_field_work(csff_plan* plan, double* executed);
    extra_arrivals = 1 makes the next far fields' contraction wait for an arrival
    that never comes, so its waits run out after wait_ms milliseconds (0 = the
    default limit of 500) and the FP64 kernels form the map instead; 0 restores
-   normal runs.  *gave_up (host, may be NULL)
-   receives 1 if a wait of the plan's last far field ran out, else 0, which
-   synchronises the plan's stream.  Errors: CSFF_ERR_INVALID_ARG, CSFF_ERR_CUDA. */
+   normal runs.  *gave_up (host, may be NULL) receives 1 if a wait of the plan's
+   last far field ran out, else 0, which synchronises the plan's stream.  Errors: CSFF_ERR_INVALID_ARG, CSFF_ERR_CUDA. */
 csff_status csff_far_field_debug_waits(csff_plan* plan, int extra_arrivals, int wait_ms, int* gave_up);
 
 /* ---- user coefficients and right-hand sides (Sec. 5.2-5.3) ---------------
