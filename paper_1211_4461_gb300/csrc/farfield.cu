@@ -19,6 +19,7 @@
 #include <algorithm>
 #include <cmath>
 #include <map>
+#include <type_traits>
 #include <vector>
 
 #include "csff_internal.h"
@@ -222,6 +223,7 @@ __device__ __forceinline__ bool df_selected(const int* __restrict__ spread) {
 __device__ __forceinline__ bool digits_selected(const int* __restrict__ spread) {
   return spread[0] < DF_NONFINITE && spread[1] < DF_NONFINITE && spread[2] <= digits::MARGIN;
 }
+__device__ __forceinline__ bool seven_digits(const int* __restrict__ spread) { return spread[2] <= digits::MARGIN_7; }
 
 __global__ void __launch_bounds__(256) k_ff_stage1(const double2* __restrict__ X, int M,
                                                    const double2* __restrict__ G, int N, int K,
@@ -472,17 +474,16 @@ __device__ __forceinline__ void split_row(double2 x, int eb, long long o, float4
 // one warp: the digits of a block of a row for k_ff_digits, in its tile.  PHASE:
 // the two rows (P_re, -P_im), (P_im, P_re) of a phase row in tiles of TK; else a row
 // of g, tiles of TM.
-template <bool PHASE>
+template <bool PHASE, int N>
 __device__ __forceinline__ void cut_row(double2 x, int e, int row, int b, int nb, unsigned char* __restrict__ out) {
   using namespace digits;
-  using F = Form2;
-  constexpr int ND = F::ND, B_SET = F::B_SET, TR = PHASE ? TK : TM;
+  constexpr int TR = PHASE ? TK : TM;
   const int lane = threadIdx.x & 31, r = row % TR, o = (lane & 3) * 4;
-  uint32_t dig[ND];
-  cut<ND>(fixed<F::BITS>(x.x, e), fixed<F::BITS>(x.y, e), dig);
-  unsigned char* tile = out + ((long long)(row / TR) * nb + b) * (PHASE ? B_SET : ND * A_DIG);
+  uint32_t dig[N];
+  cut<N>(fixed<N>(x.x, e), fixed<N>(x.y, e), dig);
+  unsigned char* tile = out + ((long long)(row / TR) * nb + b) * (N * (PHASE ? B_DIG : A_DIG));
 #pragma unroll
-  for (int s = 0; s < ND; ++s) {
+  for (int s = 0; s < N; ++s) {
     if (PHASE) {
       *reinterpret_cast<uint32_t*>(tile + s * B_DIG + sw(r, lane >> 2) + o) = neg_hi(dig[s]);
       *reinterpret_cast<uint32_t*>(tile + s * B_DIG + sw(TK + r, lane >> 2) + o) = swap_pair(dig[s]);
@@ -512,9 +513,12 @@ __global__ void __launch_bounds__(256) k_operands(Rows X, Rows G, int m, const i
     const bool in = row < n;
     const double2 x = in && i < m ? (phase ? X.v : G.v)[(long long)row * m + i] : make_double2(0, 0);
     const int e = in ? (phase ? X.ev : G.ev)[(long long)row * nb + b] : 0;
-    if (dig) {
-      if (phase) cut_row<true>(x, e, row, b, nb, xop);
-      else cut_row<false>(x, e, row, b, nb, gop);
+    if (dig && seven_digits(spread)) {
+      if (phase) cut_row<true, 7>(x, e, row, b, nb, xop);
+      else cut_row<false, 7>(x, e, row, b, nb, gop);
+    } else if (dig) {
+      if (phase) cut_row<true, digits::ND>(x, e, row, b, nb, xop);
+      else cut_row<false, digits::ND>(x, e, row, b, nb, gop);
     } else {
       float4* const vdf = reinterpret_cast<float4*>(phase ? xop : gop);
       const long long o = ((long long)row * nb + b) * DKB + lane;
@@ -777,12 +781,12 @@ __global__ void k_cut_phase3(const double2* __restrict__ v, const int* __restric
 #pragma unroll
   for (int o = 8; o > 0; o >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
   if (row < nrows && (lane & 15) == 0) ev[((long long)row * nb + b) * F::SUB + (lane >> 4)] = block_scale(e);
-  uint32_t dig[F::ND];
-  cut<F::ND>(fixed<F::BITS>(x.x, e), fixed<F::BITS>(x.y, e), dig);
+  uint32_t dig[ND];
+  cut(fixed(x.x, e), fixed(x.y, e), dig);
   const int r = row % TK, o = (lane & 3) * 4;
-  unsigned char* tile = out + ((long long)(row / TK) * nb + b) * F::B_SET;
+  unsigned char* tile = out + ((long long)(row / TK) * nb + b) * B_SET;
 #pragma unroll
-  for (int s = 0; s < F::ND; ++s) {
+  for (int s = 0; s < ND; ++s) {
     *reinterpret_cast<uint32_t*>(tile + s * B_DIG + sw(r, lane >> 2) + o) = neg_hi(dig[s]);
     *reinterpret_cast<uint32_t*>(tile + s * B_DIG + sw(TK + r, lane >> 2) + o) = swap_pair(dig[s]);
   }
@@ -810,14 +814,14 @@ __global__ void __launch_bounds__(digits::TM) k_cut_field3(const double2* __rest
   unsigned char* tile = out + (xt * nbs + sb) * (F::A_SLOTS * A_DIG);
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
-    uint32_t d[8][F::ND];
+    uint32_t d[8][ND];
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
       const double2 x = 8 * h + k < nz ? p[(long long)(8 * h + k) * ncol] : make_double2(0, 0);
-      cut<F::ND>(fixed<F::BITS>(x.x, e), fixed<F::BITS>(x.y, e), d[k]);
+      cut(fixed(x.x, e), fixed(x.y, e), d[k]);
     }
 #pragma unroll
-    for (int s = 0; s < F::ND; ++s) {
+    for (int s = 0; s < ND; ++s) {
       unsigned char* slot = tile + (s >> 1) * A_DIG;
       const int c = 4 * (s & 1) + 2 * h;
       *reinterpret_cast<uint4*>(slot + sw(r, c)) = make_uint4(d[0][s], d[1][s], d[2][s], d[3][s]);
@@ -834,8 +838,9 @@ __global__ void __launch_bounds__(digits::TM) k_cut_field3(const double2* __rest
 // which else returns at once, then forms T again.
 // Bound by the issue of the MMAs (114 clocks each where the tensor core needs
 // 64; 150 from one thread in a divergent branch) and by the last wave: 184 tiles
-// on 152 SMs at 1025^2.  361 phase rows x 1023 x 1023, every block kept: 125 us,
-// 18 us for cutting the operands; the double-float contraction takes 538.
+// on 152 SMs at 1025^2.  361 phase rows x 1023 x 1023, every block kept: 127 us with
+// seven digits, 150 with eight, 18 us for cutting the operands; the double-float
+// contraction takes 538.
 //
 // 3D form: T1[t][col] of the z contraction, every block kept (skip and spread
 // null), columns from tile0 TM on, in chunks whose operands stay in L2.  A block
@@ -853,8 +858,9 @@ __global__ void __launch_bounds__(digits::NT, 1)
                 const unsigned char* __restrict__ skip, int skip_tiles, double2* __restrict__ T, int* __restrict__ err,
                 int tile0, const int* __restrict__ field, const int* __restrict__ map, FFWaits waits) {
   using namespace digits;
-  constexpr int ND = F::ND, DG = F::DG, NA = F::NA, SUB = F::SUB, B_SET = F::B_SET, OFF_BAR = F::OFF_BAR, OFF_ACT = F::OFF_ACT;
+  constexpr int NA = F::NA, SUB = F::SUB, OFF_BAR = F::OFF_BAR, OFF_ACT = F::OFF_ACT;
   if (spread && !digits_selected(spread)) return;      // another kernel takes this launch
+  const int n_dig = SUB == 1 && seven_digits(spread) ? 7 : ND;
   extern __shared__ __align__(1024) unsigned char dsm_raw[];
   unsigned char* base = dsm_raw + ((1024 - (saddr(dsm_raw) & 1023)) & 1023);
   const uint32_t sbase = saddr(base), bars = sbase + OFF_BAR;
@@ -921,15 +927,15 @@ __global__ void __launch_bounds__(digits::NT, 1)
       const bool first = idx % SUB == 0;
       if (first && kb >= 2) ok = bar_wait(b_empty + 8 * p, (uint32_t)((kb >> 1) - 1) & 1u, abort, waits.ns);
       if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
-      const unsigned char* src = Ad + (((long long)xt * nb + b) * SUB + idx % SUB) * (F::A_SLOTS * A_DIG);
+      const int slots = n_dig / SUB, set = n_dig * B_DIG;          // a block's A slots, bytes of its B set
+      const unsigned char* src = Ad + (((long long)xt * nb + b) * SUB + idx % SUB) * (slots * A_DIG);
       if (first) {
         if (elect_one())
-          bulk_load(sbase + NA * A_DIG + p * B_SET, Bd + ((long long)blockIdx.y * nb + b) * B_SET, B_SET, b_full + 8 * p);
+          bulk_load(sbase + NA * A_DIG + p * B_SET, Bd + ((long long)blockIdx.y * nb + b) * set, set, b_full + 8 * p);
         ++ib;
       }
       __syncwarp();
-#pragma unroll
-      for (int s = 0; s < F::A_SLOTS; ++s) {
+      for (int s = 0; s < slots; ++s) {
         if (ia >= NA) ok = ok && bar_wait(a_empty + 8 * slot, eph, abort, waits.ns);
         if (__all_sync(0xffffffffu, ok)) {
           if (elect_one()) bulk_load(sbase + slot * A_DIG, src + s * A_DIG, A_DIG, a_full + 8 * slot);
@@ -960,47 +966,51 @@ __global__ void __launch_bounds__(digits::NT, 1)
     const uint32_t tm = __reduce_max_sync(0xffffffffu, tmem);
     // FP32 accumulator, BF16 A and B, both K-major, M = 128; N per digit of A
     constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TM >> 4) << 24);
-    int slot = 0;
-    uint32_t aph = 0;
     bool ok = true;
-    for (int idx = 0; idx < n; ++idx) {
-      const int p = idx & 1;
-      if (idx >= 2) ok = bar_wait(acc_empty + 8 * p, (uint32_t)((idx >> 1) - 1) & 1u, abort, waits.ns);
-      const int kb = idx / SUB, pb = kb & 1;             // B's buffer
-      ok = ok && bar_wait(b_full + 8 * pb, (uint32_t)(kb >> 1) & 1u, abort, waits.ns);
-      if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
-      const uint32_t sB = sbase + NA * A_DIG + pb * B_SET + (SUB - 1) * 64 * (idx & 1);
+    auto issue = [&](auto digits_) {
+      constexpr int N = decltype(digits_)::value;
+      int slot = 0;
+      uint32_t aph = 0;
+      for (int idx = 0; idx < n; ++idx) {
+        const int p = idx & 1;
+        if (idx >= 2) ok = bar_wait(acc_empty + 8 * p, (uint32_t)((idx >> 1) - 1) & 1u, abort, waits.ns);
+        const int kb = idx / SUB, pb = kb & 1;             // B's buffer
+        ok = ok && bar_wait(b_full + 8 * pb, (uint32_t)(kb >> 1) & 1u, abort, waits.ns);
+        if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
+        const uint32_t sB = sbase + NA * A_DIG + pb * B_SET + (SUB - 1) * 64 * (idx & 1);
 #pragma unroll
-      for (int s = 0; s < ND; ++s) {
-        if (s % SUB == 0) ok = ok && bar_wait(a_full + 8 * slot, aph, abort, waits.ns);
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        constexpr int TKK = 2 * TK;
-        const uint32_t nd = (uint32_t)(TKK * min(ND, DG - s));       // columns: digits of B for the kept diagonals
-        const uint32_t d = tm + (uint32_t)(p * ACC + TKK * s), sA = sbase + slot * A_DIG + 64 * (s % SUB);
-        if (__all_sync(0xffffffffu, ok) && elect_one()) {
+        for (int s = 0; s < N; ++s) {
+          if (s % SUB == 0) ok = ok && bar_wait(a_full + 8 * slot, aph, abort, waits.ns);
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          constexpr int TKK = 2 * TK;
+          const uint32_t nd = (uint32_t)(TKK * min(N, ND - s));        // columns: digits of B for the kept diagonals
+          const uint32_t d = tm + (uint32_t)(p * ACC + TKK * s), sA = sbase + slot * A_DIG + 64 * (s % SUB);
+          if (__all_sync(0xffffffffu, ok) && elect_one()) {
 #pragma unroll
-          for (int kk = 0; kk < 4 / SUB; ++kk) {
-            const bool more = DG > ND && s == DG - ND;             // its last columns start a diagonal
-            const uint32_t n1 = more && kk == 0 ? nd - TKK : nd;
-            mma(d, desc(sA + 32 * kk), desc(sB + 32 * kk), idesc | ((n1 >> 3) << 17), (s > 0 || kk > 0) ? 1u : 0u);
-            if (more && kk == 0)
-              mma(d + n1, desc(sA), desc(sB + (n1 / TKK) * B_DIG), idesc | ((uint32_t)(TKK >> 3) << 17), 0u);
+            for (int kk = 0; kk < 4 / SUB; ++kk) {
+              const bool more = N < ND && s == ND - N && kk == 0;      // the last of them start a diagonal
+              const uint32_t n1 = more ? nd - TKK : nd;
+              mma(d, desc(sA + 32 * kk), desc(sB + 32 * kk), idesc | ((n1 >> 3) << 17), (s > 0 || kk > 0) ? 1u : 0u);
+              if (more) mma(d + n1, desc(sA), desc(sB + (n1 / TKK) * B_DIG), idesc | ((uint32_t)(TKK >> 3) << 17), 0u);
+            }
+            if (s % SUB == SUB - 1) commit(a_empty + 8 * slot);
           }
-          if (s % SUB == SUB - 1) commit(a_empty + 8 * slot);
+          __syncwarp();
+          if (s % SUB == SUB - 1 && ++slot == NA) {
+            slot = 0;
+            aph ^= 1u;
+          }
+        }
+        if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
+        if (elect_one()) {
+          if (idx % SUB == SUB - 1) commit(b_empty + 8 * pb);
+          commit(acc_full + 8 * p);
         }
         __syncwarp();
-        if (s % SUB == SUB - 1 && ++slot == NA) {
-          slot = 0;
-          aph ^= 1u;
-        }
       }
-      if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
-      if (elect_one()) {
-        if (idx % SUB == SUB - 1) commit(b_empty + 8 * pb);
-        commit(acc_full + 8 * p);
-      }
-      __syncwarp();
-    }
+    };
+    if (SUB == 1 && n_dig == 7) issue(std::integral_constant<int, 7>());
+    else issue(std::integral_constant<int, ND>());
     if (!ok) {
       int never = 0;
       if (elect_one()) commit(fin);
@@ -1056,9 +1066,9 @@ __global__ void __launch_bounds__(digits::NT, 1)
         // one part at a time: both take more registers than 18 warps have
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
-          uint32_t v[DG][EK];
+          uint32_t v[ND][EK];
 #pragma unroll
-          for (int d = 0; d < DG; ++d) CSFF_TMEM_LD4(v[d], tl + (uint32_t)(p * ACC + 2 * TK * d + TK * c));
+          for (int d = 0; d < ND; ++d) CSFF_TMEM_LD4(v[d], tl + (uint32_t)(p * ACC + 2 * TK * d + TK * c));
           asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
           if (c == 1) {
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -1067,18 +1077,18 @@ __global__ void __launch_bounds__(digits::NT, 1)
           }
 #pragma unroll
           for (int j = 0; j < EK; ++j) {
-            float q[DG];
+            float q[ND];
 #pragma unroll
-            for (int d = 0; d < DG; ++d) q[d] = __uint_as_float(v[d][j]);
+            for (int d = 0; d < ND; ++d) q[d] = __uint_as_float(v[d][j]);
             S[c][j] += fixed_to_double(join_fixed(q), es[j]);
           }
         }
       } else {
-        uint32_t v[2][DG][EK];
+        uint32_t v[2][ND][EK];
 #pragma unroll
         for (int c = 0; c < 2; ++c)
 #pragma unroll
-          for (int d = 0; d < DG; ++d) CSFF_TMEM_LD4(v[c][d], tl + (uint32_t)(p * ACC + 2 * TK * d + TK * c));
+          for (int d = 0; d < ND; ++d) CSFF_TMEM_LD4(v[c][d], tl + (uint32_t)(p * ACC + 2 * TK * d + TK * c));
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncwarp();
@@ -1093,9 +1103,9 @@ __global__ void __launch_bounds__(digits::NT, 1)
           E[2 * j + 1] = En1;
 #pragma unroll
           for (int c = 0; c < 2; ++c) {
-            float2 q[DG], h, l, t, e;
+            float2 q[ND], h, l, t, e;
 #pragma unroll
-            for (int d = 0; d < DG; ++d)
+            for (int d = 0; d < ND; ++d)
               q[d] = make_float2(__uint_as_float(v[c][d][2 * j]), __uint_as_float(v[c][d][2 * j + 1]));
             join(q, h, l);
             two_sum(__fmul2_rn(H[c][j], fa), __fmul2_rn(h, fs), t, e);
@@ -1610,7 +1620,7 @@ static int dig3_chunk(int m, int T) {
 static cudaError_t dig3_ensure(FFBuffers& B, int m, int T, int chunk, csff_plan* P) {
   using F = digits::Form3;
   const size_t nb = (m + digits::KB - 1) / digits::KB, kt = (T + digits::TK - 1) / digits::TK;
-  cudaError_t e = ensure((void**)&B.dxop, B.xop, kt * nb * F::B_SET, P);
+  cudaError_t e = ensure((void**)&B.dxop, B.xop, kt * nb * digits::B_SET, P);
   if (e == cudaSuccess)
     e = ensure((void**)&B.dgop, B.gop, (size_t)chunk * nb * F::SUB * F::A_SLOTS * digits::A_DIG, P);
   if (e == cudaSuccess)
@@ -1660,7 +1670,7 @@ static size_t dig3_b_ints(const YTiles& y, int m, int T) {
 static cudaError_t dig3_ensure_b(FFBuffers& B, const YTiles& y, int m, int T, csff_plan* P) {
   using F = digits::Form3;
   const size_t nb = (m + digits::KB - 1) / digits::KB, tiles = (m + digits::TM - 1) / digits::TM;
-  cudaError_t e = ensure((void**)&B.dxop, B.xop, y.field.size() * nb * F::B_SET, P);
+  cudaError_t e = ensure((void**)&B.dxop, B.xop, y.field.size() * nb * digits::B_SET, P);
   if (e == cudaSuccess)
     e = ensure((void**)&B.dgop, B.gop, T * tiles * nb * F::SUB * F::A_SLOTS * digits::A_DIG, P);
   if (e == cudaSuccess) e = ensure((void**)&B.dtce, B.tce, sizeof(int) * dig3_b_ints(y, m, T), P);
@@ -1960,10 +1970,10 @@ csff_status far_field_one(csff_plan* P, const double* eta_host, const double2* u
   const int gxt = (int)((R + digits::TM - 1) / digits::TM), gkt = (n_ux + digits::TK - 1) / digits::TK;
   const size_t xn = (size_t)n_ux * nbk * DKB, gn = (size_t)R * nbk * DKB, node = sizeof(float4) + sizeof(float2);
   bool dig = d == 2 && nbk <= digits::MAX_NB &&
-             ensure((void**)&B.dxop, B.xop, std::max(node * xn, (size_t)gkt * nbk * digits::Form2::B_SET), P) ==
+             ensure((void**)&B.dxop, B.xop, std::max(node * xn, (size_t)gkt * nbk * digits::B_SET), P) ==
                  cudaSuccess &&
              ensure((void**)&B.dgop, B.gop,
-                    std::max(node * gn, (size_t)gxt * nbk * digits::Form2::ND * digits::A_DIG), P) == cudaSuccess;
+                    std::max(node * gn, (size_t)gxt * nbk * digits::ND * digits::A_DIG), P) == cudaSuccess;
   if (!dig) {
     cudaGetLastError();
     if ((e = ensure((void**)&B.dxop, B.xop, node * xn, P)) != cudaSuccess ||

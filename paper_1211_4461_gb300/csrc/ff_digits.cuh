@@ -5,45 +5,48 @@
 //
 // Representation.  As in the double-float form, each row of either operand is
 // scaled by a power of two per block of 32 nodes, so |x'| < 1 there.  Then
-//   x' = sum_{s=1..7} d_s 2^-(8 s - 1) + r,   |d_s| <= 128,  |r| <= 2^-56,
-// digits balanced (round to nearest), stored as BF16 integers.  A product of two
-// digits is at most 2^14; a block's sum over 64 real terms (32 complex nodes)
-// and the at most 7 digit pairs (s, t) of one diagonal s + t = D stays below
-// 2^23, so the FP32 accumulators hold it exactly.  Diagonals D = 2..9 are kept (34
-// of the 49 pairs).  Cutting into slices whose products add up exactly is a
-// published method (Ozaki, Ogita, Oishi and Rump, Numer. Algorithms 59, 2012).
+//   x' = sum_{s=1..n} d_s 2^-(8 s - 1) + r,   |d_s| <= 128,  |r| <= 2^-8n,
+// n = 7 or 8, digits balanced (round to nearest), stored as BF16 integers.  A product
+// of two digits is at most 2^14; a block's sum over 64 real terms (32 complex nodes)
+// and the at most 8 digit pairs (s, t) of one diagonal s + t = D stays within
+// 2^23, so the FP32 accumulators hold it exactly.  Diagonals D = 2..9 are kept (36
+// of the 64 pairs of eight digits, 34 of seven's 49).  Cutting into slices whose
+// products add up exactly is a published method (Ozaki, Ogita, Oishi and Rump, Numer.
+// Algorithms 59, 2012).
 //
-// Error of a block, relative to the product 2^(ex + eg) of the two scales: five
-// pairs of at most 2^14 at 2^-78 are dropped for each of 64 real products (2^-55.7,
-// 2^-61 for digits of random signs), and the operands' remainders of up to
-// 2^-56 each enter 64 times (2^-49 at most; 2^-54.8 rms for dense blocks, less where
-// few values count).
+// Error of a block, relative to the product 2^(ex + eg) of the two scales: seven
+// (five) pairs of at most 2^14 at 2^-78 are dropped for each of 64 real products
+// (2^-55.2; 2^-61 for digits of random signs), and seven digits leave remainders of up
+// to 2^-56 (2^-54.8 rms for dense blocks, less where few values count).
 //
-// When it runs.  These errors are relative to the block maxima, so the kernel is
+// When it runs.  This error is relative to the block maxima, so the kernel is
 // taken when for every block that a tile keeps the scales ex + eg lie at most
 // MARGIN binades over L, the lower bound of the sum of the terms' magnitudes that
 // the skip kernel forms (-3 to 2 for constant phases, more as they vary over a block:
-// up to about k h sin(gamma) 32 = 5).  The line is where the error reaches the
-// double-float kernel's, which runs beyond it.  Both restated on the CPU on single
-// blocks against a longer sum, relative to the sum of the terms' magnitudes, by
-// margin, as binades of the rms error over the double-float kernel's (2^-48.5 to
-// 2^-45.7):
-//   fields                                margin 5     6     7     8     9     10
-//   random                                     -3.5  -3.3  -3.3  -3.2
-//   balanced against the phases                -4.1  -3.7  -3.0  -2.0  -1.4  -0.6
-//   falling three times as fast                -4.4  -3.7  -2.9  -1.9  -1.1  -0.6
-//   three nodes where the phase is smallest    -2.5  -2.2  -1.7  -0.9  +0.1  +0.7
-//   a single node there                        -2.0  -1.8  -1.5  -0.8  +0.1  +1.0
-// (with diagonals up to 8 and the line at 12 binades over a bound from single
-// nodes, as before, up to 3.9 binades larger.)
+// up to about k h sin(gamma) 32 = 9), with seven digits up to MARGIN_7 (4.5).  Up
+// to either line the error stays below the double-float kernel's, which runs beyond
+// the second.  Both restated on the CPU on single blocks against a longer sum,
+// relative to the sum of the terms' magnitudes, by margin, as binades of the rms
+// error over the double-float kernel's (2^-48.5 to 2^-45.7):
+//                          seven digits, margin 6    8     9     10   eight, 10    13    15    16    17
+//   random fields                          -3.3  -3.2                    -3.2  -3.0  -2.9  -2.9  -3.1
+//   balanced against the phases            -3.7  -2.0  -1.4  -0.6        -4.3  -3.7  -2.3  -1.5  -0.5
+//   falling three times as fast            -3.7  -1.9  -1.1  -0.6        -4.8  -3.6  -2.0  -0.9  +0.1
+//   three nodes at the smallest phase      -2.2  -0.9  +0.1  +0.7        -2.6  -2.4  -0.8  +0.1  +0.8
+//   a single node there                    -1.8  -0.8  +0.1  +1.0        -2.1  -1.9  -0.7  +0.3  +1.2
+// (Seven digits with diagonals up to 8 and the line at 12 binades over a bound from
+// single nodes, as before: up to 3.9 binades larger than the double-float kernel's.)
+// On whole maps (129^2, fields at the small end of the phases, 2 to 14 binades a
+// block) the eight digits lie 2^-50.3 of the terms from the FP64 contraction or less.
 //
 // Kernel.  D[rho][j] = sum_K A[rho][K] B[j][K], K = (re, im) of 32 nodes; a
 // CTA takes 128 rows of g (A) and 16 phase rows (B: rows j < 16 give the real
 // parts from (P_re, -P_im), 16 + j the imaginary parts from (P_im, P_re)).  The
 // 32 rows of digit t of B are rows [32 (t - 1), 32 t) of one operand, and
 // diagonal D accumulates in tensor-memory columns [32 (D - 2), 32 (D - 1)), so
-// one MMA of digit s of A against digits 1..8-s of B (N = 32 (8 - s)) adds to
-// the right diagonals: seven MMAs per 16 K values, each reading A once.
+// one MMA of digit s of A against digits 1..9-s of B (N = 32 (9 - s), at most all
+// there are) adds to the right diagonals: one MMA a digit per 16 K values, each
+// reading A once, and with seven digits one more where the last diagonal starts.
 // One thread streams digit tiles (16 KB, pre-swizzled in global memory) into a
 // ring with bulk copies, one issues the MMAs, sixteen warps read the two
 // alternating sets of accumulators and join them, all handing over through
@@ -66,31 +69,31 @@ constexpr int MAX_NB = 1024;                   // blocks of a row
 constexpr int EPI_WARPS = 16, NT = 32 * (EPI_WARPS + 2);
 constexpr int EK = TK * 4 / EPI_WARPS;           // phase rows of an epilogue warp
 constexpr int TMEM_COLS = 512, ACC = 256;      // columns of one set of accumulators, one diagonal in 32
-constexpr int MARGIN = 9;
+constexpr int MARGIN = 15, MARGIN_7 = 8;
 
-// A form of the contraction: ND digits a value, NA A slots in the ring, SUB
-// scale blocks in the 32 nodes of a row of B.
-//  2D: seven digits, one block, an A slot one digit of 32 nodes.
-//  3D (the z contraction): eight digits, two blocks, an A slot two digits of 16
-//  nodes; each block's diagonals fill a set of accumulators.
-template <int ND_, int NA_, int SUB_> struct Form {
-  static constexpr int ND = ND_, NA = NA_, SUB = SUB_;
-  static constexpr int DG = 8;                 // diagonals kept
-  static constexpr int BITS = 8 * ND - 1;      // fixed-point bits below the scale
-  static constexpr int A_SLOTS = ND / SUB;     // slots of a block
-  static constexpr int B_SET = ND * B_DIG;
+// A form of the contraction: NA A slots in the ring, SUB scale blocks in the 32 nodes
+// of a row of B.
+//  2D: one block, an A slot one digit of 32 nodes; seven or eight digits.
+//  3D (the z and y contractions): two blocks, an A slot two digits of 16 nodes, eight
+//  digits; each block's diagonals fill a set of accumulators.
+constexpr int ND = 8;                          // digits at most, and diagonals kept
+constexpr int B_SET = ND * B_DIG;
+template <int NA_, int SUB_> struct Form {
+  static constexpr int NA = NA_, SUB = SUB_;
+  static constexpr int A_SLOTS = ND / SUB;     // slots of a block of eight digits
   static constexpr int OFF_BAR = NA * A_DIG + 2 * B_SET, OFF_ACT = OFF_BAR + 512;
   static constexpr int SMEM = OFF_ACT + MAX_NB * 2 + 1024;
-  static_assert(SMEM <= 227 * 1024 && ND % SUB == 0 && ND <= DG && 2 * TK * DG <= ACC, "shared and tensor memory");
+  static_assert(SMEM <= 227 * 1024 && ND % SUB == 0 && 2 * TK * ND <= ACC, "shared and tensor memory");
 };
-using Form2 = Form<7, 10, 1>;
-using Form3 = Form<8, 9, 2>;
+using Form2 = Form<9, 1>;
+using Form3 = Form<9, 2>;
 
 // 128-byte-swizzled K-major row: byte offset of 16-byte chunk c of row r
 __device__ __forceinline__ int sw(int r, int c) { return (r >> 3) * 1024 + (r & 7) * 128 + ((c ^ (r & 7)) << 4); }
 
-// x 2^(BITS - e) rounded to an integer, |x| < 2^e, from the IEEE fields
-template <int BITS> __device__ __forceinline__ long long fixed(double x, int e) {
+// x 2^(8 N - 1 - e) rounded to an integer, |x| < 2^e, from the IEEE fields
+template <int N = ND> __device__ __forceinline__ long long fixed(double x, int e) {
+  constexpr int BITS = 8 * N - 1;
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
   const int E = (int)((b >> 52) & 0x7ff);
   const long long m = (long long)((b & bits::MANT_MASK) | (E ? 1ull << 52 : 0));
@@ -118,14 +121,14 @@ __device__ __forceinline__ int block_scale(int e) { return e > 1024 ? NONFINITE 
 __device__ __forceinline__ float byte_digit(unsigned v, int byte) {
   return __uint_as_float(__byte_perm(v, 0x4B000000u, 0x7440 | byte)) - 8388736.f;      // 2^23 + 128
 }
-template <int ND> __device__ __forceinline__ void cut(long long p, long long q, uint32_t (&dig)[ND]) {
-  constexpr int SH = 8 * (ND - 1);
+template <int N = ND> __device__ __forceinline__ void cut(long long p, long long q, uint32_t (&dig)[N]) {
+  constexpr int SH = 8 * (N - 1);
   constexpr unsigned long long LOW = (1ull << SH) - 1, HALF = 0x8080808080808080ull & LOW;
   const unsigned long long lp = ((unsigned long long)p & LOW) + HALF, lq = ((unsigned long long)q & LOW) + HALF;
   auto pack = [](float a, float b) { return __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x7632); };
 #pragma unroll
-  for (int s = 1; s < ND; ++s) {
-    const int byte = ND - 1 - s;
+  for (int s = 1; s < N; ++s) {
+    const int byte = N - 1 - s;
     const unsigned a = (unsigned)(byte < 4 ? lp : lp >> 32), b = (unsigned)(byte < 4 ? lq : lq >> 32);
     dig[s] = pack(byte_digit(a, byte & 3), byte_digit(b, byte & 3));
   }
@@ -207,20 +210,21 @@ __device__ __forceinline__ void two_sum(float2 x, float2 y, float2& t, float2& e
 __device__ __forceinline__ float pow2_or_0(int d) { return __int_as_float(max(d + 127, 0) << 23); }
 __device__ __forceinline__ float2 both(float a) { return make_float2(a, a); }
 
-// h + l = sum_{d=0..7} p[d] 2^-8d: the four leading terms by exact sums (their
-// digit sums reach 2^23, eight bits apart), the four trailing ones, whose
-// roundings lie below 2^-55 of the scale, by multiply-adds
+// h + l = sum_{d=0..7} p[d] 2^-8d: the six leading terms by exact sums (their digit
+// sums reach 2^23, eight bits apart), the two trailing ones, whose roundings lie
+// below 2^-49 of p[0]'s unit, the size of the last bits of a value 15 binades under
+// the scales, by multiply-adds
 __device__ __forceinline__ void join(const float2 (&p)[8], float2& h, float2& l) {
   const float2 w = both(0x1p-8f);
-  float2 q = __ffma2_rn(p[7], w, p[6]);
-  q = __ffma2_rn(q, w, p[5]);
-  q = __ffma2_rn(q, w, p[4]);
-  float2 e3, e2, e1, t;
-  two_sum(p[3], __fmul2_rn(q, w), t, e3);
-  two_sum(p[2], __fmul2_rn(t, w), t, e2);
-  two_sum(p[1], __fmul2_rn(t, w), t, e1);
+  float2 t = __ffma2_rn(p[7], w, p[6]), e, c;
+  two_sum(p[5], __fmul2_rn(t, w), t, c);
+#pragma unroll
+  for (int d = 4; d >= 1; --d) {
+    two_sum(p[d], __fmul2_rn(t, w), t, e);
+    c = __ffma2_rn(c, w, e);
+  }
   two_sum(p[0], __fmul2_rn(t, w), h, l);
-  l = __fadd2_rn(l, __fmul2_rn(__ffma2_rn(__ffma2_rn(e3, w, e2), w, e1), w));
+  l = __fadd2_rn(l, __fmul2_rn(c, w));
 }
 
 // 3D form: sum_{d=0..7} p[d] 2^(43 - 8 d) as an integer (the block's sum times

@@ -57,7 +57,7 @@ def test_nan_direction_3d_gives_nan(csff, component):
 # digit form's line.  The contraction against the FP64 one of the same call (the
 # waits made to run out), whose rounding is 2^-52: no further apart than the
 # double-float form's rms error of 2^-48
-@pytest.mark.parametrize("var", [2.0, 4.5, 5.5, 6.5, 8.3, 9.5])
+@pytest.mark.parametrize("var", [2.0, 4.5, 6.5, 8.3, 9.5, 11.0, 12.5, 14.0])
 @pytest.mark.parametrize("nodes", [1, 3, 32])
 def test_far_field_2d_of_unbalanced_blocks(csff, var, nodes):
     n, R, g = 129, 10.0, math.pi / 6
@@ -77,7 +77,7 @@ def test_far_field_2d_of_unbalanced_blocks(csff, var, nodes):
     F64, E64 = _far(plan, eta, u, al)
     digits = plan.debug_far_field_waits(0)
     plan.close()
-    assert digits or var > 4.5
+    assert digits or var > 9.5
     tn, e2 = O.far_field(O.problem_from_dict(prob), u, eta[0], al, return_terms_norm=True)[:0:-1]
     diff = np.abs(F * 2.0 ** (E.astype(np.float64) - e2) - F64 * 2.0 ** (E64.astype(np.float64) - e2)) / tn
     assert np.sqrt(np.mean(diff ** 2)) <= 2.0 ** -48
@@ -95,7 +95,7 @@ def test_far_field_2d_holds_one_set_of_operands(csff):
     rows, nb = len(np.unique(al[:, 0])), (m + 31) // 32
     tiles_x, tiles_g = (rows + 15) // 16, (m + 127) // 128
     field = 16 * m * m + 16 * m * (rows + 2 * ang) + 16 * m * rows           # g, phase tables, sums
-    digits = nb * (tiles_x * 7 * 4096 + tiles_g * 7 * 16384)
+    digits = nb * (tiles_x * 8 * 4096 + tiles_g * 8 * 16384)
     words = 8 * nb * (rows + m) + tiles_x * ((m + 31) // 32) * nb + 8 * 3 * (rows + ang) + 4 * ang
     assert grown <= field + digits + words
 
