@@ -48,7 +48,6 @@ def _peaks():
 
 # FP64 FMA throughput of this part, measured with an FMA-loop kernel
 # (0.599e12 DFMA/s over 152 SMs; 2 flops per FMA).
-FP64_PEAK_TFLOPS = 1.198
 # DRAM bytes (read + write) per launch of the dominant kernels, from one ncu
 # capture of the current kernels on this workload (None when no capture of
 # the current kernels exists): the fused FP32 V(1,1) tiles (all levels, and those
@@ -556,7 +555,7 @@ def run_ours(args, rank, world, local_rank):
             runner.close()
         line["cpu_baseline"] = cpu_baseline_record(r, runner.workers)
     if args.details:
-        with open(args.details, "w") as f:
+        with open(os.path.join(ROOT, args.details), "w") as f:
             json.dump(line, f, indent=1)
     print(json.dumps(compact_line(line, args.details)), flush=True)
 
@@ -872,7 +871,6 @@ def measure_3d(csff, torch, dev, stream, flush):
             out[f"ff_{name}_ms_per_16_maps"] = ff_ms
             out[f"ff_{name}_stageA_ms_per_map"] = prof["ms"] / max(1, nr)
             out[f"ff_{name}_stageA_tflops"] = prof["alg_flops"] / (prof["ms"] * 1e-3) / 1e12 if prof["ms"] else 0.0
-    out["ff_fp64_stageA_fp64_frac"] = out["ff_fp64_stageA_tflops"] / FP64_PEAK_TFLOPS
     rel = np.linalg.norm(maps["tc_bf16x4"] - maps["fp64"], axis=1) / np.linalg.norm(maps["fp64"], axis=1)
     out["tc_vs_fp64_rel_l2"] = {"max": float(rel.max()), "median": float(np.median(rel)),
                                 "maps_below_1e-5": int((rel <= 1e-5).sum())}
@@ -1285,8 +1283,8 @@ def main():
     ap.add_argument("--no-cpu-baseline", dest="cpu_baseline", action="store_false")
     ap.add_argument("--no-variants", dest="variants", action="store_false",
                     help="skip the plain-FP64 and batched comparison runs")
-    ap.add_argument("--details", default=os.path.join(ROOT, "bench_details.json"),
-                    help="file for the whole record (rooflines, per-map solves, every variant); empty: none")
+    ap.add_argument("--details", default="bench_details.json",
+                    help="file (from this folder) for the whole record: rooflines, per-map solves, every variant; empty: none")
     ap.add_argument("--ks", default="", help="comma-separated subset of the wavenumbers (profiling runs)")
     ap.add_argument("--inner-cycles", type=int, default=INNER_CYCLES,
                     help="FP32 V-cycles per refinement step of the mixed solve")
