@@ -560,8 +560,8 @@ __device__ __forceinline__ void batch_body(const BArgs& A, unsigned char* smem, 
 // 64 registers a thread, four CTAs an SM (with the learned step, whose operands
 // leave shared memory for three, 80; the autotuner picks between one and the
 // occupancy maximum).  32 instances of 129^2 to 1025^2: 20.4 ms at three CTAs, 18.2
-// at four; in an earlier build 20.2 at three, 19.1 at four, 18.6 at five of 48 registers, whose spills cost 24 instances of up to
-// 257^2 more (4.24 ms against 3.93).  LEARNED: the
+// at four (same build); five of 48 registers took 18.6 against 19.1, but their
+// spills cost 24 instances of up to 257^2 more (4.24 ms against 3.93).  LEARNED: the
 // learned step ends every cycle; each CTA holds the network's weight operands
 // for the whole launch, and the activation planes share the tiles' shared
 // memory.  The network runs on the warp-level MMA instructions: the occupancy

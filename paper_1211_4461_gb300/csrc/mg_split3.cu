@@ -10,7 +10,7 @@
 // the other), HP slots a row (a multiple of four; slots outside the domain are
 // zero).  The six neighbours of slot j lie in the other colour's array: slots
 // j + o - 1 and j + o of the same row, slot j of the rows above, below, before
-// and behind.  A thread takes two slots of a row (one 16-byte access in FP32).
+// and behind.  A thread takes two slots of a row (one 16-byte access).
 //
 // A cycle has four passes per level instead of eight:
 //  - the red half sweep from zero, u = d^{-1} b, is folded into the full
@@ -27,11 +27,12 @@
 //    adds the interpolated correction's neighbour sum, formed from the coarse
 //    values directly;
 //  - the last black half sweep writes both colours in natural order.
-// 257^3 FP32 cycle through the public call (natural order in and out): 362 us,
-// 670 with interleaved colours.  A half sweep of 255^3 39 us (the copy rate), 53
-// with the black change, 61 prolonging, 59 into natural order (80 before, 125 with
-// the prolongation's pass); the 38-point full weighting 32 us, residual and full
-// weighting 123 before.
+// 257^3 FP32 cycle through the public call (natural order in and out): 358 us,
+// 670 with interleaved colours.  Passes of 255^3 from a cold L2 (share of DRAM's
+// peak): half sweep 42 us (75 %), with the black change 55 (82 %), prolonging 64
+// (52 %), into natural order 57 (66 %); the 38-point full weighting 37 (28 %: load
+// latency).  Interleaved: 80 a half sweep, 125 with the prolongation's pass, 123 for
+// residual and full weighting.
 #include "csff_internal.h"
 
 #include <cmath>
